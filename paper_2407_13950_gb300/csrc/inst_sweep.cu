@@ -1,7 +1,9 @@
 // Explicit instantiation of the sweep kernels (the families: one thread per fiber, a lane pair
-// per fiber and, for 2-level shapes, a lane quad per fiber) for one (levels, subsystems) shape,
+// per fiber and, for 2-level shapes, a lane quad per fiber) and of the quadrature kernel for one
+// (levels, subsystems) shape,
 // selected with -DMSQOC_L=<levels> -DMSQOC_Q=<subsystems>; this file is compiled once per
 // supported shape.
+#include "msqoc_quad.cuh"
 #include "msqoc_sweep.cuh"
 #include "msqoc_sweep_pair.cuh"
 
@@ -102,6 +104,23 @@ cudaError_t MSQOC_CAT(launch_sweep, MSQOC_L, MSQOC_Q)(const SweepArgs& a, int nt
     if (a.pair == 2) return launch_family<2>(a, ntiles, s);
 #endif
     return cudaErrorInvalidValue;
+}
+
+template <bool SPLIT>
+static cudaError_t launch_quad_one(const QuadArgs& a, int blocks, int nprob, cudaStream_t s) {
+    auto kern = k_quad<MSQOC_L, MSQOC_Q, SPLIT>;
+    constexpr size_t smem = quad_smem<MSQOC_L, MSQOC_Q>();
+    if constexpr (smem > SMEM_DEFAULT_LIMIT) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (e != cudaSuccess) return e;
+    }
+    if (blocks <= 0 || nprob <= 0) return cudaSuccess;
+    kern<<<dim3(blocks, nprob), 32 * quad_warps<MSQOC_L, MSQOC_Q>(), smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t MSQOC_CAT(launch_quad, MSQOC_L, MSQOC_Q)(const QuadArgs& a, int blocks, int nprob, cudaStream_t s) {
+    return a.split ? launch_quad_one<true>(a, blocks, nprob, s) : launch_quad_one<false>(a, blocks, nprob, s);
 }
 
 int MSQOC_CAT(sweep_occupancy, MSQOC_L, MSQOC_Q)(const SweepArgs& a) {

@@ -192,6 +192,26 @@ int max_tile_threads(int pair, int lean = 0) {
     return pair == 2 ? MAX_QUAD_TILE_THREADS : pair ? MAX_PAIR_TILE_THREADS : lean ? MAX_LEAN_TILE_THREADS : MAX_TILE_THREADS;
 }
 
+// Shared memory that admits a tile width and a history depth (200 KB at most, below): the apply
+// buffers and coefficients of a tile, two groups of `depth` steps of midpoint states, and a
+// window's part of the alpha-gradient with its product sums.  The options' range is defined by
+// this sum, whatever the sweeps hold: they stage one group and sum no products, so an admitted
+// tile always fits.
+size_t admission_bytes(int q, int L, int N, int cpt, int nthreads, int g, int solver, int pair, int depth) {
+    const bool mixed = solver == SOLVER_MIXED, two_float = !pair && mixed;
+    const size_t nslot = size_t(q) * L * 2, ncoef = pair ? 2 : 1, buf = size_t(cpt) * N + 1;
+    size_t V = 1;
+    while (V < size_t(4 * q)) V <<= 1;
+    size_t o = 0;
+    for (size_t bytes : {4 * ncoef * nslot * 16, 4 * ncoef * nslot * 8, two_float ? 4 * nslot * 16 : 0, size_t(64),
+                         size_t(16), 4 * size_t(nthreads / 32) * V * 8, size_t(4 * 4 * q * 8), size_t(2) * g * 8,
+                         two_float ? size_t(2) * g * 8 : 0, two_float ? size_t(N) * 16 : 0, buf * 16,
+                         mixed ? 0 : buf * 16, mixed ? buf * 8 : 0, mixed ? buf * 8 : 0,
+                         size_t(depth) * cpt * N * 16, size_t(depth) * cpt * N * 16})
+        o += align16(bytes);
+    return o;
+}
+
 // Is `cpt` columns per tile usable in the given kernel family?  Tiles must fit the family's
 // thread limit and the shared memory; a tile that covers two windows needs two warps (one per
 // window's coefficients), so a one-warp tile must divide the window's columns.  g: doubles of
@@ -200,9 +220,7 @@ bool tile_width_ok(int cpt, int E, int F, int q, int L, int N, int g, int solver
     if (cpt < 1 || cpt > E || (1 << pair) * cpt * F > max_tile_threads(pair, lean)) return false;
     const int nthreads = tile_threads(cpt, F, pair);
     if (nthreads == 32 && E % cpt) return false;
-    const size_t s1 = sweep_layout(q, L, N, cpt, nthreads, g, solver, true, pair).total;
-    const size_t s0 = sweep_layout(q, L, N, cpt, nthreads, g, solver, false, pair).total;
-    return std::max(s0, s1) <= 200 * 1024;
+    return admission_bytes(q, L, N, cpt, nthreads, g, solver, pair, 1) <= 200 * 1024;
 }
 
 // Lane quads serve 2-level subsystems whose exchange-coupled pairs all have precomputed sources.
@@ -394,7 +412,7 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
         pd.wsq[2 * l + 0] = std::sqrt(double(l + 1));
         pd.wsq[2 * l + 1] = std::sqrt(double(l));
     }
-    // the tiles' shared alpha-gradient: the splines active in one window (the most over the
+    // a window's part of the alpha-gradient: the splines active in one window (the most over the
     // windows, from each window's first active spline), plus a margin of two
     int span = 3;
     for (int m = pd.m_off + 1; m <= pd.m_off + pd.M; ++m) {
@@ -404,8 +422,7 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
         const int s_last = spline_index((double(n1 - 1) + 0.5) * pd.h, pd.dtau, pd.d1);
         span = std::max(span, s_last - s_first + 3);
     }
-    pd.gspan = std::min(pd.d1, span + 2);
-    pd.glocal = 2 * nfsum * pd.gspan;
+    pd.glocal = 2 * nfsum * std::min(pd.d1, span + 2);
     if (layout < MSQOC_LAYOUT_AUTO || layout > MSQOC_LAYOUT_FIBER_LEAN)
         return fail(MSQOC_ERR_INVALID_ARG, "layout %d is not an MSQOC_LAYOUT_* value", layout);
     if (layout == MSQOC_LAYOUT_QUAD && !quad_admitted(pd))
@@ -431,25 +448,33 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
     const int64_t max_ns = (nsteps + nwindows - 1) / nwindows;
     pd.kseg = static_cast<int>(max_ns);
     pd.nseg = 1;
+    pd.kadj = pd.kseg;
+    pd.nsub = 1;
     pd.hdepth = 1;
     return MSQOC_OK;
 }
 
-// the sweeps' shared memory fits with history groups of `depth` steps
+// history groups of `depth` steps are admitted
 bool history_depth_ok(const ProbDev& pd, int depth) {
     if (depth < 1 || depth > MAX_HDEPTH) return false;
-    for (int bwd = 0; bwd < 2; ++bwd)
-        if (sweep_layout(pd.q, pd.L, pd.N, pd.cb, pd.nthreads, pd.glocal, pd.solver, bwd != 0, pd.pair, depth).total >
-            200 * 1024)
-            return false;
-    return true;
+    return admission_bytes(pd.q, pd.L, pd.N, pd.cb, pd.nthreads, pd.glocal, pd.solver, pd.pair, depth) <= 200 * 1024;
 }
+
+// The adjoint midpoint states kept between an adjoint launch and the quadrature of its steps: at
+// most this many bytes (a longer segment is cut into chunks of equal length; a chunk has at least
+// 16 steps).  1 GiB holds a whole segment of every workload but the largest, whose launches last
+// milliseconds a chunk.
+constexpr size_t ADJ_CHUNK_BYTES = size_t(1) << 30;
 
 // history segmentation for a checkpoint interval K (1 = keep every midpoint state)
 void set_segments(ProbDev& pd, int K) {
     const int64_t max_ns = (pd.nsteps + pd.M_glob - 1) / pd.M_glob;
     pd.kseg = (K <= 1 || K >= max_ns) ? static_cast<int>(max_ns) : K;
     pd.nseg = static_cast<int>((max_ns + pd.kseg - 1) / pd.kseg);
+    const size_t step = size_t(pd.M) * pd.N * pd.E * sizeof(double2);
+    const int64_t most = std::max<int64_t>(16, static_cast<int64_t>(ADJ_CHUNK_BYTES / step));
+    pd.nsub = static_cast<int>((pd.kseg + most - 1) / most);
+    pd.kadj = (pd.kseg + pd.nsub - 1) / pd.nsub;
 }
 
 // sweep launch arguments of a single problem
@@ -499,7 +524,7 @@ void free_problem(msqoc_problem* p) {
     void* bufs[] = {p->tiles_ro, p->lanemap_ro,
                     p->pds,   p->tiles, p->lanemap, p->P,     p->emb,   p->V,     p->alpha_dev, p->W_dev,
                     p->ctrl,  p->spl,   p->phase,   p->hist,  p->ckpt,  p->Lstate, p->Uend,     p->Lterm,
-                    p->Lam0,  p->term,  p->gpart,   p->status, p->out_dev, p->reg_dev};
+                    p->Lam0,  p->term,  p->lhist,   p->quad,  p->status, p->out_dev, p->reg_dev};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (p->status_host) cudaFreeHost(p->status_host);
@@ -527,14 +552,20 @@ struct Mark {
 // doubles of the regularization scratch: alpha[d], gradient[d], energy shares[q d1], R
 size_t reg_doubles(const ProbDev& pd) { return 2 * size_t(pd.d) + size_t(pd.q) * pd.d1 + 2; }
 
-// device bytes of the history, checkpoints and segment state of one problem
+// device bytes of the histories, checkpoints and segment state of one problem:
 // 16-byte blocks after the history that hold its column scale exponents ([M][nseg][E] ints)
 size_t hist_scale_blocks(const ProbDev& pd) { return (size_t(pd.M) * pd.nseg * pd.E * sizeof(int) + 15) / 16; }
+
+// the same after the adjoint's ([M][E] ints)
+size_t adj_scale_blocks(const ProbDev& pd) { return (size_t(pd.M) * pd.E * sizeof(int) + 15) / 16; }
 
 size_t gradient_bytes(const ProbDev& pd) {
     const size_t ne = size_t(pd.N) * pd.E;
     size_t b = (size_t(pd.M) * pd.kseg * ne + hist_scale_blocks(pd)) * sizeof(double2);
-    if (pd.nseg > 1) b += (size_t(pd.M) * pd.nseg * ne + size_t(pd.M) * ne) * sizeof(double2);
+    b += (size_t(pd.M) * pd.kadj * ne + adj_scale_blocks(pd)) * sizeof(double2);
+    b += size_t(pd.q) * pd.nsteps * sizeof(double2);
+    if (pd.nseg > 1) b += size_t(pd.M) * pd.nseg * ne * sizeof(double2);
+    if (pd.nseg * pd.nsub > 1) b += size_t(pd.M) * ne * sizeof(double2);
     return b;
 }
 
@@ -675,7 +706,6 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     A(dalloc(&p->Lterm, M * p->ne), "Lterm");
     A(dalloc(&p->Lam0, M * p->ne), "Lam0");
     A(dalloc(&p->term, M), "terms");
-    A(dalloc(&p->gpart, size_t(pd.ntiles) * pd.d), "gradient partials");
     A(dalloc(&p->status, 1), "status");
     A(dalloc(&p->out_dev, out_layout(p->npen, pd.d, p->nW).total), "outputs");
     A(dalloc(&p->reg_dev, reg_doubles(pd)), "regularization scratch");
@@ -698,7 +728,6 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
         pd.Lterm = p->Lterm;
         pd.Lam0 = p->Lam0;
         pd.term = p->term;
-        pd.gpart = p->gpart;
         pd.status = p->status;
         A(cudaMemcpy(p->tiles, tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice), "tiles copy");
         A(cudaMemcpy(p->lanemap, maps.data(), maps.size() * sizeof(int), cudaMemcpyHostToDevice), "lane map copy");
@@ -721,8 +750,7 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     }
     if (st != MSQOC_OK) return st;
     p->bytes = sizeof(double2) * (N + p->ne * (1 + 3 * M) + size_t(nsteps) * (q + nfsum)) +
-               sizeof(Spline4) * size_t(nsteps) + sizeof(double) * (pd.d + p->nW + M + size_t(pd.ntiles) * pd.d + out_layout(p->npen, pd.d, p->nW).total +
-                                reg_doubles(pd)) +
+               sizeof(Spline4) * size_t(nsteps) + sizeof(double) * (pd.d + p->nW + M + out_layout(p->npen, pd.d, p->nW).total + reg_doubles(pd)) +
                sizeof(int) * (E + 1 + maps.size() + maps_ro.size()) + sizeof(Tile) * (tiles.size() + tiles_ro.size()) +
                sizeof(ProbDev);
     p->grad_bytes = gradient_bytes(pd);
@@ -782,24 +810,30 @@ msqoc_status stage_inputs(msqoc_problem* p, const double* alpha, const double* W
     return MSQOC_OK;
 }
 
-// the history, checkpoints and segment state, on the first gradient evaluation
+// the histories, checkpoints and segment state, on the first gradient evaluation
 msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s) {
     if (p->hist) return MSQOC_OK;
     ProbDev& pd = p->pd;
     const size_t M = pd.M;
     cudaError_t e = dalloc(&p->hist, M * pd.kseg * p->ne + hist_scale_blocks(pd));
+    if (e == cudaSuccess) e = dalloc(&p->lhist, M * pd.kadj * p->ne + adj_scale_blocks(pd));
+    if (e == cudaSuccess) e = dalloc(&p->quad, size_t(pd.q) * pd.nsteps);
     if (e == cudaSuccess && pd.nseg > 1) e = dalloc(&p->ckpt, M * pd.nseg * p->ne);
-    if (e == cudaSuccess && pd.nseg > 1) e = dalloc(&p->Lstate, M * p->ne);
+    if (e == cudaSuccess && pd.nseg * pd.nsub > 1) e = dalloc(&p->Lstate, M * p->ne);
     if (e != cudaSuccess) {
-        for (void* b : {static_cast<void*>(p->hist), static_cast<void*>(p->ckpt), static_cast<void*>(p->Lstate)})
-            if (b) cudaFree(b);
-        p->hist = p->ckpt = p->Lstate = nullptr;
+        for (double2** b : {&p->hist, &p->lhist, &p->quad, &p->ckpt, &p->Lstate}) {
+            if (*b) cudaFree(*b);
+            *b = nullptr;
+        }
         cudaGetLastError();
         return fail(MSQOC_ERR_OUT_OF_MEMORY, "history buffers (%zu bytes, checkpoint interval %d): %s", p->grad_bytes,
                     p->ckpt_interval, cudaGetErrorString(e));
     }
     pd.hist = p->hist;
     pd.hsh = reinterpret_cast<int*>(p->hist + M * pd.kseg * p->ne);
+    pd.lhist = p->lhist;
+    pd.lsh = reinterpret_cast<int*>(p->lhist + M * pd.kadj * p->ne);
+    pd.quad = p->quad;
     pd.ckpt = p->ckpt;
     pd.Lstate = p->Lstate;
     p->bytes += p->grad_bytes;
@@ -808,8 +842,30 @@ msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s) {
     return MSQOC_OK;
 }
 
-msqoc_status sweep(msqoc_problem* p, int mode, int seg, cudaStream_t s) {
-    const SweepArgs a = sweep_args(p->pd, p->pds, p->tiles, p->lanemap, mode, seg);
+bool split_history(const ProbDev& pd) { return pd.solver == SOLVER_MIXED && pd.pair == 0; }
+
+// blocks of the quadrature kernel: per window, the chunk's steps in groups of 32 lanes
+int quad_blocks(const ProbDev& pd) {
+    int lanes = 1;
+    while (lanes < pd.E && lanes < 32) lanes <<= 1;
+    const int per = 32 / lanes;
+    return pd.M * ((pd.kadj + per - 1) / per);
+}
+
+QuadArgs quad_args(const ProbDev& pd, const ProbDev* pds_dev, int seg, int sub) {
+    QuadArgs a{};
+    a.pds = pds_dev;
+    a.L = pd.L;
+    a.q = pd.q;
+    a.split = split_history(pd) ? 1 : 0;
+    a.seg = seg;
+    a.sub = sub;
+    return a;
+}
+
+msqoc_status sweep(msqoc_problem* p, int mode, int seg, cudaStream_t s, int sub = 0) {
+    SweepArgs a = sweep_args(p->pd, p->pds, p->tiles, p->lanemap, mode, seg);
+    a.sub = sub;
     CUDA_TRY(launch_sweep(a, p->pd.ntiles, s));
     return MSQOC_OK;
 }
@@ -838,7 +894,7 @@ msqoc_status launch_terminal(msqoc_problem* p, bool want_lambda, cudaStream_t s)
 
 msqoc_status launch_objective_outputs(msqoc_problem* p, double* P, double* J, double* pen, cudaStream_t s) {
     Mark mk(p, MSQOC_KERNEL_FINALIZE, s);
-    k_finalize_scalars<<<1, 32, 0, s>>>(p->pd, P, J, p->npen > 0 ? pen : nullptr, nullptr);
+    k_objective_outputs<<<1, OUT_THREADS, 0, s>>>(p->pd, P, J, p->npen > 0 ? pen : nullptr);
     CUDA_TRY(cudaGetLastError());
     return MSQOC_OK;
 }
@@ -846,14 +902,11 @@ msqoc_status launch_objective_outputs(msqoc_problem* p, double* P, double* J, do
 msqoc_status launch_gradient_outputs(msqoc_problem* p, double* P, double* ga, double* gw, cudaStream_t s) {
     const ProbDev& pd = p->pd;
     Mark mk(p, MSQOC_KERNEL_FINALIZE, s);
-    k_finalize_scalars<<<std::max(1, (pd.d + 255) / 256), 256, 0, s>>>(pd, P, nullptr, nullptr, ga);
+    const size_t total = p->nWs > 0 ? p->ne * size_t(p->nWs) : 0;
+    const int wblocks = static_cast<int>(std::min<size_t>((total + OUT_THREADS - 1) / OUT_THREADS, 8192));
+    k_gradient_outputs<<<1 + pd.nfsum * pd.d1 + wblocks, OUT_THREADS, 0, s>>>(
+        pd, P, ga, reinterpret_cast<double2*>(gw), wblocks, p->nWs);
     CUDA_TRY(cudaGetLastError());
-    if (p->nWs > 0) {
-        const size_t total = p->ne * size_t(p->nWs);
-        const int blocks = static_cast<int>(std::min<size_t>((total + 255) / 256, 8192));
-        k_grad_W<<<blocks, 256, 0, s>>>(pd, reinterpret_cast<double2*>(gw), p->nWs);
-        CUDA_TRY(cudaGetLastError());
-    }
     return MSQOC_OK;
 }
 
@@ -874,8 +927,6 @@ msqoc_status status_error(int st) {
     if (st & ST_TIMEOUT) return fail(MSQOC_ERR_TIMEOUT, "a bounded device wait gave up (status %d)", st);
     if (st & ST_SOLVER_RANGE)
         return fail(MSQOC_ERR_UNSUPPORTED, "time step too large for the step solver (h*|H_c|/2 >= 0.5)");
-    if (st & ST_GRAD_RANGE)
-        return fail(MSQOC_ERR_INTERNAL, "a gradient spline index fell outside its tile's window range (status %d)", st);
     return fail(MSQOC_ERR_INTERNAL, "device status %d", st);
 }
 
@@ -903,7 +954,6 @@ msqoc_status msqoc_eval_objective(msqoc_problem* p, const double* alpha, const d
     if (st) return st;
     st = launch_forward_part(p, SWEEP_OBJECTIVE, s);
     if (st) return st;
-    const ProbDev& pd = p->pd;
     const bool dP = is_device_ptr(P_out), dJ = !J_out || is_device_ptr(J_out), dpen = !pen_out || is_device_ptr(pen_out);
     double* o = p->out_dev;
     st = launch_objective_outputs(p, dP ? P_out : o, J_out ? (dJ ? J_out : o + 1) : nullptr,
@@ -940,8 +990,11 @@ msqoc_status msqoc_eval_gradient(msqoc_problem* p, const double* alpha, const do
                 st = sweep(p, SWEEP_RECOMPUTE, seg, s);
                 if (st) return st;
             }
-            st = sweep(p, SWEEP_ADJOINT, seg, s);
-            if (st) return st;
+            for (int sub = pd.nsub - 1; sub >= 0; --sub) {
+                st = sweep(p, SWEEP_ADJOINT, seg, s, sub);
+                if (st) return st;
+                CUDA_TRY(launch_quad(quad_args(pd, p->pds, seg, sub), quad_blocks(pd), 1, s));
+            }
         }
     }
     const bool dP = !P_out || is_device_ptr(P_out), dga = is_device_ptr(grad_alpha),
@@ -1342,7 +1395,7 @@ msqoc_status eval_objective_noalloc(const msqoc_hamiltonian* H, const msqoc_cont
     CUDA_TRY(launch_sweep(sweep_args(pd, pd_d, tiles_d, map_d, SWEEP_OBJECTIVE, 0), pd.ntiles, s));
     k_terminal<<<pd.M, TERM_THREADS, 0, s>>>(pd, 0);
     CUDA_TRY(cudaGetLastError());
-    k_finalize_scalars<<<1, 32, 0, s>>>(pd, outs, outs + 1, M > 1 ? outs + 2 : nullptr, nullptr);
+    k_objective_outputs<<<1, OUT_THREADS, 0, s>>>(pd, outs, outs + 1, M > 1 ? outs + 2 : nullptr);
     CUDA_TRY(cudaGetLastError());
 
     // ---- results to the caller (host or device) and the device status word

@@ -185,27 +185,29 @@ __global__ void __launch_bounds__(TERM_THREADS) k_terminal(const ProbDev pd, con
     }
 }
 
-// P = J + sum_m pen_m (window order), J and pen outputs, and the alpha-gradient as the sum of
-// the per-tile partials in tile order.  A shard sums its own windows' terms; J is 0 unless its
-// last window is the problem's last.
-__global__ void k_finalize_scalars(const ProbDev pd, double* P_out, double* J_out, double* pen_out,
-                                   double* galpha_out) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const bool has_last = pd.m_off + pd.M == pd.M_glob;
-        double P = 0.0;
-        for (int m = 1; m <= pd.M; ++m) P += pd.term[m - 1];
+// P = J + sum_m pen_m (fixed order), J and pen outputs.  A shard sums its own windows' terms; J is
+// 0 unless its last window is the problem's last.  One block.
+constexpr int OUT_THREADS = 128;
+__device__ __forceinline__ void objective_outputs(const ProbDev& pd, double* P_out, double* J_out, double* pen_out,
+                                                  double* sh) {
+    const bool has_last = pd.m_off + pd.M == pd.M_glob;
+    const int npen = pd.M - (has_last ? 1 : 0);
+    double P = 0.0;
+    for (int m = threadIdx.x; m < pd.M; m += OUT_THREADS) {
+        const double t = pd.term[m];
+        P += t;
+        if (pen_out && m < npen) pen_out[m] = t;
+    }
+    P = block_sum<OUT_THREADS>(P, sh);
+    if (threadIdx.x == 0) {
         if (P_out) *P_out = P;
         if (J_out) *J_out = has_last ? pd.term[pd.M - 1] : 0.0;
-        if (pen_out)
-            for (int m = 1; m <= pd.M - (has_last ? 1 : 0); ++m) pen_out[m - 1] = pd.term[m - 1];
     }
-    if (galpha_out) {
-        for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < pd.d; l += gridDim.x * blockDim.x) {
-            double s = 0.0;
-            for (int t = 0; t < pd.ntiles; ++t) s += pd.gpart[size_t(t) * pd.d + l];
-            galpha_out[l] = s;
-        }
-    }
+}
+__global__ void __launch_bounds__(OUT_THREADS) k_objective_outputs(const ProbDev pd, double* P_out, double* J_out,
+                                                                    double* pen_out) {
+    __shared__ double sh[OUT_THREADS];
+    objective_outputs(pd, P_out, J_out, pen_out, sh);
 }
 
 // Roll-out infidelity estimate (Eq. rollout-infid-est) from the last evaluation's window terms:
@@ -221,16 +223,61 @@ __global__ void k_rollout_estimate(const ProbDev pd, double* est) {
     }
 }
 
-// dP/dW^k = mu (W^k - U^k(t_k)) - 2 Lambda^{k+1}(t_k) = 2 (Lambda^k(t_k) - Lambda^{k+1}(t_k))
-// (Eq. dP-dW with the factor of Appendix B, Eq. dT-dW-j), k = 1..M-1.  A shard (global windows
-// m_off + 1 .. m_off + M) writes, for the window states it reads (k = max(m_off, 1) ..
-// min(m_off + M, M_glob - 1)), the terms it owns: 2 Lambda^k(t_k) if window k is its own,
-// -2 Lambda^{k+1}(t_k) if window k + 1 is.
-__global__ void k_grad_W(const ProbDev pd, double2* gW, int nblocks) {
+// The outputs of a gradient evaluation, one launch:
+//   block 0                 P;
+//   blocks 1 .. nfsum d1    the alpha-gradient (Eq. grad-int), one block per (carrier f of subsystem
+//     k, spline s) over the steps where the spline is active (its weight B = w_{s - s0}):
+//       dP/dalpha1_kfs = -2h sum_n B (p.x A_k + p.y B_k), dP/dalpha2_kfs = -2h sum_n B (p.x B_k - p.y A_k)
+//     with (A_k, B_k) the step's products (k_quad) and p = e^{i Omega_f t} its carrier phase; FP64
+//     sums in a fixed order;
+//   the other blocks        dP/dW^k = mu (W^k - U^k(t_k)) - 2 Lambda^{k+1}(t_k) = 2 (Lambda^k(t_k) -
+//     Lambda^{k+1}(t_k)) (Eq. dP-dW with the factor of Appendix B, Eq. dT-dW-j), k = 1..M-1.  A shard
+//     (global windows m_off + 1 .. m_off + M) writes, for the window states it reads
+//     (k = max(m_off, 1) .. min(m_off + M, M_glob - 1)), the terms it owns: 2 Lambda^k(t_k) if
+//     window k is its own, -2 Lambda^{k+1}(t_k) if window k + 1 is.
+__global__ void __launch_bounds__(OUT_THREADS) k_gradient_outputs(const ProbDev pd, double* P_out, double* ga,
+                                                                   double2* gW, int wblocks, int nstates) {
+    __shared__ double sh[OUT_THREADS];
+    if (blockIdx.x == 0) {
+        objective_outputs(pd, P_out, nullptr, nullptr, sh);
+        return;
+    }
+    const int nfold = pd.nfsum * pd.d1;
+    if (blockIdx.x <= nfold) {
+        const int fi = (blockIdx.x - 1) / pd.d1, s = (blockIdx.x - 1) % pd.d1;
+        int k = 0;
+        while (pd.cof[k + 1] <= fi) ++k;
+        // steps whose midpoint lies in [(s - 2) dtau, (s + 1) dtau), widened by two steps on each
+        // side (membership is decided by the step table), within this problem's windows
+        const double r = pd.dtau / pd.h;
+        const int64_t w0 = (int64_t(pd.m_off) * pd.nsteps) / pd.M_glob;
+        const int64_t w1 = (int64_t(pd.m_off + pd.M) * pd.nsteps) / pd.M_glob;
+        const int64_t lo = max(w0, int64_t(floor((s - 2) * r - 0.5)) - 2);
+        const int64_t hi = min(w1, int64_t(ceil((s + 1) * r)) + 2);
+        double g1 = 0.0, g2 = 0.0;
+        for (int64_t n = lo + threadIdx.x; n < hi; n += OUT_THREADS) {
+            const Spline4 sp = pd.spl[n];
+            const int j = s - sp.s;
+            if (j < 0 || j > 2) continue;
+            const double w = j == 0 ? sp.w0 : (j == 1 ? sp.w1 : sp.w2);
+            const double2 ab = pd.quad[size_t(k) * pd.nsteps + n], ph = pd.phase[size_t(n) * pd.nfsum + fi];
+            g1 = fma(w, fma(ph.x, ab.x, ph.y * ab.y), g1);
+            g2 = fma(w, fma(ph.x, ab.y, -ph.y * ab.x), g2);
+        }
+        g1 = block_sum<OUT_THREADS>(g1, sh);
+        g2 = block_sum<OUT_THREADS>(g2, sh);
+        if (threadIdx.x == 0) {
+            const size_t i = (size_t(fi) * pd.d1 + s) * 2;
+            ga[i] = -2.0 * pd.h * g1;
+            ga[i + 1] = -2.0 * pd.h * g2;
+        }
+        return;
+    }
     const size_t ne = size_t(pd.N) * pd.E;
-    const size_t total = ne * size_t(nblocks);
+    const size_t total = ne * size_t(nstates);
     const int kfirst = pd.m_off > 1 ? pd.m_off : 1;
-    for (size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += size_t(gridDim.x) * blockDim.x) {
+    for (size_t e = size_t(blockIdx.x - 1 - nfold) * OUT_THREADS + threadIdx.x; e < total;
+         e += size_t(wblocks) * OUT_THREADS) {
         const int k = kfirst + static_cast<int>(e / ne);
         const size_t i = e % ne;
         const int jk = k - pd.m_off;                  // local index of window k (own if >= 1)

@@ -24,7 +24,8 @@ struct msqoc_batch {
         std::vector<int> members;     // indices into probs
         SweepArgs args{};             // pds / tiles / lanemap / geometry of the group's launches
         int ntiles = 0;
-        int nseg_max = 1;
+        int nseg_max = 1, nsub_max = 1;
+        int quad_blocks = 0;          // blocks of a row of the quadrature launch: the most of the members
         ProbDev* pds = nullptr;
         Tile* tiles = nullptr;
         int* lanemap = nullptr;
@@ -32,6 +33,8 @@ struct msqoc_batch {
         std::vector<int> first, count;        // per member: its tiles in host_tiles (by member k)
         Tile* slot_tiles[MSQOC_BATCH_SLOTS] = {};   // per slot: the tiles of a subset evaluation
         Tile* slot_host[MSQOC_BATCH_SLOTS] = {};    // pinned staging of those tiles
+        int* slot_list[MSQOC_BATCH_SLOTS] = {};     // per slot: the subset's members (rows of the
+        int* slot_lhost[MSQOC_BATCH_SLOTS] = {};    // quadrature launch), and their pinned staging
     };
     std::vector<msqoc_problem*> probs;
     std::vector<int> group_of, member_of;   // per problem: its group and index within it
@@ -58,6 +61,8 @@ void free_batch(msqoc_batch* b) {
         for (int k = 0; k < MSQOC_BATCH_SLOTS; ++k) {
             if (g.slot_tiles[k]) cudaFree(g.slot_tiles[k]);
             if (g.slot_host[k]) cudaFreeHost(g.slot_host[k]);
+            if (g.slot_list[k]) cudaFree(g.slot_list[k]);
+            if (g.slot_lhost[k]) cudaFreeHost(g.slot_lhost[k]);
         }
     }
     for (auto& e : b->slot_done)
@@ -101,9 +106,10 @@ msqoc_status for_groups(msqoc_batch* b, const int* ntiles, int set, cudaStream_t
 }
 
 // The launch sequence of one batched evaluation of the problems `sel` (all when sel is empty);
-// tiles[g] / ntiles[g] are the tiles of group g to launch; set: the stream set of the groups.
+// tiles[g] / ntiles[g] are the tiles of group g to launch, list[g] / nlist[g] its members (device
+// array; nullptr: every member, in order); set: the stream set of the groups.
 msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, Tile* const* tiles, const int* ntiles,
-                     bool grad, int set, cudaStream_t s) {
+                     int* const* list, const int* nlist, bool grad, int set, cudaStream_t s) {
     msqoc_status st;
     for (msqoc_problem* p : sel)
         if ((st = launch_controls(p, s))) return st;
@@ -135,9 +141,16 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, Til
                 const cudaError_t e = launch_sweep(a, ntiles[gi], gs);
                 if (e != cudaSuccess) return e;
             }
-            a.mode = SWEEP_ADJOINT;
-            const cudaError_t e = launch_sweep(a, ntiles[gi], gs);
-            if (e != cudaSuccess) return e;
+            for (int sub = g.nsub_max - 1; sub >= 0; --sub) {
+                a.mode = SWEEP_ADJOINT;
+                a.sub = sub;
+                cudaError_t e = launch_sweep(a, ntiles[gi], gs);
+                if (e != cudaSuccess) return e;
+                QuadArgs qa = quad_args(b->probs[g.members[0]]->pd, g.pds, seg, sub);
+                qa.list = list[gi];
+                e = launch_quad(qa, g.quad_blocks, nlist[gi], gs);
+                if (e != cudaSuccess) return e;
+            }
         }
         return cudaSuccess;
     });
@@ -152,12 +165,14 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, Til
 
 msqoc_status enqueue_all(msqoc_batch* b, bool grad, cudaStream_t s) {
     std::vector<Tile*> tiles;
-    std::vector<int> ntiles;
+    std::vector<int> ntiles, nlist;
+    std::vector<int*> list(b->groups.size(), nullptr);
     for (auto& g : b->groups) {
         tiles.push_back(g.tiles);
         ntiles.push_back(g.ntiles);
+        nlist.push_back(static_cast<int>(g.members.size()));
     }
-    return enqueue(b, b->probs, tiles.data(), ntiles.data(), grad, MSQOC_BATCH_SLOTS, s);
+    return enqueue(b, b->probs, tiles.data(), ntiles.data(), list.data(), nlist.data(), grad, MSQOC_BATCH_SLOTS, s);
 }
 
 msqoc_status eval(msqoc_batch* b, bool grad, cudaStream_t s) {
@@ -257,6 +272,8 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
             cpt = std::max(cpt, pd.cb);
             gmax = std::max(gmax, pd.glocal);
             g.nseg_max = std::max(g.nseg_max, pd.nseg);
+            g.nsub_max = std::max(g.nsub_max, pd.nsub);
+            g.quad_blocks = std::max(g.quad_blocks, quad_blocks(pd));
         }
         std::vector<ProbDev> pds;
         std::vector<Tile> tiles;
@@ -296,6 +313,8 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         for (int k = 0; k < MSQOC_BATCH_SLOTS && e == cudaSuccess; ++k) {
             e = cudaMalloc(reinterpret_cast<void**>(&g.slot_tiles[k]), tiles.size() * sizeof(Tile));
             if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&g.slot_host[k]), tiles.size() * sizeof(Tile));
+            if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&g.slot_list[k]), g.members.size() * sizeof(int));
+            if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&g.slot_lhost[k]), g.members.size() * sizeof(int));
         }
         if (e != cudaSuccess) {
             st = fail(e == cudaErrorMemoryAllocation ? MSQOC_ERR_OUT_OF_MEMORY : MSQOC_ERR_CUDA, "batch tables: %s",
@@ -311,13 +330,14 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         g.args.nthreads = nthreads;
         SweepArgs adj = g.args;
         adj.mode = SWEEP_ADJOINT;
-        if (std::max(sweep_smem_bytes(g.args), sweep_smem_bytes(adj)) > 227 * 1024) {
+        if (admission_bytes(g.q, g.L, p0.N, cpt, nthreads, gmax, g.solver, g.pair, g.args.hdepth) > 227 * 1024) {
             st = fail(MSQOC_ERR_UNSUPPORTED, "batched tiles need too much shared memory");
             break;
         }
         // set the kernels' shared-memory limits now (a launch of no tiles only does that), so
         // that a graph capture later makes no attribute calls
-        if (launch_sweep(g.args, 0, nullptr) != cudaSuccess || launch_sweep(adj, 0, nullptr) != cudaSuccess)
+        if (launch_sweep(g.args, 0, nullptr) != cudaSuccess || launch_sweep(adj, 0, nullptr) != cudaSuccess ||
+            launch_quad(quad_args(p0, g.pds, 0, 0), 0, 0, nullptr) != cudaSuccess)
             st = fail(MSQOC_ERR_CUDA, "sweep kernel attributes could not be set");
     }
     if (!st && (flags & MSQOC_BATCH_GRAPH) && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
@@ -360,7 +380,8 @@ msqoc_status batch_eval_subset(msqoc_batch* b, const int32_t* members, int32_t n
     CUDA_TRY(cudaEventSynchronize(b->slot_done[slot]));
     std::vector<msqoc_problem*> sel;
     std::vector<Tile*> tiles(b->groups.size());
-    std::vector<int> ntiles(b->groups.size(), 0);
+    std::vector<int> ntiles(b->groups.size(), 0), nlist(b->groups.size(), 0);
+    std::vector<int*> list(b->groups.size());
     for (int i = 0; i < n; ++i) sel.push_back(b->probs[members[i]]);
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         auto& g = b->groups[gi];
@@ -371,6 +392,7 @@ msqoc_status batch_eval_subset(msqoc_batch* b, const int32_t* members, int32_t n
             const int k = b->member_of[members[i]];
             std::copy(g.host_tiles.begin() + g.first[k], g.host_tiles.begin() + g.first[k] + g.count[k], h + cnt);
             cnt += g.count[k];
+            g.slot_lhost[slot][nlist[gi]++] = k;
         }
         auto tile_len = [&](const Tile& x) {
             const ProbDev& pd = b->probs[g.members[x.prob]]->pd;
@@ -378,11 +400,15 @@ msqoc_status batch_eval_subset(msqoc_batch* b, const int32_t* members, int32_t n
         };
         std::stable_sort(h, h + cnt, [&](const Tile& x, const Tile& y) { return tile_len(x) > tile_len(y); });
         if (cnt) CUDA_TRY(cudaMemcpyAsync(g.slot_tiles[slot], h, cnt * sizeof(Tile), cudaMemcpyHostToDevice, s));
+        if (cnt && gradient)
+            CUDA_TRY(cudaMemcpyAsync(g.slot_list[slot], g.slot_lhost[slot], nlist[gi] * sizeof(int),
+                                     cudaMemcpyHostToDevice, s));
         tiles[gi] = g.slot_tiles[slot];
         ntiles[gi] = cnt;
+        list[gi] = g.slot_list[slot];
     }
     CUDA_TRY(cudaEventRecord(b->slot_done[slot], s));
-    return enqueue(b, sel, tiles.data(), ntiles.data(), gradient != 0, slot, s);
+    return enqueue(b, sel, tiles.data(), ntiles.data(), list.data(), nlist.data(), gradient != 0, slot, s);
 }
 
 }  // namespace

@@ -40,7 +40,8 @@ struct msqoc_problem {
     double2* Lterm = nullptr;
     double2* Lam0 = nullptr;
     double* term = nullptr;
-    double* gpart = nullptr;
+    double2* lhist = nullptr;      // (with hist) adjoint midpoint states of one chunk
+    double2* quad = nullptr;       // (with hist) the steps' gradient products
     int* status = nullptr;
     double* out_dev = nullptr;     // outputs of the last evaluation: P, J, pen[M-1], galpha[d], gW[nW]
     double* reg_dev = nullptr;     // regularization: alpha[d], gradient[d], energy shares[q d1], R
@@ -92,6 +93,11 @@ Tile tile_at(long t, int M, int E, int cpt, int prob);
 long tile_count(int M, int E, int cpt);
 SweepArgs sweep_args(const ProbDev& pd, const ProbDev* pds_dev, const Tile* tiles, const int* lanemap, int mode,
                      int seg);
+
+// quadrature launch arguments (SweepArgs of the same segment and chunk), see k_quad
+QuadArgs quad_args(const ProbDev& pd, const ProbDev* pds_dev, int seg, int sub);
+// shared memory that admits a tile (see msqoc_api.cu)
+size_t admission_bytes(int q, int L, int N, int cpt, int nthreads, int g, int solver, int pair, int depth);
 
 // Output staging layout in out_dev (doubles): P, J, pen[npen], grad_alpha[d], grad_W[nW].
 // grad_alpha and grad_W start at even offsets: grad_W is written as double2 (16-byte aligned).

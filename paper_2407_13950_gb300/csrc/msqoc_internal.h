@@ -26,11 +26,10 @@ static_assert(MAX_TILE_THREADS <= MAX_ANY_TILE_THREADS && MAX_LEAN_TILE_THREADS 
 enum Solver { SOLVER_FP64 = 1, SOLVER_MIXED = 2 };
 
 // device status word bits
-enum Status { ST_OK = 0, ST_TIMEOUT = 1, ST_BAD_LAUNCH = 2, ST_SOLVER_RANGE = 4, ST_GRAD_RANGE = 8 };
+enum Status { ST_OK = 0, ST_TIMEOUT = 1, ST_BAD_LAUNCH = 2, ST_SOLVER_RANGE = 4 };
 
 // Index of the first of the three quadratic B-splines (spacing dtau, d1 of them) active at time
-// t, clamped to the grid.  The controls kernel, the sweeps and the host's sizing of the shared
-// gradient all take it from here.
+// t, clamped to the grid.  The controls kernel and the host take it from here.
 __host__ __device__ inline int spline_index(double t, double dtau, int d1) {
     const int s0 = static_cast<int>(floor(t / dtau));
     return s0 < 0 ? 0 : (s0 > d1 - 3 ? d1 - 3 : s0);
@@ -59,15 +58,16 @@ struct ProbDev {
                    // 2-level fiber)
     int lean;      // one thread per fiber compiled for 168 registers (more warps per SM), pair = 0
     int ntiles;    // tiles of the problem's sweeps
-    int gspan;     // splines per carrier in a tile's shared alpha-gradient: every spline active in
-                   // one window (from the window's first active spline), with a margin
-    int glocal;    // doubles of that gradient per window slot: nfsum gspan 2
+    int glocal;    // doubles of a window's part of the alpha-gradient (its active splines with a
+                   // margin of two, every carrier): enters the admission of tiles only
     int solver;
     int kseg;      // steps per history segment (checkpoint interval; >= the longest window when
                    // every midpoint state is kept)
     int nseg;      // segments per window: ceil(longest window / kseg)
-    int hdepth;    // steps per history synchronisation: midpoint states staged and stored (forward)
-                   // or fetched (adjoint) in groups of hdepth steps, one wait per group
+    int kadj;      // steps per adjoint launch (a chunk of a segment; kseg when it is not cut)
+    int nsub;      // chunks per segment: ceil(kseg / kadj)
+    int hdepth;    // steps per history synchronisation: midpoint states staged and stored in
+                   // groups of hdepth steps, one wait per group
     int64_t nsteps;
     double T, h, mu, dtau;
     double lam;    // ||a + a^+|| on L levels (bound of the ladder-term norm per unit |d|)
@@ -100,13 +100,17 @@ struct ProbDev {
                                  // two-float split of Ubar 2^-hsh, hsh the column's scale exponent)
     int* hsh;                    // [M][nseg][E] column scale exponent of each window segment's
                                  // history (mixed solver, one thread per fiber), after hist
+    double2* lhist;              // [M][kadj][E][N] adjoint midpoint states Lbar of one chunk of every
+                                 // window, in the form of hist
+    int* lsh;                    // [M][E] their column scale exponents, after lhist
+    double2* quad;               // [q][nsteps] the step's gradient products (A_k, B_k) of every step
+                                 // (msqoc_quad.cuh)
     double2* ckpt;               // [M][nseg][E][N] states at the segment starts (kseg < longest window)
     double2* Uend;               // [M][E][N] U^m(t_m)
     double2* Lterm;              // [M][E][N] Lambda^m(t_m)
     double2* Lam0;               // [M][E][N] Lambda^m(t_{m-1})
     double2* Lstate;             // [M][E][N] adjoint state between segments
     double* term;                // [M] pen_m (m < M), J (m = M)
-    double* gpart;               // [ntiles][d] per-tile alpha-gradient partials
     int* status;                 // status word (ST_* bits)
 };
 
@@ -114,7 +118,7 @@ struct ProbDev {
 // order, starting at column c0 of window m0 (1-based).  The first `ncol0` columns belong to
 // window m0, the rest to window m0 + 1 (a tile covers at most two windows).  `map` selects the
 // thread -> (column, fiber) assignment in the launch's lane maps; `tloc` is the tile's index
-// among its problem's tiles (row of the problem's gradient partials).
+// among its problem's tiles.
 struct Tile {
     int prob, m0, c0, ncol, ncol0, map, tloc, pad;
 };
@@ -127,7 +131,7 @@ enum SweepMode {
                           // starts (checkpoints, more segments)
     SWEEP_RECOMPUTE = 3,  // forward over segment `seg` from its checkpoint; midpoint states
                           // (no work for a problem with one segment)
-    SWEEP_ADJOINT = 4,    // adjoint over segment `seg` with the fused gradient quadrature
+    SWEEP_ADJOINT = 4,    // adjoint over chunk `sub` of segment `seg`; its midpoint states
     SWEEP_ROLLOUT = 5     // forward over the whole time grid as one window from the identity
                           // embedding; the state at every window boundary t_m into `out`
 };
@@ -138,9 +142,10 @@ struct SweepArgs {
     const Tile* tiles;    // [tiles] one per CTA
     const int* lanemap;   // [maps][threads]: (column << 16 | fiber), ~value for idle lanes
     int cpt;              // columns of the widest tile (shared-memory sizing)
-    int gmax;             // largest shared alpha-gradient per window slot (doubles) over the problems
+    int gmax;             // largest ProbDev::glocal over the problems (admission)
     int mode;             // SweepMode
     int seg;              // segment (SWEEP_RECOMPUTE, SWEEP_ADJOINT)
+    int sub;              // chunk of the segment (SWEEP_ADJOINT)
     int L, q, solver, nthreads;
     int pair;             // kernel family: log2 of the threads per fiber (0, 1 or 2)
     int lean;             // pair = 0 with the 168-register build (ProbDev::lean)
@@ -153,6 +158,19 @@ size_t sweep_smem_bytes(const SweepArgs& a);
 
 // launcher (dispatches on L, q, solver, direction); returns cudaError_t
 cudaError_t launch_sweep(const SweepArgs& a, int ntiles, cudaStream_t s);
+
+// Arguments of one quadrature launch: the gradient products of chunk `sub` of segment `seg` of
+// every problem listed (problems share shape, solver and kernel family).
+struct QuadArgs {
+    const ProbDev* pds;   // device copies
+    const int* list;      // [blocks in y] problem of each row of blocks; nullptr: row y is problem y
+    int L, q, split;      // split: the midpoint states are stored split (two floats)
+    int seg, sub;
+};
+// blocks a problem needs for its windows' chunks
+int quad_blocks(const ProbDev& pd);
+// nprob rows of `blocks` blocks each (0 blocks: only sets the kernel's attributes)
+cudaError_t launch_quad(const QuadArgs& a, int blocks, int nprob, cudaStream_t s);
 
 // resident CTAs per SM of a sweep kernel at this launch shape (0 on error)
 int sweep_ctas_per_sm(const SweepArgs& a);

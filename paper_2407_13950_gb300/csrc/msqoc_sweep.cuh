@@ -31,7 +31,7 @@
 //   dP/dalpha2_kfs += -2h B_s Re(e^{i W t} z_k - e^{-i W t} y_k).
 #pragma once
 
-#include <type_traits>
+#include <climits>
 
 #include "msqoc_sweep_common.cuh"
 
@@ -50,13 +50,6 @@ __device__ __forceinline__ void cmac(float2& w, float2 c, float2 x) {
     w.x = fmaf(-c.y, x.y, w.x);
     w.y = fmaf(c.x, x.y, w.y);
     w.y = fmaf(c.y, x.x, w.y);
-}
-// w += conj(a) * b
-__device__ __forceinline__ void cjmac(double2& w, double2 a, double2 b) {
-    w.x = fma(a.x, b.x, w.x);
-    w.x = fma(a.y, b.y, w.x);
-    w.y = fma(a.x, b.y, w.y);
-    w.y = fma(-a.y, b.x, w.y);
 }
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
@@ -254,42 +247,6 @@ __device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, d
     }
 }
 
-// sums of the gradient products: FP64 (FP64 solver) or two-float (mixed solver; exact two-sums
-// of the leading parts, no FP64 instruction)
-__device__ __forceinline__ double gsum_add(double a, double b) { return a + b; }
-__device__ __forceinline__ DF gsum_add(DF a, DF b) { return df_add(a, b); }
-__device__ __forceinline__ double gsum_shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ DF gsum_shfl_xor(DF v, int o) {
-    return DF{__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.c, o)};
-}
-__device__ __forceinline__ void gsum_zero(double& v) { v = 0.0; }
-__device__ __forceinline__ void gsum_zero(DF& v) { v = DF{0.f, 0.f}; }
-
-// warp reduce-scatter of V values: lane ends with value (lane >> (5 - NH)) summed over the warp
-template <int V, int NH, typename T>
-__device__ __forceinline__ T warp_reduce_scatter(T (&acc)[V], int lane) {
-    int cnt = V;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (cnt > 1) {
-            const int half = cnt >> 1;
-            const bool upper = (lane & o) != 0;
-#pragma unroll
-            for (int q2 = 0; q2 < V / 2; ++q2) {
-                if (q2 < half) {
-                    const T send = upper ? acc[q2] : acc[q2 + half];
-                    const T keep = upper ? acc[q2 + half] : acc[q2];
-                    acc[q2] = gsum_add(keep, gsum_shfl_xor(send, o));
-                }
-            }
-            cnt = half;
-        } else {
-            acc[0] = gsum_add(acc[0], gsum_shfl_xor(acc[0], o));
-        }
-    }
-    return acc[0];
-}
-
 // ------------------------------------------------------------------ compensated apply
 // w += c x for split complex operands (hi.x, hi.y, lo.x, lo.y); w[0] real, w[1] imaginary part
 __device__ __forceinline__ void cmac_df(DF (&w)[2], const float4& c, const float4& x) {
@@ -402,182 +359,6 @@ static __device__ __noinline__ ResidOut<L> resid_fp64(const double2* D0, const d
     return o;
 }
 
-// ------------------------------------------------------------------ gradient products, split form
-// (R, I) += (Re, Im) of conj(x) u for split entries x, u = (hi.x, hi.y, lo.x, lo.y); sr = -1
-// subtracts the real part instead
-template <int SR>
-__device__ __forceinline__ void cjmac_split(DF& R, DF& I, const float4& x, const float4& u) {
-    if constexpr (SR > 0) {
-        df_mac(R, x.x, x.z, u.x, u.z);
-        df_mac(R, x.y, x.w, u.y, u.w);
-    } else {
-        df_mac(R, -x.x, -x.z, u.x, u.z);
-        df_mac(R, -x.y, -x.w, u.y, u.w);
-    }
-    df_mac(I, x.x, x.z, u.y, u.w);
-    df_mac(I, -x.y, -x.w, u.x, u.z);
-}
-// the same as the first term of the sums (R = SR Re(conj(x) u), I = Im(conj(x) u)): no
-// two-sum with zero
-template <int SR>
-__device__ __forceinline__ void cjmul_split(DF& R, DF& I, const float4& x, const float4& u) {
-    if constexpr (SR > 0)
-        R = dot2_df(x.x, x.z, u.x, u.z, x.y, x.w, u.y, u.w);
-    else
-        R = dot2_df(-x.x, -x.z, u.x, u.z, -x.y, -x.w, u.y, u.w);
-    I = dot2_df(x.x, x.z, u.y, u.w, -x.y, -x.w, u.x, u.z);
-}
-
-// The mixed solver's gradient products of one fiber (the FP64 form is in the adjoint below):
-// acc[2k] = A_k and acc[2k + 1] = B_k, the fiber's rows of A_k = Im z_k + Im y_k and
-// B_k = Re z_k - Re y_k with z_k = <Lbar, a_k Ubar>, y_k = <Lbar, a_k^+ Ubar>.  Lbar comes split
-// into two floats (zs, in units of its column's scale 2^shL), the midpoint states Ubar split by
-// the forward sweep (ub, scale 2^shU).  Each value is a compensated FP32 sum (about 2^-47 times
-// its terms' magnitudes) in units 2^(shL + shU), multiplied by pscale (a power of two) into the
-// tile's common units.
-//   last subsystem, weight class j = 1 .. L-1 (weight sqrt j): the pairs (Lbar_{j-1}, Ubar_j)
-//     (a_k, real part +) and (Lbar_j, Ubar_{j-1}) (a_k^+, real part -);
-//   other subsystems: entry 1 of the neighbour list (weight sqrt(l_k + 1) for a_k, real part +;
-//     sqrt(l_k) for a_k^+ at the top level, real part -) and, at interior levels, entry 2
-//     (a_k^+, weight sqrt(l_k), real part -).
-template <int L, int Q>
-__device__ __forceinline__ void products_split(const float4 (&zs)[L], const float4* __restrict__ ub,
-                                               const Fiber<L, Q>& fb, float pscale, DF* acc) {
-    {
-        constexpr int kl = Q - 1;
-        DF A{0.f, 0.f}, B{0.f, 0.f};
-#pragma unroll
-        for (int j = 1; j < L; ++j) {
-            DF R, I;
-            cjmul_split<+1>(R, I, zs[j - 1], ub[fb.xo + j]);
-            cjmac_split<-1>(R, I, zs[j], ub[fb.xo + j - 1]);
-            if (j == 1) {
-                A = I;
-                B = R;
-            } else {
-                A = df_add(A, df_scale_sqrt(I, j));
-                B = df_add(B, df_scale_sqrt(R, j));
-            }
-        }
-        acc[2 * kl + 0] = DF{fmul_n(A.s, pscale), fmul_n(A.c, pscale)};
-        acc[2 * kl + 1] = DF{fmul_n(B.s, pscale), fmul_n(B.c, pscale)};
-    }
-#pragma unroll
-    for (int k = 0; k < Fiber<L, Q>::NFIX; ++k) {
-        const int lk = (fb.f / ipow_c(L, Q - 2 - k)) % L;   // the fiber's level in subsystem k
-        DF R, I;
-        const float4* u1 = ub + fb.nb1[k];
-        cjmul_split<+1>(R, I, zs[0], u1[0]);
-#pragma unroll
-        for (int l = 1; l < L; ++l) cjmac_split<+1>(R, I, zs[l], u1[l]);
-        // entry 1: a_k (weight sqrt(l_k + 1)) or, at the top level, a_k^+ (sqrt(l_k), real part -)
-        DF A = df_scale_sqrt(I, fb.plus1[k] ? lk + 1 : lk);
-        DF B = df_scale_sqrt(R, fb.plus1[k] ? lk + 1 : lk);
-        if (!fb.plus1[k]) B = df_neg(B);
-        if (fb.two[k]) {   // an interior level (warp-uniform: lanes are sorted by class)
-            DF R2, I2;
-            const float4* u2 = ub + fb.nb2[k];
-            cjmul_split<-1>(R2, I2, zs[0], u2[0]);
-#pragma unroll
-            for (int l = 1; l < L; ++l) cjmac_split<-1>(R2, I2, zs[l], u2[l]);
-            A = df_add(A, df_scale_sqrt(I2, lk));
-            B = df_add(B, df_scale_sqrt(R2, lk));
-        }
-        acc[2 * k + 0] = DF{fmul_n(A.s, pscale), fmul_n(A.c, pscale)};
-        acc[2 * k + 1] = DF{fmul_n(B.s, pscale), fmul_n(B.c, pscale)};
-    }
-}
-
-// ------------------------------------------------------------------ gradient fold (adjoint)
-// One step's fold of a window slot, run by that slot's folding warp: the warps' partial sums
-// red[w][v] (fixed order) of A_k = Im z_k + Im y_k and B_k = Re z_k - Re y_k into zy, then, per
-// (carrier kf, active spline jw) entry, dP/dalpha1_kfs += -2h B_s (p.x A + p.y B) and
-// dP/dalpha2_kfs += -2h B_s (p.x B - p.y A) with p = e^{i W t} at the midpoint (Eq. grad-int).
-// Kept out of line: it runs once per step on one warp, and inlined it enlarged the adjoint's
-// step loop, whose instruction fetches already stall its warps.
-template <int Q, int V>
-static __device__ __noinline__ void fold_step(const ProbDev& pd, const double* red, double* zy, double* ga,
-                                              int nwarps, int64_t np, Spline4 sp, double2 ph_lane, bool prefetched,
-                                              int s0, int lane) {
-    if (lane < 2 * Q) {
-        const double* r = red + lane;
-        double s_even = 0.0, s_odd = 0.0;
-        for (int w2 = 0; w2 < nwarps; w2 += 2) {
-            s_even += r[w2 * V];
-            if (w2 + 1 < nwarps) s_odd += r[(w2 + 1) * V];
-        }
-        zy[lane] = s_even + s_odd;
-    }
-    __syncwarp();
-    const int nscat = pd.nfsum * 3;
-    const double m2h = -2.0 * pd.h;
-    for (int i = lane; i < nscat; i += 32) {
-        const int kf = i / 3, jw = i % 3;
-        int k = 0;
-        while (k + 1 < Q && pd.cof[k + 1] <= kf) ++k;
-        const double2 ph = (prefetched && i == lane) ? ph_lane : pd.phase[size_t(np) * pd.nfsum + kf];
-        const double wgt = m2h * (jw == 0 ? sp.w0 : (jw == 1 ? sp.w1 : sp.w2));
-        const double A = zy[2 * k], B = zy[2 * k + 1];
-        const int idx = (kf * pd.gspan + s0 + jw) * 2;
-        ga[idx + 0] = fma(wgt, fma(ph.x, A, ph.y * B), ga[idx + 0]);
-        ga[idx + 1] = fma(wgt, fma(ph.x, B, -ph.y * A), ga[idx + 1]);
-    }
-}
-
-// The mixed solver's fold (the same sums as fold_step): the partial sums and zy are two-float
-// sums in units of 2^S (the tile's product scale, see the adjoint), the phase and spline weight
-// are split on the fly, and each step's contribution goes into a two-float copy gdf of the
-// slot's gradient, which is added into the FP64 gradient ga every FOLD_FLUSH steps (flush: one
-// FP64 add and FMA per element), so a window's hundreds of steps still accumulate in FP64.
-__device__ __forceinline__ void df_mac_full(DF& a, float xh, float xl, float yh, float yl) {
-    df_mac(a, xh, xl, yh, yl);
-    a.c = ffma_n(xl, yl, a.c);   // the low parts' product too: y may be a sum that cancelled
-}
-template <int Q, int V>
-static __device__ __noinline__ void fold_step_df(const ProbDev& pd, const DF* red, DF* zy, double* ga, DF* gdf,
-                                                 int gmax, int nwarps, int64_t np, Spline4 sp, double2 ph_lane,
-                                                 bool prefetched, int s0, int S, bool flush, int lane) {
-    if (lane < 2 * Q) {
-        const DF* r = red + lane;
-        DF s_even{0.f, 0.f}, s_odd{0.f, 0.f};
-        for (int w2 = 0; w2 < nwarps; w2 += 2) {
-            s_even = df_add(s_even, r[w2 * V]);
-            if (w2 + 1 < nwarps) s_odd = df_add(s_odd, r[(w2 + 1) * V]);
-        }
-        zy[lane] = df_add(s_even, s_odd);
-    }
-    __syncwarp();
-    const int nscat = pd.nfsum * 3;
-    for (int i = lane; i < nscat; i += 32) {
-        const int kf = i / 3, jw = i % 3;
-        int k = 0;
-        while (k + 1 < Q && pd.cof[k + 1] <= kf) ++k;
-        const double2 ph = (prefetched && i == lane) ? ph_lane : pd.phase[size_t(np) * pd.nfsum + kf];
-        const float2 px = split_scaled(ph.x, 0), py = split_scaled(ph.y, 0);
-        const float2 wg = split_scaled(jw == 0 ? sp.w0 : (jw == 1 ? sp.w1 : sp.w2), 0);
-        const DF A = zy[2 * k], B = zy[2 * k + 1];
-        DF t1{0.f, 0.f}, t2{0.f, 0.f};
-        df_mac_full(t1, px.x, px.y, A.s, A.c);
-        df_mac_full(t1, py.x, py.y, B.s, B.c);
-        df_mac_full(t2, px.x, px.y, B.s, B.c);
-        df_mac_full(t2, -py.x, -py.y, A.s, A.c);
-        DF* g = gdf + (kf * pd.gspan + s0 + jw) * 2;
-        g[0] = df_add(g[0], df_scale(t1, wg.x, wg.y));
-        g[1] = df_add(g[1], df_scale(t2, wg.x, wg.y));
-    }
-    if (flush) {
-        __syncwarp();
-        const double m2h = -2.0 * pd.h;
-        for (int e = lane; e < gmax; e += 32) {
-            const DF v = gdf[e];
-            if (v.s != 0.f || v.c != 0.f) {
-                ga[e] = fma(m2h, df_to_f64_scaled(v, S), ga[e]);
-                gdf[e] = DF{0.f, 0.f};
-            }
-        }
-    }
-}
-
 // ------------------------------------------------------------------ the sweep kernel
 // One CTA per tile.  A tile covers one or two windows ("slots"); each slot has its own step
 // range, per-step coefficients and iteration counts, computed by warp `slot`, and gradient fold,
@@ -591,40 +372,25 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     constexpr int N = ipow_c(L, Q);
     constexpr int NSLOT = Q * L * 2;
     constexpr int S = BWD ? +1 : -1;       // sign of the preconditioned off-diagonal term
-    // reduced gradient values per subsystem: A_k = Im z_k + Im y_k and B_k = Re z_k - Re y_k, the
-    // only combinations of the products the quadrature needs (padded to a power of two)
-    constexpr int V = next_pow2_c(2 * Q);
-    constexpr int NH = log2_c(V);          // halving levels of the warp reduce-scatter
 
     const Tile tile = a.tiles[blockIdx.x];
     const ProbDev& pd = a.pds[tile.prob];
 
     extern __shared__ __align__(128) unsigned char smem[];
-    const SweepSmem lay = sweep_layout(Q, L, N, a.cpt, blockDim.x, a.gmax, SOLVER, BWD, 0, a.hdepth);
+    const SweepSmem lay = sweep_layout(Q, L, N, a.cpt, SOLVER, 0, a.hdepth);
     double2* coef_d = reinterpret_cast<double2*>(smem + lay.coef_d);
     float2* coef_f = reinterpret_cast<float2*>(smem + lay.coef_f);
     float4* coef_s = SOLVER == SOLVER_MIXED ? reinterpret_cast<float4*>(smem + lay.coef_s) : nullptr;
     int* params = reinterpret_cast<int*>(smem + lay.params);
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + lay.mbar);
-    // sums of the gradient products: two-float (mixed solver, in units 2^S_tile) or FP64; the
-    // tile's window gradients are FP64
-    using GT = std::conditional_t<SOLVER == SOLVER_MIXED, DF, double>;
-    GT* red = reinterpret_cast<GT*>(smem + lay.red);
-    GT* zy = reinterpret_cast<GT*>(smem + lay.zy);
-    double* galpha = reinterpret_cast<double*>(smem + lay.galpha);
-    DF* gdf = reinterpret_cast<DF*>(smem + lay.gdf);   // two-float gradient terms (mixed solver)
     double2* D0 = reinterpret_cast<double2*>(smem + lay.D0);
     double2* D1 = reinterpret_cast<double2*>(smem + lay.D1);
     float2* FA = reinterpret_cast<float2*>(smem + lay.FA);
     float2* FB = reinterpret_cast<float2*>(smem + lay.FB);
     double2* H = reinterpret_cast<double2*>(smem + lay.H);
-    double2* UB0 = reinterpret_cast<double2*>(smem + lay.UB0);
-    double2* UB1 = reinterpret_cast<double2*>(smem + lay.UB1);
 
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int warp = tid >> 5;
-    const int nwarps = blockDim.x >> 5;
     const int E = pd.E;
     const int ncol = tile.ncol, ncol0 = tile.ncol0;
     const int nslot = ncol0 < ncol ? 2 : 1;
@@ -637,27 +403,17 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     const int wns_0 = rollout ? static_cast<int>(pd.nsteps) : static_cast<int>(win_start(pd, tile.m0 + 1) - wn0_0);
     const int64_t wn0_1 = nslot > 1 ? win_start(pd, tile.m0 + 1) : 0;
     const int wns_1 = nslot > 1 ? static_cast<int>(win_start(pd, tile.m0 + 2) - wn0_1) : 0;
-    const int lo_0 = segmented ? a.seg * pd.kseg : 0;
-    const int lo_1 = lo_0;
-    const int cnt_0 = idle_launch ? 0 : max(0, (segmented ? min(wns_0, lo_0 + pd.kseg) : wns_0) - lo_0);
-    const int cnt_1 = nslot > 1 && !idle_launch ? max(0, (segmented ? min(wns_1, lo_1 + pd.kseg) : wns_1) - lo_1) : 0;
+    // (an adjoint launch covers chunk `sub` of its segment)
+    const int seg_hi = segmented ? (a.seg + 1) * pd.kseg : INT_MAX;
+    const int lo = segmented ? a.seg * pd.kseg + (BWD ? a.sub * pd.kadj : 0) : 0;
+    const int hi = BWD ? min(seg_hi, lo + pd.kadj) : seg_hi;
+    const int cnt_0 = idle_launch ? 0 : max(0, min(wns_0, hi) - lo);
+    const int cnt_1 = nslot > 1 && !idle_launch ? max(0, min(wns_1, hi) - lo) : 0;
     const int nit = max(cnt_0, cnt_1);
-    // first spline active in each slot's window: the origin of the slot's window-local
-    // alpha-gradient (adjoint)
-    const int slo_0 = BWD ? spline_first(pd, wn0_0) : 0;
-    const int slo_1 = BWD && nslot > 1 ? spline_first(pd, wn0_1) : 0;
-    // every step's splines fit the slot's window-local range (the index grows with the step, so
-    // a window's last step bounds them all; the host sizes the range with a margin): checked
-    // once per launch, a failure reported in the status word and the gradient left unfolded
-    const bool grad_fits =
-        !BWD || (spline_first(pd, wn0_0 + wns_0 - 1) - slo_0 + 2 < pd.gspan &&
-                 (nslot < 2 || spline_first(pd, wn0_1 + wns_1 - 1) - slo_1 + 2 < pd.gspan));
-    if (!grad_fits && threadIdx.x == 0) atomicOr(pd.status, ST_GRAD_RANGE);
     // global step of slot s at iteration jj, clamped into the slot's range (a slot without steps
     // in this launch maps to its window's first step, which exists)
     auto step_of = [&](int s, int jj) -> int64_t {
         const int cnt = s ? cnt_1 : cnt_0;
-        const int lo = s ? lo_1 : lo_0;
         const int64_t n0 = s ? wn0_1 : wn0_0;
         if (cnt <= 0) return n0;
         const int jc = min(jj, cnt - 1);
@@ -674,7 +430,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     const int m = tile.m0 + slot;                   // window, 1-based
     const int col = slot == 0 ? tile.c0 + c : c - ncol0;
     const int my_cnt = slot ? cnt_1 : cnt_0;
-    const int my_lo = slot ? lo_1 : lo_0;
     const int my_ns = slot ? wns_1 : wns_0;
     const size_t wcol = (size_t(m - 1) * E + col) * N;   // (window, column) in [M][E][N] arrays
 
@@ -740,7 +495,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
         if (my_cnt == 0) {
             u[l] = make_double2(0.0, 0.0);
         } else if (BWD) {
-            u[l] = (my_lo + my_cnt == my_ns) ? pd.Lterm[wcol + i] : pd.Lstate[wcol + i];
+            u[l] = (lo + my_cnt == my_ns) ? pd.Lterm[wcol + i] : pd.Lstate[wcol + i];
         } else if (a.mode == SWEEP_RECOMPUTE) {
             u[l] = pd.ckpt[((size_t(m - 1) * pd.nseg + a.seg) * E + col) * N + i];
         } else if (m + pd.m_off == 1) {
@@ -764,47 +519,34 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
         sh = column_shift(colexp_s[c < MAX_TILE_COLS ? c : 0]);
     }
     const ColScale cs = col_scale(sh);
-    // the history's column scale exponent: written by the forward launch that stores the
-    // segment's midpoint states, read by the adjoint launch of the segment
-    const int hseg = a.mode == SWEEP_HISTORY ? 0 : a.seg;
-    int* const hsh_col = pd.hsh + (size_t(m - 1) * pd.nseg + hseg) * E + col;
-    int shU = 0;
-    // adjoint, mixed solver: the gradient products of column c are in units 2^(sh + shU); the
-    // tile sums them in units 2^S_tile, the largest over its columns (pscale = 2^(sh + shU -
-    // S_tile) <= 1, set after the barrier below)
-    __shared__ int stile_s;
-    int S_tile = 0;
-    float pscale = 1.f;
+    // the midpoint states' column scale exponent, read by the quadrature kernel: per segment for
+    // the forward's history, per launch for the adjoint's
     if constexpr (SOLVER == SOLVER_MIXED) {
-        if (!BWD && ((a.mode == SWEEP_HISTORY && pd.nseg == 1) || a.mode == SWEEP_RECOMPUTE) && act && f == 0 &&
-            my_cnt > 0)
-            *hsh_col = sh;
-        if (BWD) {
-            if (tid == 0) stile_s = -(1 << 20);
-            tile_sync();
-            if (my_cnt > 0) shU = *hsh_col;
-            if (act && my_cnt > 0) atomicMax(&stile_s, sh + shU);
+        if (act && f == 0 && my_cnt > 0) {
+            if (BWD)
+                pd.lsh[size_t(m - 1) * E + col] = sh;
+            else if ((a.mode == SWEEP_HISTORY && pd.nseg == 1) || a.mode == SWEEP_RECOMPUTE)
+                pd.hsh[(size_t(m - 1) * pd.nseg + (a.mode == SWEEP_HISTORY ? 0 : a.seg)) * E + col] = sh;
         }
     }
 
     // ---- history blocks: slot s of a tile covers a contiguous column range of its window
-    const bool want_hist = !BWD && ((a.mode == SWEEP_HISTORY && pd.nseg == 1) || a.mode == SWEEP_RECOMPUTE);
+    const bool want_hist = BWD || (a.mode == SWEEP_HISTORY && pd.nseg == 1) || a.mode == SWEEP_RECOMPUTE;
     const bool want_ckpt = !BWD && a.mode == SWEEP_HISTORY && pd.nseg > 1;
     const uint32_t bytes_0 = static_cast<uint32_t>(size_t(ncol0) * N * sizeof(double2));
     const uint32_t bytes_1 = static_cast<uint32_t>(size_t(ncol - ncol0) * N * sizeof(double2));
     auto hist_ptr = [&](int s, int jj) -> double2* {
         const int64_t n0 = s ? wn0_1 : wn0_0;
-        const int lo = s ? lo_1 : lo_0;
-        const int jr = static_cast<int>(step_of(s, jj) - n0) - lo;   // step within the segment
-        return pd.hist + ((size_t(tile.m0 + s - 1) * pd.kseg + jr) * E + (s ? 0 : tile.c0)) * N;
+        const int jr = static_cast<int>(step_of(s, jj) - n0) - lo;   // step within the segment (chunk)
+        return (BWD ? pd.lhist : pd.hist) +
+               ((size_t(tile.m0 + s - 1) * (BWD ? pd.kadj : pd.kseg) + jr) * E + (s ? 0 : tile.c0)) * N;
     };
-    // Steps per history synchronisation: the midpoint states move in groups of hd iterations
-    // (iterations g hd .. g hd + hd - 1), one block of the tile's cpt N states per iteration.  The
-    // forward stages a group in H and stores it with one wait per group; the adjoint fetches
-    // group g into UB0 / UB1 (g even / odd) on mbar[g & 1], one group ahead.
+    // Steps per history synchronisation: the midpoint states are staged in H in groups of hd
+    // iterations (g hd .. g hd + hd - 1), one block of the tile's cpt N states per iteration, and
+    // a group is stored with one wait.
     const int hd = a.hdepth;
     const size_t hstride = size_t(a.cpt) * N;
-    // forward (thread 0): store the staged group starting at iteration g0 (every slot with a step)
+    // thread 0: store the staged group starting at iteration g0 (every slot with a step)
     auto publish_group = [&](int g0) {
         const int g1 = min(g0 + hd, nit);
         for (int j = g0; j < g1; ++j) {
@@ -813,44 +555,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
             if (j < cnt_1) bulk_s2g(hist_ptr(1, j), src + size_t(ncol0) * N, bytes_1);
         }
     };
-    // adjoint (thread 0): fetch the group starting at iteration g0 into dst, completing on bar
-    auto fetch_group = [&](double2* dst, int g0, uint64_t* bar) {
-        const int g1 = min(g0 + hd, nit);
-        uint32_t total = 0;
-        for (int j = g0; j < g1; ++j) total += (j < cnt_0 ? bytes_0 : 0u) + (j < cnt_1 ? bytes_1 : 0u);
-        mbar_expect_tx(bar, total);
-        for (int j = g0; j < g1; ++j) {
-            double2* d = dst + size_t(j - g0) * hstride;
-            if (j < cnt_0) bulk_g2s(d, hist_ptr(0, j), bytes_0, bar);
-            if (j < cnt_1) bulk_g2s(d + size_t(ncol0) * N, hist_ptr(1, j), bytes_1, bar);
-        }
-    };
-
-    if (BWD) {
-        for (int j = tid; j < 2 * a.gmax; j += blockDim.x) galpha[j] = 0.0;
-        if constexpr (SOLVER == SOLVER_MIXED)
-            for (int j = tid; j < 2 * a.gmax; j += blockDim.x) gdf[j] = DF{0.f, 0.f};
-        if (tid == 0) {
-            mbar_init(&mbar[0], 1);
-            mbar_init(&mbar[1], 1);
-            fence_mbar_init();
-        }
-        tile_sync();
-        if (tid == 0 && nit > 0) fetch_group(UB0, 0, &mbar[0]);
-        if constexpr (SOLVER == SOLVER_MIXED) {
-            S_tile = stile_s > -(1 << 20) ? stile_s : 0;
-            const int k = sh + shU - S_tile;   // <= 0
-            pscale = k >= -126 ? float_of(static_cast<uint32_t>(127 + k) << 23)
-                               : (k >= -149 ? float_of(1u << (k + 149)) : 0.f);
-        }
-    }
-
     // warp s < nslot computes slot s's coefficients and keeps d_k and the iteration counts of
-    // the slot's next step in registers (lane -> subsystem of its slot); warp nwarps - 1 - s folds
-    // the slot's gradient (the two extra jobs of a step on different warps where there are two)
+    // the slot's next step in registers (lane -> subsystem of its slot)
     const bool coef_warp = warp < nslot;
-    const bool fold_warp = nwarps - 1 - warp < nslot;
-    const int fslot = fold_warp ? nwarps - 1 - warp : 0;
     const int cslot = coef_warp ? warp : 0;
     const int my_k = (lane < NSLOT) ? (lane / (2 * L)) : 0;
     double2 dk_next = make_double2(0.0, 0.0);
@@ -862,34 +569,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
             cnt_next = pd.spl[n].cnt;
         }
     };
-    // gradient entries of a step: (carrier, spline of the 3 active) pairs, one per lane of the
-    // folding warp (whose phases are prefetched for the lane's first entry)
-    const int nscat = pd.nfsum * 3;
-    // warps whose lanes belong to both slots reduce each slot separately
-    const unsigned mask1 = __ballot_sync(0xffffffffu, act && slot == 1);
-    const unsigned mask0 = __ballot_sync(0xffffffffu, act && slot == 0);
-
-    // fold slot s's reduced products of step np (parity pp of the reduction buffers) into the
-    // slot's alpha-gradient: dP/dalpha1_kfs += -2h B_s Im(e^{iWt} z_k + e^{-iWt} y_k),
-    // dP/dalpha2_kfs += -2h B_s Re(e^{iWt} z_k - e^{-iWt} y_k)  (Eq. grad-int at the midpoint),
-    // i.e. with (A, B) = (Im z + Im y, Re z - Re y) and the phase p: -2h B_s (p.x A + p.y B) and
-    // -2h B_s (p.x B - p.y A)
-    auto fold = [&](int s, int pp, int64_t np, const Spline4& sp, double2 ph_lane, bool prefetched, bool flush) {
-        if (!grad_fits) {
-            // the sums are not needed; keep the warp's lanes together as fold_step would
-            __syncwarp();
-            return;
-        }
-        if constexpr (SOLVER == SOLVER_MIXED)
-            fold_step_df<Q, V>(pd, red + ((pp * 2 + s) * nwarps) * V, zy + (pp * 2 + s) * 4 * Q,
-                               galpha + size_t(s) * a.gmax, gdf + size_t(s) * a.gmax, a.gmax, nwarps, np, sp,
-                               ph_lane, prefetched, sp.s - (s ? slo_1 : slo_0), S_tile, flush, lane);
-        else
-            fold_step<Q, V>(pd, red + ((pp * 2 + s) * nwarps) * V, zy + (pp * 2 + s) * 4 * Q,
-                            galpha + size_t(s) * a.gmax, nwarps, np, sp, ph_lane, prefetched,
-                            sp.s - (s ? slo_1 : slo_0), lane);
-    };
-
     // the step's state update: 2 z - u (FP64 solver); R u + 2 d in FP64 or the compensated form
     // with the carry (mixed solver; the FP64 form reads R's P from the table: rare)
     auto state_update = [&](double2 (&uu)[L], const double2 (&zz)[L], const DF (&br)[L], const DF (&bi)[L],
@@ -915,17 +594,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     // the state as stored (u + carry)
     auto state_out = [&](int l) { return carry_upd ? carry_finish(u[l], car[l], sh) : u[l]; };
 
-    __shared__ int tflag_s;   // a bounded history wait gave up (adjoint)
-    int* tflag = &tflag_s;
-    if (tid == 0) tflag_s = 0;
-    // (the first barrier of the loop orders this store before every read of the flag)
-    bool timed_out = false;
     int fsel = 0;
     double2* Dc = D0;   // FP64-solver ping-pong buffers
     double2* Dn = D1;
     if (nit > 0) load_ctrl(0);
 
-    int hpos = 0, hgrp = 0;   // iteration jj = hgrp hd + hpos (history group and position)
+    int hpos = 0;   // position of iteration jj in its history group
     for (int jj = 0; jj < nit; ++jj) {
         const int par = jj & 1;
         const bool live = jj < my_cnt;
@@ -937,15 +611,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
                                     coef_f + (par * 2 + cslot) * NSLOT,
                                     coef_s ? coef_s + (par * 2 + cslot) * NSLOT : nullptr,
                                     params + (par * 2 + cslot) * 4);
-        }
-        // adjoint: the folding warps fetch what the fold of iteration jj - 1 needs now, so the
-        // loads are in flight during the solve
-        Spline4 sp_prev{};
-        double2 ph_prev = make_double2(0.0, 0.0);
-        if (BWD && jj > 0 && fold_warp && jj - 1 < (fslot ? cnt_1 : cnt_0)) {
-            const int64_t np = step_of(fslot, jj - 1);
-            sp_prev = pd.spl[np];
-            if (lane < nscat) ph_prev = pd.phase[size_t(np) * pd.nfsum + lane / 3];
         }
         // checkpoint: the state at the start of every segment (forward over whole windows)
         // (the carry is folded into u there, so that a segment recomputed from its checkpoint
@@ -981,25 +646,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
         DF bre[L], bim[L];   // mixed solver: b = P u (conj(P) for the adjoint), two-float
 
         // first barrier of the step: the coefficients are published; thread 0 stores the
-        // previous iteration's midpoints (forward) or fetches the next iteration's (adjoint)
-        // the folding warps add iteration jj - 1's reduced products into the alpha-gradient right
-        // after this iteration's first barrier (which published red[par ^ 1]): the other warps
-        // then run FP32 sweeps, so the fold's FP64 chain does not queue behind the FP64 work
-        // every warp issues at the ends of a step
-        auto fold_previous = [&]() {
-            if (BWD && jj > 0 && fold_warp && jj - 1 < (fslot ? cnt_1 : cnt_0))
-                fold(fslot, par ^ 1, step_of(fslot, jj - 1), sp_prev, ph_prev, true,
-                     ((jj - 1) & (FOLD_FLUSH - 1)) == FOLD_FLUSH - 1 || jj == (fslot ? cnt_1 : cnt_0));
-        };
+        // previous group's midpoints
         auto first_sync_work = [&]() {
-            if (BWD && *tflag) timed_out = true;   // uniform: read after a barrier
-            if (!BWD && want_hist && tid == 0 && jj > 0 && hpos == 0) {
+            if (want_hist && tid == 0 && jj > 0 && hpos == 0) {
                 fence_proxy_async_smem();
                 publish_group(jj - hd);
-            }
-            if (BWD && tid == 0 && hpos == 0 && jj + hd < nit) {
-                const int gn = hgrp + 1;
-                fetch_group((gn & 1) ? UB1 : UB0, jj + hd, &mbar[gn & 1]);
             }
         };
 
@@ -1018,8 +669,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
             }
             tile_sync();
             first_sync_work();
-            if (timed_out) break;
-            fold_previous();
             const int Kown = prm[0];
             const int Kmax = nslot > 1 ? max(prm0[0], prm1[0]) : prm0[0];
             for (int it = 0; it < Kmax; ++it) {
@@ -1070,8 +719,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
                 }
                 tile_sync();
                 first_sync_work();
-                if (timed_out) break;
-                fold_previous();
                 float2 w[L];
                 apply_off<L, Q, float2>(Fb, cff, fb, y, w, pd);
 #pragma unroll
@@ -1129,10 +776,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
                     for (int l = 0; l < L; ++l) zv.v[l] = zs[l];
                     store_z64<L>(D0 + fb.xo, zv, sh);
                 }
-                // forward: the staged midpoints of the previous step must have been read by their
+                // the staged midpoints of the previous step must have been read by their
                 // bulk store (issued at this step's first barrier) before this step's are staged;
                 // waiting here, ahead of a barrier every step has, makes the staging barrier-free
-                if (!BWD && want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
+                if (want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
                 tile_sync();
                 float2 rf[L], e[L];
                 if (dfa) {
@@ -1196,29 +843,28 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
         // the step is solved: what follows (history, gradient products) needs only the midpoint
         if (live) state_update(u, z, bre, bim, dre, dim);
 
-        if constexpr (!BWD) {
-            // ---- midpoint states for the adjoint sweep (async bulk store at the next step)
-            if (want_hist) {
-                if constexpr (SOLVER == SOLVER_FP64) {
-                    // (the FP64 solver's step may have no barrier after the first one)
-                    if (hpos == 0) {
-                        if (tid == 0) bulk_wait_read_all();
-                        tile_sync();
-                    }
+        // ---- midpoint states for the quadrature (async bulk store at the next step)
+        if (want_hist) {
+            if constexpr (SOLVER == SOLVER_FP64) {
+                // (the FP64 solver's step may have no barrier after the first one)
+                if (hpos == 0) {
+                    if (tid == 0) bulk_wait_read_all();
+                    tile_sync();
                 }
-                if (act && live) {
-                    if constexpr (SOLVER == SOLVER_MIXED) {
-                        // the adjoint's gradient products read the split form (products_split)
-                        float4* Hs = reinterpret_cast<float4*>(H) + size_t(hpos) * hstride + fb.xo;
-#pragma unroll
-                        for (int l = 0; l < L; ++l) Hs[l] = zf[l];
-                    } else {
-#pragma unroll
-                        for (int l = 0; l < L; ++l) H[size_t(hpos) * hstride + fb.xo + l] = z[l];
-                    }
-                }
-                fence_proxy_async_smem();
             }
+            if (act && live) {
+                if constexpr (SOLVER == SOLVER_MIXED) {
+                    float4* Hs = reinterpret_cast<float4*>(H) + size_t(hpos) * hstride + fb.xo;
+#pragma unroll
+                    for (int l = 0; l < L; ++l) Hs[l] = zf[l];
+                } else {
+#pragma unroll
+                    for (int l = 0; l < L; ++l) H[size_t(hpos) * hstride + fb.xo + l] = z[l];
+                }
+            }
+            fence_proxy_async_smem();
+        }
+        if constexpr (!BWD) {
             // roll-out: U(t_m) when the step ends on a window boundary t_m, i.e. when n + 1 =
             // floor(m N_T / M) for some 1 <= m < M; the only candidate is m = ceil((n+1) M / N_T)
             if (rollout && live && act) {
@@ -1230,170 +876,22 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
                     for (int l = 0; l < L; ++l) dst[l] = state_out(l);
                 }
             }
-        } else {
-            // ---- gradient quadrature on the midpoints (fused): needs Ubar_n of the tile
-            double2* UB = ((hgrp & 1) ? UB1 : UB0) + size_t(hpos) * hstride;
-            // a wait that gives up raises the tile's flag, read after the next barrier (the
-            // products below then use whatever landed; the evaluation reports the timeout)
-            if (hpos == 0 && !mbar_wait(&mbar[hgrp & 1], (hgrp >> 1) & 1)) *tflag = 1;
-            GT acc[V];
-#pragma unroll
-            for (int v = 0; v < V; ++v) gsum_zero(acc[v]);
-            if constexpr (SOLVER == SOLVER_MIXED) {
-                products_split<L, Q>(zf, reinterpret_cast<const float4*>(UB), fb, pscale, acc);
-            } else {
-            {
-                // last subsystem (stride 1) from the fiber itself, grouped by entry l of Lbar:
-                // A += Im(conj(Lbar_l) v+), B += Re(conj(Lbar_l) v-) with
-                // v+- = sqrt(l+1) Ubar_{l+1} +- sqrt(l) Ubar_{l-1} (the z and y terms of entry l)
-                constexpr int kl = Q - 1;
-                double A = 0.0, B = 0.0;
-#pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    constexpr double kOne = 1.0;
-                    const double wp = l < L - 1 ? sqrt_small(l + 1) : 0.0;   // folded after unrolling
-                    const double wm = l > 0 ? sqrt_small(l) : 0.0;
-                    const double2 zl = z[l];
-                    if (wp != 0.0 && wm != 0.0) {
-                        const double2 up = UB[fb.xo + l + 1], um = UB[fb.xo + l - 1];
-                        double2 vp, vm;
-                        if (wp == kOne) {
-                            vp = make_double2(up.x + wm * um.x, up.y + wm * um.y);
-                            vm = make_double2(up.x - wm * um.x, up.y - wm * um.y);
-                        } else if (wm == kOne) {
-                            vp = make_double2(fma(wp, up.x, um.x), fma(wp, up.y, um.y));
-                            vm = make_double2(fma(wp, up.x, -um.x), fma(wp, up.y, -um.y));
-                        } else {
-                            vp = make_double2(fma(wp, up.x, wm * um.x), fma(wp, up.y, wm * um.y));
-                            vm = make_double2(fma(wp, up.x, -wm * um.x), fma(wp, up.y, -wm * um.y));
-                        }
-                        A = fma(zl.x, vp.y, fma(-zl.y, vp.x, A));
-                        B = fma(zl.x, vm.x, fma(zl.y, vm.y, B));
-                    } else {
-                        // one term: plus (first entry) or minus (last), weight w
-                        const bool plus = wp != 0.0;
-                        const double w = plus ? wp : wm;
-                        const double2 u = UB[fb.xo + (plus ? l + 1 : l - 1)];
-                        if (w == kOne) {
-                            A = fma(zl.x, u.y, fma(-zl.y, u.x, A));
-                            B = plus ? fma(zl.x, u.x, fma(zl.y, u.y, B)) : fma(-zl.x, u.x, fma(-zl.y, u.y, B));
-                        } else {
-                            const double ti = fma(zl.x, u.y, -zl.y * u.x), tr = fma(zl.x, u.x, zl.y * u.y);
-                            A = fma(w, ti, A);
-                            B = fma(plus ? w : -w, tr, B);
-                        }
-                    }
-                }
-                acc[2 * kl + 0] = A;
-                acc[2 * kl + 1] = B;
-            }
-#pragma unroll
-            for (int k = 0; k < Fiber<L, Q>::NFIX; ++k) {
-                double2 p = make_double2(0.0, 0.0);
-                const double2* q1 = UB + fb.nb1[k];
-#pragma unroll
-                for (int l = 0; l < L; ++l) cjmac(p, z[l], q1[l]);
-                // entry 1 is a z_k term (a_k) or, for a fiber at the top level, a y_k term
-                // (a_k^+); entry 2, where there is one, a y_k term: A = Im z + Im y, B = Re z - Re y
-                double A, B;
-                if (fb.two[k]) {   // an interior level (warp-uniform: lanes are sorted by class)
-                    double2 p2 = make_double2(0.0, 0.0);
-                    const double2* q2 = UB + fb.nb2[k];
-#pragma unroll
-                    for (int l = 0; l < L; ++l) cjmac(p2, z[l], q2[l]);
-                    if constexpr (L == 3) {   // level 1 of 3: weights sqrt(2) (a_k) and 1 (a_k^+)
-                        A = fma(fb.w1[k], p.y, p2.y);
-                        B = fma(fb.w1[k], p.x, -p2.x);
-                    } else {
-                        A = fma(fb.w1[k], p.y, fb.w2[k] * p2.y);
-                        B = fma(fb.w1[k], p.x, -fb.w2[k] * p2.x);
-                    }
-                } else {
-                    const double sw1 = fb.plus1[k] ? fb.w1[k] : -fb.w1[k];
-                    A = fb.w1[k] * p.y;
-                    B = sw1 * p.x;
-                }
-                acc[2 * k + 0] = A;
-                acc[2 * k + 1] = B;
-            }
-            }   // FP64 products
-            if (!act || !live) {
-#pragma unroll
-                for (int v = 0; v < V; ++v) gsum_zero(acc[v]);
-            }
-            // per-slot warp sums: lane (lane >> (5 - NH)) == v holds value v
-            {
-                const int vi = lane >> (5 - NH);
-                const bool writer = (lane & ((1 << (5 - NH)) - 1)) == 0;
-                GT* r0 = red + ((par * 2 + 0) * nwarps + warp) * V;
-                GT* r1 = red + ((par * 2 + 1) * nwarps + warp) * V;
-                GT zero;
-                gsum_zero(zero);
-                // a warp with lanes of both windows reduces each window's lanes in a pass of its
-                // own (one copy of the reduction in the code: the step loop's instruction fetches
-                // already stall the adjoint's warps)
-                const bool both = mask0 && mask1;
-                for (int pass = 0; pass < (both ? 2 : 1); ++pass) {
-                    GT t[V];
-#pragma unroll
-                    for (int v = 0; v < V; ++v) t[v] = (!both || slot == pass) ? acc[v] : zero;
-                    const GT sv = warp_reduce_scatter<V, NH>(t, lane);
-                    if (writer) {
-                        if (!both) {
-                            r0[vi] = mask1 ? zero : sv;
-                            if (nslot > 1) r1[vi] = mask1 ? sv : zero;
-                        } else {
-                            (pass == 0 ? r0 : r1)[vi] = sv;
-                        }
-                    }
-                }
-            }
         }
-
-        if (++hpos == hd) {
-            hpos = 0;
-            ++hgrp;
-        }
+        if (++hpos == hd) hpos = 0;
     }
 
-    if (!timed_out) {
-        tile_sync();
-        if (BWD && *tflag) timed_out = true;   // the last step's wait (uniform: after the barrier)
+    tile_sync();
+    if (want_hist && tid == 0 && nit > 0) {
+        fence_proxy_async_smem();
+        publish_group(((nit - 1) / hd) * hd);
+        bulk_wait_all();
     }
-    if (!timed_out) {
-        if constexpr (!BWD) {
-            if (want_hist && tid == 0 && nit > 0) {
-                fence_proxy_async_smem();
-                publish_group(((nit - 1) / hd) * hd);
-                bulk_wait_all();
-            }
-            if (a.mode != SWEEP_RECOMPUTE && !rollout && act && my_cnt > 0) {
+    if (act && my_cnt > 0 && !rollout && a.mode != SWEEP_RECOMPUTE) {
+        // forward: U^m(t_m); adjoint: Lambda at the launch's first step (Lambda^m(t_{m-1}) for
+        // the window's first)
+        double2* dst = !BWD ? pd.Uend : (lo == 0 ? pd.Lam0 : pd.Lstate);
 #pragma unroll
-                for (int l = 0; l < L; ++l) pd.Uend[wcol + f * L + l] = state_out(l);
-            }
-        } else {
-            // the last fold of every slot whose range ends at the last iteration
-            if (fold_warp && nit > 0 && (fslot ? cnt_1 : cnt_0) == nit) {
-                const int64_t np = step_of(fslot, nit - 1);
-                fold(fslot, (nit - 1) & 1, np, pd.spl[np], make_double2(0.0, 0.0), false, true);
-            }
-            tile_sync();
-            // the tile's alpha-gradient partial, accumulated over the segment launches (the first
-            // adjoint launch is the last segment's)
-            double* gp = pd.gpart + size_t(tile.tloc) * pd.d;
-            const bool first_launch = a.seg == pd.nseg - 1;
-            store_grad_partial(gp, galpha, pd, a.gmax, slo_0, nslot > 1 ? slo_1 : -1, first_launch);
-            // Lambda at the segment start: Lambda^m(t_{m-1}) for the window's first segment
-            if (act && my_cnt > 0) {
-                double2* dst = my_lo == 0 ? pd.Lam0 : pd.Lstate;
-#pragma unroll
-                for (int l = 0; l < L; ++l) dst[wcol + f * L + l] = state_out(l);
-            }
-        }
-    } else if (tid == 0) {
-        atomicOr(pd.status, ST_TIMEOUT);
-        // let the bulk copies this tile issued land before its shared memory is released
-        for (int p2 = 0; p2 < 2; ++p2) (void)mbar_wait(&mbar[p2], 0), (void)mbar_wait(&mbar[p2], 1);
+        for (int l = 0; l < L; ++l) dst[wcol + f * L + l] = state_out(l);
     }
 }
 

@@ -1,8 +1,7 @@
 // Pieces shared by the sweep kernel families (msqoc_sweep.cuh: one thread per fiber;
-// msqoc_sweep_pair.cuh: a lane pair, or for 2-level subsystems a lane quad, per fiber):
-// precision conversions, 1D bulk async copies and bounded mbarrier waits, the per-thread
-// neighbour lists, the shared-memory layout, the tile barrier, the spline origin of a window
-// and the write-out of a tile's gradient partial.
+// msqoc_sweep_pair.cuh: a lane pair, or for 2-level subsystems a lane quad, per fiber) and the
+// quadrature kernel (msqoc_quad.cuh): precision conversions, 1D bulk async copies and bounded
+// mbarrier waits, the per-thread neighbour lists, the shared-memory layout and the tile barrier.
 #pragma once
 
 #include <cstdint>
@@ -132,18 +131,6 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-// global -> shared bulk copy completing on an mbarrier (bytes multiple of 16, 16B-aligned)
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
 // shared -> global bulk copy (bulk-group completion)
 __device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)),
@@ -268,21 +255,15 @@ struct Fiber {
 // keep each coefficient in the form of either part, so their coefficient arrays are twice as
 // large.
 struct SweepSmem {
-    size_t coef_d, coef_f, coef_s, params, mbar, red, zy, galpha, gdf, cq, D0, D1, FA, FB, H, UB0, UB1, total;
+    size_t coef_d, coef_f, coef_s, params, cq, D0, D1, FA, FB, H, total;
 };
-// steps between flushes of the mixed solver's two-float gradient accumulator into the FP64 one
-constexpr int FOLD_FLUSH = 8;
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
-__host__ __device__ inline SweepSmem sweep_layout(int q, int L, int N, int cpt, int nthreads, int gmax, int solver,
-                                                  bool bwd, int pair, int hdepth = 1) {
+__host__ __device__ inline SweepSmem sweep_layout(int q, int L, int N, int cpt, int solver, int pair, int hdepth = 1) {
     SweepSmem s{};
     const int nslot = q * L * 2;
-    const int nwarps = nthreads / 32;
     const int ncoef = pair ? 2 : 1;
-    int V = 1;
-    while (V < 4 * q) V <<= 1;
     // apply buffers hold cpt N entries plus a zero entry (index cpt N, never written by the
     // sweeps: the source of the exchange terms an entry does not have)
     const size_t buf_d = (size_t(cpt) * N + 1) * 16, buf_f = (size_t(cpt) * N + 1) * 8;
@@ -293,12 +274,6 @@ __host__ __device__ inline SweepSmem sweep_layout(int q, int L, int N, int cpt, 
     // solver's one-thread families
     s.coef_s = o; o = align16(o + (!pair && solver == SOLVER_MIXED ? size_t(2) * 2 * nslot * 16 : 0));
     s.params = o; o = align16(o + 2 * 2 * 4 * 4);                      // [parity][slot][4]
-    s.mbar = o;   o = align16(o + 2 * 8);
-    s.red = o;    o = align16(o + (bwd ? size_t(2) * 2 * nwarps * V * 8 : 0));   // [parity][slot][warp][V]
-    s.zy = o;     o = align16(o + (bwd ? size_t(2) * 2 * 4 * q * 8 : 0));        // [parity][slot][4q]
-    s.galpha = o; o = align16(o + (bwd ? size_t(2) * gmax * 8 : 0));             // [slot][nfsum][gspan][2]
-    // the mixed solver's one-thread families: the same, two-float, holding the last steps' terms
-    s.gdf = o;    o = align16(o + (bwd && !pair && solver == SOLVER_MIXED ? size_t(2) * gmax * 8 : 0));
     // the mixed solver's one-thread families: per fiber entry the third parts of the splits of
     // 2 kappa and P (the compensated state update)
     s.cq = o;     o = align16(o + (!pair && solver == SOLVER_MIXED ? size_t(N) * 16 : 0));
@@ -306,11 +281,7 @@ __host__ __device__ inline SweepSmem sweep_layout(int q, int L, int N, int cpt, 
     s.D1 = o;     o = align16(o + (solver == SOLVER_FP64 ? buf_d : 0));
     s.FA = o;     o = align16(o + (solver == SOLVER_MIXED ? buf_f : 0));
     s.FB = o;     o = align16(o + (solver == SOLVER_MIXED ? buf_f : 0));
-    // history staging: hdepth blocks of cpt N states (forward H; adjoint UB0 / UB1, one group each)
-    const size_t hist_b = size_t(hdepth) * cpt * N * 16;
-    s.H = o;      o = align16(o + (bwd ? 0 : hist_b));
-    s.UB0 = o;    o = align16(o + (bwd ? hist_b : 0));
-    s.UB1 = o;    o = align16(o + (bwd ? hist_b : 0));
+    s.H = o;      o = align16(o + size_t(hdepth) * cpt * N * 16);   // history staging: hdepth blocks of cpt N states
     s.total = o;
     return s;
 }
@@ -326,30 +297,6 @@ __device__ __forceinline__ void tile_sync() {
 __device__ __forceinline__ int tile_sync_or(int p) {
     if (blockDim.x == 32) return __any_sync(0xffffffffu, p);
     return __syncthreads_or(p);
-}
-
-
-// first spline active at the midpoint of global step n (the controls kernel's spline table
-// holds the same index for every step)
-__device__ __forceinline__ int spline_first(const ProbDev& pd, int64_t n) {
-    return spline_index((double(n) + 0.5) * pd.h, pd.dtau, pd.d1);
-}
-
-// The tile's alpha-gradient partial gp[d] ([carrier][spline][re, im]) from the window-local
-// sums of its slots (slot s holds splines [slo_s, slo_s + gspan) of every carrier at
-// galpha + s gmax; slo_1 < 0: one slot), stored (first launch of the adjoint) or added.  Kept
-// out of line: it runs once per launch, and inlined into the lane-pair adjoint of some shapes
-// it crashed the assembler.
-static __device__ __noinline__ void store_grad_partial(double* gp, const double* galpha, const ProbDev& pd, int gmax,
-                                                int slo_0, int slo_1, bool first) {
-    for (int jx = threadIdx.x; jx < pd.d; jx += blockDim.x) {
-        const int kf = jx / (2 * pd.d1), sx = (jx >> 1) - kf * pd.d1;
-        const int l0 = sx - slo_0, l1 = sx - slo_1;
-        double v = 0.0;
-        if (l0 >= 0 && l0 < pd.gspan) v += galpha[(kf * pd.gspan + l0) * 2 + (jx & 1)];
-        if (slo_1 >= 0 && l1 >= 0 && l1 < pd.gspan) v += galpha[gmax + (kf * pd.gspan + l1) * 2 + (jx & 1)];
-        gp[jx] = first ? v : gp[jx] + v;
-    }
 }
 
 // first global step of local window m (1-based); window m owns [win_start(m), win_start(m + 1))

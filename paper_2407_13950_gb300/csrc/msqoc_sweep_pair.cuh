@@ -18,6 +18,8 @@
 // budget cost the adjoint 2-4%).
 #pragma once
 
+#include <climits>
+
 #include "msqoc_sweep_common.cuh"
 
 namespace msqoc {
@@ -201,33 +203,6 @@ __device__ __forceinline__ void step_coefficients_pair(const ProbDev& pd, int la
     }
 }
 
-// Reduce-scatter of VH values over the 16 lanes of one part (lanes of equal parity): the
-// halving levels use lane bits 4..1, so lane ends with value (lane >> (5 - NH)) of its part
-// summed over the part's lanes (NH = log2 VH <= 4); bit 0, the part, is never mixed.
-template <int VH, int NH>
-__device__ __forceinline__ double part_reduce_scatter(double (&acc)[VH], int lane) {
-    int cnt = VH;
-#pragma unroll
-    for (int o = 16; o > 1; o >>= 1) {
-        if (cnt > 1) {
-            const int half = cnt >> 1;
-            const bool upper = (lane & o) != 0;
-#pragma unroll
-            for (int q2 = 0; q2 < VH / 2; ++q2) {
-                if (q2 < half) {
-                    const double send = upper ? acc[q2] : acc[q2 + half];
-                    const double keep = upper ? acc[q2 + half] : acc[q2];
-                    acc[q2] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-                }
-            }
-            cnt = half;
-        } else {
-            acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
-        }
-    }
-    return acc[0];
-}
-
 // ------------------------------------------------------------------ the sweep kernel
 // One CTA per tile.  A tile covers one or two windows ("slots"); each slot has its own step
 // range, per-step coefficients, iteration counts and gradient fold, computed by warp `slot`
@@ -244,34 +219,24 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     constexpr int N = ipow_c(L, Q);
     constexpr int NSLOT = Q * L * 2;
     constexpr int S = BWD ? +1 : -1;       // sign of the preconditioned off-diagonal term
-    constexpr int V = next_pow2_c(4 * Q);  // padded count of reduced gradient values (both parts)
-    constexpr int VH = V / 2;              // values of one part: z_k and y_k components, k < Q
-    constexpr int NH = log2_c(VH);         // halving levels of the part reduce-scatter
 
     const Tile tile = a.tiles[blockIdx.x];
     const ProbDev& pd = a.pds[tile.prob];
 
     extern __shared__ __align__(128) unsigned char smem[];
-    const SweepSmem lay = sweep_layout(Q, L, N, a.cpt, blockDim.x, a.gmax, SOLVER, BWD, SPLIT, a.hdepth);
+    const SweepSmem lay = sweep_layout(Q, L, N, a.cpt, SOLVER, SPLIT, a.hdepth);
     double2* coef_d = reinterpret_cast<double2*>(smem + lay.coef_d);
     float2* coef_f = reinterpret_cast<float2*>(smem + lay.coef_f);
     int* params = reinterpret_cast<int*>(smem + lay.params);
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + lay.mbar);
-    double* red = reinterpret_cast<double*>(smem + lay.red);
-    double* zy = reinterpret_cast<double*>(smem + lay.zy);
-    double* galpha = reinterpret_cast<double*>(smem + lay.galpha);
     double2* D0 = reinterpret_cast<double2*>(smem + lay.D0);
     double2* D1 = reinterpret_cast<double2*>(smem + lay.D1);
     float2* FA = reinterpret_cast<float2*>(smem + lay.FA);
     float2* FB = reinterpret_cast<float2*>(smem + lay.FB);
     double2* H = reinterpret_cast<double2*>(smem + lay.H);
-    double2* UB0 = reinterpret_cast<double2*>(smem + lay.UB0);
-    double2* UB1 = reinterpret_cast<double2*>(smem + lay.UB1);
 
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int warp = tid >> 5;
-    const int nwarps = blockDim.x >> 5;
     const int part = tid & 1;              // component this thread computes (0: re, 1: im)
     const int le = SPLIT > 1 ? ((tid >> 1) & (SPLIT - 1)) * LS : 0;   // first entry it holds
     const int E = pd.E;
@@ -286,27 +251,17 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     const int wns_0 = rollout ? static_cast<int>(pd.nsteps) : static_cast<int>(win_start(pd, tile.m0 + 1) - wn0_0);
     const int64_t wn0_1 = nslot > 1 ? win_start(pd, tile.m0 + 1) : 0;
     const int wns_1 = nslot > 1 ? static_cast<int>(win_start(pd, tile.m0 + 2) - wn0_1) : 0;
-    const int lo_0 = segmented ? a.seg * pd.kseg : 0;
-    const int lo_1 = lo_0;
-    const int cnt_0 = idle_launch ? 0 : max(0, (segmented ? min(wns_0, lo_0 + pd.kseg) : wns_0) - lo_0);
-    const int cnt_1 = nslot > 1 && !idle_launch ? max(0, (segmented ? min(wns_1, lo_1 + pd.kseg) : wns_1) - lo_1) : 0;
+    // (an adjoint launch covers chunk `sub` of its segment)
+    const int seg_hi = segmented ? (a.seg + 1) * pd.kseg : INT_MAX;
+    const int lo = segmented ? a.seg * pd.kseg + (BWD ? a.sub * pd.kadj : 0) : 0;
+    const int hi = BWD ? min(seg_hi, lo + pd.kadj) : seg_hi;
+    const int cnt_0 = idle_launch ? 0 : max(0, min(wns_0, hi) - lo);
+    const int cnt_1 = nslot > 1 && !idle_launch ? max(0, min(wns_1, hi) - lo) : 0;
     const int nit = max(cnt_0, cnt_1);
-    // first spline active in each slot's window: the origin of the slot's window-local
-    // alpha-gradient (adjoint)
-    const int slo_0 = BWD ? spline_first(pd, wn0_0) : 0;
-    const int slo_1 = BWD && nslot > 1 ? spline_first(pd, wn0_1) : 0;
-    // every step's splines fit the slot's window-local range (the index grows with the step, so
-    // a window's last step bounds them all; the host sizes the range with a margin): checked
-    // once per launch, a failure reported in the status word and the gradient left unfolded
-    const bool grad_fits =
-        !BWD || (spline_first(pd, wn0_0 + wns_0 - 1) - slo_0 + 2 < pd.gspan &&
-                 (nslot < 2 || spline_first(pd, wn0_1 + wns_1 - 1) - slo_1 + 2 < pd.gspan));
-    if (!grad_fits && threadIdx.x == 0) atomicOr(pd.status, ST_GRAD_RANGE);
     // global step of slot s at iteration jj, clamped into the slot's range (a slot without steps
     // in this launch maps to its window's first step, which exists)
     auto step_of = [&](int s, int jj) -> int64_t {
         const int cnt = s ? cnt_1 : cnt_0;
-        const int lo = s ? lo_1 : lo_0;
         const int64_t n0 = s ? wn0_1 : wn0_0;
         if (cnt <= 0) return n0;
         const int jc = min(jj, cnt - 1);
@@ -323,7 +278,6 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     const int m = tile.m0 + slot;                   // window, 1-based
     const int col = slot == 0 ? tile.c0 + c : c - ncol0;
     const int my_cnt = slot ? cnt_1 : cnt_0;
-    const int my_lo = slot ? lo_1 : lo_0;
     const int my_ns = slot ? wns_1 : wns_0;
     const size_t wcol = (size_t(m - 1) * E + col) * N;   // (window, column) in [M][E][N] arrays
 
@@ -373,7 +327,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
         if (my_cnt == 0) {
             u[l] = 0.0;
         } else if (BWD) {
-            u[l] = comp((my_lo + my_cnt == my_ns) ? pd.Lterm[wcol + i] : pd.Lstate[wcol + i], part);
+            u[l] = comp((lo + my_cnt == my_ns) ? pd.Lterm[wcol + i] : pd.Lstate[wcol + i], part);
         } else if (a.mode == SWEEP_RECOMPUTE) {
             u[l] = comp(pd.ckpt[((size_t(m - 1) * pd.nseg + a.seg) * E + col) * N + i], part);
         } else if (m + pd.m_off == 1) {
@@ -404,23 +358,22 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     };
 
     // ---- history blocks: slot s of a tile covers a contiguous column range of its window
-    const bool want_hist = !BWD && ((a.mode == SWEEP_HISTORY && pd.nseg == 1) || a.mode == SWEEP_RECOMPUTE);
+    const bool want_hist = BWD || (a.mode == SWEEP_HISTORY && pd.nseg == 1) || a.mode == SWEEP_RECOMPUTE;
     const bool want_ckpt = !BWD && a.mode == SWEEP_HISTORY && pd.nseg > 1;
     const uint32_t bytes_0 = static_cast<uint32_t>(size_t(ncol0) * N * sizeof(double2));
     const uint32_t bytes_1 = static_cast<uint32_t>(size_t(ncol - ncol0) * N * sizeof(double2));
     auto hist_ptr = [&](int s, int jj) -> double2* {
         const int64_t n0 = s ? wn0_1 : wn0_0;
-        const int lo = s ? lo_1 : lo_0;
-        const int jr = static_cast<int>(step_of(s, jj) - n0) - lo;   // step within the segment
-        return pd.hist + ((size_t(tile.m0 + s - 1) * pd.kseg + jr) * E + (s ? 0 : tile.c0)) * N;
+        const int jr = static_cast<int>(step_of(s, jj) - n0) - lo;   // step within the segment (chunk)
+        return (BWD ? pd.lhist : pd.hist) +
+               ((size_t(tile.m0 + s - 1) * (BWD ? pd.kadj : pd.kseg) + jr) * E + (s ? 0 : tile.c0)) * N;
     };
-    // Steps per history synchronisation: the midpoint states move in groups of hd iterations
-    // (iterations g hd .. g hd + hd - 1), one block of the tile's cpt N states per iteration.  The
-    // forward stages a group in H and stores it with one wait per group; the adjoint fetches
-    // group g into UB0 / UB1 (g even / odd) on mbar[g & 1], one group ahead.
+    // Steps per history synchronisation: the midpoint states are staged in H in groups of hd
+    // iterations (g hd .. g hd + hd - 1), one block of the tile's cpt N states per iteration, and
+    // a group is stored with one wait.
     const int hd = a.hdepth;
     const size_t hstride = size_t(a.cpt) * N;
-    // forward (thread 0): store the staged group starting at iteration g0 (every slot with a step)
+    // thread 0: store the staged group starting at iteration g0 (every slot with a step)
     auto publish_group = [&](int g0) {
         const int g1 = min(g0 + hd, nit);
         for (int j = g0; j < g1; ++j) {
@@ -429,32 +382,8 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
             if (j < cnt_1) bulk_s2g(hist_ptr(1, j), src + size_t(ncol0) * N, bytes_1);
         }
     };
-    // adjoint (thread 0): fetch the group starting at iteration g0 into dst, completing on bar
-    auto fetch_group = [&](double2* dst, int g0, uint64_t* bar) {
-        const int g1 = min(g0 + hd, nit);
-        uint32_t total = 0;
-        for (int j = g0; j < g1; ++j) total += (j < cnt_0 ? bytes_0 : 0u) + (j < cnt_1 ? bytes_1 : 0u);
-        mbar_expect_tx(bar, total);
-        for (int j = g0; j < g1; ++j) {
-            double2* d = dst + size_t(j - g0) * hstride;
-            if (j < cnt_0) bulk_g2s(d, hist_ptr(0, j), bytes_0, bar);
-            if (j < cnt_1) bulk_g2s(d + size_t(ncol0) * N, hist_ptr(1, j), bytes_1, bar);
-        }
-    };
-
-    if (BWD) {
-        for (int j = tid; j < 2 * a.gmax; j += blockDim.x) galpha[j] = 0.0;
-        if (tid == 0) {
-            mbar_init(&mbar[0], 1);
-            mbar_init(&mbar[1], 1);
-            fence_mbar_init();
-        }
-        tile_sync();
-        if (tid == 0 && nit > 0) fetch_group(UB0, 0, &mbar[0]);
-    }
-
-    // warp s < nslot computes slot s's coefficients and folds its gradient; it keeps d_k and
-    // the iteration counts of the slot's next step in registers (lane -> subsystem of its slot)
+    // warp s < nslot computes slot s's coefficients and keeps d_k and the iteration counts of
+    // the slot's next step in registers (lane -> subsystem of its slot)
     const bool coef_warp = warp < nslot;
     const int cslot = coef_warp ? warp : 0;
     const int my_k = (lane < NSLOT) ? (lane / (2 * L)) : 0;
@@ -467,63 +396,12 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
             cnt_next = pd.spl[n].cnt;
         }
     };
-    // gradient entries of a step: (carrier, spline of the 3 active) pairs, one per lane; the
-    // carrier, spline offset and subsystem of this lane's first entry are fixed for the launch
-    const int nscat = pd.nfsum * 3;
-    const int f_kf = lane / 3, f_jw = lane % 3;
-    int f_k = 0;
-    while (f_k + 1 < Q && pd.cof[f_k + 1] <= f_kf) ++f_k;
-    // warps whose lanes belong to both slots reduce each slot separately
-    const unsigned mask1 = __ballot_sync(0xffffffffu, act && slot == 1);
-    const unsigned mask0 = __ballot_sync(0xffffffffu, act && slot == 0);
-
-    // fold slot s's reduced products of step np (parity pp of the reduction buffers) into the
-    // slot's alpha-gradient: dP/dalpha1_kfs += -2h B_s Im(e^{iWt} z_k + e^{-iWt} y_k),
-    // dP/dalpha2_kfs += -2h B_s Re(e^{iWt} z_k - e^{-iWt} y_k)  (Eq. grad-int at the midpoint).
-    // Value v = 4k + j (j: Re z, Im z, Re y, Im y) was reduced by part j & 1 at index 2k + (j >> 1).
-    auto fold = [&](int s, int pp, int64_t np, const Spline4& sp, double2 ph_lane, bool prefetched) {
-        if (lane < 4 * Q) {
-            const int j = lane & 3, kk = lane >> 2;
-            const int pos = (j & 1) * VH + 2 * kk + (j >> 1);
-            double sum = 0.0;
-            for (int w2 = 0; w2 < nwarps; ++w2) sum += red[((pp * 2 + s) * nwarps + w2) * V + pos];
-            zy[(pp * 2 + s) * 4 * Q + lane] = sum;
-        }
-        __syncwarp();
-        if (!grad_fits) return;
-        const int s0 = sp.s - (s ? slo_1 : slo_0);   // first active spline, window-local
-        double* ga = galpha + size_t(s) * a.gmax;
-        for (int i = lane; i < nscat; i += 32) {
-            int kf = f_kf, jw = f_jw, k = f_k;   // this lane's first entry, precomputed
-            if (i != lane) {
-                kf = i / 3;
-                jw = i % 3;
-                k = 0;
-                while (k + 1 < Q && pd.cof[k + 1] <= kf) ++k;
-            }
-            const double* zyk = zy + (pp * 2 + s) * 4 * Q + 4 * k;
-            const double2 zk = make_double2(zyk[0], zyk[1]);
-            const double2 yk = make_double2(zyk[2], zyk[3]);
-            const double2 ph = (prefetched && i == lane) ? ph_lane : pd.phase[size_t(np) * pd.nfsum + kf];
-            const double wgt = -2.0 * pd.h * (jw == 0 ? sp.w0 : (jw == 1 ? sp.w1 : sp.w2));
-            const double A = zk.y + yk.y, B = zk.x - yk.x;
-            const int idx = (kf * pd.gspan + s0 + jw) * 2;
-            ga[idx + 0] += wgt * fma(ph.x, A, ph.y * B);
-            ga[idx + 1] += wgt * fma(ph.x, B, -ph.y * A);
-        }
-    };
-
-    __shared__ int tflag_s;   // a bounded history wait gave up (adjoint)
-    int* tflag = &tflag_s;
-    if (tid == 0) tflag_s = 0;
-    // (the first barrier of the loop orders this store before every read of the flag)
-    bool timed_out = false;
     int fsel = 0;
     double2* Dc = D0;   // FP64-solver ping-pong buffers
     double2* Dn = D1;
     if (nit > 0) load_ctrl(0);
 
-    int hpos = 0, hgrp = 0;   // iteration jj = hgrp hd + hpos (history group and position)
+    int hpos = 0;   // position of iteration jj in its history group
     for (int jj = 0; jj < nit; ++jj) {
         const int par = jj & 1;
         const bool live = jj < my_cnt;
@@ -533,15 +411,6 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
             if (jj + 1 < nit) load_ctrl(jj + 1);
             step_coefficients_pair<L, Q>(pd, lane, dk, cnt, coef_d + (par * 2 + cslot) * 2 * NSLOT,
                                     coef_f + (par * 2 + cslot) * 2 * NSLOT, params + (par * 2 + cslot) * 4);
-        }
-        // adjoint: the folding warps fetch what the fold of iteration jj - 1 needs now, so the
-        // loads are in flight during the solve
-        Spline4 sp_prev{};
-        double2 ph_prev = make_double2(0.0, 0.0);
-        if (BWD && jj > 0 && coef_warp && jj - 1 < (cslot ? cnt_1 : cnt_0)) {
-            const int64_t np = step_of(cslot, jj - 1);
-            sp_prev = pd.spl[np];
-            if (lane < nscat) ph_prev = pd.phase[size_t(np) * pd.nfsum + lane / 3];
         }
         // checkpoint: the state at the start of every segment (forward over whole windows)
         if (want_ckpt && live && act && jj % pd.kseg == 0)
@@ -563,16 +432,11 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
         double z[LS];   // this part of the midpoint state being solved for (Ubar or Lbar)
 
         // first barrier of the step: the coefficients are published; thread 0 stores the
-        // previous iteration's midpoints (forward) or fetches the next iteration's (adjoint)
+        // previous group's midpoints
         auto first_sync_work = [&]() {
-            if (BWD && *tflag) timed_out = true;   // uniform: read after a barrier
-            if (!BWD && want_hist && tid == 0 && jj > 0 && hpos == 0) {
+            if (want_hist && tid == 0 && jj > 0 && hpos == 0) {
                 fence_proxy_async_smem();
                 publish_group(jj - hd);
-            }
-            if (BWD && tid == 0 && hpos == 0 && jj + hd < nit) {
-                const int gn = hgrp + 1;
-                fetch_group((gn & 1) ? UB1 : UB0, jj + hd, &mbar[gn & 1]);
             }
         };
 
@@ -584,7 +448,6 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
             if (act) store_part<LS, double2>(Dc, fb.xo + le, part, z);
             tile_sync();
             first_sync_work();
-            if (timed_out) break;
             const int Kown = prm[0];
             const int Kmax = nslot > 1 ? max(prm0[0], prm1[0]) : prm0[0];
             for (int it = 0; it < Kmax; ++it) {
@@ -619,7 +482,6 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 if (act) store_part<LS, float2>(Fb, fb.xo + le, part, y);
                 tile_sync();
                 first_sync_work();
-                if (timed_out) break;
                 float w[LS];
                 apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, exo, pd);
 #pragma unroll
@@ -658,10 +520,10 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
             }
             for (int pass = 0;; ++pass) {
                 if (act) store_part<LS, double2>(D0, fb.xo + le, part, z);
-                // forward: the staged midpoints of the previous step must have been read by their
+                // the staged midpoints of the previous step must have been read by their
                 // bulk store (issued at this step's first barrier) before this step's are staged;
                 // waiting here, ahead of a barrier every step has, makes the staging barrier-free
-                if (!BWD && want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
+                if (want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
                 tile_sync();
                 double w[LS];
                 apply_off_pair<L, Q, double2, SPLIT>(D0, cfd, fb, z, w, part, le, exo, pd);
@@ -707,23 +569,23 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
 
         if (tid == 0 && (prm0[3] || (nslot > 1 && prm1[3]))) atomicOr(pd.status, ST_SOLVER_RANGE);
 
-        if constexpr (!BWD) {
-            // ---- midpoint states for the adjoint sweep (async bulk store at the next step)
-            if (want_hist) {
-                if constexpr (SOLVER == SOLVER_FP64) {
-                    // (the FP64 solver's step may have no barrier after the first one)
-                    if (hpos == 0) {
-                        if (tid == 0) bulk_wait_read_all();
-                        tile_sync();
-                    }
+        // ---- midpoint states for the quadrature (async bulk store at the next step)
+        if (want_hist) {
+            if constexpr (SOLVER == SOLVER_FP64) {
+                // (the FP64 solver's step may have no barrier after the first one)
+                if (hpos == 0) {
+                    if (tid == 0) bulk_wait_read_all();
+                    tile_sync();
                 }
-                if (act && live) store_part<LS, double2>(H + size_t(hpos) * hstride, fb.xo + le, part, z);
-                fence_proxy_async_smem();
             }
-            if (live) {
+            if (act && live) store_part<LS, double2>(H + size_t(hpos) * hstride, fb.xo + le, part, z);
+            fence_proxy_async_smem();
+        }
+        if (live) {
 #pragma unroll
-                for (int l = 0; l < LS; ++l) u[l] = fma(2.0, z[l], -u[l]);
-            }
+            for (int l = 0; l < LS; ++l) u[l] = fma(2.0, z[l], -u[l]);
+        }
+        if constexpr (!BWD) {
             // roll-out: U(t_m) when the step ends on a window boundary t_m, i.e. when n + 1 =
             // floor(m N_T / M) for some 1 <= m < M; the only candidate is m = ceil((n+1) M / N_T)
             if (rollout && live && act) {
@@ -732,156 +594,20 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 if (mb >= 1 && mb < pd.M && (mb * pd.nsteps) / pd.M == n1)
                     store_fiber(a.out + (size_t(mb - 1) * E + col) * N);
             }
-        } else {
-            // ---- gradient quadrature on the midpoints (fused): needs Ubar_n of the tile
-            double2* UB = ((hgrp & 1) ? UB1 : UB0) + size_t(hpos) * hstride;
-            // this part's products conj(Lbar) x Ubar: Re (part 0) = Lr Ur + Li Ui = za Ur + zb Ui,
-            // Im (part 1) = Lr Ui - Li Ur = za Ur + zb Ui with (za, zb) = (-Li, Lr)
-            double za[LS], zb[LS];
-#pragma unroll
-            for (int l = 0; l < LS; ++l) {
-                const double zo = partner(z[l]);
-                za[l] = part ? -z[l] : z[l];
-                zb[l] = zo;
-            }
-            // a wait that gives up raises the tile's flag, read after the next barrier (the
-            // products below then use whatever landed; the evaluation reports the timeout)
-            if (hpos == 0 && !mbar_wait(&mbar[hgrp & 1], (hgrp >> 1) & 1)) *tflag = 1;
-            double acc[VH];   // index 2k: z_k, 2k + 1: y_k (this part's component)
-#pragma unroll
-            for (int v = 0; v < VH; ++v) acc[v] = 0.0;
-            auto prod = [&](double s0, int l, double2 x) { return fma(za[l], x.x, fma(zb[l], x.y, s0)); };
-            if constexpr (SPLIT > 1) {
-                // last subsystem, lane quads (L = 2): entry 0 gives z (conj(Lbar_0) Ubar_1),
-                // entry 1 gives y (conj(Lbar_1) Ubar_0); every weight is 1
-                constexpr int kl = Q - 1;
-                const double pq = prod(0.0, 0, UB[fb.xo + 1 - le]);
-                acc[2 * kl + 0] = le ? 0.0 : pq;
-                acc[2 * kl + 1] = le ? pq : 0.0;
-            } else {
-                // last subsystem (stride 1) from the fiber itself
-                constexpr int kl = Q - 1;
-                double zq = 0.0, yq = 0.0;
-#pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    // z: conj(Lbar_l) sqrt(l+1) Ubar_{l+1};  y: conj(Lbar_l) sqrt(l) Ubar_{l-1}
-                    if (l < L - 1) {
-                        const double wz = sqrt_small(l + 1);   // folded after unrolling
-                        if (wz == 1.0)
-                            zq = prod(zq, l, UB[fb.xo + l + 1]);
-                        else
-                            zq = fma(wz, prod(0.0, l, UB[fb.xo + l + 1]), zq);
-                    }
-                    if (l > 0) {
-                        const double wy = sqrt_small(l);
-                        if (wy == 1.0)
-                            yq = prod(yq, l, UB[fb.xo + l - 1]);
-                        else
-                            yq = fma(wy, prod(0.0, l, UB[fb.xo + l - 1]), yq);
-                    }
-                }
-                acc[2 * kl + 0] = zq;
-                acc[2 * kl + 1] = yq;
-            }
-#pragma unroll
-            for (int k = 0; k < Fiber<L, Q>::NFIX; ++k) {
-                double p1 = 0.0;
-                const double2* q1 = UB + fb.nb1[k] + le;
-#pragma unroll
-                for (int l = 0; l < LS; ++l) p1 = prod(p1, l, q1[l]);
-                const double pv = fb.w1[k] * p1;
-                acc[2 * k + 0] = fb.plus1[k] ? pv : 0.0;
-                acc[2 * k + 1] = fb.plus1[k] ? 0.0 : pv;
-                if (fb.two[k]) {
-                    double p2 = 0.0;
-                    const double2* q2 = UB + fb.nb2[k] + le;
-#pragma unroll
-                    for (int l = 0; l < LS; ++l) p2 = prod(p2, l, q2[l]);
-                    acc[2 * k + 1] = fb.w2[k] * p2;
-                }
-            }
-            if (!act || !live) {
-#pragma unroll
-                for (int v = 0; v < VH; ++v) acc[v] = 0.0;
-            }
-            // per-slot sums over each part's lanes: lane (lane >> (5 - NH)) == vi of part p holds
-            // value vi of part p, stored at p VH + vi
-            {
-                const int vi = lane >> (5 - NH);
-                const bool writer = (lane & ((1 << (5 - NH)) - 2)) == 0;
-                const int pos = part * VH + vi;
-                double* r0 = red + ((par * 2 + 0) * nwarps + warp) * V;
-                double* r1 = red + ((par * 2 + 1) * nwarps + warp) * V;
-                if (mask0 && mask1) {
-                    // lanes of both windows: reduce the window-1 lanes on a copy first
-                    double t[VH];
-#pragma unroll
-                    for (int v = 0; v < VH; ++v) t[v] = slot == 1 ? acc[v] : 0.0;
-                    const double s1 = part_reduce_scatter<VH, NH>(t, lane);
-#pragma unroll
-                    for (int v = 0; v < VH; ++v) acc[v] = slot == 0 ? acc[v] : 0.0;
-                    const double s0 = part_reduce_scatter<VH, NH>(acc, lane);
-                    if (writer) {
-                        r0[pos] = s0;
-                        r1[pos] = s1;
-                    }
-                } else {
-                    const double sv = part_reduce_scatter<VH, NH>(acc, lane);
-                    if (writer) {
-                        r0[pos] = mask1 ? 0.0 : sv;
-                        if (nslot > 1) r1[pos] = mask1 ? sv : 0.0;
-                    }
-                }
-            }
-            // Lambda_n = 2 Lbar - Lambda_{n+1}
-            if (live) {
-#pragma unroll
-                for (int l = 0; l < LS; ++l) u[l] = fma(2.0, z[l], -u[l]);
-            }
         }
-
-        // the folding warps add iteration jj - 1's reduced products into the alpha-gradient
-        // (the barrier that published red[par ^ 1] was this iteration's first one)
-        if (BWD && jj > 0 && coef_warp && jj - 1 < (cslot ? cnt_1 : cnt_0))
-            fold(cslot, par ^ 1, step_of(cslot, jj - 1), sp_prev, ph_prev, true);
-        if (++hpos == hd) {
-            hpos = 0;
-            ++hgrp;
-        }
+        if (++hpos == hd) hpos = 0;
     }
 
-    if (!timed_out) {
-        tile_sync();
-        if (BWD && *tflag) timed_out = true;   // the last step's wait (uniform: after the barrier)
+    tile_sync();
+    if (want_hist && tid == 0 && nit > 0) {
+        fence_proxy_async_smem();
+        publish_group(((nit - 1) / hd) * hd);
+        bulk_wait_all();
     }
-    if (!timed_out) {
-        if constexpr (!BWD) {
-            if (want_hist && tid == 0 && nit > 0) {
-                fence_proxy_async_smem();
-                publish_group(((nit - 1) / hd) * hd);
-                bulk_wait_all();
-            }
-            if (a.mode != SWEEP_RECOMPUTE && !rollout && act && my_cnt > 0) store_fiber(pd.Uend + wcol);
-        } else {
-            // the last fold of every slot whose range ends at the last iteration
-            if (coef_warp && nit > 0 && (cslot ? cnt_1 : cnt_0) == nit) {
-                const int64_t np = step_of(cslot, nit - 1);
-                fold(cslot, (nit - 1) & 1, np, pd.spl[np], make_double2(0.0, 0.0), false);
-            }
-            tile_sync();
-            // the tile's alpha-gradient partial, accumulated over the segment launches (the first
-            // adjoint launch is the last segment's)
-            double* gp = pd.gpart + size_t(tile.tloc) * pd.d;
-            const bool first_launch = a.seg == pd.nseg - 1;
-            store_grad_partial(gp, galpha, pd, a.gmax, slo_0, nslot > 1 ? slo_1 : -1, first_launch);
-            // Lambda at the segment start: Lambda^m(t_{m-1}) for the window's first segment
-            if (act && my_cnt > 0) store_fiber((my_lo == 0 ? pd.Lam0 : pd.Lstate) + wcol);
-        }
-    } else if (tid == 0) {
-        atomicOr(pd.status, ST_TIMEOUT);
-        // let the bulk copies this tile issued land before its shared memory is released
-        for (int p2 = 0; p2 < 2; ++p2) (void)mbar_wait(&mbar[p2], 0), (void)mbar_wait(&mbar[p2], 1);
-    }
+    // forward: U^m(t_m); adjoint: Lambda at the launch's first step (Lambda^m(t_{m-1}) for the
+    // window's first)
+    if (act && my_cnt > 0 && !rollout && a.mode != SWEEP_RECOMPUTE)
+        store_fiber((!BWD ? pd.Uend : (lo == 0 ? pd.Lam0 : pd.Lstate)) + wcol);
 }
 
 }  // namespace msqoc
