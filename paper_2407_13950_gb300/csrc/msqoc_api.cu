@@ -406,6 +406,8 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
                     pd.rho_ex += pd.h * (L - 1) * std::fabs(H->jx[j * q + k]);
                     ++pd.nex;
                 }
+    pd.kap = 0.0;
+    for (int i = 0; i < pd.N; ++i) pd.kap = std::max(pd.kap, std::fabs(0.5 * pd.h * drift_entry(H, q, L, i)));
     for (int l = 0; l < MAXL; ++l) {
         pd.sc[2 * l + 0] = 0.5 * pd.h * std::sqrt(double(l + 1));
         pd.sc[2 * l + 1] = 0.5 * pd.h * std::sqrt(double(l));
@@ -844,11 +846,12 @@ msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s) {
 
 bool split_history(const ProbDev& pd) { return pd.solver == SOLVER_MIXED && pd.pair == 0; }
 
-// blocks of the quadrature kernel: per window, the chunk's steps in groups of 32 lanes
+// blocks of the quadrature kernel: per window, the chunk's steps in groups of its staged lanes
 int quad_blocks(const ProbDev& pd) {
+    const int most = pd.N <= 128 ? 32 : 16;   // quad_lanes
     int lanes = 1;
-    while (lanes < pd.E && lanes < 32) lanes <<= 1;
-    const int per = 32 / lanes;
+    while (lanes < pd.E && lanes < most) lanes <<= 1;
+    const int per = most / lanes;
     return pd.M * ((pd.kadj + per - 1) / per);
 }
 

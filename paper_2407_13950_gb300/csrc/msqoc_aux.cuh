@@ -8,33 +8,41 @@ namespace msqoc {
 
 // Iteration counts of the implicit-midpoint solve of one step from the contraction bound
 // rho = ||P iX_C|| <= (h/2) lam sum_k |d_k(t_{n+1/2})| of the diagonally preconditioned
-// fixed point (P = (I + i h/2 D)^-1).  Packed as j1 | j2 << 8 | passes << 16 | bad << 24.
+// fixed point (P = (I + i kappa)^-1, kappa = (h/2) D) and kap = max |kappa|.  Packed as j1 | j2 << 8 |
+// passes << 16 | bad << 24 | coarse << 25.
 //   FP64 solver : j1 = K sweeps with rho^(K+1) <= 2^-56.
-//   mixed solver: the FP32 stage leaves the error e1 = c u32 rho + rho^(j1+1) relative to
-//     |P rhs| (FP32 rounding of the right-hand side and of the sweeps, times the contraction,
-//     plus truncation); each FP64 residual + FP32 correction multiplies it by
-//     phi = c u32 + rho^(j2+1).  c = 4 rounding units per FP32 sweep output; target: the FP64
-//     unit roundoff 2^-53.  An FP64 pass costs far more than FP32 sweeps, so the fewest passes R
-//     are taken first, then the fewest FP32 sweeps j1 + j2 (each sweep is a barrier of the
-//     tile), then the smaller j2.
+//   mixed solver, one thread per fiber: the FP32 estimate m0 of the increment m = z - U leaves the
+//     error e1 = u32 (2 kap + c rho) + rho^(j1+1) relative to |U| (its roundings plus truncation);
+//     a pass forms the increment at U + m0 in compensated FP32 and solves for the correction in
+//     FP32, whose part that is added to the increment carries the same factor
+//     phi = u32 (2 kap + c rho) + rho^(j2+1).  c = 4 rounding units per FP32 sweep output; target:
+//     the FP64 unit roundoff 2^-53.  The fewest passes are taken first (a pass costs far more than
+//     a sweep), then the fewest sweeps j1 + j2 (each is a barrier of the tile), then the smaller j2.
+//   mixed solver, lane pairs and quads: the FP32 stage leaves e1 = c u32 rho + rho^(j1+1) relative to
+//     |P rhs|; each FP64 residual + FP32 correction multiplies it by phi = c u32 + rho^(j2+1).
+//   coarse (one thread per fiber): the compensated increment's error, about 2^-49 of its leading
+//     terms (rms), stays below the FP64 rounding of the state where kap <= 2^-4 and rho <= 2^-5;
+//     other steps are taken in FP64 (j1 = K sweeps as the FP64 solver).
 //   bad: rho >= 1/2, outside the range the counts are derived for.
-__device__ inline int step_counts(int solver, float rho) {
+__device__ inline int step_counts(int solver, int pair, float rho, float kap) {
     int a = 1, b = 1, r = 1, bad = 0;
+    const int coarse = solver == SOLVER_MIXED && !pair && (rho > 0.03125f || kap > 0.0625f) ? 1 : 0;
     if (rho > 1e-30f) {
         const float lr = logf(rho);
-        if (solver == SOLVER_FP64) {
+        if (solver == SOLVER_FP64 || coarse) {
             a = int(ceilf(-38.8162f / lr)) - 1;   // log(2^-56) = -38.816
             a = a < 1 ? 1 : (a > 60 ? 60 : a);
         } else {
             const float u32 = 5.9604645e-8f, c = 4.f, target = 1.1102230e-16f;
+            const float f1 = pair ? c * u32 * rho : u32 * (2.f * kap + c * rho), f2 = pair ? c * u32 : f1;
             const int j0 = max(1, min(30, int(ceilf(logf(u32) / lr))));   // rho^j0 <= u32
             r = 0;
             for (int pass = 1; pass <= 6 && r == 0; ++pass) {
                 int best = 0;
                 for (int ja = 1; ja <= j0 + 2; ++ja) {
-                    const float e1 = c * u32 * rho + __powf(rho, float(ja + 1));
+                    const float e1 = f1 + __powf(rho, float(ja + 1));
                     for (int jb = 1; jb <= j0 + 1; ++jb) {
-                        const float phi = c * u32 + __powf(rho, float(jb + 1));
+                        const float phi = f2 + __powf(rho, float(jb + 1));
                         float e = e1;
                         for (int t = 0; t < pass; ++t) e *= phi;
                         if (e <= target && (best == 0 || ja + jb < best || (ja + jb == best && jb < b))) {
@@ -54,10 +62,7 @@ __device__ inline int step_counts(int solver, float rho) {
         }
         if (rho >= 0.5f) bad = 1;
     }
-    // the compensated FP32 apply of the residual (error about 2^-47 |P iX_C z| <= 2^-47 rho |z|)
-    // stays below the FP64 rounding of z (2^-53 |z|) for rho <= 2^-7; above, the FP64 apply
-    const int f64_apply = rho > 0.0078125f ? 1 : 0;
-    return a | (b << 8) | (r << 16) | (bad << 24) | (f64_apply << 25);
+    return a | (b << 8) | (r << 16) | (bad << 24) | (coarse << 25);
 }
 
 // The quadratic cardinal B-splines active at time t: on [j dtau, (j+1) dtau) the three
@@ -101,7 +106,7 @@ __global__ void k_controls(const ProbDev pd) {
             mag += sqrt(dk.x * dk.x + dk.y * dk.y);
         }
         const float rho = float(0.5 * pd.h * pd.lam * mag + pd.rho_ex) * 1.0001f;
-        pd.spl[n] = Spline4{sp.s0, step_counts(pd.solver, rho), sp.w0, sp.w1, sp.w2};
+        pd.spl[n] = Spline4{sp.s0, step_counts(pd.solver, pd.pair, rho, float(pd.kap)), sp.w0, sp.w1, sp.w2};
     }
 }
 

@@ -81,6 +81,7 @@ struct ProbDev {
     int ex_j[MAXEX], ex_k[MAXEX];
     double ex_c[MAXEX];
     double rho_ex;
+    double kap;                  // max |(h/2) D_i| over the rows: the largest diagonal rotation of a step
     double wsq[2 * MAXL];        // sqrt(l+1) [dir +] and sqrt(l) [dir -]: product weights
     // constant tables
     const double2* P;            // [N] (1 + i h/2 D_i)^-1

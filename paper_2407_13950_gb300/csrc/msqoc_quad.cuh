@@ -8,12 +8,20 @@
 // Unlike the sweeps, the steps here are independent: the products run at the GPU's throughput
 // instead of adding to the latency of every adjoint step.
 //
-// One CTA takes SPW consecutive steps of a window, SPW = 32 / EL with EL = the columns rounded up
-// to a power of two (at most 32; more columns run in blocks of 32).  A lane is one column of
-// one step, a warp one fiber (the L entries that differ in the last subsystem's level) at a time,
-// so every branch on a level is warp-uniform and every lane of a warp does the same products.  The
-// states are staged in shared memory transposed to [row][lane] (33 lanes a row: conflict-free
-// both ways) with 16-byte asynchronous copies, and each product operand is one 16-byte load.
+// One CTA takes SPW consecutive steps of a window, SPW = LN / EL with EL = the columns rounded up to
+// a power of two (at most LN; more columns run in blocks of LN).  A lane is one column of one step.
+// The terms of subsystem k and weight sqrt(j) are the N / L row pairs (i, i') with l_k = j - 1 and
+// j: a warp takes one (k, j) and does, per pair, conj(L_i) U_i' (the a_k term) and conj(L_i') U_i (the
+// a_k^+ term), so every lane of a warp does the same eight real products, there is no branch in
+// the loop and every warp has the same work.  The states are staged in shared memory transposed
+// to [row][lane] (one padding lane a row: conflict-free both ways) with 16-byte asynchronous copies.
+// Split states sum a few pairs at a time in fresh two-float sums (their low parts round relative
+// to the partial sum) before those join the running sum.
+// 4 transmons, 100000 steps: 2.08 ms (4.1 GB read, 2.0 TB/s; the products' FP32 operations alone
+// would take 0.8 ms), against 2.71 ms for one fiber a warp with a branch per level and 37% more
+// instructions.  Issue-bound: a staged CTA holds 85 KB, so two are resident on an SM.
+// LN = 32, or 16 for shapes whose staging would not fit (the half-warps then take alternate groups
+// of pairs).
 #pragma once
 
 #include <type_traits>
@@ -32,23 +40,33 @@ __device__ __forceinline__ DF gsum_shfl_xor(DF v, int o) {
 }
 __device__ __forceinline__ void gsum_zero(double& v) { v = 0.0; }
 __device__ __forceinline__ void gsum_zero(DF& v) { v = DF{0.f, 0.f}; }
-__device__ __forceinline__ double gsum_weight(double v, int j) { return j == 1 ? v : v * sqrt_small(j); }
-__device__ __forceinline__ DF gsum_weight(DF v, int j) { return df_scale_sqrt(v, j); }
-
-// (R, I) += (SR Re, Im) of conj(x) u
-template <int SR>
-__device__ __forceinline__ void cjmac_acc(DF& R, DF& I, const float4& x, const float4& u) {
-    df_mac(R, SR > 0 ? x.x : -x.x, SR > 0 ? x.z : -x.z, u.x, u.z);
-    df_mac(R, SR > 0 ? x.y : -x.y, SR > 0 ? x.w : -x.w, u.y, u.w);
-    df_mac(I, x.x, x.z, u.y, u.w);
-    df_mac(I, -x.y, -x.w, u.x, u.z);
+// R = Re(conj(x) u') - Re(conj(x') u), I = Im(conj(x) u') + Im(conj(x') u): added to R, I, or (FIRST)
+// the first terms of those sums
+template <bool FIRST>
+__device__ __forceinline__ void pair_products(DF& R, DF& I, const float4& x, const float4& x2, const float4& u,
+                                              const float4& u2) {
+    if constexpr (FIRST) {
+        R = dot2_df(x.x, x.z, u2.x, u2.z, x.y, x.w, u2.y, u2.w);
+        I = dot2_df(x.x, x.z, u2.y, u2.w, -x.y, -x.w, u2.x, u2.z);
+    } else {
+        df_mac(R, x.x, x.z, u2.x, u2.z);
+        df_mac(R, x.y, x.w, u2.y, u2.w);
+        df_mac(I, x.x, x.z, u2.y, u2.w);
+        df_mac(I, -x.y, -x.w, u2.x, u2.z);
+    }
+    df_mac(R, -x2.x, -x2.z, u.x, u.z);
+    df_mac(R, -x2.y, -x2.w, u.y, u.w);
+    df_mac(I, x2.x, x2.z, u.y, u.w);
+    df_mac(I, -x2.y, -x2.w, u.x, u.z);
 }
-template <int SR>
-__device__ __forceinline__ void cjmac_acc(double& R, double& I, const double2& x, const double2& u) {
-    R = fma(SR > 0 ? x.x : -x.x, u.x, R);
-    R = fma(SR > 0 ? x.y : -x.y, u.y, R);
-    I = fma(x.x, u.y, I);
-    I = fma(-x.y, u.x, I);
+template <bool FIRST>
+__device__ __forceinline__ void pair_products(double& R, double& I, const double2& x, const double2& x2,
+                                              const double2& u, const double2& u2) {
+    if constexpr (FIRST) R = I = 0.0;
+    R = fma(x.x, u2.x, fma(x.y, u2.y, R));
+    I = fma(x.x, u2.y, fma(-x.y, u2.x, I));
+    R = fma(-x2.x, u.x, fma(-x2.y, u.y, R));
+    I = fma(x2.x, u.y, fma(-x2.y, u.x, I));
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -56,40 +74,40 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// warps of a CTA: a divisor of the fibers (3-level shapes: 1, 3, 9 a shape of 3^(q-1) fibers)
+// staged lanes, warps and staging bytes of a CTA
 template <int L, int Q>
-__host__ __device__ constexpr int quad_warps() {
-    constexpr int F = ipow_c(L, Q - 1);
-    return L == 3 ? (F < 9 ? F : 9) : (F < 8 ? F : 8);
+__host__ __device__ constexpr int quad_lanes() { return ipow_c(L, Q) <= 128 ? 32 : 16; }
+template <int L, int Q>
+__host__ __device__ constexpr int quad_split() {   // warps that share one (k, j)
+    return ipow_c(L, Q) > 128 ? 2 : 1;
 }
-// states of at most this many rows are staged for both operands; of larger ones only Ubar (every
-// entry of Lbar is read by one thread, every entry of Ubar by up to 2 q)
-constexpr int QUAD_STAGE_ROWS = 128;
+template <int L, int Q>
+__host__ __device__ constexpr int quad_warps() { return Q * (L - 1) * quad_split<L, Q>(); }
 template <int L, int Q>
 __host__ __device__ constexpr size_t quad_smem() {
-    constexpr int N = ipow_c(L, Q);
-    constexpr size_t stage = size_t(N) * 33 * 16 * (N <= QUAD_STAGE_ROWS ? 2 : 1);
-    constexpr size_t sums = size_t(quad_warps<L, Q>()) * 32 * 2 * Q * 8;   // at one column a step
+    constexpr size_t stage = size_t(ipow_c(L, Q)) * (quad_lanes<L, Q>() + 1) * 16 * 2;
+    constexpr size_t sums = size_t(quad_warps<L, Q>()) * 32 * 2 * 8;   // at one column a step
     return stage > sums ? stage : sums;
 }
 
 template <int L, int Q, bool SPLIT>
 __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs a) {
-    constexpr int N = ipow_c(L, Q), F = N / L, NW = quad_warps<L, Q>();
-    constexpr int V = next_pow2_c(2 * Q);
-    constexpr bool STAGE_L = N <= QUAD_STAGE_ROWS;
+    constexpr int N = ipow_c(L, Q), F = N / L, NW = quad_warps<L, Q>(), LN = quad_lanes<L, Q>();
+    constexpr int WS = quad_split<L, Q>();
+    constexpr int UN = L == 3 ? (F < 3 ? 1 : 3) : (F < 4 ? F : 4);   // pairs summed afresh; divides F
+    constexpr int ROW = LN + 1;
     using GT = std::conditional_t<SPLIT, DF, double>;
     using ET = std::conditional_t<SPLIT, float4, double2>;
     const ProbDev& pd = a.pds[a.list ? a.list[blockIdx.y] : blockIdx.y];
     const int E = pd.E;
-    const int EL = E >= 32 ? 32 : (E <= 1 ? 1 : 1 << (32 - __clz(E - 1)));
+    const int EL = E >= LN ? LN : (E <= 1 ? 1 : 1 << (32 - __clz(E - 1)));
     extern __shared__ __align__(128) unsigned char smem[];
     ET* Us = reinterpret_cast<ET*>(smem);
-    ET* Ls = Us + (STAGE_L ? N * 33 : 0);
-    GT* red = reinterpret_cast<GT*>(smem);                   // [NW][spw][2 Q], over the staged states
+    ET* Ls = Us + N * ROW;
+    GT* red = reinterpret_cast<GT*>(smem);                   // [NW][spw][2], over the staged states
 
     // ---- this CTA's steps: group g of window m, local steps [j0, j0 + spw) of the chunk
-    const int spw = 32 / EL;
+    const int spw = LN / EL;
     const int groups = (pd.kadj + spw - 1) / spw;
     const int m = blockIdx.x / groups;                       // window, 0-based
     if (m >= pd.M) return;
@@ -100,8 +118,15 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
     const int hi = min(min(ns, (a.seg + 1) * pd.kseg), lo + pd.kadj);
     if (lo + j0 >= hi) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int sl = lane / EL, cl = lane % EL;                // step and column of the lane
+    const int half = lane / LN;                              // 0, or the half-warp (LN = 16)
+    const int ln = lane % LN, sl = ln / EL, cl = ln % EL;    // staged lane; its step and column
     const bool live = lo + j0 + sl < hi;
+    const int k = warp / ((L - 1) * WS), j = 1 + (warp / WS) % (L - 1);
+    const int st = [&] {                                     // the stride of subsystem k's level
+        int t = 1;
+        for (int e = k; e < Q - 1; ++e) t *= L;
+        return t;
+    }();
 
     // power-of-two units: the products of column c are in units 2^(shL + shU), the same at every
     // step of the chunk; a step sums them in units 2^S, the largest over its columns
@@ -114,12 +139,12 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
         for (int o = EL >> 1; o > 0; o >>= 1) S = max(S, __shfl_xor_sync(0xffffffffu, S, o));
     }
 
-    GT tot[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) gsum_zero(tot[v]);
-    for (int cb = 0; cb < E; cb += 32) {
-        const int nc = min(E - cb, 32);                      // columns of this block
-        // ---- stage Ubar (and Lbar) transposed
+    GT A, B;
+    gsum_zero(A);
+    gsum_zero(B);
+    for (int cb = 0; cb < E; cb += LN) {
+        const int nc = min(E - cb, LN);                      // columns of this block
+        // ---- stage Ubar and Lbar transposed
         if (cb) __syncthreads();
         const int per = nc * N, steps = min(spw, hi - lo - j0);
         for (int s = 0; s < steps; ++s) {
@@ -128,118 +153,82 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
             const ET* gl = reinterpret_cast<const ET*>(pd.lhist) + ((size_t(m) * pd.kadj + j0 + s) * E + cb) * N;
             for (int e = threadIdx.x; e < per; e += 32 * NW) {
                 const int c = e / N, i = e - c * N;
-                cp_async16(Us + i * 33 + s * EL + c, gu + e);
-                if (STAGE_L) cp_async16(Ls + i * 33 + s * EL + c, gl + e);
+                cp_async16(Us + i * ROW + s * EL + c, gu + e);
+                cp_async16(Ls + i * ROW + s * EL + c, gl + e);
             }
         }
         cp_async_wait_all();
         __syncthreads();
-        const bool on = live && cl < nc;
-        const ET* lg = reinterpret_cast<const ET*>(pd.lhist) +
-                       ((size_t(m) * pd.kadj + j0 + (live ? sl : 0)) * E + cb + (on ? cl : 0)) * N;
-        // ---- products: acc[k][j - 1] sums the terms of weight sqrt(j) of subsystem k
-        GT R[Q][L - 1], I[Q][L - 1];
+        // ---- the pairs, UN at a time; the warps (and half-warps) that share a (k, j) take turns
+        GT R, I;
+        gsum_zero(R);
+        gsum_zero(I);
+        constexpr int TURNS = WS * (32 / LN);
+        for (int p0 = UN * ((warp % WS) * (32 / LN) + half); p0 < F; p0 += UN * TURNS) {
+            GT r, q;
 #pragma unroll
-        for (int k = 0; k < Q; ++k)
-#pragma unroll
-            for (int j = 0; j < L - 1; ++j) {
-                gsum_zero(R[k][j]);
-                gsum_zero(I[k][j]);
+            for (int t = 0; t < UN; ++t) {
+                const int p = p0 + t, ph = p / st;
+                const int i = (ph * (L - 1) + j - 1) * st + p;   // digit j - 1 inserted at k
+                const ET x = Ls[i * ROW + ln], x2 = Ls[(i + st) * ROW + ln];
+                const ET u = Us[i * ROW + ln], u2 = Us[(i + st) * ROW + ln];
+                if (t == 0)
+                    pair_products<true>(r, q, x, x2, u, u2);
+                else
+                    pair_products<false>(r, q, x, x2, u, u2);
             }
-        for (int f = warp; f < F; f += NW) {
-            ET x[L], u[L];
-#pragma unroll
-            for (int l = 0; l < L; ++l) {
-                x[l] = STAGE_L ? Ls[(f * L + l) * 33 + lane] : lg[f * L + l];
-                u[l] = Us[(f * L + l) * 33 + lane];
-            }
-            // the last subsystem: a_k pairs (Lbar_{j-1}, Ubar_j), a_k^+ pairs (Lbar_j, Ubar_{j-1})
-#pragma unroll
-            for (int j = 1; j < L; ++j) {
-                cjmac_acc<+1>(R[Q - 1][j - 1], I[Q - 1][j - 1], x[j - 1], u[j]);
-                cjmac_acc<-1>(R[Q - 1][j - 1], I[Q - 1][j - 1], x[j], u[j - 1]);
-            }
-#pragma unroll
-            for (int k = 0; k < Q - 1; ++k) {
-                const int sf = ipow_c(L, Q - 2 - k);
-                const int lk = (f / sf) % L;                 // warp-uniform
-#pragma unroll
-                for (int j = 1; j < L; ++j) {
-                    if (lk == j - 1) {                       // a_k: the fiber one level up
-                        const ET* un = Us + (f + sf) * L * 33 + lane;
-#pragma unroll
-                        for (int l = 0; l < L; ++l) cjmac_acc<+1>(R[k][j - 1], I[k][j - 1], x[l], un[l * 33]);
-                    }
-                    if (lk == j) {                           // a_k^+: one level down
-                        const ET* un = Us + (f - sf) * L * 33 + lane;
-#pragma unroll
-                        for (int l = 0; l < L; ++l) cjmac_acc<-1>(R[k][j - 1], I[k][j - 1], x[l], un[l * 33]);
-                    }
-                }
-            }
+            R = gsum_add(R, r);
+            I = gsum_add(I, q);
         }
-        float ps = 1.f;
-        if constexpr (SPLIT) {
-            const int d = on ? lsh[cb + cl] + hsh[cb + cl] - S : 0;   // <= 0
-            ps = d >= -126 ? float_of(static_cast<uint32_t>(127 + d) << 23)
-                           : (d >= -149 ? float_of(1u << (d + 149)) : 0.f);
-        }
-#pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            GT A = I[k][0], B = R[k][0];
-#pragma unroll
-            for (int j = 2; j < L; ++j) {
-                A = gsum_add(A, gsum_weight(I[k][j - 1], j));
-                B = gsum_add(B, gsum_weight(R[k][j - 1], j));
-            }
+        // (a lane without a column or a step holds whatever its shared words held: dropped)
+        if (live && cl < nc) {
             if constexpr (SPLIT) {
-                A = DF{fmul_n(A.s, ps), fmul_n(A.c, ps)};
-                B = DF{fmul_n(B.s, ps), fmul_n(B.c, ps)};
+                const int d = lsh[cb + cl] + hsh[cb + cl] - S;   // <= 0
+                const float ps = d >= -126 ? float_of(static_cast<uint32_t>(127 + d) << 23)
+                                           : (d >= -149 ? float_of(1u << (d + 149)) : 0.f);
+                R = DF{fmul_n(R.s, ps), fmul_n(R.c, ps)};
+                I = DF{fmul_n(I.s, ps), fmul_n(I.c, ps)};
             }
-            // (a lane without a column holds whatever its shared words held: dropped)
-            if (on) {
-                tot[2 * k] = gsum_add(tot[2 * k], A);
-                tot[2 * k + 1] = gsum_add(tot[2 * k + 1], B);
-            }
+            A = gsum_add(A, I);
+            B = gsum_add(B, R);
         }
     }
 
-    // ---- sums over the step's lanes (halving the values a lane carries while there are several),
-    // then over the warps, in a fixed order
-    int base = 0;
-#pragma unroll
-    for (int o = 1, half = V / 2; o < 32; o <<= 1, half >>= 1) {
-        if (o < EL) {                                        // uniform
-            if (half >= 1) {
-                const bool upper = (lane & o) != 0;
-#pragma unroll
-                for (int v = 0; v < half; ++v) {
-                    const GT send = upper ? tot[v] : tot[v + half], keep = upper ? tot[v + half] : tot[v];
-                    tot[v] = gsum_add(keep, gsum_shfl_xor(send, o));
-                }
-                if (upper) base += half;
-            } else {
-                tot[0] = gsum_add(tot[0], gsum_shfl_xor(tot[0], o));
-            }
-        }
+    // ---- sums over the step's lanes (and half-warps), weighted, then over the warps, fixed order
+    for (int o = EL >> 1; o > 0; o >>= 1) {
+        A = gsum_add(A, gsum_shfl_xor(A, o));
+        B = gsum_add(B, gsum_shfl_xor(B, o));
+    }
+    if constexpr (LN < 32) {
+        A = gsum_add(A, gsum_shfl_xor(A, LN));
+        B = gsum_add(B, gsum_shfl_xor(B, LN));
+    }
+    if constexpr (SPLIT) {
+        A = df_scale_sqrt(A, j);
+        B = df_scale_sqrt(B, j);
+    } else {
+        A *= sqrt_small(j);
+        B *= sqrt_small(j);
     }
     __syncthreads();
-    const int left = EL >= V ? 1 : V / EL;                   // values a lane ends with
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-        if (v < left && cl < V && base + v < 2 * Q) red[(warp * spw + sl) * 2 * Q + base + v] = tot[v];
+    if (half == 0 && cl == 0) {
+        red[(warp * spw + sl) * 2] = A;
+        red[(warp * spw + sl) * 2 + 1] = B;
+    }
     __syncthreads();
     for (int e = threadIdx.x; e < spw * 2 * Q; e += 32 * NW) {
-        const int s = e / (2 * Q), v = e % (2 * Q);
+        const int kk = e / (2 * spw), r = e % (2 * spw), s = r >> 1;
         if (lo + j0 + s >= hi) continue;
-        GT t = red[e];
-        for (int w = 1; w < NW; ++w) t = gsum_add(t, red[w * spw * 2 * Q + e]);
-        double r;
+        const GT* q = red + size_t(kk) * (L - 1) * WS * spw * 2 + r;
+        GT t = q[0];
+#pragma unroll
+        for (int w = 1; w < (L - 1) * WS; ++w) t = gsum_add(t, q[w * spw * 2]);
+        double v;
         if constexpr (SPLIT)
-            r = df_to_f64_scaled(t, S);
+            v = df_to_f64_scaled(t, S);
         else
-            r = t;
-        reinterpret_cast<double*>(pd.quad)[2 * (size_t(v >> 1) * pd.nsteps + n0 + lo + j0 + s) + (v & 1)] = r;
+            v = t;
+        reinterpret_cast<double*>(pd.quad)[2 * (size_t(kk) * pd.nsteps + n0 + lo + j0 + s) + (r & 1)] = v;
     }
 }
 

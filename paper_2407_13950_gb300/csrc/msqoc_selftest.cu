@@ -1,11 +1,11 @@
-// Self-tests of pieces of the sweeps:
-//  * the failure path: the bounded mbarrier wait (the one the adjoint sweep uses for its
-//    midpoint-history fetches) on a barrier that nothing completes gives up after its spin
+// Self-tests:
+//  * the failure path: a bounded mbarrier wait on a barrier that nothing completes gives up after its spin
 //    limit, and the launch reports it through the status word as MSQOC_ERR_TIMEOUT instead of
 //    hanging the GPU.  The context stays usable afterwards.
 //  * the compensated FP32 arithmetic of the mixed solver (msqoc_split.cuh), on the host or in a
 //    one-thread kernel: the split of doubles into two floats, a real dot product formed the way
-//    the adjoint forms its gradient products, and steps of the compensated state update.
+//    the gradient products are, and steps of the state update with an FP32 carry (the form of the
+//    update on an FP64 state, which the exported self-test defines).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -51,6 +51,49 @@ __host__ __device__ double dot_split(const double* x, const double* y, int64_t n
 
 __global__ void k_dot_probe(const double* x, const double* y, int64_t n, int shx, int shy, double* out) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *out = dot_split(x, y, n, shx, shy);
+}
+
+// ------------------------------------------------------------------ the compensated state update
+// The mixed solver's implicit-midpoint state update U_{n+1} = 2 Ubar - U_n = R U_n + 2 d, with
+// R = 2P - 1, P = 1 / (1 + i kappa) the diagonal preconditioner entry (kappa = (h/2) D real) and d
+// the step's correction (Ubar = P U_n + d).  Since R - 1 = -2 i kappa P, where |2 kappa| <= 2^-4.5
+// the state is kept as an FP64 part u and an FP32 carry (units 2^-sh) and
+//   u' + carry' = u + carry + 2 kappa (Im b, -Re b) + 2 d,   b = P (u + carry),
+// the increment formed as a two-float sum s + c and renormalised: u' = u + s (one FP64 add; s is
+// exact as a double), carry' = c.  b is the step's right-hand side (carry_rhs); its compensated
+// error (about 2^-47 |b|) enters times |2 kappa|, of the order of the FP64 rounding of u.
+constexpr double CARRY_UPDATE_K2 = 0.001953125;   // (2 kappa)^2 <= 2^-9
+
+// b = P (u + carry) from the split u (units 2^-sh), the split P and its third parts P3; the
+// carry (at most half an FP32 unit of the last increment) goes into the low parts
+__host__ __device__ __forceinline__ void carry_rhs(const float4& us, const float4& P, float2 P3, float2 car, DF& bre,
+                                                   DF& bim) {
+    cmul_df(us, P, bre, bim);
+    const float cr = ffma_n(P.x, car.x, ffma_n(-P.y, car.y, ffma_n(P3.x, us.x, fmul_n(-P3.y, us.y))));
+    const float ci = ffma_n(P.x, car.y, ffma_n(P.y, car.x, ffma_n(P3.x, us.y, fmul_n(P3.y, us.x))));
+    bre.c = fadd_n(bre.c, cr);
+    bim.c = fadd_n(bim.c, ci);
+}
+// u' (returned) and carry' from u, b = (bre, bim), the split 2 kappa (k2) and its third part k3,
+// and d = (dre, dim)
+__host__ __device__ __forceinline__ double2 carry_update(double2 u, DF bre, DF bim, float2 k2, float k3, DF dre, DF dim,
+                                                         int sh, float2& car) {
+    DF qr = df_scale(bim, k2.x, k2.y), qi = df_neg(df_scale(bre, k2.x, k2.y));
+    qr.c = fadd_n(qr.c, ffma_n(k3, bim.s, car.x));
+    qi.c = fadd_n(qi.c, ffma_n(-k3, bre.s, car.y));
+    const DF ar = df_add(qr, DF{fadd_n(dre.s, dre.s), fadd_n(dre.c, dre.c)});
+    const DF ai = df_add(qi, DF{fadd_n(dim.s, dim.s), fadd_n(dim.c, dim.c)});
+    // renormalised, so that u takes all but the last rounding of the increment and the carry
+    // stays within half an FP32 unit of it (else it would gather the low parts of every step)
+    // (a fast two-sum: |ar.c| is below |ar.s| but where ar.s cancels to nothing, and there the
+    // carry's error is of the order of the cancelled parts' rounding)
+    const DF xr = fast_two_sum(ar.s, ar.c), xi = fast_two_sum(ai.s, ai.c);
+    car = make_float2(xr.c, xi.c);
+    return make_double2(u.x + f64_of_float_scaled_normal(xr.s, sh), u.y + f64_of_float_scaled_normal(xi.s, sh));
+}
+// the state u + carry as one double (one FP64 add a component)
+__host__ __device__ __forceinline__ double2 carry_finish(double2 u, float2 car, int sh) {
+    return make_double2(u.x + f64_of_float_scaled_normal(car.x, sh), u.y + f64_of_float_scaled_normal(car.y, sh));
 }
 
 // n steps of the compensated state update on one complex entry from u0 with the preconditioner

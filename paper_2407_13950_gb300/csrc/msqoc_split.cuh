@@ -1,7 +1,6 @@
-// Double values as unevaluated sums of two floats, and compensated FP32 arithmetic on them: the
-// mixed solver forms the right-hand side of its steps, the residual apply, the gradient products
-// of Eq. grad-int and the state update of the implicit midpoint rule with these instead of FP64
-// multiply-adds.  On this GPU a warp's FP64 instruction occupies the issuing warp for ~60 cycles
+// Double values as unevaluated sums of two or three floats, and compensated FP32 arithmetic on
+// them: the mixed solver holds its state, forms the midpoint increment and the gradient products of
+// Eq. grad-int with these instead of FP64 multiply-adds.  On this GPU a warp's FP64 instruction occupies the issuing warp for ~60 cycles
 // and the SM retires ~2 FP64 lanes a cycle, against 128 FP32 lanes.  Every function here runs on
 // the host too (the CPU tests pin them);
 // the host side must be compiled without floating-point contraction (-ffp-contract=off), the
@@ -99,18 +98,21 @@ __host__ __device__ __forceinline__ float4 split_scaled(double2 v, int sh) {
 struct DF {
     float s, c;
 };
-// a += x y for x = xh + xl, y = yh + yl: xh yh = p + e exactly (FMA), p added to s with an exact
-// two-sum, e, the two-sum's error and the cross terms xh yl + xl yh added to c; xl yl
+// a += x y for x = xh + xl, y = yh + yl: p = RN(xh yh) is added to s by a two-sum, whose error is
+// (s - a') + (p - b) with b the part of p that reached the sum; p - b and the rounding of p
+// together are xh yh - b, one FMA.  Both and the cross terms xh yl + xl yh go into c; xl yl
 // (<= 2^-48 |x y|) is dropped.  Error of the finished sum: about 2^-47 times the sum of the
-// magnitudes of its terms and partial sums.
+// magnitudes of its terms and partial sums.  (Accumulating s by an FMA of xh yh would save one
+// more operation but is wrong where s is close to -p: the sum then keeps low bits of the product
+// that b cannot hold.)
 __host__ __device__ __forceinline__ void df_mac(DF& a, float xh, float xl, float yh, float yl) {
     const float p = fmul_n(xh, yh);
-    const float e = ffma_n(xh, yh, -p);
     const float s = fadd_n(a.s, p);
-    const float bp = fsub_n(s, a.s);
-    const float t = fadd_n(fsub_n(a.s, fsub_n(s, bp)), fsub_n(p, bp));
+    const float b = fsub_n(s, a.s);
+    const float t = fsub_n(a.s, fsub_n(s, b));
+    const float e = ffma_n(xh, yh, -b);
     a.s = s;
-    a.c = fadd_n(a.c, fadd_n(t, ffma_n(xh, yl, ffma_n(xl, yh, e))));
+    a.c = fadd_n(ffma_n(xl, yh, ffma_n(xh, yl, a.c)), fadd_n(e, t));
 }
 // a + b (exact two-sum of the leading parts)
 __host__ __device__ __forceinline__ DF df_add(DF a, DF b) {
@@ -215,53 +217,47 @@ __host__ __device__ __forceinline__ double df_to_f64_scaled(DF a, int sh) {
     return f64_of_float_scaled(a.s, sh) + f64_of_float_scaled(a.c, sh);
 }
 
-// ------------------------------------------------------------------ the compensated state update
-// The mixed solver's implicit-midpoint state update U_{n+1} = 2 Ubar - U_n = R U_n + 2 d, with
-// R = 2P - 1, P = 1 / (1 + i kappa) the diagonal preconditioner entry (kappa = (h/2) D real) and d
-// the step's correction (Ubar = P U_n + d).  Since R - 1 = -2 i kappa P, where |2 kappa| <= 2^-4.5
-// the state is kept as an FP64 part u and an FP32 carry (units 2^-sh) and
-//   u' + carry' = u + carry + 2 kappa (Im b, -Re b) + 2 d,   b = P (u + carry),
-// the increment formed as a two-float sum s + c and renormalised: u' = u + s (one FP64 add; s is
-// exact as a double), carry' = c.  b is the step's right-hand side (carry_rhs); its compensated
-// error (about 2^-47 |b|) enters times |2 kappa|, of the order of the FP64 rounding of u.
-constexpr double CARRY_UPDATE_K2 = 0.001953125;   // (2 kappa)^2 <= 2^-9
-
-// The constants P and 2 kappa enter every step, so their splits are made exact with a third part
-// (x - hi - lo, at most 5 bits: exact as a float): otherwise the 2^-48 remainders of the splits
-// would act as a constant error of P and kappa and add up over the steps.
+// ------------------------------------------------------------------ the state as three floats
+// The mixed solver holds every component of the state as the exact sum of three floats a + b + c
+// (units 2^-sh): a the value rounded to 24 bits, b the remainder likewise, c the rest.  A double
+// splits exactly (24 + 24 + 5 bits).
+struct TF {
+    float a, b, c;
+};
+// x 2^-sh, exactly (down to 2^-126 2^sh; smaller remainders become zero)
+__host__ __device__ __forceinline__ TF tf_split(double x, int sh) {
+    const float2 h = split_scaled(x, sh);
+    const double r = (x - f64_of_float_scaled(h.x, sh)) - f64_of_float_scaled(h.y, sh);
+    return TF{h.x, h.y, split_scaled(r, sh).x};
+}
+// u += s + t for an increment s + t (|t| <= ulp(s)) below the state's size: every sum is exact
+// (two-sums) but the last part's, about 2^-72 |u|.  The closing fast two-sums renormalise; their
+// operands are ordered but where the leading part cancels to nothing, and what they drop there is
+// below 2^-48 of the cancelled increment.
+__host__ __device__ __forceinline__ void tf_add(TF& u, float s, float t) {
+    const DF x = two_sum(u.a, s);
+    const DF y = two_sum(u.b, x.c);
+    const DF z = two_sum(y.s, t);
+    const float r = fadd_n(u.c, fadd_n(y.c, z.c));
+    const DF p = fast_two_sum(x.s, z.s);
+    const DF q = fast_two_sum(p.c, r);
+    u = TF{p.s, q.s, q.c};
+}
+// u 2^sh rounded to a double (|sh| <= 896)
+__host__ __device__ __forceinline__ double tf_to_f64(TF u, int sh) {
+    return f64_of_float_scaled_normal(u.a, sh) +
+           (f64_of_float_scaled_normal(u.b, sh) + f64_of_float_scaled_normal(u.c, sh));
+}
+// x - hi - lo of a split constant: at most 5 bits, exact as a float.  A constant that enters every
+// step keeps it: its 2^-48 remainder would otherwise act the same way each step and add up.
 __host__ __device__ __forceinline__ float split_third(double x, float2 s) {
     return static_cast<float>((x - static_cast<double>(s.x)) - static_cast<double>(s.y));
 }
-// b = P (u + carry) from the split u (units 2^-sh), the split P and its third parts P3; the
-// carry (at most half an FP32 unit of the last increment) goes into the low parts
-__host__ __device__ __forceinline__ void carry_rhs(const float4& us, const float4& P, float2 P3, float2 car, DF& bre,
-                                                   DF& bim) {
-    cmul_df(us, P, bre, bim);
-    const float cr = ffma_n(P.x, car.x, ffma_n(-P.y, car.y, ffma_n(P3.x, us.x, fmul_n(-P3.y, us.y))));
-    const float ci = ffma_n(P.x, car.y, ffma_n(P.y, car.x, ffma_n(P3.x, us.y, fmul_n(P3.y, us.x))));
-    bre.c = fadd_n(bre.c, cr);
-    bim.c = fadd_n(bim.c, ci);
-}
-// u' (returned) and carry' from u, b = (bre, bim), the split 2 kappa (k2) and its third part k3,
-// and d = (dre, dim)
-__host__ __device__ __forceinline__ double2 carry_update(double2 u, DF bre, DF bim, float2 k2, float k3, DF dre, DF dim,
-                                                         int sh, float2& car) {
-    DF qr = df_scale(bim, k2.x, k2.y), qi = df_neg(df_scale(bre, k2.x, k2.y));
-    qr.c = fadd_n(qr.c, ffma_n(k3, bim.s, car.x));
-    qi.c = fadd_n(qi.c, ffma_n(-k3, bre.s, car.y));
-    const DF ar = df_add(qr, DF{fadd_n(dre.s, dre.s), fadd_n(dre.c, dre.c)});
-    const DF ai = df_add(qi, DF{fadd_n(dim.s, dim.s), fadd_n(dim.c, dim.c)});
-    // renormalised, so that u takes all but the last rounding of the increment and the carry
-    // stays within half an FP32 unit of it (else it would gather the low parts of every step)
-    // (a fast two-sum: |ar.c| is below |ar.s| but where ar.s cancels to nothing, and there the
-    // carry's error is of the order of the cancelled parts' rounding)
-    const DF xr = fast_two_sum(ar.s, ar.c), xi = fast_two_sum(ai.s, ai.c);
-    car = make_float2(xr.c, xi.c);
-    return make_double2(u.x + f64_of_float_scaled_normal(xr.s, sh), u.y + f64_of_float_scaled_normal(xi.s, sh));
-}
-// the state u + carry as one double (one FP64 add a component)
-__host__ __device__ __forceinline__ double2 carry_finish(double2 u, float2 car, int sh) {
-    return make_double2(u.x + f64_of_float_scaled_normal(car.x, sh), u.y + f64_of_float_scaled_normal(car.y, sh));
+// kappa z for kappa = kh + kl + k3 and z = s + c
+__host__ __device__ __forceinline__ DF kappa_mul(float kh, float kl, float k3, float s, float c) {
+    const float p = fmul_n(kh, s);
+    const float e = ffma_n(kh, s, -p);
+    return DF{p, ffma_n(kh, c, ffma_n(kl, s, ffma_n(k3, s, e)))};
 }
 
 }  // namespace msqoc

@@ -18,17 +18,18 @@
 // factor rho_n = ||P iX_C|| <= (h/2) lam sum_k |d_k(t)| is evaluated every step and sets the
 // iteration counts (warp-uniform).
 //   SOLVER_FP64 : K fixed-point sweeps in FP64, K = ceil(log(2^-56)/log rho) - 1.
-//   SOLVER_MIXED: mixed-precision iterative refinement.  FP32 sweeps give d = Ubar - P rhs,
-//     the FP64 residual r = P rhs - z + s P (iX_C) z of z = P rhs + d is formed once with an
-//     FP64 apply, and the FP32 correction e (I + ...)e = r is added in FP64.  Conversions
-//     between f64 and f32 are done with integer bit operations because the hardware
-//     conversions issue on the (slow) FP64 pipe; they carry a per-column binary scale taken
-//     from the launch's initial state (the step preserves column norms), so the FP32 stage
-//     works relative to the column norm whatever the state's magnitude.
-// The adjoint sweep fuses the gradient quadrature of Eq. grad-int at the midpoints:
-//   z_k = <Lbar, a_k Ubar>_F, y_k = <Lbar, a_k^+ Ubar>_F (summed over the tile's columns),
-//   dP/dalpha1_kfs += -2h B_s Im(e^{i W t} z_k + e^{-i W t} y_k),
-//   dP/dalpha2_kfs += -2h B_s Re(e^{i W t} z_k - e^{-i W t} y_k).
+//   SOLVER_MIXED: the increment m = Ubar - U is estimated in FP32 sweeps, formed once at the
+//     estimate in compensated FP32 (two-float sums) and corrected by FP32 sweeps on its residual;
+//     the state is the exact sum of three floats, so a step has no FP64 instruction.  Everything is
+//     in units of a per-column power of two taken from the launch's initial state (the step
+//     preserves column norms), so the FP32 arithmetic works relative to the column norm whatever
+//     the state's magnitude.
+// Both sweeps store the midpoint states, from which msqoc_quad.cuh forms the gradient products.
+//
+// What bounds the mixed step: instruction issue and the dependency latency inside its 4-5 barrier-
+// separated phases (no pipe is saturated).  4 transmons, 100000 steps at 256 windows on one GB300:
+// a forward sweep 5.22 -> 4.43 ms against the form with an FP64 state, an FP32 carry and two more
+// sweeps a step; at 64 windows 6.97 -> 5.52 ms.
 #pragma once
 
 #include <climits>
@@ -80,97 +81,16 @@ __device__ __forceinline__ float2 cadd_scaled(float2 acc, float2 c, float2 w) {
     return r;
 }
 
-// -d + s * (c * w): the FP64 residual of the refinement when the current iterate is b + d
-// (the negations are FMA operand modifiers; nothing is materialized)
-template <int S>
-__device__ __forceinline__ double2 resid_from(double2 d, double2 c, double2 w) {
-    double2 r;
-    if constexpr (S > 0) {
-        r.x = fma(c.x, w.x, fma(-c.y, w.y, -d.x));
-        r.y = fma(c.x, w.y, fma(c.y, w.x, -d.y));
-    } else {
-        r.x = fma(-c.x, w.x, fma(c.y, w.y, -d.x));
-        r.y = fma(-c.x, w.y, fma(-c.y, w.x, -d.y));
-    }
-    return r;
-}
 // 2 z - u as one FMA per component
 __device__ __forceinline__ double2 reflect(double2 z, double2 u) {
     return make_double2(fma(2.0, z.x, -u.x), fma(2.0, z.y, -u.y));
 }
-// the mixed solver's 2 z - u for z = P u + d: R u + 2 d with R = 2P - 1 (FP64; d a two-float
-// sum in units 2^-sh, doubled exactly through the scale): three FP64 instructions a component
-__device__ __forceinline__ double2 cayley_update(double2 R, double2 u, DF dre, DF dim, int sh) {
-    const double tx = df_to_f64_scaled(dre, sh + 1), ty = df_to_f64_scaled(dim, sh + 1);
-    return make_double2(fma(R.x, u.x, fma(-R.y, u.y, tx)), fma(R.x, u.y, fma(R.y, u.x, ty)));
-}
-
-// Dipole exchange on the fiber (fiber index f, entries at fb.xo of a [cols][N] buffer):
-// w += i (h/2) J_jk (a_k^+ a_j + a_k a_j^+) x for every coupled pair j < k.  a_k^+ a_j moves one
-// quantum from j to k: the source has l_j + 1 and l_k - 1, weight sqrt(l_k) sqrt(l_j + 1); a_k a_j^+
-// the opposite, weight sqrt(l_k + 1) sqrt(l_j).  When k is the last subsystem the source is an
-// entry of the neighbour fiber in subsystem j at the shifted level; otherwise a fiber that
-// differs in both digits, at the same level.  The pairs are warp-uniform; the level tests are
-// per lane.
-template <int L, int Q, typename T2>
-__device__ __forceinline__ void apply_exchange(const T2* __restrict__ buf, const ProbDev& pd, int f, int xo,
-                                               T2 (&w)[L]) {
-    using R = typename cx<T2>::T;
-    for (int e = 0; e < pd.nex; ++e) {
-        const int j = pd.ex_j[e], k = pd.ex_k[e];
-        int sfj = 1, sfk = 1;                                  // fiber strides (j is never the last)
-        for (int t = j; t < Q - 2; ++t) sfj *= L;
-        for (int t = k; t < Q - 2; ++t) sfk *= L;
-        const int lj = (f / sfj) % L;
-        const R c = static_cast<R>(pd.ex_c[e]);
-        if (k == Q - 1) {
-#pragma unroll
-            for (int l = 0; l < L; ++l) {
-                // a_k^+ a_j: from (l_j + 1, l - 1)
-                if (l >= 1 && lj <= L - 2) {
-                    const R wt = c * static_cast<R>(sqrt_small(l) * sqrt_small(lj + 1));
-                    const T2 x = buf[xo + sfj * L + (l - 1)];
-                    w[l].x -= wt * x.y;
-                    w[l].y += wt * x.x;
-                }
-                // a_k a_j^+: from (l_j - 1, l + 1)
-                if (l <= L - 2 && lj >= 1) {
-                    const R wt = c * static_cast<R>(sqrt_small(l + 1) * sqrt_small(lj));
-                    const T2 x = buf[xo - sfj * L + (l + 1)];
-                    w[l].x -= wt * x.y;
-                    w[l].y += wt * x.x;
-                }
-            }
-        } else {
-            const int lk = (f / sfk) % L;
-            if (lk >= 1 && lj <= L - 2) {
-                const R wt = c * static_cast<R>(sqrt_small(lk) * sqrt_small(lj + 1));
-                const T2* src = buf + xo + (sfj - sfk) * L;
-#pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    w[l].x -= wt * src[l].y;
-                    w[l].y += wt * src[l].x;
-                }
-            }
-            if (lk <= L - 2 && lj >= 1) {
-                const R wt = c * static_cast<R>(sqrt_small(lk + 1) * sqrt_small(lj));
-                const T2* src = buf + xo + (sfk - sfj) * L;
-#pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    w[l].x -= wt * src[l].y;
-                    w[l].y += wt * src[l].x;
-                }
-            }
-        }
-    }
-}
-
 // w = (iX_C x) on the fiber: ladder terms of the last subsystem from registers (xr), the
 // others from the shared buffer.  cf: per-slot coefficients i(h/2)sqrt(.)d_k for this step.
 template <int L, int Q, typename T2>
 __device__ __forceinline__ void apply_off(const T2* __restrict__ buf, const T2* __restrict__ cf,
                                           const Fiber<L, Q>& fb, const T2 (&xr)[L], T2 (&w)[L],
-                                          const ProbDev& pd) {
+                                          const ExTab& ex) {
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         w[l].x = 0;
@@ -196,22 +116,21 @@ __device__ __forceinline__ void apply_off(const T2* __restrict__ buf, const T2* 
         }
     }
     // exchange-coupled problems are 2-level qubit models (the only shapes compiled with it):
-    // w += i (h/2) J x_src from the fiber's precomputed sources, or the general form
+    // w += i (h/2) J x_src
     if constexpr (L == 2 && Q >= 2) {
-        if (pd.nex > MAXEXF) {
-            apply_exchange<L, Q, T2>(buf, pd, fb.f, fb.xo, w);
-        } else if (pd.nex) {
-            using R = typename cx<T2>::T;
+        using R = typename cx<T2>::T;
+        for (int e = 0; e < ex.n; ++e) {                       // uniform
+            R c;
+            if constexpr (sizeof(R) == 4)
+                c = ex.cs[e].x;
+            else
+                c = ex.cd[e];
+            const int mask = ex.mask[e];
 #pragma unroll
-            for (int e = 0; e < MAXEXF; ++e) {
-                if (e >= pd.nex) break;                        // warp-uniform
-                const R c = static_cast<R>(pd.ex_c[e]);
-#pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    const T2 x = buf[fb.exs[e][l]];            // the zero entry where no term
-                    w[l].x -= c * x.y;
-                    w[l].y += c * x.x;
-                }
+            for (int l = 0; l < L; ++l) {
+                const T2 x = buf[fb.exsrc(e, l, mask)];        // the zero entry where no term
+                w[l].x -= c * x.y;
+                w[l].y += c * x.x;
             }
         }
     }
@@ -221,10 +140,10 @@ __device__ __forceinline__ void apply_off(const T2* __restrict__ buf, const T2* 
 // ------------------------------------------------------------------ per-step coefficients
 // Warp 0: slot (k, l, dir) -> i (h/2) sqrt(l+1) d_k (dir 0, a_k) or i (h/2) sqrt(l) conj(d_k)
 // (dir 1, a_k^+); lane k' < NSLOT holds d_k of its slot's subsystem.  The coefficients go out
-// in FP64, FP32 and (mixed solver, cfs != nullptr) split into two floats.  The iteration counts
+// in FP64 (FP64 solver) or in FP32 and split into two floats (mixed solver).  The iteration counts
 // of the step (packed by step_counts in the controls kernel) are unpacked into prm; prm[3] holds
-// the solver-range flag (bit 0) and the FP64-apply flag (bit 1).
-template <int L, int Q>
+// the solver-range flag (bit 0) and the coarse-step flag (bit 1).
+template <int L, int Q, int SOLVER>
 __device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, double2 dk, int cnt, double2* cfd,
                                                   float2* cff, float4* cfs, int* prm) {
     constexpr int NSLOT = Q * L * 2;
@@ -235,9 +154,13 @@ __device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, d
         const double s = pd.sc[2 * l + dir];
         double2 v = make_double2(0.0, 0.0);
         if (valid) v = dir == 0 ? make_double2(-s * dk.y, s * dk.x) : make_double2(s * dk.y, s * dk.x);
-        cfd[lane] = v;
-        cff[lane] = f32_of(v);
-        if (cfs) cfs[lane] = split_scaled(v, 0);
+        if constexpr (SOLVER == SOLVER_FP64) {
+            cfd[lane] = v;
+        } else {
+            const float4 sp = split_scaled(v, 0);
+            cff[lane] = make_float2(sp.x, sp.y);
+            cfs[lane] = sp;
+        }
     }
     if (lane == 0) {
         prm[0] = cnt & 0xff;
@@ -255,16 +178,12 @@ __device__ __forceinline__ void cmac_df(DF (&w)[2], const float4& c, const float
     df_mac(w[1], c.x, c.z, x.y, x.w);
     df_mac(w[1], c.y, c.w, x.x, x.z);
 }
-// w = iX_C x on the fiber (apply_off without exchange terms) from split entries: the fiber's own
-// in xr, the neighbours' in buf, the coefficients in cf; compensated FP32 sums (about 2^-47 of
-// the terms' magnitudes).  The mixed solver's residual needs P w to within 2^-53 |x| only, and
-// |P w| <= rho |x| with rho <= 2^-7 wherever this form is used.
-// exc / nex: the exchange pairs' coefficients (h/2) J split into two floats and their count
-// (2-level problems with at most MAXEXF pairs; terms i (h/2) J x_src from the fiber's sources)
+// w = iX_C x on the fiber (apply_off) from split entries: the fiber's own in xr, the neighbours'
+// in buf, the coefficients in cf; compensated FP32 sums (about 2^-47 of the terms' magnitudes)
 template <int L, int Q>
 __device__ __forceinline__ void apply_off_df(const float4* __restrict__ buf, const float4* __restrict__ cf,
                                              const Fiber<L, Q>& fb, const float4 (&xr)[L], DF (&w)[L][2],
-                                             const float2 (&exc)[MAXEXF], int nex) {
+                                             const ExTab& ex) {
     // the first term of each entry's sum initialises it (no two-sum with zero)
     constexpr int kl = Q - 1;
 #pragma unroll
@@ -291,79 +210,84 @@ __device__ __forceinline__ void apply_off_df(const float4* __restrict__ buf, con
         }
     }
     if constexpr (L == 2 && Q >= 2) {
-#pragma unroll
-        for (int e = 0; e < MAXEXF; ++e) {
-            if (e >= nex) break;   // uniform
+        for (int e = 0; e < ex.n; ++e) {   // uniform
+            const float2 c = ex.cs[e];
+            const int mask = ex.mask[e];
 #pragma unroll
             for (int l = 0; l < L; ++l) {
-                const float4 x = buf[fb.exs[e][l]];   // the zero entry where the pair gives no term
-                df_mac(w[l][0], -exc[e].x, -exc[e].y, x.y, x.w);
-                df_mac(w[l][1], exc[e].x, exc[e].y, x.x, x.z);
+                const float4 x = buf[fb.exsrc(e, l, mask)];   // the zero entry where the pair gives no term
+                df_mac(w[l][0], -c.x, -c.y, x.y, x.w);
+                df_mac(w[l][1], c.x, c.y, x.x, x.z);
             }
         }
     }
 }
-// the residual -d + s P w of the refinement in scaled units, rounded to FP32: d = dh + dl and
-// P = (hi, lo) split, w from apply_off_df
-template <int S>
-__device__ __forceinline__ float2 resid_df(float2 dh, float2 dl, const float4& P, const DF (&w)[2]) {
-    DF re{-dh.x, -dl.x}, im{-dh.y, -dl.y};
-    constexpr float s = S > 0 ? 1.f : -1.f;
-    df_mac(re, s * P.x, s * P.z, w[0].s, w[0].c);
-    df_mac(re, -s * P.y, -s * P.w, w[1].s, w[1].c);
-    df_mac(im, s * P.x, s * P.z, w[1].s, w[1].c);
-    df_mac(im, s * P.y, s * P.w, w[0].s, w[0].c);
-    return make_float2(fadd_n(re.s, re.c), fadd_n(im.s, im.c));
-}
 
-// ------------------------------------------------------------------ FP64 residual, out of line
-// The mixed solver's refinement residual in FP64, for the steps whose contraction factor is
-// above the compensated form's bound (step_counts) and for exchange-coupled problems.  Out of
-// line: it is rare on the workloads that fill the GPU, and inlined into the step loop (with the
-// FP64 midpoint state and the FP64 apply it needs) it slowed the common path by 4-9%.  Values
-// travel by value; the fiber's neighbour list is rebuilt from (column, fiber).
-template <int L> struct SplitVals { float4 v[L]; };
-template <int L> struct ResidIn { float4 zs[L]; DF dre[L], dim[L]; };
-template <int L> struct ResidOut { float2 r[L]; };
-
-// the midpoint state z = zs 2^sh in FP64 into the shared apply buffer (the fiber's entries)
-template <int L>
-static __device__ __noinline__ void store_z64(double2* dst, SplitVals<L> zs, int sh) {
-#pragma unroll
-    for (int l = 0; l < L; ++l)
-        dst[l] = make_double2(df_to_f64_scaled(DF{zs.v[l].x, zs.v[l].z}, sh),
-                              df_to_f64_scaled(DF{zs.v[l].y, zs.v[l].w}, sh));
-}
-// r = s P (iX_C) z - d_total in FP64, rounded to FP32 in the column's scaled units
+// ------------------------------------------------------------------ coarse steps, out of line
+// The mixed solver's step in FP64, for the steps step_counts flags as coarse: where the rotation
+// of a drift entry or the contraction factor is so large that the compensated increment's 2^-48
+// relative error would exceed the FP64 rounding of the state.  The fixed point z = P u + s P w(z)
+// takes K sweeps, U' = 2 z - U.  Out of line: it is rare, and everything it needs would cost the
+// common step registers.  Every thread of the tile takes part in the barriers; `mine` says
+// whether the thread's slot is coarse at this step.  The buffer's zero entry stays zero.
+template <int L> struct CoarseIO {
+    TF u[L][2];
+    float4 z[L];
+};
 template <int L, int Q, int S, bool BWD>
-static __device__ __noinline__ ResidOut<L> resid_fp64(const double2* D0, const double2* cfd, const ProbDev& pd, int c,
-                                                      int f, int zero, ResidIn<L> in, int sh) {
+static __device__ __noinline__ void coarse_step(double2* D0, double2* cfd, const ProbDev& pd, const ExTab& ex, int c,
+                                                int f, int zero, int64_t n0, int64_t n1, int nslot, int slot, bool act,
+                                                bool mine, int K, int Kmax, int sh, CoarseIO<L>& io) {
+    constexpr int NSLOT = Q * L * 2;
     Fiber<L, Q> fb;
     fb.init(c, f, pd, zero);
-    double2 z[L];
-#pragma unroll
-    for (int l = 0; l < L; ++l)
-        z[l] = make_double2(df_to_f64_scaled(DF{in.zs[l].x, in.zs[l].z}, sh),
-                            df_to_f64_scaled(DF{in.zs[l].y, in.zs[l].w}, sh));
-    double2 w[L];
-    apply_off<L, Q, double2>(D0, cfd, fb, z, w, pd);
-    const ColScale cs = col_scale(sh);
-    ResidOut<L> o;
+    // the step's coefficients of both slots in FP64
+    for (int t = threadIdx.x; t < nslot * NSLOT; t += blockDim.x) {
+        const int i = t % NSLOT, dir = i & 1, l = (i >> 1) % L;
+        const double2 d = pd.ctrl[size_t(t < NSLOT ? n0 : n1) * pd.q + i / (2 * L)];
+        const double s = (dir == 0 ? l < L - 1 : l > 0) ? pd.sc[2 * l + dir] : 0.0;
+        cfd[t] = dir == 0 ? make_double2(-s * d.y, s * d.x) : make_double2(s * d.y, s * d.x);
+    }
+    double2 u[L], b[L], z[L], P[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
-        double2 p = pd.P[f * L + l];
-        if (BWD) p.y = -p.y;
-        const double2 dacc = make_double2(df_to_f64_scaled(in.dre[l], sh), df_to_f64_scaled(in.dim[l], sh));
-        o.r[l] = f32_of_scaled(resid_from<S>(dacc, p, w[l]), cs);
+        P[l] = pd.P[f * L + l];
+        if (BWD) P[l].y = -P[l].y;
+        u[l] = make_double2(tf_to_f64(io.u[l][0], sh), tf_to_f64(io.u[l][1], sh));
+        b[l] = cmul(P[l], u[l]);
+        z[l] = b[l];
     }
-    return o;
+    for (int it = 0; it < Kmax; ++it) {
+        tile_sync();   // the buffer's readers are done (and the coefficients written)
+        if (act) {
+#pragma unroll
+            for (int l = 0; l < L; ++l) D0[fb.xo + l] = z[l];
+        }
+        tile_sync();
+        double2 w[L];
+        apply_off<L, Q, double2>(D0, cfd + (nslot > 1 ? slot : 0) * NSLOT, fb, z, w, ex);
+        if (it < K) {
+#pragma unroll
+            for (int l = 0; l < L; ++l) z[l] = cadd_scaled<S>(b[l], P[l], w[l]);
+        }
+    }
+    tile_sync();
+    if (mine) {
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            io.z[l] = split_scaled(z[l], sh);
+            const double2 v = reflect(z[l], u[l]);
+            io.u[l][0] = tf_split(v.x, sh);
+            io.u[l][1] = tf_split(v.y, sh);
+        }
+    }
 }
 
 // ------------------------------------------------------------------ the sweep kernel
 // One CTA per tile.  A tile covers one or two windows ("slots"); each slot has its own step
-// range, per-step coefficients and iteration counts, computed by warp `slot`, and gradient fold,
-// run by warp nwarps - 1 - slot (the host only builds two-slot tiles with at least two warps).  Loops run to the longer of
-// the slots' ranges; a thread whose slot has no step at an iteration keeps its state.
+// range, per-step coefficients and iteration counts, computed by warp `slot` (the host only builds
+// two-slot tiles with at least two warps).  Loops run to the longer of the slots' ranges; a thread
+// whose slot has no step at an iteration keeps its state.
 // MAXT: the largest tile the instantiation serves; it sets the register budget (255 registers a
 // thread for MAX_TILE_THREADS, 168 for MAX_LEAN_TILE_THREADS: 12 warps on an SM).
 template <int L, int Q, int SOLVER, bool BWD, bool ROLLOUT = false, int MAXT = MAX_TILE_THREADS>
@@ -380,7 +304,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     const SweepSmem lay = sweep_layout(Q, L, N, a.cpt, SOLVER, 0, a.hdepth);
     double2* coef_d = reinterpret_cast<double2*>(smem + lay.coef_d);
     float2* coef_f = reinterpret_cast<float2*>(smem + lay.coef_f);
-    float4* coef_s = SOLVER == SOLVER_MIXED ? reinterpret_cast<float4*>(smem + lay.coef_s) : nullptr;
+    float4* coef_s = reinterpret_cast<float4*>(smem + lay.coef_s);
     int* params = reinterpret_cast<int*>(smem + lay.params);
     double2* D0 = reinterpret_cast<double2*>(smem + lay.D0);
     double2* D1 = reinterpret_cast<double2*>(smem + lay.D1);
@@ -435,11 +359,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
 
     Fiber<L, Q> fb;
     fb.init(c, f, pd, a.cpt * N);
-    // the exchange coefficients split for the compensated apply (2-level problems)
-    float2 exc[MAXEXF];
-#pragma unroll
-    for (int e = 0; e < MAXEXF; ++e)
-        exc[e] = (L == 2 && Q >= 2 && e < pd.nex) ? split_scaled(pd.ex_c[e], 0) : make_float2(0.f, 0.f);
+    __shared__ ExTab ex_s;   // (ordered before its first read by the first barrier of the time loop)
+    fill_exchange(ex_s, pd);
     // the apply buffers' zero entry (read by the exchange terms a fiber entry does not have; the
     // first barrier of the time loop orders these stores before any read)
     if (tid == 0) {
@@ -452,35 +373,27 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
         }
     }
 
-    // preconditioner on the fiber: P (forward) or conj(P) (adjoint)
+    // FP64 solver: the preconditioner on the fiber, P (forward) or conj(P) (adjoint).  Mixed solver:
+    // kappa (-kappa for the adjoint) of P = 1 / (1 + i kappa) as three floats, and G = P - 1 =
+    // (Im P) (-Im P / Re P + i) ... = -i kappa P in FP32, formed in FP64 without cancellation
     double2 Pd[L];
-    float2 Pf[L];
-    float4 Ps[L];   // split (mixed solver's right-hand side and compensated residual)
-    // 2 kappa = -2 Im P / Re P split (P = 1 / (1 + i kappa)), for the mixed solver's state update
-    float2 k2s[L];
-    float4* cq = SOLVER == SOLVER_MIXED ? reinterpret_cast<float4*>(smem + lay.cq) : nullptr;
-    bool carry_ok = true;
+    float kh[L], kl[L], k3[L];
+    float2 Gf[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         double2 p = pd.P[f * L + l];
         if (BWD) p.y = -p.y;
-        Pd[l] = p;
-        Ps[l] = split_scaled(p, 0);
-        Pf[l] = make_float2(Ps[l].x, Ps[l].y);   // p rounded to FP32
-        const double k2 = -2.0 * p.y / p.x;
-        k2s[l] = split_scaled(k2, 0);
-        carry_ok = carry_ok && k2 * k2 <= CARRY_UPDATE_K2;
-        // the splits' third parts, per entry of the fiber (the same for every column)
-        if (SOLVER == SOLVER_MIXED && act && c == 0)
-            cq[f * L + l] = make_float4(split_third(k2, k2s[l]), split_third(p.x, make_float2(Ps[l].x, Ps[l].z)),
-                                        split_third(p.y, make_float2(Ps[l].y, Ps[l].w)), 0.f);
+        if constexpr (SOLVER == SOLVER_FP64) {
+            Pd[l] = p;
+        } else {
+            const double kap = -p.y / p.x;
+            const float2 ks = split_scaled(kap, 0);
+            kh[l] = ks.x;
+            kl[l] = ks.y;
+            k3[l] = split_third(kap, ks);
+            Gf[l] = make_float2(f32_of(kap * p.y), f32_of(p.y));   // -i kappa P = kappa Im P - i kappa Re P
+        }
     }
-    // the compensated state update for the whole tile (the same P table for every tile of the
-    // problem, so the same choice), else R u + 2 d in FP64
-    const bool carry_upd = SOLVER == SOLVER_MIXED && tile_sync_or(act && !carry_ok) == 0;
-    float2 car[L];   // the state's FP32 carry (compensated update), zero otherwise
-#pragma unroll
-    for (int l = 0; l < L; ++l) car[l] = make_float2(0.f, 0.f);
 
     // ---- initial state
     //   forward, whole window : U^m(t_{m-1}) = W^{m-1} (identity embedding for the first window
@@ -518,7 +431,15 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
         tile_sync();
         sh = column_shift(colexp_s[c < MAX_TILE_COLS ? c : 0]);
     }
-    const ColScale cs = col_scale(sh);
+    // the mixed solver's state, units 2^sh
+    TF v[L][2];
+    if constexpr (SOLVER == SOLVER_MIXED) {
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            v[l][0] = tf_split(u[l].x, sh);
+            v[l][1] = tf_split(u[l].y, sh);
+        }
+    }
     // the midpoint states' column scale exponent, read by the quadrature kernel: per segment for
     // the forward's history, per launch for the adjoint's
     if constexpr (SOLVER == SOLVER_MIXED) {
@@ -569,30 +490,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
             cnt_next = pd.spl[n].cnt;
         }
     };
-    // the step's state update: 2 z - u (FP64 solver); R u + 2 d in FP64 or the compensated form
-    // with the carry (mixed solver; the FP64 form reads R's P from the table: rare)
-    auto state_update = [&](double2 (&uu)[L], const double2 (&zz)[L], const DF (&br)[L], const DF (&bi)[L],
-                            const DF (&dr)[L], const DF (&di)[L]) {
-        if constexpr (SOLVER == SOLVER_MIXED) {
-            if (carry_upd) {
-#pragma unroll
-                for (int l = 0; l < L; ++l)
-                    uu[l] = carry_update(uu[l], br[l], bi[l], k2s[l], cq[f * L + l].x, dr[l], di[l], sh, car[l]);
-            } else {
-#pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    double2 p = pd.P[f * L + l];
-                    if (BWD) p.y = -p.y;
-                    uu[l] = cayley_update(make_double2(fma(2.0, p.x, -1.0), 2.0 * p.y), uu[l], dr[l], di[l], sh);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int l = 0; l < L; ++l) uu[l] = reflect(zz[l], uu[l]);
-        }
+    // the state as stored
+    auto state_out = [&](int l) {
+        if constexpr (SOLVER == SOLVER_MIXED)
+            return make_double2(tf_to_f64(v[l][0], sh), tf_to_f64(v[l][1], sh));
+        else
+            return u[l];
     };
-    // the state as stored (u + carry)
-    auto state_out = [&](int l) { return carry_upd ? carry_finish(u[l], car[l], sh) : u[l]; };
 
     int fsel = 0;
     double2* Dc = D0;   // FP64-solver ping-pong buffers
@@ -607,26 +511,23 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
             const double2 dk = dk_next;
             const int cnt = cnt_next;
             if (jj + 1 < nit) load_ctrl(jj + 1);
-            step_coefficients<L, Q>(pd, lane, dk, cnt, coef_d + (par * 2 + cslot) * NSLOT,
-                                    coef_f + (par * 2 + cslot) * NSLOT,
-                                    coef_s ? coef_s + (par * 2 + cslot) * NSLOT : nullptr,
-                                    params + (par * 2 + cslot) * 4);
+            step_coefficients<L, Q, SOLVER>(pd, lane, dk, cnt, coef_d + (par * 2 + cslot) * NSLOT,
+                                            coef_f + (par * 2 + cslot) * NSLOT, coef_s + (par * 2 + cslot) * NSLOT,
+                                            params + (par * 2 + cslot) * 4);
         }
         // checkpoint: the state at the start of every segment (forward over whole windows)
-        // (the carry is folded into u there, so that a segment recomputed from its checkpoint
+        // (the state is rounded to what is stored, so that a segment recomputed from its checkpoint
         // repeats these steps bit for bit)
         if (want_ckpt && live && jj % pd.kseg == 0) {
-            if (carry_upd) {
+            double2* ck = pd.ckpt + ((size_t(m - 1) * pd.nseg + jj / pd.kseg) * E + col) * N + f * L;
 #pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    u[l] = carry_finish(u[l], car[l], sh);
-                    car[l] = make_float2(0.f, 0.f);
+            for (int l = 0; l < L; ++l) {
+                const double2 o = state_out(l);
+                if (act) ck[l] = o;
+                if constexpr (SOLVER == SOLVER_MIXED) {
+                    v[l][0] = tf_split(o.x, sh);
+                    v[l][1] = tf_split(o.y, sh);
                 }
-            }
-            if (act) {
-                double2* ck = pd.ckpt + ((size_t(m - 1) * pd.nseg + jj / pd.kseg) * E + col) * N + f * L;
-#pragma unroll
-                for (int l = 0; l < L; ++l) ck[l] = u[l];
             }
         }
         const double2* cfd = coef_d + (par * 2 + slot) * NSLOT;
@@ -636,14 +537,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
         const int* prm0 = params + (par * 2) * 4;
         const int* prm1 = params + (par * 2 + 1) * 4;
 
-        // the midpoint state being solved for (Ubar or Lbar): FP64 (FP64 solver) or, for the
-        // mixed solver, the two-float sum zf = b + d_total in the column's scaled units (about
-        // 2^-47 |z|), which the forward's history and the adjoint's gradient products use; the
-        // mixed solver's state update needs only the correction d_total (dre, dim: two-float)
+        // the midpoint state (Ubar or Lbar) the history keeps: FP64, or split (mixed solver)
         double2 z[L];
         float4 zf[L];
-        DF dre[L], dim[L];
-        DF bre[L], bim[L];   // mixed solver: b = P u (conj(P) for the adjoint), two-float
 
         // first barrier of the step: the coefficients are published; thread 0 stores the
         // previous group's midpoints
@@ -680,7 +576,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
                     tile_sync();
                 }
                 double2 w[L];
-                apply_off<L, Q, double2>(Dc, cfd, fb, z, w, pd);
+                apply_off<L, Q, double2>(Dc, cfd, fb, z, w, ex_s);
                 if (it < Kown) {
 #pragma unroll
                     for (int l = 0; l < L; ++l) z[l] = cadd_scaled<S>(b[l], Pd[l], w[l]);
@@ -690,158 +586,170 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
                 Dn = tmp;
             }
         } else {
-            // ---- b = P u (conj(P) for the adjoint) as a two-float sum in the column's scaled
-            // units: the FP32 stage's right-hand side and the point at which the refinement
-            // evaluates the off-diagonal apply.  The residual below is that of the exact P u
-            // (it is formed as s P w(z) - d_total), so b's 2^-47 error enters the solve only
-            // through the evaluation point of a term of size rho.  The state update takes R u
-            // either in FP64 (R = 2P - 1) or, compensated, as u + 2 kappa (Im b, -Re b), where
-            // b's error enters times |2 kappa| <= 2^-4.5; there the state is u + carry, and
-            // P carry (|carry| <= half an FP32 unit of the last increment) joins the low parts.
+            // The midpoint increment m = z - U of (I + iX) z = U solves m = -i kappa z + s w(z) with
+            // w = iX_C z (s = -1; the adjoint has -kappa and s = +1), and U' = U + 2 m.  An FP32
+            // estimate m0 gives z = U + m0 exactly (two floats), the right-hand side at that z is
+            // formed once in compensated FP32 (m1), and the correction delta = z* - z solves
+            // (I + i kappa - s w) delta = R = m1 - m0, small (the FP32 rounding of m0 and what its
+            // sweeps left) and therefore FP32: m = m1 + (delta - R).  The state and every
+            // increment's leading part are never rounded; see step_counts for the counts.
+            float2 m0[L], d[L], y[L];
 #pragma unroll
             for (int l = 0; l < L; ++l) {
-                const float4 t = cq[f * L + l];
-                carry_rhs(split_scaled(u[l], sh), Ps[l], make_float2(t.y, t.z), car[l], bre[l], bim[l]);
+                // G u0 and, as the first sweep's point, P u0 = u0 + G u0
+                m0[l] = make_float2(fmaf(Gf[l].x, v[l][0].a, -Gf[l].y * v[l][1].a),
+                                    fmaf(Gf[l].x, v[l][1].a, Gf[l].y * v[l][0].a));
+                y[l] = make_float2(v[l][0].a + m0[l].x, v[l][1].a + m0[l].y);
             }
-            // ---- FP32 stage: d = Ubar - b from the preconditioned fixed point d = s P w(b + d)
-            float2 bf[L], df[L], y[L];
-#pragma unroll
-            for (int l = 0; l < L; ++l) {
-                bf[l] = make_float2(fadd_n(bre[l].s, bre[l].c), fadd_n(bim[l].s, bim[l].c));
-                y[l] = bf[l];
-            }
-            {
+            // s P w for P = 1 + G
+            auto precond = [&](int l, const float2& w) {
+                const float x = fmaf(Gf[l].x, w.x, fmaf(-Gf[l].y, w.y, w.x)), yy = fmaf(Gf[l].x, w.y, fmaf(Gf[l].y, w.x, w.y));
+                return S > 0 ? make_float2(x, yy) : make_float2(-x, -yy);
+            };
+            auto exchange = [&](const float2 (&x)[L]) {
                 float2* Fb = fsel ? FB : FA;
                 fsel ^= 1;
                 if (act) {
 #pragma unroll
-                    for (int l = 0; l < L; ++l) Fb[fb.xo + l] = y[l];
+                    for (int l = 0; l < L; ++l) Fb[fb.xo + l] = x[l];
                 }
                 tile_sync();
-                first_sync_work();
-                float2 w[L];
-                apply_off<L, Q, float2>(Fb, cff, fb, y, w, pd);
+                return Fb;
+            };
+            float2* Fb = exchange(y);
+            first_sync_work();
+            // coarse steps (uniform over a slot) go to FP64 below
+            const bool coarse0 = prm0[3] & 2, coarse1 = nslot > 1 ? (prm1[3] & 2) != 0 : coarse0;
+            if (!coarse0 || !coarse1) {
+                const int j1 = prm[0], j2 = prm[1], R = prm[2];
+                const bool two = nslot > 1 && !coarse0 && !coarse1;
+                const int* pm = coarse0 ? prm1 : prm0;
+                const int j1max = two ? max(prm0[0], prm1[0]) : pm[0];
+                const int j2max = two ? max(prm0[1], prm1[1]) : pm[1];
+                const int Rmax = two ? max(prm0[2], prm1[2]) : pm[2];
+                for (int it = 0;;) {
+                    float2 w[L];
+                    apply_off<L, Q, float2>(Fb, cff, fb, y, w, ex_s);
+                    if (it < j1) {
 #pragma unroll
-                for (int l = 0; l < L; ++l) df[l] = cadd_scaled<S>(make_float2(0.f, 0.f), Pf[l], w[l]);
-            }
-            const int j1 = prm[0], j2 = prm[1], R = prm[2];
-            const int j1max = nslot > 1 ? max(prm0[0], prm1[0]) : prm0[0];
-            const int j2max = nslot > 1 ? max(prm0[1], prm1[1]) : prm0[1];
-            const int Rmax = nslot > 1 ? max(prm0[2], prm1[2]) : prm0[2];
-            for (int it = 1; it < j1max; ++it) {
+                        for (int l = 0; l < L; ++l) d[l] = precond(l, w[l]);
+                    }
+                    if (++it >= j1max) break;
 #pragma unroll
-                for (int l = 0; l < L; ++l) y[l] = make_float2(bf[l].x + df[l].x, bf[l].y + df[l].y);
-                float2* Fb = fsel ? FB : FA;
-                fsel ^= 1;
-                if (act) {
-#pragma unroll
-                    for (int l = 0; l < L; ++l) Fb[fb.xo + l] = y[l];
+                    for (int l = 0; l < L; ++l)
+                        y[l] = make_float2((v[l][0].a + m0[l].x) + d[l].x, (v[l][1].a + m0[l].y) + d[l].y);
+                    Fb = exchange(y);
                 }
-                tile_sync();
-                float2 w[L];
-                apply_off<L, Q, float2>(Fb, cff, fb, y, w, pd);
-                if (it < j1) {
-#pragma unroll
-                    for (int l = 0; l < L; ++l) df[l] = cadd_scaled<S>(make_float2(0.f, 0.f), Pf[l], w[l]);
-                }
-            }
-            // ---- refinement: z = b + d_total, residual r = s P w(z) - d_total (that of the exact
-            // P u), an FP32 correction e added to d_total (two-float, scaled units)
-#pragma unroll
-            for (int l = 0; l < L; ++l) {
-                dre[l] = DF{df[l].x, 0.f};
-                dim[l] = DF{df[l].y, 0.f};
-            }
-            // the residual's apply in compensated FP32 (split entries in D0) where the step's
-            // contraction factor (exchange included) allows it (step_counts) and the exchange
-            // terms, if any, have precomputed sources, else in FP64; uniform over a slot, so a
-            // column's entries in D0 have one form
-            const bool dfa = (pd.nex == 0 || (L == 2 && pd.nex <= MAXEXF)) && !(prm[3] & 2);
-            float4* D0s = reinterpret_cast<float4*>(D0);
-            for (int pass = 0;; ++pass) {
-                float4 zs[L];
+                float4* D0s = reinterpret_cast<float4*>(D0);
+                DF mr[L], mi[L];   // the current z - U
 #pragma unroll
                 for (int l = 0; l < L; ++l) {
-                    const DF zr = df_add(bre[l], dre[l]), zi = df_add(bim[l], dim[l]);
-                    zs[l] = make_float4(zr.s, zi.s, zr.c, zi.c);
+                    mr[l] = DF{m0[l].x + d[l].x, 0.f};
+                    mi[l] = DF{m0[l].y + d[l].y, 0.f};
+                    const DF zr = two_sum(v[l][0].a, mr[l].s), zi = two_sum(v[l][1].a, mi[l].s);
+                    zf[l] = make_float4(zr.s, zi.s, fadd_n(zr.c, v[l][0].b), fadd_n(zi.c, v[l][1].b));
                 }
-                if (dfa) {
+                for (int pass = 0;; ++pass) {
                     if (act) {
 #pragma unroll
-                        for (int l = 0; l < L; ++l) D0s[fb.xo + l] = zs[l];
+                        for (int l = 0; l < L; ++l) D0s[fb.xo + l] = zf[l];
                     }
-                } else if (act) {
-                    SplitVals<L> zv;
-#pragma unroll
-                    for (int l = 0; l < L; ++l) zv.v[l] = zs[l];
-                    store_z64<L>(D0 + fb.xo, zv, sh);
-                }
-                // the staged midpoints of the previous step must have been read by their
-                // bulk store (issued at this step's first barrier) before this step's are staged;
-                // waiting here, ahead of a barrier every step has, makes the staging barrier-free
-                if (want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
-                tile_sync();
-                float2 rf[L], e[L];
-                if (dfa) {
-                    DF w[L][2];
-                    apply_off_df<L, Q>(D0s, cfs, fb, zs, w, exc, pd.nex);
-#pragma unroll
-                    for (int l = 0; l < L; ++l) {
-                        rf[l] = resid_df<S>(make_float2(dre[l].s, dim[l].s), make_float2(dre[l].c, dim[l].c), Ps[l],
-                                            w[l]);
-                        e[l] = rf[l];
-                    }
-                } else {
-                    ResidIn<L> in;
-#pragma unroll
-                    for (int l = 0; l < L; ++l) {
-                        in.zs[l] = zs[l];
-                        in.dre[l] = dre[l];
-                        in.dim[l] = dim[l];
-                    }
-                    const ResidOut<L> o = resid_fp64<L, Q, S, BWD>(D0, cfd, pd, c, f, a.cpt * N, in, sh);
-#pragma unroll
-                    for (int l = 0; l < L; ++l) {
-                        rf[l] = o.r[l];
-                        e[l] = rf[l];
-                    }
-                }
-                for (int it = 0; it < j2max; ++it) {
-                    float2* Fb = fsel ? FB : FA;
-                    fsel ^= 1;
-                    if (act) {
-#pragma unroll
-                        for (int l = 0; l < L; ++l) Fb[fb.xo + l] = e[l];
-                    }
+                    // the staged midpoints of the previous step must have been read by their bulk
+                    // store (issued at this step's first barrier) before this step's are staged;
+                    // waiting here, ahead of a barrier every step has, makes the staging
+                    // barrier-free
+                    if (want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
                     tile_sync();
-                    float2 wf[L];
-                    apply_off<L, Q, float2>(Fb, cff, fb, e, wf, pd);
-                    if (it < j2) {
+                    float2 r[L], pr[L], e[L];
+                    {
+                        DF w[L][2];
+                        apply_off_df<L, Q>(D0s, cfs, fb, zf, w, ex_s);
 #pragma unroll
-                        for (int l = 0; l < L; ++l) e[l] = cadd_scaled<S>(rf[l], Pf[l], wf[l]);
+                        for (int l = 0; l < L; ++l) {
+                            // m1 = -i kappa z + s w
+                            DF kr = kappa_mul(kh[l], kl[l], k3[l], zf[l].y, zf[l].w);
+                            DF ki = df_neg(kappa_mul(kh[l], kl[l], k3[l], zf[l].x, zf[l].z));
+                            kr = df_add(kr, S > 0 ? w[l][0] : df_neg(w[l][0]));
+                            ki = df_add(ki, S > 0 ? w[l][1] : df_neg(w[l][1]));
+                            r[l] = make_float2(fadd_n(fsub_n(kr.s, mr[l].s), fsub_n(kr.c, mr[l].c)),
+                                               fadd_n(fsub_n(ki.s, mi[l].s), fsub_n(ki.c, mi[l].c)));
+                            if (pass < R) {
+                                mr[l] = kr;
+                                mi[l] = ki;
+                            }
+                            // P R, the first sweep's point
+                            pr[l] = make_float2(fmaf(Gf[l].x, r[l].x, fmaf(-Gf[l].y, r[l].y, r[l].x)),
+                                                fmaf(Gf[l].x, r[l].y, fmaf(Gf[l].y, r[l].x, r[l].y)));
+                            e[l] = pr[l];
+                        }
                     }
+                    for (int it = 0; it < j2max; ++it) {
+                        float2* Fe = exchange(e);
+                        float2 w[L];
+                        apply_off<L, Q, float2>(Fe, cff, fb, e, w, ex_s);
+                        if (it < j2) {
+#pragma unroll
+                            for (int l = 0; l < L; ++l) {
+                                const float2 t = precond(l, w[l]);
+                                e[l] = make_float2(pr[l].x + t.x, pr[l].y + t.y);
+                            }
+                        }
+                    }
+                    if (pass < R) {
+#pragma unroll
+                        for (int l = 0; l < L; ++l) {
+                            mr[l].c = fadd_n(mr[l].c, fsub_n(e[l].x, r[l].x));
+                            mi[l].c = fadd_n(mi[l].c, fsub_n(e[l].y, r[l].y));
+                            const DF zr = two_sum(zf[l].x, e[l].x), zi = two_sum(zf[l].y, e[l].y);
+                            zf[l] = make_float4(zr.s, zi.s, fadd_n(zf[l].z, zr.c), fadd_n(zf[l].w, zi.c));
+                        }
+                    }
+                    if (pass + 1 >= Rmax) break;
+                    // another pass rewrites D0: every thread must be done reading it
+                    tile_sync();
                 }
-                if (pass < R) {
+                // U' = U + 2 m
+                if (live && !(prm[3] & 2)) {
 #pragma unroll
                     for (int l = 0; l < L; ++l) {
-                        dre[l] = df_add(dre[l], DF{e[l].x, 0.f});
-                        dim[l] = df_add(dim[l], DF{e[l].y, 0.f});
+                        tf_add(v[l][0], fadd_n(mr[l].s, mr[l].s), fadd_n(mr[l].c, mr[l].c));
+                        tf_add(v[l][1], fadd_n(mi[l].s, mi[l].s), fadd_n(mi[l].c, mi[l].c));
                     }
                 }
-                if (pass + 1 >= Rmax) break;
-                // another pass rewrites D0: every thread must be done reading it
-                tile_sync();
+            } else if (want_hist && tid == 0 && hpos == 0) {
+                bulk_wait_read_all();   // (the coarse step's barriers follow)
             }
+            if (coarse0 || coarse1) {
+                const bool mine = prm[3] & 2;
+                const int Kmax = max(coarse0 ? prm0[0] : 0, coarse1 ? (nslot > 1 ? prm1[0] : prm0[0]) : 0);
+                CoarseIO<L> io;
 #pragma unroll
-            for (int l = 0; l < L; ++l) {
-                const DF zr = df_add(bre[l], dre[l]), zi = df_add(bim[l], dim[l]);
-                zf[l] = make_float4(zr.s, zi.s, zr.c, zi.c);
+                for (int l = 0; l < L; ++l) {
+                    io.u[l][0] = v[l][0];
+                    io.u[l][1] = v[l][1];
+                }
+                coarse_step<L, Q, S, BWD>(D0, coef_d, pd, ex_s, c, f, a.cpt * N, step_of(0, jj), step_of(nslot - 1, jj),
+                                          nslot, slot, act, mine, mine ? prm[0] : 0, Kmax, sh, io);
+                if (mine) {
+#pragma unroll
+                    for (int l = 0; l < L; ++l) {
+                        zf[l] = io.z[l];
+                        if (live) {
+                            v[l][0] = io.u[l][0];
+                            v[l][1] = io.u[l][1];
+                        }
+                    }
+                }
             }
         }
         if (tid == 0 && ((prm0[3] & 1) || (nslot > 1 && (prm1[3] & 1)))) atomicOr(pd.status, ST_SOLVER_RANGE);
-        // the state update (U_{n+1} = 2 Ubar - U_n; Lambda_n = 2 Lbar - Lambda_{n+1}) as soon as
-        // the step is solved: what follows (history, gradient products) needs only the midpoint
-        if (live) state_update(u, z, bre, bim, dre, dim);
+        if constexpr (SOLVER == SOLVER_FP64) {
+            // U_{n+1} = 2 Ubar - U_n; Lambda_n = 2 Lbar - Lambda_{n+1}
+            if (live) {
+#pragma unroll
+                for (int l = 0; l < L; ++l) u[l] = reflect(z[l], u[l]);
+            }
+        }
 
         // ---- midpoint states for the quadrature (async bulk store at the next step)
         if (want_hist) {

@@ -162,8 +162,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int64_
 }
 
 // ------------------------------------------------------------------ per-thread neighbour lists
-// exchange-coupled pairs whose sources a fiber keeps precomputed (more use the general form)
+// exchange-coupled pairs up to which lane quads are admitted
 constexpr int MAXEXF = 6;
+// The dipole exchange of a 2-level problem, per tile in shared memory: pair e couples the rows
+// whose two digits differ to the row with both digits flipped (mask: the two digits' bits), with
+// the coefficient i (h/2) J.
+struct ExTab {
+    int n;
+    int mask[MAXEX];
+    float2 cs[MAXEX];   // (h/2) J split into two floats; x is its FP32 rounding
+    double cd[MAXEX];
+};
+__device__ __forceinline__ void fill_exchange(ExTab& t, const ProbDev& pd) {
+    for (int e = threadIdx.x; e < pd.nex; e += blockDim.x) {
+        t.mask[e] = (1 << (pd.q - 1 - pd.ex_j[e])) | (1 << (pd.q - 1 - pd.ex_k[e]));
+        t.cs[e] = split_scaled(pd.ex_c[e], 0);
+        t.cd[e] = pd.ex_c[e];
+    }
+    if (threadIdx.x == 0) t.n = pd.nex;
+}
 template <int L, int Q>
 struct Fiber {
     static constexpr int NFIX = Q - 1;
@@ -178,10 +195,10 @@ struct Fiber {
     bool plus1[NA];    // entry 1 is the a_k (lowering, "+") term
     double w1[NA];     // product weight sqrt(level factor) of entry 1
     double w2[NA];
-    // dipole exchange of a 2-level (qubit) problem with at most MAXEXF coupled pairs: the source
-    // of pair e's term for entry l (an entry index in a [cb][N] buffer, or the buffer's zero
-    // entry when the pair gives that entry no term), so the apply is the same for every lane
-    int exs[MAXEXF][L];
+    // dipole exchange of 2-level subsystems: the column's first entry, the buffers' zero entry and,
+    // per entry of the fiber, the pairs that give it a term
+    int eb, zero;
+    unsigned exm[L];
 
     // c: tile column, f: fiber, zero: index of the shared buffers' zero entry
     __device__ void init(int c, int f, const ProbDev& pd, int zero) {
@@ -212,41 +229,21 @@ struct Fiber {
                 w2[k] = 0.0;
             }
         }
-        if constexpr (L == 2 && Q >= 2) init_exchange(pd, zero);
-    }
-
-    // For 2 levels every weight of the exchange terms is 1 and a coupled pair (j, k) gives the
-    // fiber at most one term.  k the last subsystem: level 1 of the fiber takes level 0 of the
-    // fiber with l_j + 1 (a_k^+ a_j, when l_j = 0), or level 0 takes level 1 of the fiber with
-    // l_j - 1 (a_k a_j^+, when l_j = 1).  k not the last: every entry takes the same level of
-    // the fiber with (l_j + 1, l_k - 1) when (l_j, l_k) = (0, 1), or (l_j - 1, l_k + 1) when
-    // (1, 0).  Computed once per launch instead of in every apply.
-    __device__ void init_exchange(const ProbDev& pd, int zero) {
+        eb = c * N;
+        this->zero = zero;
 #pragma unroll
-        for (int e = 0; e < MAXEXF; ++e) {
-#pragma unroll
-            for (int l = 0; l < L; ++l) exs[e][l] = zero;
-            if (e < pd.nex) {
-                const int j = pd.ex_j[e], k = pd.ex_k[e];
-                int sfj = 1, sfk = 1;                          // fiber strides (j is never the last)
-                for (int t = j; t < Q - 2; ++t) sfj *= 2;
-                for (int t = k; t < Q - 2; ++t) sfk *= 2;
-                const int lj = (f / sfj) % 2;
-                if (k == Q - 1) {
-                    if (lj == 0)
-                        exs[e][1] = xo + sfj * 2;
-                    else
-                        exs[e][0] = xo - sfj * 2 + 1;
-                } else {
-                    const int lk = (f / sfk) % 2;
-#pragma unroll
-                    for (int l = 0; l < L; ++l) {
-                        if (lk == 1 && lj == 0) exs[e][l] = xo + (sfj - sfk) * 2 + l;
-                        if (lk == 0 && lj == 1) exs[e][l] = xo + (sfk - sfj) * 2 + l;
-                    }
-                }
+        for (int l = 0; l < L; ++l) {
+            exm[l] = 0;
+            if constexpr (L == 2 && Q >= 2) {
+                const int i = f * 2 + l;
+                for (int e = 0; e < pd.nex; ++e)
+                    if (((i >> (Q - 1 - pd.ex_j[e])) ^ (i >> (Q - 1 - pd.ex_k[e]))) & 1) exm[l] |= 1u << e;
             }
         }
+    }
+    // buffer entry of pair e's term for entry l of the fiber (the zero entry where it has none)
+    __device__ __forceinline__ int exsrc(int e, int l, int mask) const {
+        return (exm[l] >> e) & 1u ? eb + ((f * L + l) ^ mask) : zero;
     }
 };
 
@@ -255,7 +252,7 @@ struct Fiber {
 // keep each coefficient in the form of either part, so their coefficient arrays are twice as
 // large.
 struct SweepSmem {
-    size_t coef_d, coef_f, coef_s, params, cq, D0, D1, FA, FB, H, total;
+    size_t coef_d, coef_f, coef_s, params, D0, D1, FA, FB, H, total;
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -274,9 +271,6 @@ __host__ __device__ inline SweepSmem sweep_layout(int q, int L, int N, int cpt, 
     // solver's one-thread families
     s.coef_s = o; o = align16(o + (!pair && solver == SOLVER_MIXED ? size_t(2) * 2 * nslot * 16 : 0));
     s.params = o; o = align16(o + 2 * 2 * 4 * 4);                      // [parity][slot][4]
-    // the mixed solver's one-thread families: per fiber entry the third parts of the splits of
-    // 2 kappa and P (the compensated state update)
-    s.cq = o;     o = align16(o + (!pair && solver == SOLVER_MIXED ? size_t(N) * 16 : 0));
     s.D0 = o;     o = align16(o + buf_d);
     s.D1 = o;     o = align16(o + (solver == SOLVER_FP64 ? buf_d : 0));
     s.FA = o;     o = align16(o + (solver == SOLVER_MIXED ? buf_f : 0));

@@ -47,70 +47,18 @@ __device__ __forceinline__ float pmac(float acc, float2 c, float xa, float xb) {
     return fmaf(c.x, xa, fmaf(c.y, xb, acc));
 }
 
-// Dipole exchange on the fiber (fiber index f, entries at fb.xo of a [cols][N] buffer), part p:
-// w += (i (h/2) J_jk (a_k^+ a_j + a_k a_j^+) x)_p for every coupled pair j < k.  a_k^+ a_j moves
-// one quantum from j to k: the source has l_j + 1 and l_k - 1, weight sqrt(l_k) sqrt(l_j + 1);
-// a_k a_j^+ the opposite, weight sqrt(l_k + 1) sqrt(l_j).  When k is the last subsystem the
-// source is an entry of the neighbour fiber in subsystem j at the shifted level; otherwise a
-// fiber that differs in both digits, at the same level.  (i c x)_p = (p ? c : -c) x_{1-p}, so
-// only the other component of each source is read (xb: the buffer's component 1 - p).  The
-// pairs are warp-uniform; the level tests are per lane.
-template <int L, int Q, typename R>
-__device__ __forceinline__ void apply_exchange_pair(const R* __restrict__ xb, const ProbDev& pd, int f, int xo, int p,
-                                               R (&w)[L]) {
-    for (int e = 0; e < pd.nex; ++e) {
-        const int j = pd.ex_j[e], k = pd.ex_k[e];
-        int sfj = 1, sfk = 1;                                  // fiber strides (j is never the last)
-        for (int t = j; t < Q - 2; ++t) sfj *= L;
-        for (int t = k; t < Q - 2; ++t) sfk *= L;
-        const int lj = (f / sfj) % L;
-        const R c = static_cast<R>(p ? pd.ex_c[e] : -pd.ex_c[e]);
-        if (k == Q - 1) {
-#pragma unroll
-            for (int l = 0; l < L; ++l) {
-                // a_k^+ a_j: from (l_j + 1, l - 1)
-                if (l >= 1 && lj <= L - 2) {
-                    const R wt = c * static_cast<R>(sqrt_small(l) * sqrt_small(lj + 1));
-                    w[l] += wt * xb[2 * (xo + sfj * L + (l - 1))];
-                }
-                // a_k a_j^+: from (l_j - 1, l + 1)
-                if (l <= L - 2 && lj >= 1) {
-                    const R wt = c * static_cast<R>(sqrt_small(l + 1) * sqrt_small(lj));
-                    w[l] += wt * xb[2 * (xo - sfj * L + (l + 1))];
-                }
-            }
-        } else {
-            const int lk = (f / sfk) % L;
-            if (lk >= 1 && lj <= L - 2) {
-                const R wt = c * static_cast<R>(sqrt_small(lk) * sqrt_small(lj + 1));
-                const int o = 2 * (xo + (sfj - sfk) * L);
-#pragma unroll
-                for (int l = 0; l < L; ++l) w[l] += wt * xb[o + 2 * l];
-            }
-            if (lk <= L - 2 && lj >= 1) {
-                const R wt = c * static_cast<R>(sqrt_small(lk + 1) * sqrt_small(lj));
-                const int o = 2 * (xo + (sfk - sfj) * L);
-#pragma unroll
-                for (int l = 0; l < L; ++l) w[l] += wt * xb[o + 2 * l];
-            }
-        }
-    }
-}
-
 // w = (iX_C x)_p on the fiber, part p: ladder terms of the last subsystem from the fiber itself,
 // the others from the shared buffer (entries interleaved re, im; both parts of the pair have
 // written theirs before the barrier).  xa: this part's components of the fiber (registers);
 // cf: this part's coefficient pairs of the step's slots, i(h/2)sqrt(.)d_k.
 //
 // SPLIT = 2 (lane quads, L = 2): the thread holds entry le of the fiber only (xa[0], w[0]); the
-// other entry of the in-fiber ladder term comes from the buffer, and exo[e] is the source of
-// exchange pair e for entry le (the problem has at most MAXEXF pairs: the host admits the
-// family only then).
+// other entry of the in-fiber ladder term comes from the buffer.
 template <int L, int Q, typename T2, int SPLIT>
 __device__ __forceinline__ void apply_off_pair(const T2* __restrict__ buf, const T2* __restrict__ cf,
                                                const Fiber<L, Q>& fb, const typename cx<T2>::T (&xa)[L / SPLIT],
                                                typename cx<T2>::T (&w)[L / SPLIT], int p, int le,
-                                               const int (&exo)[MAXEXF], const ProbDev& pd) {
+                                               const ExTab& ex) {
     using R = typename cx<T2>::T;
     constexpr int LS = L / SPLIT;
     const R* ba = reinterpret_cast<const R*>(buf) + p;        // component p of entry i: ba[2 i]
@@ -144,21 +92,17 @@ __device__ __forceinline__ void apply_off_pair(const T2* __restrict__ buf, const
         }
     }
     // exchange-coupled problems are 2-level qubit models (the only shapes compiled with it):
-    // w += (i (h/2) J x_src)_p from the fiber's precomputed sources (a zero entry where a pair
-    // gives an entry no term), or, lane pairs only, the general form beyond MAXEXF pairs
+    // w += (i (h/2) J x_src)_p, and (i c x)_p = (p ? c : -c) x_{1-p}
     if constexpr (L == 2 && Q >= 2) {
-        bool general = false;
-        if constexpr (SPLIT == 1) general = pd.nex > MAXEXF;
-        if (general) {
-            if constexpr (SPLIT == 1) apply_exchange_pair<L, Q, R>(bb, pd, fb.f, fb.xo, p, w);
-        } else if (pd.nex) {
+        for (int e = 0; e < ex.n; ++e) {                       // uniform
+            R c;
+            if constexpr (sizeof(R) == 4)
+                c = p ? ex.cs[e].x : -ex.cs[e].x;
+            else
+                c = p ? ex.cd[e] : -ex.cd[e];
+            const int mask = ex.mask[e];
 #pragma unroll
-            for (int e = 0; e < MAXEXF; ++e) {
-                if (e >= pd.nex) break;                        // warp-uniform
-                const R c = static_cast<R>(p ? pd.ex_c[e] : -pd.ex_c[e]);
-#pragma unroll
-                for (int l = 0; l < LS; ++l) w[l] += c * bb[2 * (SPLIT == 1 ? fb.exs[e][l] : exo[e])];
-            }
+            for (int l = 0; l < LS; ++l) w[l] += c * bb[2 * fb.exsrc(e, le + l, mask)];
         }
     }
 }
@@ -283,12 +227,8 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
 
     Fiber<L, Q> fb;
     fb.init(c, f, pd, a.cpt * N);
-    // lane quads: the exchange sources of this thread's entry
-    int exo[MAXEXF] = {};
-    if constexpr (SPLIT > 1) {
-#pragma unroll
-        for (int e = 0; e < MAXEXF; ++e) exo[e] = le ? fb.exs[e][1] : fb.exs[e][0];
-    }
+    __shared__ ExTab ex_s;   // (ordered before its first read by the first barrier of the time loop)
+    fill_exchange(ex_s, pd);
     // the apply buffers' zero entry (read by the exchange terms a fiber entry does not have; the
     // first barrier of the time loop orders these stores before any read)
     if (tid == 0) {
@@ -456,7 +396,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                     tile_sync();
                 }
                 double w[LS];
-                apply_off_pair<L, Q, double2, SPLIT>(Dc, cfd, fb, z, w, part, le, exo, pd);
+                apply_off_pair<L, Q, double2, SPLIT>(Dc, cfd, fb, z, w, part, le, ex_s);
                 double wo[LS];
 #pragma unroll
                 for (int l = 0; l < LS; ++l) wo[l] = partner(w[l]);
@@ -483,7 +423,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 tile_sync();
                 first_sync_work();
                 float w[LS];
-                apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, exo, pd);
+                apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, ex_s);
 #pragma unroll
                 for (int l = 0; l < LS; ++l) {
                     const float wo = partner(w[l]);
@@ -502,7 +442,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 if (act) store_part<LS, float2>(Fb, fb.xo + le, part, y);
                 tile_sync();
                 float w[LS], wo[LS];
-                apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, exo, pd);
+                apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, ex_s);
 #pragma unroll
                 for (int l = 0; l < LS; ++l) wo[l] = partner(w[l]);
                 if (it < j1) {
@@ -526,7 +466,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 if (want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
                 tile_sync();
                 double w[LS];
-                apply_off_pair<L, Q, double2, SPLIT>(D0, cfd, fb, z, w, part, le, exo, pd);
+                apply_off_pair<L, Q, double2, SPLIT>(D0, cfd, fb, z, w, part, le, ex_s);
                 float rf[LS], e[LS];
 #pragma unroll
                 for (int l = 0; l < LS; ++l) {
@@ -541,7 +481,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                     if (act) store_part<LS, float2>(Fb, fb.xo + le, part, e);
                     tile_sync();
                     float wf[LS], wfo[LS];
-                    apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, e, wf, part, le, exo, pd);
+                    apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, e, wf, part, le, ex_s);
 #pragma unroll
                     for (int l = 0; l < LS; ++l) wfo[l] = partner(wf[l]);
                     if (it < j2) {
