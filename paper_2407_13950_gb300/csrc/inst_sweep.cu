@@ -21,16 +21,20 @@ namespace msqoc {
 
 // FAM: log2 of the threads per fiber (0: k_sweep; 1, 2: k_sweep_pair with one or two entry groups),
 // or 3: k_sweep with the 168-register budget (one thread per fiber, up to 12 warps an SM)
-template <int SOLVER, bool BWD, bool ROLLOUT, int FAM>
+// BOTH: k_sweep_both
+template <int SOLVER, bool BWD, bool PROP, int FAM, bool BOTH = false>
 static auto kernel_of() {
-    if constexpr (FAM == 3)
-        return k_sweep<MSQOC_L, MSQOC_Q, SOLVER, BWD, ROLLOUT, MAX_LEAN_TILE_THREADS>;
-    else if constexpr (FAM == 2)
-        return k_sweep_pair<MSQOC_L, MSQOC_Q, SOLVER, BWD, ROLLOUT, 2>;
-    else if constexpr (FAM == 1)
-        return k_sweep_pair<MSQOC_L, MSQOC_Q, SOLVER, BWD, ROLLOUT, 1>;
+    if constexpr (BOTH)
+        return k_sweep_both<MSQOC_L, MSQOC_Q, FAM == 3 ? MAX_LEAN_TILE_THREADS : MAX_TILE_THREADS>;
     else
-        return k_sweep<MSQOC_L, MSQOC_Q, SOLVER, BWD, ROLLOUT>;
+    if constexpr (FAM == 3)
+        return k_sweep<MSQOC_L, MSQOC_Q, SOLVER, BWD, PROP, MAX_LEAN_TILE_THREADS>;
+    else if constexpr (FAM == 2)
+        return k_sweep_pair<MSQOC_L, MSQOC_Q, SOLVER, BWD, 2>;
+    else if constexpr (FAM == 1)
+        return k_sweep_pair<MSQOC_L, MSQOC_Q, SOLVER, BWD, 1>;
+    else
+        return k_sweep<MSQOC_L, MSQOC_Q, SOLVER, BWD, PROP>;
 }
 
 // Dynamic shared memory above 48 KB needs the kernel's opt-in attribute, and the 48 KB limit
@@ -40,27 +44,27 @@ static auto kernel_of() {
 constexpr size_t SMEM_DEFAULT_LIMIT = 48 * 1024;
 
 // one static per kernel instantiation (the template parameters name the kernel)
-template <int SOLVER, bool BWD, bool ROLLOUT, int FAM>
+template <int SOLVER, bool BWD, bool PROP, int FAM, bool BOTH = false>
 static bool needs_opt_in(size_t smem) {
     static const size_t static_bytes = [] {
         cudaFuncAttributes fa{};
         // an unreadable attribute counts as the largest static size, so the opt-in is taken
-        return cudaFuncGetAttributes(&fa, kernel_of<SOLVER, BWD, ROLLOUT, FAM>()) == cudaSuccess ? fa.sharedSizeBytes
+        return cudaFuncGetAttributes(&fa, kernel_of<SOLVER, BWD, PROP, FAM, BOTH>()) == cudaSuccess ? fa.sharedSizeBytes
                                                                                                  : SMEM_DEFAULT_LIMIT;
     }();
     return smem + static_bytes > SMEM_DEFAULT_LIMIT;
 }
 
-template <int SOLVER, bool BWD, bool ROLLOUT, int FAM>
+template <int SOLVER, bool BWD, bool PROP, int FAM, bool BOTH = false>
 static cudaError_t launch_one(const SweepArgs& a, int ntiles, cudaStream_t s) {
-    auto kern = kernel_of<SOLVER, BWD, ROLLOUT, FAM>();
+    auto kern = kernel_of<SOLVER, BWD, PROP, FAM, BOTH>();
     const size_t smem = sweep_smem_bytes(a);
-    if (needs_opt_in<SOLVER, BWD, ROLLOUT, FAM>(smem)) {
+    if (needs_opt_in<SOLVER, BWD, PROP, FAM, BOTH>(smem)) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
     }
     if (ntiles <= 0) return cudaSuccess;
-    kern<<<ntiles, a.nthreads, smem, s>>>(a);
+    kern<<<BOTH ? 2 * ntiles : ntiles, a.nthreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -78,9 +82,13 @@ static int occupancy_one(const SweepArgs& a) {
 
 template <int FAM>
 static cudaError_t launch_family(const SweepArgs& a, int ntiles, cudaStream_t s) {
-    if (a.mode == SWEEP_ROLLOUT)
-        return a.solver == SOLVER_FP64 ? launch_one<SOLVER_FP64, false, true, FAM>(a, ntiles, s)
-                                       : launch_one<SOLVER_MIXED, false, true, FAM>(a, ntiles, s);
+    if constexpr (FAM == 0 || FAM == 3)
+        if (a.mode == SWEEP_PROP)
+            return a.solver == SOLVER_FP64 ? launch_one<SOLVER_FP64, false, true, FAM>(a, ntiles, s)
+                                           : launch_one<SOLVER_MIXED, false, true, FAM>(a, ntiles, s);
+    if constexpr (FAM == 0 || FAM == 3)
+        if (a.mode == SWEEP_BOTH && a.solver == SOLVER_MIXED)
+            return launch_one<SOLVER_MIXED, false, false, FAM, true>(a, ntiles, s);
     const bool bwd = a.mode == SWEEP_ADJOINT;
     if (a.solver == SOLVER_FP64)
         return bwd ? launch_one<SOLVER_FP64, true, false, FAM>(a, ntiles, s)
@@ -106,9 +114,9 @@ cudaError_t MSQOC_CAT(launch_sweep, MSQOC_L, MSQOC_Q)(const SweepArgs& a, int nt
     return cudaErrorInvalidValue;
 }
 
-template <bool SPLIT>
+template <int MODE>
 static cudaError_t launch_quad_one(const QuadArgs& a, int blocks, int nprob, cudaStream_t s) {
-    auto kern = k_quad<MSQOC_L, MSQOC_Q, SPLIT>;
+    auto kern = k_quad<MSQOC_L, MSQOC_Q, MODE>;
     constexpr size_t smem = quad_smem<MSQOC_L, MSQOC_Q>();
     if constexpr (smem > SMEM_DEFAULT_LIMIT) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
@@ -120,7 +128,9 @@ static cudaError_t launch_quad_one(const QuadArgs& a, int blocks, int nprob, cud
 }
 
 cudaError_t MSQOC_CAT(launch_quad, MSQOC_L, MSQOC_Q)(const QuadArgs& a, int blocks, int nprob, cudaStream_t s) {
-    return a.split ? launch_quad_one<true>(a, blocks, nprob, s) : launch_quad_one<false>(a, blocks, nprob, s);
+    return a.mode == 2   ? launch_quad_one<2>(a, blocks, nprob, s)
+           : a.mode == 1 ? launch_quad_one<1>(a, blocks, nprob, s)
+                         : launch_quad_one<0>(a, blocks, nprob, s);
 }
 
 int MSQOC_CAT(sweep_occupancy, MSQOC_L, MSQOC_Q)(const SweepArgs& a) {

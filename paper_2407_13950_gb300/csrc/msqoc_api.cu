@@ -186,6 +186,20 @@ void build_lanemaps(int L, int q, int M, int E, int cpt, int nthreads, int pair,
     build_lanemap(L, q, last.ncol, last.ncol0, nthreads, pair, out + size_t(cpt) * nthreads);
 }
 
+// tiles and lane maps of a sweep over V windows of E columns
+struct TileTables {
+    std::vector<Tile> tiles;
+    std::vector<int> maps;
+};
+TileTables tile_tables(int L, int q, int V, int E, int cpt, int nthreads, int pair) {
+    TileTables t;
+    t.tiles.resize(tile_count(V, E, cpt));
+    for (size_t i = 0; i < t.tiles.size(); ++i) t.tiles[i] = tile_at(static_cast<long>(i), V, E, cpt, 0);
+    t.maps.resize(size_t(cpt + 1) * nthreads);
+    build_lanemaps(L, q, V, E, cpt, nthreads, pair, t.maps.data());
+    return t;
+}
+
 // one thread, a lane pair or a lane quad (2^pair threads) per (column, fiber)
 int tile_threads(int cpt, int F, int pair) { return (((1 << pair) * cpt * F + 31) / 32) * 32; }
 int max_tile_threads(int pair, int lean = 0) {
@@ -226,64 +240,50 @@ bool tile_width_ok(int cpt, int E, int F, int q, int L, int N, int g, int solver
 // Lane quads serve 2-level subsystems whose exchange-coupled pairs all have precomputed sources.
 bool quad_admitted(const ProbDev& pd) { return pd.L == 2 && pd.nex <= MAXEXF; }
 
-// Kernel family and columns per tile.  Makespan model, from FP64 throughput probes and sweep
-// timings on this GPU: a warp issues one FP64 instruction per 64 cycles on its SM sub-partition,
-// an SM with four or more warps of FP64 work runs at its full rate, and every thread of a tile
-// does the same FP64 work per step (idle lanes cost as much as busy ones).  In units of the
-// step time of one one-thread-per-fiber warp alone on a sub-partition, a step of an SM holding
-// w warps costs max(w c / 4, c0): c = c0 = 1 for that family; for lane pairs (half the FP64
-// instructions a thread, plus shuffles) c = 0.6 at full SM load and c0 = 0.7 alone (measured:
-// equal to the one-thread family on the 4-transmon tiles, 1.4x faster steps on small
-// problems); for lane quads (2-level subsystems, a quarter of a fiber's work a thread)
-// c = 0.38 and c0 = 0.52 (measured on the paper's QFT cases: steps 1.33-1.38x faster than lane
-// pairs where the tiles are too few to fill the GPU; under load, from QFT-16 at 64 windows,
-// seven one-warp quad tiles per SM take 0.73 of the time of one-thread tiles at the floor).
-// Tiles that do not fit at once run in waves of the CTAs an SM holds (the kernels'
-// occupancy at that width).  A tile over two windows pays a second coefficient set, gradient
-// reduction and fold each step and wider class mixing in its warps: about one more warp's work
-// per step, so its cost is taken (w + 1) / w times that of w warps (measured on the 4-transmon
-// tiles: 6-warp two-window tiles as slow as 7-warp one-window ones, at 64 windows; 8-warp
-// two-window tiles in three waves 7% faster than 7-warp one-window tiles in four, at 256
-// windows, where (w + 1) / w predicts 4%).  Candidates are ranked by
+// Kernel family and columns per tile.  Makespan model calibrated on sweep timings, in units of the
+// step time of one one-thread-per-fiber warp alone on a sub-partition.
+//   Mixed solver: a step of an SM holding w warps of the one-thread families costs 1 up to four
+//     warps and 0.09 more for each further one (4 transmons: 3.3 us a step at 4 warps, 4.1 at 7, 6.0
+//     at 12: the steps are latency-bound).  One-warp tiles of at least two columns without
+//     idle lanes step without tile barriers and fall out of step: 0.85 (QFT-16 at 64 windows: 2.24
+//     us a step with 4-column one-warp tiles, 2.85 with 8-column ones).  The lane families do
+//     their arithmetic in FP64 and are slower even alone (64-step probes of a gradient: QFT-4 315 us
+//     against 474 with lane pairs and 381 with lane quads, 2 transmons 290 / 417, 3 transmons
+//     372 / 538, QFT-8 367 / 567 / 413, 4 transmons at 256 windows 1902 / 4952): max(w c / 4, c0)
+//     with c = 2.4, c0 = 1.45 for lane pairs, c = 2.2, c0 = 1.2 for lane quads.
+//   FP64 solver: max(w c / 4, c0), c = c0 = 1 with one thread per fiber, c = 0.6 and c0 = 0.7 with
+//     lane pairs (half the FP64 instructions a thread, plus shuffles), c = 0.38 and c0 = 0.52 with
+//     lane quads.
+// Tiles that do not fit at once run in waves of the CTAs an SM holds (the kernels' occupancy at
+// that width).
+// A tile over two windows pays a second coefficient set each step and wider class mixing in its
+// warps: about one more warp's work per step, so its cost is taken (w + 1) / w times that of w
+// warps (measured on the 4-transmon tiles: 6-warp two-window tiles as slow as 7-warp one-window
+// ones, at 64 windows; 8-warp two-window tiles in three waves 7% faster than 7-warp one-window
+// tiles in four, at 256 windows, where (w + 1) / w predicts 4%).  Candidates are ranked by
 //   1. the makespan: an SM's ceil(tiles / SMs) tiles in waves of `resident`, summed over the
 //      waves;
 //   2. tiles that stay inside one window;
 //   3. where every wave sits at the single-warp floor (problems too small to fill the GPU, whose
-//      candidates all tie there): tiles of 2 or 3 warps, then of 1, then of more (measured
-//      there, 2-3 warp tiles step fastest:
-//      fewer threads meet at each barrier than in wider tiles, and the coefficient and gradient
-//      work of a tile is not serialised with the step as in one-warp tiles);
+//      candidates all tie there): more warps, up to the four of the floor (4 transmons at 16
+//      windows: 3.41 us a step with 4-column tiles, 3.50 with 2, 3.67 with 1; FP64 solver: 2 or 3);
 //   4. the idle-lane fraction of a tile.
-// fixed_cpt > 0 restricts the width, layout (MSQOC_LAYOUT_*) the family; quad_ok: the problem
-// admits lane quads.  cpt = -1: none fits.
-constexpr double QUAD_C = 0.38, QUAD_C0 = 0.52;
-// the one-thread family with 168 registers a thread: an SM holds 12 warps.  While the sweeps
-// were bound by the FP64 pipe, two or more of its tiles on an SM did better than their warp
-// count (each has its own barriers, so one tile's FP32 sweeps overlapped another's FP64 work)
-// and a warp of such tiles counted 0.9.  With the mixed solver's compensated FP32 arithmetic
-// the sweeps are bound by issue and dependency latency instead, and on the 4-transmon tiles one
-// 14-column tile of 12 warps per SM steps 5% faster than two 7-column tiles (autotuner probes at
-// 256 windows: 2.78 against 2.93 ms), so the lean build's warps count like any others
-constexpr double LEAN_C = 1.0;
-TileChoice choose_tile_layout(int M, int E, int F, int q, int L, int N, int g, int solver, int sms, int fixed_cpt,
-                              int layout, bool quad_ok) {
-    TileChoice best{-1, 0, 0};
-    double best_a = 0.0, best_c = 0.0;
-    int best_b = 0, best_w = 0;
+struct TileCand {
+    int cpt, pair, lean, threads, warps;
+    long resident;   // CTAs an SM holds
+};
+// every usable (family, width); layout (MSQOC_LAYOUT_*) restricts the family; quad_ok: the problem
+// admits lane quads.  Widths up to N columns (a propagator's).
+std::vector<TileCand> tile_candidates(int F, int q, int L, int N, int g, int solver, int layout, bool quad_ok) {
+    std::vector<TileCand> out;
     for (int fam = MSQOC_LAYOUT_FIBER; fam <= MSQOC_LAYOUT_FIBER_LEAN; ++fam) {
         if (layout != MSQOC_LAYOUT_AUTO && layout != fam) continue;
         const int pair = fam == MSQOC_LAYOUT_FIBER_LEAN ? 0 : fam - MSQOC_LAYOUT_FIBER;
         const int lean = fam == MSQOC_LAYOUT_FIBER_LEAN ? 1 : 0;
         if (pair == 2 && !quad_ok) continue;
-        const double c_load = pair == 2 ? QUAD_C : pair ? 0.6 : 1.0;
-        const double c_alone = pair == 2 ? QUAD_C0 : pair ? 0.7 : 1.0;
-        const int hi = fixed_cpt > 0 ? fixed_cpt : std::min(E, max_tile_threads(pair, lean) / ((1 << pair) * F));
-        const int lo = fixed_cpt > 0 ? fixed_cpt : 1;
-        for (int cpt = hi; cpt >= lo; --cpt) {
-            if (!tile_width_ok(cpt, E, F, q, L, N, g, solver, pair, lean)) continue;
-            const long tiles = (long(M) * E + cpt - 1) / cpt;
+        for (int cpt = std::min(N, max_tile_threads(pair, lean) / ((1 << pair) * F)); cpt >= 1; --cpt) {
             const int threads = tile_threads(cpt, F, pair);
-            const int warps = threads / 32;
+            if (admission_bytes(q, L, N, cpt, threads, g, solver, pair, 1) > 200 * 1024) continue;
             SweepArgs a{};
             a.cpt = cpt;
             a.gmax = g;
@@ -298,32 +298,109 @@ TileChoice choose_tile_layout(int M, int E, int F, int q, int L, int N, int g, i
             const int r0 = sweep_ctas_per_sm(a);
             a.mode = SWEEP_ADJOINT;
             const int r1 = sweep_ctas_per_sm(a);
-            const long resident = std::max(1, std::min(r0, r1));
-            const long per_sm = (tiles + sms - 1) / sms;
-            const long waves = (per_sm + resident - 1) / resident;
-            const long last = per_sm - (waves - 1) * resident;
-            const int cb = (E % cpt) ? 1 : 0;
-            const double two = cb ? double(warps + 1) / double(warps) : 1.0;
-            // a wave of n tiles on an SM; the lean build's warps count LEAN_C when two or more
-            // of its tiles share the SM (independent tiles fall out of step)
-            auto wave = [&](long n) {
-                const double c = (lean && n >= 2 && warps >= 4) ? LEAN_C : c_load;
-                return std::max(double(n * warps) * c / 4.0, c_alone);
-            };
-            const double ca = two * (double(waves - 1) * wave(resident) + wave(last));
-            const double cc = 1.0 - double((1 << pair) * cpt * F) / (32.0 * warps);
-            const bool at_floor = ca <= two * double(waves) * c_alone + 1e-9;
-            const int cw = !at_floor ? 0 : ((warps == 2 || warps == 3) ? 0 : (warps == 1 ? 1 : 2));
-            const bool tie_a = ca < best_a + 1e-9, tie_b = cb == best_b, tie_w = cw == best_w;
-            const bool better = best.cpt < 0 || ca < best_a - 1e-9 ||
-                                (tie_a && (cb < best_b || (tie_b && (cw < best_w || (tie_w && cc < best_c - 1e-9)))));
-            if (better) {
-                best = TileChoice{cpt, pair, lean};
-                best_a = ca;
-                best_b = cb;
-                best_w = cw;
-                best_c = cc;
-            }
+            out.push_back(TileCand{cpt, pair, lean, threads, threads / 32, std::max(1, std::min(r0, r1))});
+        }
+    }
+    return out;
+}
+// the best of them for M windows of E columns (cpt = -1: none fits); fixed_cpt > 0 restricts the
+// width, fiber_only the families to one thread per fiber
+TileChoice choose_tile_layout(const std::vector<TileCand>& cands, int M, int E, int F, int solver, int sms,
+                              int fixed_cpt, bool fiber_only = false) {
+    TileChoice best{-1, 0, 0, 0.0};
+    double best_c = 0.0;
+    int best_b = 0, best_w = 0;
+    const bool fp64 = solver == SOLVER_FP64;
+    for (const TileCand& t : cands) {
+        if (t.cpt > E || (fixed_cpt > 0 && t.cpt != fixed_cpt) || (fiber_only && t.pair)) continue;
+        if (t.threads == 32 && E % t.cpt) continue;   // a one-warp tile must not cover two windows
+        const double c_load = t.pair == 2 ? (fp64 ? 0.38 : 2.2) : t.pair ? (fp64 ? 0.6 : 2.4) : 1.0;
+        const double c_alone = t.pair == 2 ? (fp64 ? 0.52 : 1.2) : t.pair ? (fp64 ? 0.7 : 1.45) : 1.0;
+        const long tiles = (long(M) * E + t.cpt - 1) / t.cpt;
+        const long per_sm = (tiles + sms - 1) / sms;
+        const long waves = (per_sm + t.resident - 1) / t.resident;
+        const long last = per_sm - (waves - 1) * t.resident;
+        const int cb = (E % t.cpt) ? 1 : 0;
+        const double two = cb ? double(t.warps + 1) / double(t.warps) : 1.0;
+        const bool free_warps = !fp64 && !t.pair && t.warps == 1 && t.cpt >= 2 && t.cpt * F == 32;
+        auto wave = [&](long n) {
+            const double w = double(n * t.warps);
+            if (fp64 || t.pair) return std::max(w * c_load / 4.0, c_alone);
+            return (w <= 4.0 ? 1.0 : 1.0 + 0.09 * (w - 4.0)) * (free_warps ? 0.85 : 1.0);
+        };
+        const double ca = two * (double(waves - 1) * wave(t.resident) + wave(last));
+        const double cc = 1.0 - double((1 << t.pair) * t.cpt * F) / (32.0 * t.warps);
+        const bool at_floor = ca <= two * double(waves) * c_alone + 1e-9;
+        const int cw = !at_floor ? 0
+                       : fp64    ? ((t.warps == 2 || t.warps == 3) ? 0 : (t.warps == 1 ? 1 : 2))
+                                 : -std::min(t.warps, 4);
+        const bool tie_a = ca < best.cost + 1e-9, tie_b = cb == best_b, tie_w = cw == best_w;
+        const bool better = best.cpt < 0 || ca < best.cost - 1e-9 ||
+                            (tie_a && (cb < best_b || (tie_b && (cw < best_w || (tie_w && cc < best_c - 1e-9)))));
+        if (better) {
+            best = TileChoice{t.cpt, t.pair, t.lean, ca};
+            best_b = cb;
+            best_w = cw;
+            best_c = cc;
+        }
+    }
+    return best;
+}
+
+// ------------------------------------------------------------------ slices of a window
+// Slices a window (k_compose): the count with the least estimated time of a gradient and half an
+// objective, over doublings and their 1.5-folds; 1 where slicing does not pay.  From measured sweeps
+// and chains: a step of one tile-model unit takes 1.2 us plus 0.13 us for each of a fiber's 2 q (L - 1)
+// terms (QFT-16 2.3 us, 3 transmons 2.6, 4 transmons 3.3), a launch LAUNCH us (its own start and a
+// sweep's set-up), and a link of the chain 0.35 us plus N^2 complex products at the FP64 rate of one
+// SM.  Slices have at least 4 steps, the propagators of a problem stay below SLICE_BYTES.
+constexpr double SLICE_LAUNCH = 5.0;
+double slice_unit_us(const ProbDev& pd) { return 1.2 + 0.13 * 2 * pd.q * (pd.L - 1); }
+constexpr size_t SLICE_BYTES = size_t(256) << 20;
+// propagators a roll-out holds at a time (whole windows; at least one)
+constexpr size_t ROLLOUT_BYTES = size_t(32) << 20;
+double slice_link_us(int N) { return 0.35 + double(N) * N * 4.0 / (1.9 * 2070.0); }
+int choose_slices(const std::vector<TileCand>& cands, const ProbDev& pd, int M, int64_t steps, int sms) {
+    const double unit = slice_unit_us(pd);
+    auto sweep_us = [&](int windows, int cols, double n) {
+        const TileChoice t = choose_tile_layout(cands, windows, cols, pd.F, pd.solver, sms, 0, true);
+        return t.cpt < 0 ? 1e30 : SLICE_LAUNCH + t.cost * n * unit;
+    };
+    const double ns = double(steps) / M;
+    const double whole = sweep_us(M, pd.E, ns);
+    int best = 1;
+    double best_us = 2.5 * whole;
+    if (M > 32768) return 1;   // (a grid dimension of the chain)
+    for (int c2 = 4; c2 / 2 <= ns / 4.0; c2 += (c2 & (c2 - 1)) ? c2 / 3 : c2 / 2) {   // C = 2, 3, 4, 6, 8, 12, ..
+        const int C = c2 / 2;
+        if (size_t(M) * C * pd.N * pd.N * sizeof(double2) > SLICE_BYTES || int64_t(M) * C > (1 << 20)) break;
+        const double n = std::ceil(ns / C), chain = SLICE_LAUNCH + C * slice_link_us(pd.N);
+        const double objective = sweep_us(M * C, pd.N, n) + chain;
+        if (objective > whole) continue;
+        // (the history and adjoint sweeps run at the same time)
+        const double us = 1.5 * objective + chain + sweep_us(2 * M * C, pd.E, n);
+        if (us < best_us) {
+            best_us = us;
+            best = C;
+        }
+    }
+    return best;
+}
+// slices a window of the roll-out, M windows in all (it has no form without them)
+int choose_rollout_slices(const std::vector<TileCand>& cands, const ProbDev& pd, int sms) {
+    int best = 1;
+    double best_us = 1e30;
+    const double ns = double(pd.nsteps) / pd.M;
+    for (int c2 = 2; c2 == 2 || c2 / 2 <= ns / 4.0; c2 += c2 < 4 ? 2 : (c2 & (c2 - 1)) ? c2 / 3 : c2 / 2) {
+        const int C = c2 / 2;
+        if (C > 1 && size_t(C) * pd.N * pd.N * sizeof(double2) > SLICE_BYTES) break;
+        const double V = double(pd.M) * C;
+        if (V > (1 << 20) && C > 1) break;
+        const TileChoice t = choose_tile_layout(cands, static_cast<int>(V), pd.N, pd.F, pd.solver, sms, 0, true);
+        const double us = t.cost * std::ceil(ns / C) * slice_unit_us(pd) + V * slice_link_us(pd.N);
+        if (us < best_us) {
+            best_us = us;
+            best = C;
         }
     }
     return best;
@@ -362,7 +439,8 @@ msqoc_status check_description(const msqoc_hamiltonian* H, const msqoc_controls*
 // of pd except the device pointers and the history segmentation).  col_block 0 = automatic.
 msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, double T, int64_t nsteps,
                            int32_t nwindows, double mu, int solver, int col_block, int layout, int sms, ProbDev& pd,
-                           int wfirst = 0, int wlast = 0) {
+                           int wfirst = 0, int wlast = 0, bool slices = false,
+                           std::vector<TileCand>* plans = nullptr) {
     const int q = H->nqubits, L = H->nlevels, ness = H->ness;
     int nfsum = 0;
     for (int k = 0; k < q; ++k) nfsum += C->ncarriers[k];
@@ -431,8 +509,21 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
         return fail(MSQOC_ERR_INVALID_ARG, "lane quads need 2-level subsystems and at most %d exchange-coupled pairs",
                     MAXEXF);
     if (col_block < 0) return fail(MSQOC_ERR_INVALID_ARG, "column block %d < 0", col_block);
-    const TileChoice tc =
-        choose_tile_layout(pd.M, pd.E, pd.F, q, L, pd.N, pd.glocal, solver, sms, col_block, layout, quad_admitted(pd));
+    const std::vector<TileCand> cands =
+        tile_candidates(pd.F, q, L, pd.N, pd.glocal, solver, layout, quad_admitted(pd));
+    // the tiles of M windows of E columns, sliced or not
+    TileChoice tc = choose_tile_layout(cands, pd.M, pd.E, pd.F, solver, sms, col_block);
+    pd.C = 1;
+    if (slices && tc.cpt > 0 && tc.pair == 0 && solver == SOLVER_MIXED) {
+        // (from the whole problem's windows, so that a shard has its problem's slices)
+        const int C = choose_slices(cands, pd, pd.M_glob, nsteps, sms);
+        const TileChoice ts = choose_tile_layout(cands, pd.M * C, pd.E, pd.F, solver, sms, col_block, true);
+        if (C > 1 && ts.cpt > 0) {
+            pd.C = C;
+            tc = ts;
+        }
+    }
+    if (plans) *plans = cands;
     if (tc.cpt < 0)
         return fail(MSQOC_ERR_INVALID_ARG,
                     "column block %d invalid for E=%d (needs 1 <= cb <= E, cb N/L <= %d threads with one thread "
@@ -445,10 +536,10 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
     pd.pair = tc.pair;
     pd.lean = tc.lean;
     pd.nthreads = tile_threads(cpt, pd.F, tc.pair);
-    pd.ntiles = static_cast<int>((long(pd.M) * pd.E + cpt - 1) / cpt);
-    // whole windows in one history segment unless a checkpoint interval is set later
+    pd.ntiles = static_cast<int>((long(pd.M) * pd.C * pd.E + cpt - 1) / cpt);
+    // whole windows (slices) in one history segment unless a checkpoint interval is set later
     const int64_t max_ns = (nsteps + nwindows - 1) / nwindows;
-    pd.kseg = static_cast<int>(max_ns);
+    pd.kseg = static_cast<int>((max_ns + pd.C - 1) / pd.C);
     pd.nseg = 1;
     pd.kadj = pd.kseg;
     pd.nsub = 1;
@@ -468,12 +559,13 @@ bool history_depth_ok(const ProbDev& pd, int depth) {
 // milliseconds a chunk.
 constexpr size_t ADJ_CHUNK_BYTES = size_t(1) << 30;
 
-// history segmentation for a checkpoint interval K (1 = keep every midpoint state)
+// history segmentation for a checkpoint interval K (1 = keep every midpoint state); slices come
+// with K = 1 only
 void set_segments(ProbDev& pd, int K) {
-    const int64_t max_ns = (pd.nsteps + pd.M_glob - 1) / pd.M_glob;
+    const int64_t max_ns = ((pd.nsteps + pd.M_glob - 1) / pd.M_glob + pd.C - 1) / pd.C;
     pd.kseg = (K <= 1 || K >= max_ns) ? static_cast<int>(max_ns) : K;
     pd.nseg = static_cast<int>((max_ns + pd.kseg - 1) / pd.kseg);
-    const size_t step = size_t(pd.M) * pd.N * pd.E * sizeof(double2);
+    const size_t step = size_t(pd.M) * pd.C * pd.N * pd.E * sizeof(double2);
     const int64_t most = std::max<int64_t>(16, static_cast<int64_t>(ADJ_CHUNK_BYTES / step));
     pd.nsub = static_cast<int>((pd.kseg + most - 1) / most);
     pd.kadj = (pd.kseg + pd.nsub - 1) / pd.nsub;
@@ -523,7 +615,7 @@ bool is_shard(const ProbDev& pd) { return pd.M != pd.M_glob; }
 namespace {
 
 void free_problem(msqoc_problem* p) {
-    void* bufs[] = {p->tiles_ro, p->lanemap_ro,
+    void* bufs[] = {p->tiles_ro, p->lanemap_ro, p->phi_ro, p->tiles_prop, p->lanemap_prop, p->Phi, p->Ubeg, p->Lend,
                     p->pds,   p->tiles, p->lanemap, p->P,     p->emb,   p->V,     p->alpha_dev, p->W_dev,
                     p->ctrl,  p->spl,   p->phase,   p->hist,  p->ckpt,  p->Lstate, p->Uend,     p->Lterm,
                     p->Lam0,  p->term,  p->lhist,   p->quad,  p->status, p->out_dev, p->reg_dev};
@@ -556,19 +648,24 @@ size_t reg_doubles(const ProbDev& pd) { return 2 * size_t(pd.d) + size_t(pd.q) *
 
 // device bytes of the histories, checkpoints and segment state of one problem:
 // 16-byte blocks after the history that hold its column scale exponents ([M][nseg][E] ints)
-size_t hist_scale_blocks(const ProbDev& pd) { return (size_t(pd.M) * pd.nseg * pd.E * sizeof(int) + 15) / 16; }
+size_t hist_scale_blocks(const ProbDev& pd) { return (size_t(pd.M) * pd.C * pd.nseg * pd.E * sizeof(int) + 15) / 16; }
 
 // the same after the adjoint's ([M][E] ints)
-size_t adj_scale_blocks(const ProbDev& pd) { return (size_t(pd.M) * pd.E * sizeof(int) + 15) / 16; }
+size_t adj_scale_blocks(const ProbDev& pd) { return (size_t(pd.M) * pd.C * pd.E * sizeof(int) + 15) / 16; }
 
 size_t gradient_bytes(const ProbDev& pd) {
-    const size_t ne = size_t(pd.N) * pd.E;
-    size_t b = (size_t(pd.M) * pd.kseg * ne + hist_scale_blocks(pd)) * sizeof(double2);
-    b += (size_t(pd.M) * pd.kadj * ne + adj_scale_blocks(pd)) * sizeof(double2);
+    const size_t ne = size_t(pd.N) * pd.E, V = size_t(pd.M) * pd.C;
+    size_t b = (V * pd.kseg * ne + hist_scale_blocks(pd)) * sizeof(double2);
+    b += (V * pd.kadj * ne + adj_scale_blocks(pd)) * sizeof(double2);
     b += size_t(pd.q) * pd.nsteps * sizeof(double2);
+    if (pd.C > 1) b += V * ne * sizeof(double2);
     if (pd.nseg > 1) b += size_t(pd.M) * pd.nseg * ne * sizeof(double2);
     if (pd.nseg * pd.nsub > 1) b += size_t(pd.M) * ne * sizeof(double2);
     return b;
+}
+// propagators and slice states of a sliced problem
+size_t slice_bytes(const ProbDev& pd) {
+    return pd.C > 1 ? size_t(pd.M) * pd.C * pd.N * (pd.N + pd.E) * sizeof(double2) : 0;
 }
 
 }  // namespace
@@ -649,6 +746,14 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     }
     p->ckpt_interval = K;
     set_segments(pd, K);
+    // slices of the windows where every midpoint state is kept
+    std::vector<TileCand> cands;
+    if (pd.nseg == 1) {
+        st0 = shape_problem(H, C, T, nsteps, nwindows, mu, solver, o.col_block, o.layout, sms, pd, o.window_first,
+                            o.window_last, true, &cands);
+        if (st0 != MSQOC_OK) return st0;
+        set_segments(pd, pd.C > 1 ? 1 : K);
+    }
     // steps per history synchronisation: 0 = one (every step)
     pd.hdepth = o.steps_per_sync > 0 ? o.steps_per_sync : 1;
     if (!history_depth_ok(pd, pd.hdepth))
@@ -672,16 +777,30 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
         for (int j = 0; j < E; ++j)
             for (int e = 0; e < E; ++e) Vh[size_t(j) * N + emb[e]] = qft_entry(E, e, j);
     }
-    std::vector<Tile> tiles(pd.ntiles);
-    for (int t = 0; t < pd.ntiles; ++t) tiles[t] = tile_at(t, pd.M, E, pd.cb, 0);
-    std::vector<int> maps(size_t(pd.cb + 1) * pd.nthreads);
-    build_lanemaps(L, q, pd.M, E, pd.cb, pd.nthreads, pd.pair, maps.data());
-    // the roll-out sweep's tiles: the same widths over a single window
-    p->ntiles_ro = static_cast<int>(tile_count(1, E, pd.cb));
-    std::vector<Tile> tiles_ro(p->ntiles_ro);
-    for (int t = 0; t < p->ntiles_ro; ++t) tiles_ro[t] = tile_at(t, 1, E, pd.cb, 0);
-    std::vector<int> maps_ro(size_t(pd.cb + 1) * pd.nthreads);
-    build_lanemaps(L, q, 1, E, pd.cb, pd.nthreads, pd.pair, maps_ro.data());
+    const int V = pd.M * pd.C;   // (virtual) windows of the sweeps
+    const TileTables tabs = tile_tables(L, q, V, E, pd.cb, pd.nthreads, pd.pair);
+    // propagators of the slices, and of the roll-out's (one thread per fiber whatever the layout)
+    TileTables tabs_prop, tabs_ro;
+    if (pd.C > 1) {
+        const TileChoice t = choose_tile_layout(cands, V, N, pd.F, solver, sms, 0, true);
+        if (t.cpt < 0) return fail(MSQOC_ERR_INTERNAL, "no tiles for the propagators");
+        p->prop = SweepPlan{t.cpt, tile_threads(t.cpt, pd.F, 0), t.lean, 0};
+        tabs_prop = tile_tables(L, q, V, N, t.cpt, p->prop.nthreads, 0);
+        p->prop.ntiles = static_cast<int>(tabs_prop.tiles.size());
+    }
+    if (pd.M > 1 && !is_shard(pd)) {
+        if (pd.pair || cands.empty())
+            cands = tile_candidates(pd.F, q, L, N, pd.glocal, solver, MSQOC_LAYOUT_AUTO, false);
+        p->ro_slices = choose_rollout_slices(cands, pd, sms);
+        p->ro_windows = static_cast<int>(std::min<size_t>(
+            size_t(pd.M - 1), std::max<size_t>(1, ROLLOUT_BYTES / (size_t(p->ro_slices) * N * N * sizeof(double2)))));
+        const int v = p->ro_windows * p->ro_slices;
+        const TileChoice t = choose_tile_layout(cands, v, N, pd.F, solver, sms, 0, true);
+        if (t.cpt < 0) return fail(MSQOC_ERR_INTERNAL, "no tiles for the roll-out");
+        p->ro = SweepPlan{t.cpt, tile_threads(t.cpt, pd.F, 0), t.lean, 0};
+        tabs_ro = tile_tables(L, q, v, N, t.cpt, p->ro.nthreads, 0);
+        p->ro.ntiles = static_cast<int>(tabs_ro.tiles.size());
+    }
 
     // ---- device buffers
     const size_t M = pd.M;
@@ -692,10 +811,18 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
                       "allocating %s: %s", what, cudaGetErrorString(e));
     };
     A(dalloc(&p->pds, 1), "problem record");
-    A(dalloc(&p->tiles, tiles.size()), "tiles");
-    A(dalloc(&p->lanemap, maps.size()), "lane maps");
-    A(dalloc(&p->tiles_ro, tiles_ro.size()), "roll-out tiles");
-    A(dalloc(&p->lanemap_ro, maps_ro.size()), "roll-out lane maps");
+    A(dalloc(&p->tiles, tabs.tiles.size()), "tiles");
+    A(dalloc(&p->lanemap, tabs.maps.size()), "lane maps");
+    A(dalloc(&p->tiles_prop, tabs_prop.tiles.size()), "propagator tiles");
+    A(dalloc(&p->lanemap_prop, tabs_prop.maps.size()), "propagator lane maps");
+    A(dalloc(&p->tiles_ro, tabs_ro.tiles.size()), "roll-out tiles");
+    A(dalloc(&p->lanemap_ro, tabs_ro.maps.size()), "roll-out lane maps");
+    const size_t phi_ro = size_t(p->ro_windows) * p->ro_slices * N * N;
+    A(dalloc(&p->phi_ro, phi_ro), "roll-out propagators");
+    if (pd.C > 1) {
+        A(dalloc(&p->Phi, size_t(V) * N * N), "propagators");
+        A(dalloc(&p->Ubeg, size_t(V) * p->ne), "slice states");
+    }
     A(dalloc(&p->P, N), "P");
     A(dalloc(&p->emb, E), "embedding");
     A(dalloc(&p->V, p->ne), "target");
@@ -731,12 +858,17 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
         pd.Lam0 = p->Lam0;
         pd.term = p->term;
         pd.status = p->status;
-        A(cudaMemcpy(p->tiles, tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice), "tiles copy");
-        A(cudaMemcpy(p->lanemap, maps.data(), maps.size() * sizeof(int), cudaMemcpyHostToDevice), "lane map copy");
-        A(cudaMemcpy(p->tiles_ro, tiles_ro.data(), tiles_ro.size() * sizeof(Tile), cudaMemcpyHostToDevice),
-          "roll-out tiles copy");
-        A(cudaMemcpy(p->lanemap_ro, maps_ro.data(), maps_ro.size() * sizeof(int), cudaMemcpyHostToDevice),
-          "roll-out lane map copy");
+        pd.Phi = p->Phi;
+        pd.Ubeg = p->Ubeg;
+        auto up = [&](auto* dst, const auto& v, const char* what) {
+            if (!v.empty()) A(cudaMemcpy(dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice), what);
+        };
+        up(p->tiles, tabs.tiles, "tiles copy");
+        up(p->lanemap, tabs.maps, "lane map copy");
+        up(p->tiles_prop, tabs_prop.tiles, "propagator tiles copy");
+        up(p->lanemap_prop, tabs_prop.maps, "propagator lane map copy");
+        up(p->tiles_ro, tabs_ro.tiles, "roll-out tiles copy");
+        up(p->lanemap_ro, tabs_ro.maps, "roll-out lane map copy");
         A(cudaMemcpy(p->P, P.data(), N * sizeof(double2), cudaMemcpyHostToDevice), "P copy");
         A(cudaMemcpy(p->emb, emb.data(), E * sizeof(int), cudaMemcpyHostToDevice), "emb copy");
         A(cudaMemcpy(p->V, Vh.data(), p->ne * sizeof(double2), cudaMemcpyHostToDevice), "target copy");
@@ -753,8 +885,9 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     if (st != MSQOC_OK) return st;
     p->bytes = sizeof(double2) * (N + p->ne * (1 + 3 * M) + size_t(nsteps) * (q + nfsum)) +
                sizeof(Spline4) * size_t(nsteps) + sizeof(double) * (pd.d + p->nW + M + out_layout(p->npen, pd.d, p->nW).total + reg_doubles(pd)) +
-               sizeof(int) * (E + 1 + maps.size() + maps_ro.size()) + sizeof(Tile) * (tiles.size() + tiles_ro.size()) +
-               sizeof(ProbDev);
+               sizeof(int) * (E + 1 + tabs.maps.size() + tabs_prop.maps.size() + tabs_ro.maps.size()) +
+               sizeof(Tile) * (tabs.tiles.size() + tabs_prop.tiles.size() + tabs_ro.tiles.size()) +
+               sizeof(double2) * phi_ro + slice_bytes(pd) + sizeof(ProbDev);
     p->grad_bytes = gradient_bytes(pd);
     *out = owner.release();
     return MSQOC_OK;
@@ -816,14 +949,15 @@ msqoc_status stage_inputs(msqoc_problem* p, const double* alpha, const double* W
 msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s) {
     if (p->hist) return MSQOC_OK;
     ProbDev& pd = p->pd;
-    const size_t M = pd.M;
-    cudaError_t e = dalloc(&p->hist, M * pd.kseg * p->ne + hist_scale_blocks(pd));
-    if (e == cudaSuccess) e = dalloc(&p->lhist, M * pd.kadj * p->ne + adj_scale_blocks(pd));
+    const size_t M = pd.M, V = M * pd.C;
+    cudaError_t e = dalloc(&p->hist, V * pd.kseg * p->ne + hist_scale_blocks(pd));
+    if (e == cudaSuccess) e = dalloc(&p->lhist, V * pd.kadj * p->ne + adj_scale_blocks(pd));
+    if (e == cudaSuccess && pd.C > 1) e = dalloc(&p->Lend, V * p->ne);
     if (e == cudaSuccess) e = dalloc(&p->quad, size_t(pd.q) * pd.nsteps);
     if (e == cudaSuccess && pd.nseg > 1) e = dalloc(&p->ckpt, M * pd.nseg * p->ne);
     if (e == cudaSuccess && pd.nseg * pd.nsub > 1) e = dalloc(&p->Lstate, M * p->ne);
     if (e != cudaSuccess) {
-        for (double2** b : {&p->hist, &p->lhist, &p->quad, &p->ckpt, &p->Lstate}) {
+        for (double2** b : {&p->hist, &p->lhist, &p->Lend, &p->quad, &p->ckpt, &p->Lstate}) {
             if (*b) cudaFree(*b);
             *b = nullptr;
         }
@@ -832,9 +966,10 @@ msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s) {
                     p->ckpt_interval, cudaGetErrorString(e));
     }
     pd.hist = p->hist;
-    pd.hsh = reinterpret_cast<int*>(p->hist + M * pd.kseg * p->ne);
+    pd.hsh = reinterpret_cast<int*>(p->hist + V * pd.kseg * p->ne);
     pd.lhist = p->lhist;
-    pd.lsh = reinterpret_cast<int*>(p->lhist + M * pd.kadj * p->ne);
+    pd.lsh = reinterpret_cast<int*>(p->lhist + V * pd.kadj * p->ne);
+    pd.Lend = p->Lend;
     pd.quad = p->quad;
     pd.ckpt = p->ckpt;
     pd.Lstate = p->Lstate;
@@ -852,7 +987,15 @@ int quad_blocks(const ProbDev& pd) {
     int lanes = 1;
     while (lanes < pd.E && lanes < most) lanes <<= 1;
     const int per = most / lanes;
-    return pd.M * ((pd.kadj + per - 1) / per);
+    return pd.M * pd.C * ((pd.kadj + per - 1) / per);
+}
+
+// FP64 products up to this many real products an evaluation: about 7 us of the FP64 pipe (0.6 T/s).
+// Such problems have few steps a window, whose states are then more exact than two-float sums of
+// the products (QFT-4 at 256 windows: gradient error 3.5e-15 with two-float sums, against 1.0e-15).
+constexpr double QUAD_FP64_MOST = 4e6;
+bool quad_fp64(const ProbDev& pd) {
+    return double(pd.nsteps) * pd.E * pd.q * (pd.N - pd.N / pd.L) * 8.0 <= QUAD_FP64_MOST;
 }
 
 QuadArgs quad_args(const ProbDev& pd, const ProbDev* pds_dev, int seg, int sub) {
@@ -860,7 +1003,7 @@ QuadArgs quad_args(const ProbDev& pd, const ProbDev* pds_dev, int seg, int sub) 
     a.pds = pds_dev;
     a.L = pd.L;
     a.q = pd.q;
-    a.split = split_history(pd) ? 1 : 0;
+    a.mode = !split_history(pd) ? 0 : quad_fp64(pd) ? 2 : 1;
     a.seg = seg;
     a.sub = sub;
     return a;
@@ -873,17 +1016,38 @@ msqoc_status sweep(msqoc_problem* p, int mode, int seg, cudaStream_t s, int sub 
     return MSQOC_OK;
 }
 
+// threads of a block of the chain over the propagators
+int compose_threads(int N) {
+    const ComposeGeom g = compose_geom(N);
+    return std::max(32, g.R * g.JG);
+}
+SweepArgs prop_args(const SweepPlan& plan, const ProbDev& pd, const ProbDev* pds_dev, const Tile* tiles,
+                    const int* lanemap) {
+    SweepArgs a = sweep_args(pd, pds_dev, tiles, lanemap, SWEEP_PROP, 0);
+    a.cpt = plan.cpt;
+    a.nthreads = plan.nthreads;
+    a.lean = plan.lean;
+    a.pair = 0;
+    a.hdepth = 1;
+    return a;
+}
+cudaError_t launch_compose(const ProbDev* pds_dev, const int* list, int E, int M, int nprob, int N, bool bwd,
+                           cudaStream_t s) {
+    k_compose<<<dim3(E, M, nprob), compose_threads(N), 0, s>>>(pds_dev, list, bwd ? 1 : 0);
+    return cudaGetLastError();
+}
+
 // blocks of 256 threads for the phase table (grid-stride loop)
 int phase_blocks(const ProbDev& pd) {
     return static_cast<int>(std::min<int64_t>((pd.nsteps * pd.nfsum + 255) / 256, 4096));
 }
 
-msqoc_status launch_controls(msqoc_problem* p, cudaStream_t s) {
+msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s) {
     const ProbDev& pd = p->pd;
     Mark mk(p, MSQOC_KERNEL_CONTROLS, s);
     const int threads = 256;
     const int blocks = static_cast<int>(std::min<int64_t>((pd.nsteps + threads - 1) / threads, 4096));
-    k_controls<<<blocks, threads, 0, s>>>(pd);
+    k_controls<<<blocks, threads, 0, s>>>(pd, pair);
     CUDA_TRY(cudaGetLastError());
     return MSQOC_OK;
 }
@@ -916,12 +1080,20 @@ msqoc_status launch_gradient_outputs(msqoc_problem* p, double* P, double* ga, do
 // controls, forward sweep over whole windows, terminal conditions
 msqoc_status launch_forward_part(msqoc_problem* p, int mode, cudaStream_t s) {
     for (bool& r : p->ran) r = false;
-    msqoc_status st = launch_controls(p, s);
+    msqoc_status st = launch_controls(p, p->pd.pair, s);
     if (st) return st;
     {
         Mark mk(p, MSQOC_KERNEL_FORWARD, s);
-        st = sweep(p, mode, 0, s);
-        if (st) return st;
+        const ProbDev& pd = p->pd;
+        if (pd.C > 1) {
+            // the slices' propagators, and the chain that gives their states and the windows' ends
+            CUDA_TRY(launch_sweep(prop_args(p->prop, pd, p->pds, p->tiles_prop, p->lanemap_prop), p->prop.ntiles, s));
+            CUDA_TRY(launch_compose(p->pds, nullptr, pd.E, pd.M, 1, pd.N, false, s));
+        }
+        if (pd.C == 1 || (mode == SWEEP_HISTORY && pd.nsub > 1)) {
+            st = sweep(p, mode, 0, s);
+            if (st) return st;
+        }
     }
     return launch_terminal(p, mode != SWEEP_OBJECTIVE, s);
 }
@@ -988,13 +1160,15 @@ msqoc_status msqoc_eval_gradient(msqoc_problem* p, const double* alpha, const do
     if (st) return st;
     {
         Mark mk(p, MSQOC_KERNEL_ADJOINT, s);
+        if (pd.C > 1) CUDA_TRY(launch_compose(p->pds, nullptr, pd.E, pd.M, 1, pd.N, true, s));
         for (int seg = pd.nseg - 1; seg >= 0; --seg) {
             if (pd.nseg > 1) {
                 st = sweep(p, SWEEP_RECOMPUTE, seg, s);
                 if (st) return st;
             }
             for (int sub = pd.nsub - 1; sub >= 0; --sub) {
-                st = sweep(p, SWEEP_ADJOINT, seg, s, sub);
+                // (a sliced problem's history was not needed before: both sweeps at once)
+                st = sweep(p, pd.C > 1 && pd.nsub == 1 ? SWEEP_BOTH : SWEEP_ADJOINT, seg, s, sub);
                 if (st) return st;
                 CUDA_TRY(launch_quad(quad_args(pd, p->pds, seg, sub), quad_blocks(pd), 1, s));
             }
@@ -1029,12 +1203,22 @@ msqoc_status msqoc_rollout(msqoc_problem* p, const double* alpha, double* W_out,
     const bool dev = is_device_ptr(W_out) && reinterpret_cast<uintptr_t>(W_out) % 16 == 0;
     double* dst = dev ? W_out : p->out_dev + out_layout(p->npen, p->pd.d, p->nW).gw;
     for (bool& r : p->ran) r = false;
-    if ((st = launch_controls(p, s))) return st;
-    SweepArgs a = sweep_args(p->pd, p->pds, p->tiles_ro, p->lanemap_ro, SWEEP_ROLLOUT, 0);
-    a.out = reinterpret_cast<double2*>(dst);
+    if ((st = launch_controls(p, 0, s))) return st;   // (propagators: one thread per fiber)
     {
+        // batches of windows whose propagators fit the buffer: their sweep, then the chain
         Mark mk(p, MSQOC_KERNEL_FORWARD, s);
-        CUDA_TRY(launch_sweep(a, p->ntiles_ro, s));
+        const ProbDev& pd = p->pd;
+        SweepArgs a = prop_args(p->ro, pd, p->pds, p->tiles_ro, p->lanemap_ro);
+        a.slices = p->ro_slices;
+        a.phi = p->phi_ro;
+        for (int w0 = 0; w0 < pd.M - 1; w0 += p->ro_windows) {
+            const int nw = std::min(p->ro_windows, pd.M - 1 - w0);
+            a.voff = w0 * p->ro_slices;
+            CUDA_TRY(launch_sweep(a, p->ro.ntiles, s));
+            k_compose_rollout<<<pd.E, compose_threads(pd.N), 0, s>>>(pd, p->phi_ro, p->ro_slices, w0, nw,
+                                                                     reinterpret_cast<double2*>(dst));
+            CUDA_TRY(cudaGetLastError());
+        }
     }
     if (dev) return MSQOC_OK;
     CUDA_TRY(cudaMemcpyAsync(W_out, dst, p->nW * sizeof(double), cudaMemcpyDefault, s));
@@ -1155,11 +1339,12 @@ msqoc_status autotune(const msqoc_hamiltonian* H, const msqoc_controls* C, doubl
     // candidates: every (family, width) with one step per history synchronisation, then the
     // best pair with 2, 4 and 8 steps per synchronisation
     std::vector<std::array<int, 3>> cands;
-    for (int fam = fam_lo; fam <= fam_hi; ++fam)
+    for (int fam = fam_lo; fam <= fam_hi; ++fam) {
+        const auto fc = tile_candidates(pd.F, pd.q, pd.L, pd.N, pd.glocal, solver, fam, quad_admitted(pd));
         for (int cb = std::min(pd.E, MAX_LEAN_TILE_THREADS / pd.F); cb >= 1; --cb)
-            if (choose_tile_layout(pd.M, pd.E, pd.F, pd.q, pd.L, pd.N, pd.glocal, solver, 1, cb, fam,
-                                   quad_admitted(pd)).cpt >= 0)
+            if (choose_tile_layout(fc, pd.M, pd.E, pd.F, solver, 1, cb).cpt >= 0)
                 cands.push_back({fam, cb, o.steps_per_sync > 0 ? o.steps_per_sync : 1});
+    }
     const size_t n_first = cands.size();
     for (size_t ci = 0; ci < cands.size() && st == MSQOC_OK; ++ci) {
         const int fam = cands[ci][0], cb = cands[ci][1], dp = cands[ci][2];
@@ -1392,7 +1577,7 @@ msqoc_status eval_objective_noalloc(const msqoc_hamiltonian* H, const msqoc_cont
         const int blocks = static_cast<int>(std::min<int64_t>((pd.nsteps + threads - 1) / threads, 4096));
         k_phases<<<phase_blocks(pd), threads, 0, s>>>(pd);
         CUDA_TRY(cudaGetLastError());
-        k_controls<<<blocks, threads, 0, s>>>(pd);
+        k_controls<<<blocks, threads, 0, s>>>(pd, pd.pair);
         CUDA_TRY(cudaGetLastError());
     }
     CUDA_TRY(launch_sweep(sweep_args(pd, pd_d, tiles_d, map_d, SWEEP_OBJECTIVE, 0), pd.ntiles, s));

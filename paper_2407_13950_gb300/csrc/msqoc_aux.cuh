@@ -84,8 +84,8 @@ __device__ __forceinline__ SplineAt spline_at(const ProbDev& pd, double t) {
 // B-spline envelope of Sec. 2): d_k(t) = sum_f e^{i Omega_kf t} sum_s (a1 + i a2)_kfs B_s(t),
 // and the step solver's iteration counts (step_counts).  Also stores the spline weights for the
 // gradient quadrature of the adjoint sweep.  The carrier phases come from the problem's phase
-// table (k_phases).
-__global__ void k_controls(const ProbDev pd) {
+// table (k_phases).  pair: the kernel family the counts are for.
+__global__ void k_controls(const ProbDev pd, const int pair) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; n < pd.nsteps; n += stride) {
         const double t = (double(n) + 0.5) * pd.h;
@@ -106,7 +106,7 @@ __global__ void k_controls(const ProbDev pd) {
             mag += sqrt(dk.x * dk.x + dk.y * dk.y);
         }
         const float rho = float(0.5 * pd.h * pd.lam * mag + pd.rho_ex) * 1.0001f;
-        pd.spl[n] = Spline4{sp.s0, step_counts(pd.solver, pd.pair, rho, float(pd.kap)), sp.w0, sp.w1, sp.w2};
+        pd.spl[n] = Spline4{sp.s0, step_counts(pd.solver, pair, rho, float(pd.kap)), sp.w0, sp.w1, sp.w2};
     }
 }
 
@@ -140,6 +140,109 @@ __device__ double block_sum(double v, double* sh) {
     const double r = sh[0];
     __syncthreads();
     return r;
+}
+
+// ------------------------------------------------------------------ slices of a window
+// A window's propagation is linear in its state, so a problem with few columns for the GPU is cut
+// into C slices a window that run at the same time: a sweep of every slice from the unit vectors
+// gives its propagator Phi (N columns instead of E), a chain of C small products per (window,
+// column) gives the states at the slices' starts and the window's end, and the same chain with
+// Phi^+ the adjoint states at the slices' ends.  The history and adjoint sweeps then run all
+// slices at once, both in one launch: two sweeps of n / C steps and 2 C products in place of two
+// sweeps of n steps.  The products are FP64.
+constexpr int COMPOSE_THREADS = 256;
+// thread t works on row t / JG and the terms congruent to t % JG mod JG of its sum (JG adjacent
+// lanes share a row): short chains, since a chain of FP64 operations costs ~70 cycles each
+struct ComposeGeom {
+    int R, JG;
+};
+__host__ __device__ inline ComposeGeom compose_geom(int N) {
+    int R = 1, n2 = 1;
+    while (R < N) R <<= 1;
+    while (n2 * 2 <= N) n2 *= 2;
+    int JG = COMPOSE_THREADS / R;
+    JG = JG < 1 ? 1 : (JG > n2 ? n2 : JG);
+    return ComposeGeom{R, JG > 32 ? 32 : JG};
+}
+// xs <- Phi xs (BWD: Phi^+ xs) for one propagator; every thread of the block takes part
+template <bool BWD>
+__device__ __forceinline__ void compose_step(const double2* __restrict__ Phi, int N, const ComposeGeom& ge,
+                                             double2* xs) {
+    const int i = threadIdx.x / ge.JG, g = threadIdx.x % ge.JG;
+    double2 y0 = make_double2(0.0, 0.0), y1 = y0;
+    if (i < N) {
+        // the terms in two running sums (shorter chains)
+        const double2* p = BWD ? Phi + size_t(i) * N : Phi + i;
+        const int st = BWD ? 1 : N;
+        int j = g;
+#pragma unroll 4
+        for (; j + ge.JG < N; j += 2 * ge.JG) {
+            const double2 a = p[size_t(j) * st], b = p[size_t(j + ge.JG) * st];
+            const double2 x = xs[j], z = xs[j + ge.JG];
+            const double ai = BWD ? -a.y : a.y, bi = BWD ? -b.y : b.y;
+            y0.x = fma(a.x, x.x, fma(-ai, x.y, y0.x));
+            y0.y = fma(a.x, x.y, fma(ai, x.x, y0.y));
+            y1.x = fma(b.x, z.x, fma(-bi, z.y, y1.x));
+            y1.y = fma(b.x, z.y, fma(bi, z.x, y1.y));
+        }
+        if (j < N) {
+            const double2 a = p[size_t(j) * st], x = xs[j];
+            const double ai = BWD ? -a.y : a.y;
+            y0.x = fma(a.x, x.x, fma(-ai, x.y, y0.x));
+            y0.y = fma(a.x, x.y, fma(ai, x.x, y0.y));
+        }
+    }
+    double yr = y0.x + y1.x, yi = y0.y + y1.y;
+    for (int o = ge.JG >> 1; o > 0; o >>= 1) {
+        yr += __shfl_xor_sync(0xffffffffu, yr, o);
+        yi += __shfl_xor_sync(0xffffffffu, yi, o);
+    }
+    __syncthreads();   // xs has been read
+    if (i < N && g == 0) xs[i] = make_double2(yr, yi);
+    __syncthreads();
+}
+// One block per (column, window, problem).  Forward: Ubeg of every slice from W^{m-1} (identity
+// embedding for the whole problem's first window) and U^m(t_m); backward: Lend of every slice from
+// Lambda^m(t_m) and Lambda^m(t_{m-1}).
+__global__ void __launch_bounds__(COMPOSE_THREADS) k_compose(const ProbDev* pds, const int* list, const int bwd) {
+    __shared__ double2 xs[256];
+    const ProbDev& pd = pds[list ? list[blockIdx.z] : blockIdx.z];
+    const int col = blockIdx.x, m = blockIdx.y, N = pd.N, E = pd.E, C = pd.C;
+    if (C == 1 || m >= pd.M || col >= E) return;
+    const ComposeGeom ge = compose_geom(N);
+    const size_t wcol = (size_t(m) * E + col) * N;
+    for (int i = threadIdx.x; i < N; i += blockDim.x)
+        xs[i] = bwd ? pd.Lterm[wcol + i]
+                    : (m + pd.m_off == 0 ? make_double2(pd.emb[col] == i ? 1.0 : 0.0, 0.0)
+                                         : pd.W[(size_t(m) - 1) * E * N + size_t(col) * N + i]);
+    __syncthreads();
+    for (int s = 0; s < C; ++s) {
+        const size_t v = size_t(m) * C + (bwd ? C - 1 - s : s);
+        double2* keep = (bwd ? pd.Lend : pd.Ubeg) + (v * E + col) * N;
+        for (int i = threadIdx.x; i < N; i += blockDim.x) keep[i] = xs[i];
+        const double2* Phi = pd.Phi + v * N * N;
+        if (bwd)
+            compose_step<true>(Phi, N, ge, xs);
+        else
+            compose_step<false>(Phi, N, ge, xs);
+    }
+    for (int i = threadIdx.x; i < N; i += blockDim.x) (bwd ? pd.Lam0 : pd.Uend)[wcol + i] = xs[i];
+}
+// The roll-out's chain over the propagators of windows w0 .. w0 + nw - 1 (C a window), one block a
+// column: from the identity embedding (w0 = 0) or the state W^{w0} an earlier launch stored, the
+// states W^{w+1} at the windows' ends (but the last window's).
+__global__ void __launch_bounds__(COMPOSE_THREADS) k_compose_rollout(const ProbDev pd, const double2* Phi, int C, int w0,
+                                                                     int nw, double2* W) {
+    __shared__ double2 xs[256];
+    const int col = blockIdx.x, N = pd.N, E = pd.E;
+    const ComposeGeom ge = compose_geom(N);
+    for (int i = threadIdx.x; i < N; i += blockDim.x)
+        xs[i] = w0 == 0 ? make_double2(pd.emb[col] == i ? 1.0 : 0.0, 0.0) : W[(size_t(w0 - 1) * E + col) * N + i];
+    __syncthreads();
+    for (int w = 0; w < nw && w0 + w < pd.M - 1; ++w) {
+        for (int s = 0; s < C; ++s) compose_step<false>(Phi + (size_t(w) * C + s) * N * N, N, ge, xs);
+        for (int i = threadIdx.x; i < N; i += blockDim.x) W[(size_t(w0 + w) * E + col) * N + i] = xs[i];
+    }
 }
 
 constexpr int TERM_THREADS = 256;

@@ -21,10 +21,20 @@ struct msqoc_batch {
     struct Group {
         int L = 0, q = 0, solver = 0, pair = 0, lean = 0;   // shape, solver and kernel family of the group
         int nthreads = 0;                          // threads of its tiles
+        int pthreads = 0, plean = 0;               // propagator tiles (0: no member is sliced)
         std::vector<int> members;     // indices into probs
+        SweepArgs pargs{};            // the members' propagator sweep
+        int nptiles = 0, E_max = 1, M_max = 1;
+        Tile* ptiles = nullptr;
+        int* plmap = nullptr;
+        std::vector<Tile> host_ptiles;
+        std::vector<int> pfirst, pcount;      // per member: its tiles in host_ptiles
+        Tile* slot_ptiles[MSQOC_BATCH_SLOTS] = {};
+        Tile* slot_phost[MSQOC_BATCH_SLOTS] = {};
         SweepArgs args{};             // pds / tiles / lanemap / geometry of the group's launches
         int ntiles = 0;
         int nseg_max = 1, nsub_max = 1;
+        bool quad_small = true;       // every member takes FP64 products (quad_fp64)
         int quad_blocks = 0;          // blocks of a row of the quadrature launch: the most of the members
         ProbDev* pds = nullptr;
         Tile* tiles = nullptr;
@@ -53,14 +63,24 @@ struct msqoc_batch {
 
 namespace {
 
+int ipow(int b, int e) {
+    int r = 1;
+    while (e-- > 0) r *= b;
+    return r;
+}
+
 void free_batch(msqoc_batch* b) {
     for (auto& g : b->groups) {
         if (g.pds) cudaFree(g.pds);
         if (g.tiles) cudaFree(g.tiles);
         if (g.lanemap) cudaFree(g.lanemap);
+        if (g.ptiles) cudaFree(g.ptiles);
+        if (g.plmap) cudaFree(g.plmap);
         for (int k = 0; k < MSQOC_BATCH_SLOTS; ++k) {
             if (g.slot_tiles[k]) cudaFree(g.slot_tiles[k]);
             if (g.slot_host[k]) cudaFreeHost(g.slot_host[k]);
+            if (g.slot_ptiles[k]) cudaFree(g.slot_ptiles[k]);
+            if (g.slot_phost[k]) cudaFreeHost(g.slot_phost[k]);
             if (g.slot_list[k]) cudaFree(g.slot_list[k]);
             if (g.slot_lhost[k]) cudaFreeHost(g.slot_lhost[k]);
         }
@@ -105,20 +125,39 @@ msqoc_status for_groups(msqoc_batch* b, const int* ntiles, int set, cudaStream_t
     return MSQOC_OK;
 }
 
-// The launch sequence of one batched evaluation of the problems `sel` (all when sel is empty);
-// tiles[g] / ntiles[g] are the tiles of group g to launch, list[g] / nlist[g] its members (device
-// array; nullptr: every member, in order); set: the stream set of the groups.
-msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, Tile* const* tiles, const int* ntiles,
-                     int* const* list, const int* nlist, bool grad, int set, cudaStream_t s) {
+// What one batched evaluation launches of a group: its tiles, its propagator tiles and its members
+// (list: device array, nullptr for every member in order).
+struct GroupWork {
+    Tile* tiles = nullptr;
+    Tile* ptiles = nullptr;
+    int* list = nullptr;
+    int ntiles = 0, nptiles = 0, nlist = 0;
+};
+// The launch sequence of one batched evaluation of the problems `sel`; work[g]: the part of group g;
+// set: the stream set of the groups.
+msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, const std::vector<GroupWork>& work,
+                     bool grad, int set, cudaStream_t s) {
+    std::vector<int> ntiles;
+    for (const GroupWork& w : work) ntiles.push_back(w.ntiles);
     msqoc_status st;
     for (msqoc_problem* p : sel)
-        if ((st = launch_controls(p, s))) return st;
-    st = for_groups(b, ntiles, set, s, [&](int gi, cudaStream_t gs) {
-        SweepArgs a = b->groups[gi].args;
-        a.tiles = tiles[gi];
+        if ((st = launch_controls(p, p->pd.pair, s))) return st;
+    st = for_groups(b, ntiles.data(), set, s, [&](int gi, cudaStream_t gs) {
+        const auto& g = b->groups[gi];
+        if (g.pthreads) {
+            SweepArgs pa = g.pargs;
+            pa.tiles = work[gi].ptiles;
+            cudaError_t e = launch_sweep(pa, work[gi].nptiles, gs);
+            if (e == cudaSuccess)
+                e = launch_compose(g.pds, work[gi].list, g.E_max, g.M_max, work[gi].nlist, ipow(g.L, g.q), false, gs);
+            if (e != cudaSuccess) return e;
+        }
+        if (g.pthreads && (!grad || g.nsub_max == 1)) return cudaSuccess;   // (history: with the adjoint)
+        SweepArgs a = g.args;
+        a.tiles = work[gi].tiles;
         a.mode = grad ? SWEEP_HISTORY : SWEEP_OBJECTIVE;
         a.seg = 0;
-        return launch_sweep(a, ntiles[gi], gs);
+        return launch_sweep(a, work[gi].ntiles, gs);
     });
     if (st) return st;
     for (msqoc_problem* p : sel)
@@ -130,25 +169,31 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, Til
         }
         return MSQOC_OK;
     }
-    st = for_groups(b, ntiles, set, s, [&](int gi, cudaStream_t gs) {
+    st = for_groups(b, ntiles.data(), set, s, [&](int gi, cudaStream_t gs) {
         const auto& g = b->groups[gi];
+        if (g.pthreads) {
+            const cudaError_t e =
+                launch_compose(g.pds, work[gi].list, g.E_max, g.M_max, work[gi].nlist, ipow(g.L, g.q), true, gs);
+            if (e != cudaSuccess) return e;
+        }
         for (int seg = g.nseg_max - 1; seg >= 0; --seg) {
             SweepArgs a = g.args;
-            a.tiles = tiles[gi];
+            a.tiles = work[gi].tiles;
             a.seg = seg;
             if (g.nseg_max > 1) {
                 a.mode = SWEEP_RECOMPUTE;
-                const cudaError_t e = launch_sweep(a, ntiles[gi], gs);
+                const cudaError_t e = launch_sweep(a, work[gi].ntiles, gs);
                 if (e != cudaSuccess) return e;
             }
             for (int sub = g.nsub_max - 1; sub >= 0; --sub) {
-                a.mode = SWEEP_ADJOINT;
+                a.mode = g.pthreads && g.nsub_max == 1 ? SWEEP_BOTH : SWEEP_ADJOINT;
                 a.sub = sub;
-                cudaError_t e = launch_sweep(a, ntiles[gi], gs);
+                cudaError_t e = launch_sweep(a, work[gi].ntiles, gs);
                 if (e != cudaSuccess) return e;
                 QuadArgs qa = quad_args(b->probs[g.members[0]]->pd, g.pds, seg, sub);
-                qa.list = list[gi];
-                e = launch_quad(qa, g.quad_blocks, nlist[gi], gs);
+                if (qa.mode && !g.quad_small) qa.mode = 1;
+                qa.list = work[gi].list;
+                e = launch_quad(qa, g.quad_blocks, work[gi].nlist, gs);
                 if (e != cudaSuccess) return e;
             }
         }
@@ -164,15 +209,10 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, Til
 }
 
 msqoc_status enqueue_all(msqoc_batch* b, bool grad, cudaStream_t s) {
-    std::vector<Tile*> tiles;
-    std::vector<int> ntiles, nlist;
-    std::vector<int*> list(b->groups.size(), nullptr);
-    for (auto& g : b->groups) {
-        tiles.push_back(g.tiles);
-        ntiles.push_back(g.ntiles);
-        nlist.push_back(static_cast<int>(g.members.size()));
-    }
-    return enqueue(b, b->probs, tiles.data(), ntiles.data(), list.data(), nlist.data(), grad, MSQOC_BATCH_SLOTS, s);
+    std::vector<GroupWork> work;
+    for (auto& g : b->groups)
+        work.push_back(GroupWork{g.tiles, g.ptiles, nullptr, g.ntiles, g.nptiles, static_cast<int>(g.members.size())});
+    return enqueue(b, b->probs, work, grad, MSQOC_BATCH_SLOTS, s);
 }
 
 msqoc_status eval(msqoc_batch* b, bool grad, cudaStream_t s) {
@@ -237,12 +277,13 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         for (msqoc_problem* p : b->probs)
             if (!st) st = ensure_gradient_buffers(p, nullptr);
     if (!st && cudaDeviceSynchronize() != cudaSuccess) st = fail(MSQOC_ERR_CUDA, "synchronize failed");
-    // groups by (levels, subsystems, solver, kernel family, tile threads)
+    // groups by (levels, subsystems, solver, kernel family, tile threads, propagator tiles)
     for (int i = 0; i < n && !st; ++i) {
         const ProbDev& pd = b->probs[i]->pd;
         auto it = std::find_if(b->groups.begin(), b->groups.end(), [&](const msqoc_batch::Group& g) {
             return g.L == pd.L && g.q == pd.q && g.solver == pd.solver && g.pair == pd.pair && g.lean == pd.lean &&
-                   g.nthreads == pd.nthreads;
+                   g.nthreads == pd.nthreads && g.pthreads == b->probs[i]->prop.nthreads &&
+                   g.plean == b->probs[i]->prop.lean;
         });
         if (it == b->groups.end()) {
             b->groups.emplace_back();
@@ -253,6 +294,8 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
             it->pair = pd.pair;
             it->lean = pd.lean;
             it->nthreads = pd.nthreads;
+            it->pthreads = b->probs[i]->prop.nthreads;
+            it->plean = b->probs[i]->prop.lean;
         }
         it->members.push_back(i);
     }
@@ -274,33 +317,53 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
             g.nseg_max = std::max(g.nseg_max, pd.nseg);
             g.nsub_max = std::max(g.nsub_max, pd.nsub);
             g.quad_blocks = std::max(g.quad_blocks, quad_blocks(pd));
+            g.quad_small = g.quad_small && quad_fp64(pd);
         }
         std::vector<ProbDev> pds;
-        std::vector<Tile> tiles;
-        std::vector<int> maps;
+        std::vector<Tile> tiles, ptiles;
+        std::vector<int> maps, pmaps;
+        SweepPlan plan{0, g.pthreads, g.plean, 0};
+        // a member's tiles and lane maps (V windows of E columns) behind those of the others
+        auto append = [](std::vector<Tile>& ts, std::vector<int>& ms, const ProbDev& pd, int k, int V, int E, int cb,
+                         int nt, int pair) {
+            const int map_base = static_cast<int>(ms.size() / nt);
+            const int n = static_cast<int>(tile_count(V, E, cb));
+            for (int t = 0; t < n; ++t) {
+                Tile x = tile_at(t, V, E, cb, k);
+                x.map += map_base;
+                ts.push_back(x);
+            }
+            const Tile last = tile_at(n - 1, V, E, cb, 0);
+            ms.resize(ms.size() + size_t(cb + 1) * nt);
+            int* mp = ms.data() + size_t(map_base) * nt;
+            for (int j = 0; j <= cb; ++j)
+                build_lanemap(pd.L, pd.q, j < cb ? cb : last.ncol, j < cb ? j + 1 : last.ncol0, nt, pair,
+                              mp + size_t(j) * nt);
+            return n;
+        };
         for (size_t k = 0; k < g.members.size(); ++k) {
             const ProbDev& pd = b->probs[g.members[k]]->pd;
-            const int map_base = static_cast<int>(maps.size() / nthreads);
+            const msqoc_problem* pr = b->probs[g.members[k]];
             g.first.push_back(static_cast<int>(tiles.size()));
-            g.count.push_back(pd.ntiles);
-            for (int t = 0; t < pd.ntiles; ++t) {
-                Tile x = tile_at(t, pd.M, pd.E, pd.cb, static_cast<int>(k));
-                x.map += map_base;
-                tiles.push_back(x);
+            g.count.push_back(append(tiles, maps, pd, static_cast<int>(k), pd.M * pd.C, pd.E, pd.cb, nthreads, pd.pair));
+            g.E_max = std::max(g.E_max, pd.E);
+            g.M_max = std::max(g.M_max, pd.M);
+            if (g.pthreads) {
+                g.pfirst.push_back(static_cast<int>(ptiles.size()));
+                g.pcount.push_back(append(ptiles, pmaps, pd, static_cast<int>(k), pd.M * pd.C, pd.N, pr->prop.cpt,
+                                          g.pthreads, 0));
+                plan.cpt = std::max(plan.cpt, pr->prop.cpt);
             }
-            const Tile last = tile_at(pd.ntiles - 1, pd.M, pd.E, pd.cb, 0);
-            maps.resize(maps.size() + size_t(pd.cb + 1) * nthreads);
-            int* mp = maps.data() + size_t(map_base) * nthreads;
-            for (int j = 0; j <= pd.cb; ++j)
-                build_lanemap(pd.L, pd.q, j < pd.cb ? pd.cb : last.ncol, j < pd.cb ? j + 1 : last.ncol0, nthreads,
-                              pd.pair, mp + size_t(j) * nthreads);
             pds.push_back(pd);
         }
         // longest windows first: the CTAs that take longest start in the first wave
         auto tile_len = [&](const Tile& x) {
             const ProbDev& pd = b->probs[g.members[x.prob]]->pd;
-            return (pd.nsteps + pd.M - 1) / pd.M;
+            return (pd.nsteps + pd.M * pd.C - 1) / (pd.M * pd.C);
         };
+        g.host_ptiles = ptiles;
+        std::stable_sort(ptiles.begin(), ptiles.end(), [&](const Tile& x, const Tile& y) { return tile_len(x) > tile_len(y); });
+        g.nptiles = static_cast<int>(ptiles.size());
         g.host_tiles = tiles;
         std::stable_sort(tiles.begin(), tiles.end(), [&](const Tile& x, const Tile& y) { return tile_len(x) > tile_len(y); });
         g.ntiles = static_cast<int>(tiles.size());
@@ -310,7 +373,18 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         if (e == cudaSuccess) e = cudaMemcpy(g.pds, pds.data(), pds.size() * sizeof(ProbDev), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(g.tiles, tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(g.lanemap, maps.data(), maps.size() * sizeof(int), cudaMemcpyHostToDevice);
+        if (g.pthreads) {
+            if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&g.ptiles), ptiles.size() * sizeof(Tile));
+            if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&g.plmap), pmaps.size() * sizeof(int));
+            if (e == cudaSuccess) e = cudaMemcpy(g.ptiles, ptiles.data(), ptiles.size() * sizeof(Tile), cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaMemcpy(g.plmap, pmaps.data(), pmaps.size() * sizeof(int), cudaMemcpyHostToDevice);
+        }
         for (int k = 0; k < MSQOC_BATCH_SLOTS && e == cudaSuccess; ++k) {
+            if (g.pthreads) {
+                e = cudaMalloc(reinterpret_cast<void**>(&g.slot_ptiles[k]), ptiles.size() * sizeof(Tile));
+                if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&g.slot_phost[k]), ptiles.size() * sizeof(Tile));
+                if (e != cudaSuccess) break;
+            }
             e = cudaMalloc(reinterpret_cast<void**>(&g.slot_tiles[k]), tiles.size() * sizeof(Tile));
             if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&g.slot_host[k]), tiles.size() * sizeof(Tile));
             if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&g.slot_list[k]), g.members.size() * sizeof(int));
@@ -328,6 +402,7 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         g.args.cpt = cpt;
         g.args.gmax = gmax;
         g.args.nthreads = nthreads;
+        if (g.pthreads) g.pargs = prop_args(plan, p0, g.pds, g.ptiles, g.plmap);
         SweepArgs adj = g.args;
         adj.mode = SWEEP_ADJOINT;
         if (admission_bytes(g.q, g.L, p0.N, cpt, nthreads, gmax, g.solver, g.pair, g.args.hdepth) > 227 * 1024) {
@@ -337,7 +412,12 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         // set the kernels' shared-memory limits now (a launch of no tiles only does that), so
         // that a graph capture later makes no attribute calls
         if (launch_sweep(g.args, 0, nullptr) != cudaSuccess || launch_sweep(adj, 0, nullptr) != cudaSuccess ||
-            launch_quad(quad_args(p0, g.pds, 0, 0), 0, 0, nullptr) != cudaSuccess)
+            launch_quad(quad_args(p0, g.pds, 0, 0), 0, 0, nullptr) != cudaSuccess ||
+            (g.pthreads && (launch_sweep(g.pargs, 0, nullptr) != cudaSuccess || [&] {
+                 SweepArgs both = g.args;
+                 both.mode = SWEEP_BOTH;
+                 return launch_sweep(both, 0, nullptr);
+             }() != cudaSuccess)))
             st = fail(MSQOC_ERR_CUDA, "sweep kernel attributes could not be set");
     }
     if (!st && (flags & MSQOC_BATCH_GRAPH) && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
@@ -379,36 +459,46 @@ msqoc_status batch_eval_subset(msqoc_batch* b, const int32_t* members, int32_t n
     // the slot's staging buffers are rewritten only after its previous copies were read
     CUDA_TRY(cudaEventSynchronize(b->slot_done[slot]));
     std::vector<msqoc_problem*> sel;
-    std::vector<Tile*> tiles(b->groups.size());
-    std::vector<int> ntiles(b->groups.size(), 0), nlist(b->groups.size(), 0);
-    std::vector<int*> list(b->groups.size());
+    std::vector<GroupWork> work(b->groups.size());
     for (int i = 0; i < n; ++i) sel.push_back(b->probs[members[i]]);
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         auto& g = b->groups[gi];
+        GroupWork& w = work[gi];
         Tile* h = g.slot_host[slot];
-        int cnt = 0;
+        Tile* ph = g.slot_phost[slot];
         for (int i = 0; i < n; ++i) {
             if (b->group_of[members[i]] != static_cast<int>(gi)) continue;
             const int k = b->member_of[members[i]];
-            std::copy(g.host_tiles.begin() + g.first[k], g.host_tiles.begin() + g.first[k] + g.count[k], h + cnt);
-            cnt += g.count[k];
-            g.slot_lhost[slot][nlist[gi]++] = k;
+            std::copy(g.host_tiles.begin() + g.first[k], g.host_tiles.begin() + g.first[k] + g.count[k], h + w.ntiles);
+            w.ntiles += g.count[k];
+            if (g.pthreads) {
+                std::copy(g.host_ptiles.begin() + g.pfirst[k], g.host_ptiles.begin() + g.pfirst[k] + g.pcount[k],
+                          ph + w.nptiles);
+                w.nptiles += g.pcount[k];
+            }
+            g.slot_lhost[slot][w.nlist++] = k;
         }
-        auto tile_len = [&](const Tile& x) {
-            const ProbDev& pd = b->probs[g.members[x.prob]]->pd;
-            return (pd.nsteps + pd.M - 1) / pd.M;
+        if (!w.ntiles) continue;
+        auto longer = [&](const Tile& x, const Tile& y) {
+            auto len = [&](const Tile& t) {
+                const ProbDev& pd = b->probs[g.members[t.prob]]->pd;
+                return (pd.nsteps + pd.M * pd.C - 1) / (pd.M * pd.C);
+            };
+            return len(x) > len(y);
         };
-        std::stable_sort(h, h + cnt, [&](const Tile& x, const Tile& y) { return tile_len(x) > tile_len(y); });
-        if (cnt) CUDA_TRY(cudaMemcpyAsync(g.slot_tiles[slot], h, cnt * sizeof(Tile), cudaMemcpyHostToDevice, s));
-        if (cnt && gradient)
-            CUDA_TRY(cudaMemcpyAsync(g.slot_list[slot], g.slot_lhost[slot], nlist[gi] * sizeof(int),
-                                     cudaMemcpyHostToDevice, s));
-        tiles[gi] = g.slot_tiles[slot];
-        ntiles[gi] = cnt;
-        list[gi] = g.slot_list[slot];
+        std::stable_sort(h, h + w.ntiles, longer);
+        CUDA_TRY(cudaMemcpyAsync(g.slot_tiles[slot], h, w.ntiles * sizeof(Tile), cudaMemcpyHostToDevice, s));
+        if (w.nptiles) {
+            std::stable_sort(ph, ph + w.nptiles, longer);
+            CUDA_TRY(cudaMemcpyAsync(g.slot_ptiles[slot], ph, w.nptiles * sizeof(Tile), cudaMemcpyHostToDevice, s));
+        }
+        CUDA_TRY(cudaMemcpyAsync(g.slot_list[slot], g.slot_lhost[slot], w.nlist * sizeof(int), cudaMemcpyHostToDevice, s));
+        w.tiles = g.slot_tiles[slot];
+        w.ptiles = g.slot_ptiles[slot];
+        w.list = g.slot_list[slot];
     }
     CUDA_TRY(cudaEventRecord(b->slot_done[slot], s));
-    return enqueue(b, sel, tiles.data(), ntiles.data(), list.data(), nlist.data(), gradient != 0, slot, s);
+    return enqueue(b, sel, work, gradient != 0, slot, s);
 }
 
 }  // namespace

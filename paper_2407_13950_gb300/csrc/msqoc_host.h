@@ -8,6 +8,13 @@
 #include "../../include/msqoc.h"
 #include "msqoc_internal.h"
 
+namespace msqoc {
+// tiles of a propagator sweep: columns a tile, threads, register build, count
+struct SweepPlan {
+    int cpt = 0, nthreads = 0, lean = 0, ntiles = 0;
+};
+}  // namespace msqoc
+
 // One problem on one device: the model tables, its tile layout and every buffer an evaluation
 // needs.  Created by msqoc_create_problem, which owns all of it.
 struct msqoc_problem {
@@ -22,9 +29,17 @@ struct msqoc_problem {
     msqoc::ProbDev* pds = nullptr;   // device copy of pd (read by the sweeps)
     msqoc::Tile* tiles = nullptr;
     int* lanemap = nullptr;
-    msqoc::Tile* tiles_ro = nullptr;   // the roll-out sweep: one window over the whole grid
+    msqoc::Tile* tiles_prop = nullptr;   // the propagator sweep of a sliced problem
+    int* lanemap_prop = nullptr;
+    msqoc::SweepPlan prop;
+    msqoc::Tile* tiles_ro = nullptr;     // the roll-out's, for ro_windows windows of ro_slices slices
     int* lanemap_ro = nullptr;
-    int ntiles_ro = 0;
+    msqoc::SweepPlan ro;
+    int ro_windows = 0, ro_slices = 1;
+    double2* phi_ro = nullptr;           // [ro_windows ro_slices][N][N]
+    double2* Phi = nullptr;              // sliced problems: see ProbDev
+    double2* Ubeg = nullptr;
+    double2* Lend = nullptr;             // (with hist)
     double2* P = nullptr;
     int* emb = nullptr;
     double2* V = nullptr;
@@ -88,14 +103,22 @@ void build_lanemap(int L, int q, int ncol, int ncol0, int nthreads, int pair, in
 // kernel family (pair: log2 of the threads per fiber, 0, 1 or 2) and columns per tile of a problem
 struct TileChoice {
     int cpt, pair, lean;
+    double cost;   // the tile model's makespan of a step
 };
 Tile tile_at(long t, int M, int E, int cpt, int prob);
 long tile_count(int M, int E, int cpt);
 SweepArgs sweep_args(const ProbDev& pd, const ProbDev* pds_dev, const Tile* tiles, const int* lanemap, int mode,
                      int seg);
 
+// propagator launch arguments of a plan, and the chain over the propagators of `nprob` problems of
+// one shape (list: their indices into pds_dev, nullptr for 0 .. nprob - 1; E, M the largest)
+SweepArgs prop_args(const SweepPlan& plan, const ProbDev& pd, const ProbDev* pds_dev, const Tile* tiles,
+                    const int* lanemap);
+cudaError_t launch_compose(const ProbDev* pds_dev, const int* list, int E, int M, int nprob, int N, bool bwd,
+                           cudaStream_t s);
 // quadrature launch arguments (SweepArgs of the same segment and chunk), see k_quad
 QuadArgs quad_args(const ProbDev& pd, const ProbDev* pds_dev, int seg, int sub);
+bool quad_fp64(const ProbDev& pd);
 // shared memory that admits a tile (see msqoc_api.cu)
 size_t admission_bytes(int q, int L, int N, int cpt, int nthreads, int g, int solver, int pair, int depth);
 
@@ -116,7 +139,8 @@ bool is_shard(const ProbDev& pd);
 msqoc_status stage_inputs(msqoc_problem* p, const double* alpha, const double* W, cudaStream_t s);
 msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s);
 int phase_blocks(const ProbDev& pd);   // blocks of 256 threads for k_phases
-msqoc_status launch_controls(msqoc_problem* p, cudaStream_t s);
+// pair: the kernel family of the sweeps that follow (its iteration counts)
+msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s);
 msqoc_status launch_terminal(msqoc_problem* p, bool want_lambda, cudaStream_t s);
 // P, J (may be NULL), pen (may be NULL) of the last forward sweep into device arrays
 msqoc_status launch_objective_outputs(msqoc_problem* p, double* P, double* J, double* pen, cudaStream_t s);

@@ -61,6 +61,7 @@ struct ProbDev {
     int glocal;    // doubles of a window's part of the alpha-gradient (its active splines with a
                    // margin of two, every carrier): enters the admission of tiles only
     int solver;
+    int C;         // slices per window (1: a window is swept as a whole; see k_compose)
     int kseg;      // steps per history segment (checkpoint interval; >= the longest window when
                    // every midpoint state is kept)
     int nseg;      // segments per window: ceil(longest window / kseg)
@@ -96,6 +97,11 @@ struct ProbDev {
     double2* ctrl;               // [nsteps][q] d_k(t_{n+1/2})
     Spline4* spl;                // [nsteps] (first spline index, solver counts, w0, w1, w2)
     double2* phase;              // [nsteps][nfsum] exp(i Omega t_{n+1/2})
+    // sliced problems (C > 1): slice i of window m is virtual window m C + i (0-based) and every per-
+    // window history below is per virtual window
+    double2* Phi;                // [M C][N][N] propagators, column-major
+    double2* Ubeg;               // [M C][E][N] states at the slices' starts
+    double2* Lend;               // [M C][E][N] adjoint states at the slices' ends
     double2* hist;               // [M][kseg][E][N] midpoint states Ubar of one segment of every window
                                  // (the mixed solver's one-thread families store each entry as the
                                  // two-float split of Ubar 2^-hsh, hsh the column's scale exponent)
@@ -133,8 +139,10 @@ enum SweepMode {
     SWEEP_RECOMPUTE = 3,  // forward over segment `seg` from its checkpoint; midpoint states
                           // (no work for a problem with one segment)
     SWEEP_ADJOINT = 4,    // adjoint over chunk `sub` of segment `seg`; its midpoint states
-    SWEEP_ROLLOUT = 5     // forward over the whole time grid as one window from the identity
-                          // embedding; the state at every window boundary t_m into `out`
+    SWEEP_PROP = 5,       // forward over every slice from the N unit vectors: its propagator
+                          // (one thread per fiber)
+    SWEEP_BOTH = 6        // SWEEP_HISTORY and SWEEP_ADJOINT (chunk `sub`) of sliced problems in one
+                          // launch (one thread per fiber, mixed solver)
 };
 
 // Arguments of one sweep launch (uniform over its tiles; problems share shape and solver).
@@ -151,7 +159,9 @@ struct SweepArgs {
     int pair;             // kernel family: log2 of the threads per fiber (0, 1 or 2)
     int lean;             // pair = 0 with the 168-register build (ProbDev::lean)
     int hdepth;           // steps per history group (ProbDev::hdepth), >= 1
-    double2* out;         // SWEEP_ROLLOUT: [M-1][E][N] states at the window boundaries
+    int slices, voff;     // SWEEP_PROP with slices > 0: slices a window instead of ProbDev::C, the
+                          // first virtual window of the launch (0-based), and
+    double2* phi;         // its propagators [virtual windows of the launch][N][N]
 };
 
 // shared-memory bytes of a sweep launch
@@ -165,9 +175,18 @@ cudaError_t launch_sweep(const SweepArgs& a, int ntiles, cudaStream_t s);
 struct QuadArgs {
     const ProbDev* pds;   // device copies
     const int* list;      // [blocks in y] problem of each row of blocks; nullptr: row y is problem y
-    int L, q, split;      // split: the midpoint states are stored split (two floats)
+    int L, q, mode;       // mode: k_quad's MODE
     int seg, sub;
 };
+// First global step of virtual window v (1-based) of a problem with C slices a window; the end of the
+// grid beyond the last.
+__host__ __device__ inline int64_t slice_start(const ProbDev& pd, int C, int v) {
+    const int w = (v - 1) / C;
+    const auto win = [&](int m) { return (static_cast<int64_t>(pd.m_off + m) * pd.nsteps) / pd.M_glob; };
+    if (w >= pd.M) return win(pd.M);
+    const int64_t n0 = win(w);
+    return C == 1 ? n0 : n0 + ((v - 1 - w * C) * (win(w + 1) - n0)) / C;
+}
 // blocks a problem needs for its windows' chunks
 int quad_blocks(const ProbDev& pd);
 // nprob rows of `blocks` blocks each (0 blocks: only sets the kernel's attributes)

@@ -90,13 +90,27 @@ __host__ __device__ constexpr size_t quad_smem() {
     return stage > sums ? stage : sums;
 }
 
-template <int L, int Q, bool SPLIT>
+// operands of a product: the entry as stored, or (MODE 2) a split entry as one double a component
+template <int MODE>
+__device__ __forceinline__ double2 quad_operand(const double2& v) { return v; }
+template <int MODE>
+__device__ __forceinline__ std::conditional_t<MODE == 2, double2, float4> quad_operand(const float4& v) {
+    if constexpr (MODE == 2)
+        return make_double2(df_to_f64_scaled(DF{v.x, v.z}, 0), df_to_f64_scaled(DF{v.y, v.w}, 0));
+    else
+        return v;
+}
+
+// MODE 0: FP64 states; 1: split states, two-float sums; 2: split states, FP64 products and sums
+// (QUAD_FP64_MOST: problems so small that the FP64 pipe does not show)
+template <int L, int Q, int MODE>
 __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs a) {
     constexpr int N = ipow_c(L, Q), F = N / L, NW = quad_warps<L, Q>(), LN = quad_lanes<L, Q>();
     constexpr int WS = quad_split<L, Q>();
     constexpr int UN = L == 3 ? (F < 3 ? 1 : 3) : (F < 4 ? F : 4);   // pairs summed afresh; divides F
     constexpr int ROW = LN + 1;
-    using GT = std::conditional_t<SPLIT, DF, double>;
+    constexpr bool SPLIT = MODE > 0;
+    using GT = std::conditional_t<MODE == 1, DF, double>;
     using ET = std::conditional_t<SPLIT, float4, double2>;
     const ProbDev& pd = a.pds[a.list ? a.list[blockIdx.y] : blockIdx.y];
     const int E = pd.E;
@@ -109,11 +123,11 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
     // ---- this CTA's steps: group g of window m, local steps [j0, j0 + spw) of the chunk
     const int spw = LN / EL;
     const int groups = (pd.kadj + spw - 1) / spw;
-    const int m = blockIdx.x / groups;                       // window, 0-based
-    if (m >= pd.M) return;
+    const int m = blockIdx.x / groups;                       // (virtual) window, 0-based
+    if (m >= pd.M * pd.C) return;
     const int j0 = (blockIdx.x - m * groups) * spw;
-    const int64_t n0 = win_start(pd, m + 1);
-    const int ns = static_cast<int>(win_start(pd, m + 2) - n0);
+    const int64_t n0 = slice_start(pd, pd.C, m + 1);
+    const int ns = static_cast<int>(slice_start(pd, pd.C, m + 2) - n0);
     const int lo = a.seg * pd.kseg + a.sub * pd.kadj;        // the chunk's first step in the window
     const int hi = min(min(ns, (a.seg + 1) * pd.kseg), lo + pd.kadj);
     if (lo + j0 >= hi) return;
@@ -170,8 +184,8 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
             for (int t = 0; t < UN; ++t) {
                 const int p = p0 + t, ph = p / st;
                 const int i = (ph * (L - 1) + j - 1) * st + p;   // digit j - 1 inserted at k
-                const ET x = Ls[i * ROW + ln], x2 = Ls[(i + st) * ROW + ln];
-                const ET u = Us[i * ROW + ln], u2 = Us[(i + st) * ROW + ln];
+                const auto x = quad_operand<MODE>(Ls[i * ROW + ln]), x2 = quad_operand<MODE>(Ls[(i + st) * ROW + ln]);
+                const auto u = quad_operand<MODE>(Us[i * ROW + ln]), u2 = quad_operand<MODE>(Us[(i + st) * ROW + ln]);
                 if (t == 0)
                     pair_products<true>(r, q, x, x2, u, u2);
                 else
@@ -186,8 +200,13 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
                 const int d = lsh[cb + cl] + hsh[cb + cl] - S;   // <= 0
                 const float ps = d >= -126 ? float_of(static_cast<uint32_t>(127 + d) << 23)
                                            : (d >= -149 ? float_of(1u << (d + 149)) : 0.f);
-                R = DF{fmul_n(R.s, ps), fmul_n(R.c, ps)};
-                I = DF{fmul_n(I.s, ps), fmul_n(I.c, ps)};
+                if constexpr (MODE == 1) {
+                    R = DF{fmul_n(R.s, ps), fmul_n(R.c, ps)};
+                    I = DF{fmul_n(I.s, ps), fmul_n(I.c, ps)};
+                } else {
+                    R *= ps;
+                    I *= ps;
+                }
             }
             A = gsum_add(A, I);
             B = gsum_add(B, R);
@@ -203,7 +222,7 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
         A = gsum_add(A, gsum_shfl_xor(A, LN));
         B = gsum_add(B, gsum_shfl_xor(B, LN));
     }
-    if constexpr (SPLIT) {
+    if constexpr (MODE == 1) {
         A = df_scale_sqrt(A, j);
         B = df_scale_sqrt(B, j);
     } else {
@@ -224,10 +243,10 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
 #pragma unroll
         for (int w = 1; w < (L - 1) * WS; ++w) t = gsum_add(t, q[w * spw * 2]);
         double v;
-        if constexpr (SPLIT)
+        if constexpr (MODE == 1)
             v = df_to_f64_scaled(t, S);
         else
-            v = t;
+            v = SPLIT ? ldexp(t, S) : t;
         reinterpret_cast<double*>(pd.quad)[2 * (size_t(kk) * pd.nsteps + n0 + lo + j0 + s) + (r & 1)] = v;
     }
 }

@@ -290,14 +290,14 @@ static __device__ __noinline__ void coarse_step(double2* D0, double2* cfd, const
 // whose slot has no step at an iteration keeps its state.
 // MAXT: the largest tile the instantiation serves; it sets the register budget (255 registers a
 // thread for MAX_TILE_THREADS, 168 for MAX_LEAN_TILE_THREADS: 12 warps on an SM).
-template <int L, int Q, int SOLVER, bool BWD, bool ROLLOUT = false, int MAXT = MAX_TILE_THREADS>
-__global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
-    static_assert(!(BWD && ROLLOUT), "the roll-out is a forward sweep");
+template <int L, int Q, int SOLVER, bool BWD, bool PROP>
+__device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, const int block) {
+    static_assert(!(BWD && PROP), "propagators are forward sweeps");
     constexpr int N = ipow_c(L, Q);
     constexpr int NSLOT = Q * L * 2;
     constexpr int S = BWD ? +1 : -1;       // sign of the preconditioned off-diagonal term
 
-    const Tile tile = a.tiles[blockIdx.x];
+    const Tile tile = a.tiles[block];
     const ProbDev& pd = a.pds[tile.prob];
 
     extern __shared__ __align__(128) unsigned char smem[];
@@ -315,31 +315,35 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int warp = tid >> 5;
-    const int E = pd.E;
+    const int E = PROP ? N : pd.E;         // columns a window
+    const int C = PROP && a.slices ? a.slices : pd.C;
     const int ncol = tile.ncol, ncol0 = tile.ncol0;
     const int nslot = ncol0 < ncol ? 2 : 1;
-    const bool segmented = a.mode == SWEEP_RECOMPUTE || a.mode == SWEEP_ADJOINT;
-    const bool idle_launch = a.mode == SWEEP_RECOMPUTE && pd.nseg == 1;   // nothing to recompute
-    constexpr bool rollout = ROLLOUT;   // one window over the whole grid (compiled separately)
+    const bool segmented = mode == SWEEP_RECOMPUTE || mode == SWEEP_ADJOINT;
+    // nothing to recompute; a sliced problem's objective comes from its propagators
+    const bool idle_launch = !PROP && ((mode == SWEEP_RECOMPUTE && pd.nseg == 1) ||
+                                       (mode == SWEEP_OBJECTIVE && C > 1));
+    if (idle_launch) return;
+    const int v0 = tile.m0 + (PROP ? a.voff : 0);   // the first slot's virtual window, 1-based
 
     // ---- the slots' windows and step ranges (local step indices [lo, lo + cnt) of the window)
-    const int64_t wn0_0 = rollout ? 0 : win_start(pd, tile.m0);
-    const int wns_0 = rollout ? static_cast<int>(pd.nsteps) : static_cast<int>(win_start(pd, tile.m0 + 1) - wn0_0);
-    const int64_t wn0_1 = nslot > 1 ? win_start(pd, tile.m0 + 1) : 0;
-    const int wns_1 = nslot > 1 ? static_cast<int>(win_start(pd, tile.m0 + 2) - wn0_1) : 0;
+    const int64_t wn0_0 = slice_start(pd, C, v0);
+    const int wns_0 = static_cast<int>(slice_start(pd, C, v0 + 1) - wn0_0);
+    const int64_t wn0_1 = nslot > 1 ? slice_start(pd, C, v0 + 1) : 0;
+    const int wns_1 = nslot > 1 ? static_cast<int>(slice_start(pd, C, v0 + 2) - wn0_1) : 0;
     // (an adjoint launch covers chunk `sub` of its segment)
     const int seg_hi = segmented ? (a.seg + 1) * pd.kseg : INT_MAX;
     const int lo = segmented ? a.seg * pd.kseg + (BWD ? a.sub * pd.kadj : 0) : 0;
     const int hi = BWD ? min(seg_hi, lo + pd.kadj) : seg_hi;
-    const int cnt_0 = idle_launch ? 0 : max(0, min(wns_0, hi) - lo);
-    const int cnt_1 = nslot > 1 && !idle_launch ? max(0, min(wns_1, hi) - lo) : 0;
+    const int cnt_0 = max(0, min(wns_0, hi) - lo);
+    const int cnt_1 = nslot > 1 ? max(0, min(wns_1, hi) - lo) : 0;
     const int nit = max(cnt_0, cnt_1);
     // global step of slot s at iteration jj, clamped into the slot's range (a slot without steps
     // in this launch maps to its window's first step, which exists)
     auto step_of = [&](int s, int jj) -> int64_t {
         const int cnt = s ? cnt_1 : cnt_0;
         const int64_t n0 = s ? wn0_1 : wn0_0;
-        if (cnt <= 0) return n0;
+        if (cnt <= 0) return min(n0, pd.nsteps - 1);
         const int jc = min(jj, cnt - 1);
         return BWD ? n0 + lo + cnt - 1 - jc : n0 + lo + jc;
     };
@@ -351,7 +355,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     const int c = lmv >> 16;                        // tile column
     const int f = lmv & 0xffff;                     // fiber
     const int slot = c < ncol0 ? 0 : 1;
-    const int m = tile.m0 + slot;                   // window, 1-based
+    const int m = tile.m0 + slot;                   // (virtual) window of the launch, 1-based
     const int col = slot == 0 ? tile.c0 + c : c - ncol0;
     const int my_cnt = slot ? cnt_1 : cnt_0;
     const int my_ns = slot ? wns_1 : wns_0;
@@ -396,6 +400,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     }
 
     // ---- initial state
+    //   propagator            : unit vectors; a sliced problem: the slice's Ubeg, Lend (k_compose)
     //   forward, whole window : U^m(t_{m-1}) = W^{m-1} (identity embedding for the first window
     //                           of the whole problem)
     //   forward, recompute    : the segment's checkpoint
@@ -405,11 +410,15 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         const int i = f * L + l;
-        if (my_cnt == 0) {
+        if constexpr (PROP) {
+            u[l] = make_double2(col == i ? 1.0 : 0.0, 0.0);
+        } else if (my_cnt == 0) {
             u[l] = make_double2(0.0, 0.0);
         } else if (BWD) {
-            u[l] = (lo + my_cnt == my_ns) ? pd.Lterm[wcol + i] : pd.Lstate[wcol + i];
-        } else if (a.mode == SWEEP_RECOMPUTE) {
+            u[l] = C > 1 ? pd.Lend[wcol + i] : (lo + my_cnt == my_ns) ? pd.Lterm[wcol + i] : pd.Lstate[wcol + i];
+        } else if (C > 1) {
+            u[l] = pd.Ubeg[wcol + i];
+        } else if (mode == SWEEP_RECOMPUTE) {
             u[l] = pd.ckpt[((size_t(m - 1) * pd.nseg + a.seg) * E + col) * N + i];
         } else if (m + pd.m_off == 1) {
             u[l] = make_double2(pd.emb[col] == i ? 1.0 : 0.0, 0.0);
@@ -443,17 +452,17 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     // the midpoint states' column scale exponent, read by the quadrature kernel: per segment for
     // the forward's history, per launch for the adjoint's
     if constexpr (SOLVER == SOLVER_MIXED) {
-        if (act && f == 0 && my_cnt > 0) {
+        if (!PROP && act && f == 0 && my_cnt > 0) {
             if (BWD)
                 pd.lsh[size_t(m - 1) * E + col] = sh;
-            else if ((a.mode == SWEEP_HISTORY && pd.nseg == 1) || a.mode == SWEEP_RECOMPUTE)
-                pd.hsh[(size_t(m - 1) * pd.nseg + (a.mode == SWEEP_HISTORY ? 0 : a.seg)) * E + col] = sh;
+            else if ((mode == SWEEP_HISTORY && pd.nseg == 1) || mode == SWEEP_RECOMPUTE)
+                pd.hsh[(size_t(m - 1) * pd.nseg + (mode == SWEEP_HISTORY ? 0 : a.seg)) * E + col] = sh;
         }
     }
 
     // ---- history blocks: slot s of a tile covers a contiguous column range of its window
-    const bool want_hist = BWD || (a.mode == SWEEP_HISTORY && pd.nseg == 1) || a.mode == SWEEP_RECOMPUTE;
-    const bool want_ckpt = !BWD && a.mode == SWEEP_HISTORY && pd.nseg > 1;
+    const bool want_hist = !PROP && (BWD || (mode == SWEEP_HISTORY && pd.nseg == 1) || mode == SWEEP_RECOMPUTE);
+    const bool want_ckpt = !BWD && !PROP && mode == SWEEP_HISTORY && pd.nseg > 1;
     const uint32_t bytes_0 = static_cast<uint32_t>(size_t(ncol0) * N * sizeof(double2));
     const uint32_t bytes_1 = static_cast<uint32_t>(size_t(ncol - ncol0) * N * sizeof(double2));
     auto hist_ptr = [&](int s, int jj) -> double2* {
@@ -772,19 +781,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
             }
             fence_proxy_async_smem();
         }
-        if constexpr (!BWD) {
-            // roll-out: U(t_m) when the step ends on a window boundary t_m, i.e. when n + 1 =
-            // floor(m N_T / M) for some 1 <= m < M; the only candidate is m = ceil((n+1) M / N_T)
-            if (rollout && live && act) {
-                const int64_t n1 = wn0_0 + jj + 1;
-                const int64_t mb = (n1 * pd.M + pd.nsteps - 1) / pd.nsteps;
-                if (mb >= 1 && mb < pd.M && (mb * pd.nsteps) / pd.M == n1) {
-                    double2* dst = a.out + (size_t(mb - 1) * E + col) * N + f * L;
-#pragma unroll
-                    for (int l = 0; l < L; ++l) dst[l] = state_out(l);
-                }
-            }
-        }
         if (++hpos == hd) hpos = 0;
     }
 
@@ -794,13 +790,34 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
         publish_group(((nit - 1) / hd) * hd);
         bulk_wait_all();
     }
-    if (act && my_cnt > 0 && !rollout && a.mode != SWEEP_RECOMPUTE) {
+    if constexpr (PROP) {
+        if (act) {
+            double2* dst = (a.slices ? a.phi : pd.Phi) + wcol + f * L;
+#pragma unroll
+            for (int l = 0; l < L; ++l) dst[l] = state_out(l);
+        }
+    } else if (act && my_cnt > 0 && C == 1 && mode != SWEEP_RECOMPUTE) {
         // forward: U^m(t_m); adjoint: Lambda at the launch's first step (Lambda^m(t_{m-1}) for
         // the window's first)
         double2* dst = !BWD ? pd.Uend : (lo == 0 ? pd.Lam0 : pd.Lstate);
 #pragma unroll
         for (int l = 0; l < L; ++l) dst[wcol + f * L + l] = state_out(l);
     }
+}
+
+template <int L, int Q, int SOLVER, bool BWD, bool PROP = false, int MAXT = MAX_TILE_THREADS>
+__global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
+    sweep_tile<L, Q, SOLVER, BWD, PROP>(a, a.mode, blockIdx.x);
+}
+// The history and adjoint sweeps of sliced problems, which do not depend on each other: blocks
+// 0 .. n - 1 the forward tiles, n .. 2n - 1 the adjoint's.
+template <int L, int Q, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_sweep_both(const SweepArgs a) {
+    const int n = gridDim.x / 2;
+    if (blockIdx.x < n)
+        sweep_tile<L, Q, SOLVER_MIXED, false, false>(a, SWEEP_HISTORY, blockIdx.x);
+    else
+        sweep_tile<L, Q, SOLVER_MIXED, true, false>(a, SWEEP_ADJOINT, blockIdx.x - n);
 }
 
 }  // namespace msqoc

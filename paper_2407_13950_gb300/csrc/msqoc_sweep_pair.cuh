@@ -154,10 +154,9 @@ __device__ __forceinline__ void step_coefficients_pair(const ProbDev& pd, int la
 // the slots' ranges; a thread whose slot has no step at an iteration keeps its state.  A lane
 // pair (parts 0 and 1) works on each (column, fiber) for SPLIT = 1, on each of its entries for
 // SPLIT = 2 (lane quads).
-template <int L, int Q, int SOLVER, bool BWD, bool ROLLOUT = false, int SPLIT = 1>
+template <int L, int Q, int SOLVER, bool BWD, int SPLIT = 1>
 __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_TILE_THREADS, 1)
     k_sweep_pair(const SweepArgs a) {
-    static_assert(!(BWD && ROLLOUT), "the roll-out is a forward sweep");
     static_assert(SPLIT == 1 || (SPLIT == 2 && L == 2), "lane quads are for 2-level subsystems");
     constexpr int LS = L / SPLIT;          // entries of the fiber this thread holds
     constexpr int N = ipow_c(L, Q);
@@ -188,11 +187,10 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     const int nslot = ncol0 < ncol ? 2 : 1;
     const bool segmented = a.mode == SWEEP_RECOMPUTE || a.mode == SWEEP_ADJOINT;
     const bool idle_launch = a.mode == SWEEP_RECOMPUTE && pd.nseg == 1;   // nothing to recompute
-    constexpr bool rollout = ROLLOUT;   // one window over the whole grid (compiled separately)
 
     // ---- the slots' windows and step ranges (local step indices [lo, lo + cnt) of the window)
-    const int64_t wn0_0 = rollout ? 0 : win_start(pd, tile.m0);
-    const int wns_0 = rollout ? static_cast<int>(pd.nsteps) : static_cast<int>(win_start(pd, tile.m0 + 1) - wn0_0);
+    const int64_t wn0_0 = win_start(pd, tile.m0);
+    const int wns_0 = static_cast<int>(win_start(pd, tile.m0 + 1) - wn0_0);
     const int64_t wn0_1 = nslot > 1 ? win_start(pd, tile.m0 + 1) : 0;
     const int wns_1 = nslot > 1 ? static_cast<int>(win_start(pd, tile.m0 + 2) - wn0_1) : 0;
     // (an adjoint launch covers chunk `sub` of its segment)
@@ -525,16 +523,6 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
 #pragma unroll
             for (int l = 0; l < LS; ++l) u[l] = fma(2.0, z[l], -u[l]);
         }
-        if constexpr (!BWD) {
-            // roll-out: U(t_m) when the step ends on a window boundary t_m, i.e. when n + 1 =
-            // floor(m N_T / M) for some 1 <= m < M; the only candidate is m = ceil((n+1) M / N_T)
-            if (rollout && live && act) {
-                const int64_t n1 = wn0_0 + jj + 1;
-                const int64_t mb = (n1 * pd.M + pd.nsteps - 1) / pd.nsteps;
-                if (mb >= 1 && mb < pd.M && (mb * pd.nsteps) / pd.M == n1)
-                    store_fiber(a.out + (size_t(mb - 1) * E + col) * N);
-            }
-        }
         if (++hpos == hd) hpos = 0;
     }
 
@@ -546,7 +534,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     }
     // forward: U^m(t_m); adjoint: Lambda at the launch's first step (Lambda^m(t_{m-1}) for the
     // window's first)
-    if (act && my_cnt > 0 && !rollout && a.mode != SWEEP_RECOMPUTE)
+    if (act && my_cnt > 0 && a.mode != SWEEP_RECOMPUTE)
         store_fiber((!BWD ? pd.Uend : (lo == 0 ? pd.Lam0 : pd.Lstate)) + wcol);
 }
 

@@ -119,6 +119,18 @@ class _CudaDevice:
         self.torch.cuda.synchronize()
 
 
+def session_columns(spec) -> int:
+    """Columns per sweep tile of a served problem (0: the library's choice).  An evaluation that
+    takes milliseconds and does not fill the GPU gets the widest one-window tiles of at most 8
+    warps: it holds a quarter of the SMs that the fastest tiles for it alone would (4 transmons at
+    16 windows: 32 tiles of 8 columns, 4.1 us a step, against 64 of 4 columns, 3.4 us), and the
+    other sessions' launches run beside it."""
+    F = spec.N // spec.L
+    cb = max((c for c in range(1, spec.E + 1) if spec.E % c == 0 and c * F <= 256), default=0)
+    return cb if cb and eval_flops(spec, True) >= 1e9 and spec.M * spec.E // cb < 128 else 0
+
+
+
 class Server:
     """Sessions and the continuous-batching loop.
 
@@ -152,7 +164,13 @@ class Server:
     # ------------------------------------------------------------------ sessions
     def admit(self, spec, ckpt_interval: int = 0, solver: int = msqoc.SOLVER_DEFAULT) -> int:
         """Create a session for `spec` if its device memory fits; returns the session id."""
-        p = msqoc.Problem(spec, ckpt_interval=ckpt_interval, solver=solver)
+        cb = session_columns(spec)
+        try:
+            p = msqoc.Problem(spec, ckpt_interval=ckpt_interval, solver=solver, col_block=cb)
+        except msqoc.MsqocError:
+            if not cb:
+                raise
+            p = msqoc.Problem(spec, ckpt_interval=ckpt_interval, solver=solver)
         if self.used + p.device_bytes > self.budget:
             need = p.device_bytes
             p.close()
