@@ -615,7 +615,7 @@ bool is_shard(const ProbDev& pd) { return pd.M != pd.M_glob; }
 namespace {
 
 void free_problem(msqoc_problem* p) {
-    void* bufs[] = {p->tiles_ro, p->lanemap_ro, p->phi_ro, p->tiles_prop, p->lanemap_prop, p->Phi, p->Ubeg, p->Lend,
+    void* bufs[] = {p->tiles_ro, p->lanemap_ro, p->phi_ro, p->tiles_prop, p->lanemap_prop, p->Phi, p->Ubeg, p->Lend, p->coef,
                     p->pds,   p->tiles, p->lanemap, p->P,     p->emb,   p->V,     p->alpha_dev, p->W_dev,
                     p->ctrl,  p->spl,   p->phase,   p->hist,  p->ckpt,  p->Lstate, p->Uend,     p->Lterm,
                     p->Lam0,  p->term,  p->lhist,   p->quad,  p->status, p->out_dev, p->reg_dev};
@@ -829,6 +829,8 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     A(dalloc(&p->alpha_dev, pd.d), "alpha");
     A(dalloc(&p->W_dev, std::max<size_t>(p->nW, 2)), "W");
     A(dalloc(&p->ctrl, size_t(nsteps) * q), "controls");
+    const size_t ncoef = pd.pair == 0 && pd.solver == SOLVER_MIXED ? size_t(nsteps) * q * (L - 1) : 0;
+    A(dalloc(&p->coef, ncoef), "step coefficients");
     A(dalloc(&p->spl, size_t(nsteps)), "splines");
     A(dalloc(&p->phase, size_t(nsteps) * nfsum), "phases");
     A(dalloc(&p->Uend, M * p->ne), "Uend");
@@ -851,6 +853,7 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
         // a shard past the first window reads its first window's initial state at index -1
         pd.W = reinterpret_cast<const double2*>(p->W_dev) + (pd.m_off >= 1 ? p->ne : 0);
         pd.ctrl = p->ctrl;
+        pd.coef = p->coef;
         pd.spl = p->spl;
         pd.phase = p->phase;
         pd.Uend = p->Uend;
@@ -887,7 +890,7 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
                sizeof(Spline4) * size_t(nsteps) + sizeof(double) * (pd.d + p->nW + M + out_layout(p->npen, pd.d, p->nW).total + reg_doubles(pd)) +
                sizeof(int) * (E + 1 + tabs.maps.size() + tabs_prop.maps.size() + tabs_ro.maps.size()) +
                sizeof(Tile) * (tabs.tiles.size() + tabs_prop.tiles.size() + tabs_ro.tiles.size()) +
-               sizeof(double2) * phi_ro + slice_bytes(pd) + sizeof(ProbDev);
+               sizeof(double2) * phi_ro + sizeof(float4) * ncoef + slice_bytes(pd) + sizeof(ProbDev);
     p->grad_bytes = gradient_bytes(pd);
     *out = owner.release();
     return MSQOC_OK;
@@ -1033,7 +1036,10 @@ SweepArgs prop_args(const SweepPlan& plan, const ProbDev& pd, const ProbDev* pds
 }
 cudaError_t launch_compose(const ProbDev* pds_dev, const int* list, int E, int M, int nprob, int N, bool bwd,
                            cudaStream_t s) {
-    k_compose<<<dim3(E, M, nprob), compose_threads(N), 0, s>>>(pds_dev, list, bwd ? 1 : 0);
+    if (bwd)
+        k_compose<true><<<dim3(E, M, nprob), compose_threads(N), 0, s>>>(pds_dev, list);
+    else
+        k_compose<false><<<dim3(E, M, nprob), compose_threads(N), 0, s>>>(pds_dev, list);
     return cudaGetLastError();
 }
 
@@ -1042,12 +1048,13 @@ int phase_blocks(const ProbDev& pd) {
     return static_cast<int>(std::min<int64_t>((pd.nsteps * pd.nfsum + 255) / 256, 4096));
 }
 
+int control_blocks(const ProbDev& pd) {
+    return static_cast<int>(std::min<int64_t>((pd.nsteps + CTRL_THREADS - 3) / (CTRL_THREADS - 2), 8192));
+}
 msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s) {
     const ProbDev& pd = p->pd;
     Mark mk(p, MSQOC_KERNEL_CONTROLS, s);
-    const int threads = 256;
-    const int blocks = static_cast<int>(std::min<int64_t>((pd.nsteps + threads - 1) / threads, 4096));
-    k_controls<<<blocks, threads, 0, s>>>(pd, pair);
+    k_controls<<<control_blocks(pd), CTRL_THREADS, 0, s>>>(pd, pair);
     CUDA_TRY(cudaGetLastError());
     return MSQOC_OK;
 }
@@ -1574,10 +1581,9 @@ msqoc_status eval_objective_noalloc(const msqoc_hamiltonian* H, const msqoc_cont
     // ---- the objective's kernels (controls, forward sweep, terminal terms, reduction)
     {
         const int threads = 256;
-        const int blocks = static_cast<int>(std::min<int64_t>((pd.nsteps + threads - 1) / threads, 4096));
         k_phases<<<phase_blocks(pd), threads, 0, s>>>(pd);
         CUDA_TRY(cudaGetLastError());
-        k_controls<<<blocks, threads, 0, s>>>(pd, pd.pair);
+        k_controls<<<control_blocks(pd), CTRL_THREADS, 0, s>>>(pd, pd.pair);
         CUDA_TRY(cudaGetLastError());
     }
     CUDA_TRY(launch_sweep(sweep_args(pd, pd_d, tiles_d, map_d, SWEEP_OBJECTIVE, 0), pd.ntiles, s));

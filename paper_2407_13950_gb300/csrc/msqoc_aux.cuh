@@ -3,6 +3,7 @@
 #pragma once
 
 #include "msqoc_internal.h"
+#include "msqoc_split.cuh"
 
 namespace msqoc {
 
@@ -12,9 +13,13 @@ namespace msqoc {
 // passes << 16 | bad << 24 | coarse << 25.
 //   FP64 solver : j1 = K sweeps with rho^(K+1) <= 2^-56.
 //   mixed solver, one thread per fiber: the FP32 estimate m0 of the increment m = z - U leaves the
-//     error e1 = u32 (2 kap + c rho) + rho^(j1+1) relative to |U| (its roundings plus truncation);
+//     error e1 = u32 (2 kap + c rho) + rho^j1 del relative to |U| (its roundings plus truncation).
+//     Its sweeps start from the estimate d of the step before, off by at most
+//     del = 2 rho (kap + rho) + drho with drho = (h/2) lam sum_k |d_k(t) - d_k(t -+ h)| (the change of
+//     the state and of the controls over a step; at most rho); where there is none, FRESH_SWEEPS
+//     more make up for it (rho^(j1+3) <= rho^j1 del holds as rho <= 2^-5 gives del >= 2 rho^2 >= rho^3);
 //     a pass forms the increment at U + m0 in compensated FP32 and solves for the correction in
-//     FP32, whose part that is added to the increment carries the same factor
+//     FP32, whose part that is added to the increment carries the factor
 //     phi = u32 (2 kap + c rho) + rho^(j2+1).  c = 4 rounding units per FP32 sweep output; target:
 //     the FP64 unit roundoff 2^-53.  The fewest passes are taken first (a pass costs far more than
 //     a sweep), then the fewest sweeps j1 + j2 (each is a barrier of the tile), then the smaller j2.
@@ -24,7 +29,7 @@ namespace msqoc {
 //     terms (rms), stays below the FP64 rounding of the state where kap <= 2^-4 and rho <= 2^-5;
 //     other steps are taken in FP64 (j1 = K sweeps as the FP64 solver).
 //   bad: rho >= 1/2, outside the range the counts are derived for.
-__device__ inline int step_counts(int solver, int pair, float rho, float kap) {
+__device__ inline int step_counts(int solver, int pair, float rho, float kap, float drho) {
     int a = 1, b = 1, r = 1, bad = 0;
     const int coarse = solver == SOLVER_MIXED && !pair && (rho > 0.03125f || kap > 0.0625f) ? 1 : 0;
     if (rho > 1e-30f) {
@@ -35,21 +40,22 @@ __device__ inline int step_counts(int solver, int pair, float rho, float kap) {
         } else {
             const float u32 = 5.9604645e-8f, c = 4.f, target = 1.1102230e-16f;
             const float f1 = pair ? c * u32 * rho : u32 * (2.f * kap + c * rho), f2 = pair ? c * u32 : f1;
+            const float del = pair ? rho : fminf(rho, 2.f * rho * (kap + rho) + drho);
             const int j0 = max(1, min(30, int(ceilf(logf(u32) / lr))));   // rho^j0 <= u32
             r = 0;
             for (int pass = 1; pass <= 6 && r == 0; ++pass) {
                 int best = 0;
-                for (int ja = 1; ja <= j0 + 2; ++ja) {
-                    const float e1 = f1 + __powf(rho, float(ja + 1));
-                    for (int jb = 1; jb <= j0 + 1; ++jb) {
-                        const float phi = f2 + __powf(rho, float(jb + 1));
-                        float e = e1;
-                        for (int t = 0; t < pass; ++t) e *= phi;
-                        if (e <= target && (best == 0 || ja + jb < best || (ja + jb == best && jb < b))) {
-                            best = ja + jb;
-                            a = ja;
-                            b = jb;
-                        }
+                float p = rho * del;
+                for (int ja = 1; ja <= j0 + 2; ++ja, p *= rho) {
+                    // the least jb with e1 phi^pass <= target
+                    const float e1 = f1 + p;
+                    const float need = (pass == 1 ? target / e1 : __powf(target / e1, 1.f / float(pass))) - f2;
+                    if (!(need > 0.f)) continue;
+                    const int jb = max(1, int(ceilf(logf(need) / lr + 1e-3f)) - 1);
+                    if (jb <= j0 + 1 && (best == 0 || ja + jb < best || (ja + jb == best && jb < b))) {
+                        best = ja + jb;
+                        a = ja;
+                        b = jb;
                     }
                 }
                 if (best) r = pass;
@@ -83,30 +89,62 @@ __device__ __forceinline__ SplineAt spline_at(const ProbDev& pd, double t) {
 // Controls at every step midpoint t_{n+1/2} = (n + 1/2) h (Eq. dj-ctrl with the quadratic
 // B-spline envelope of Sec. 2): d_k(t) = sum_f e^{i Omega_kf t} sum_s (a1 + i a2)_kfs B_s(t),
 // and the step solver's iteration counts (step_counts).  Also stores the spline weights for the
-// gradient quadrature of the adjoint sweep.  The carrier phases come from the problem's phase
-// table (k_phases).  pair: the kernel family the counts are for.
-__global__ void k_controls(const ProbDev pd, const int pair) {
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; n < pd.nsteps; n += stride) {
-        const double t = (double(n) + 0.5) * pd.h;
-        const SplineAt sp = spline_at(pd, t);
-        double mag = 0.0;   // sum_k |d_k| for the contraction bound
+// gradient quadrature and the mixed solver's split coefficients.  The carrier phases come from the
+// problem's phase table (k_phases).  pair: the kernel family the counts are for.
+__device__ __forceinline__ double2 control_at(const ProbDev& pd, int64_t n, int k, const SplineAt& sp) {
+    double2 dk = make_double2(0.0, 0.0);
+    for (int fi = pd.cof[k]; fi < pd.cof[k + 1]; ++fi) {
+        const double2 ph = pd.phase[size_t(n) * pd.nfsum + fi];
+        const double cs = ph.x, sn = ph.y;
+        const double* a = pd.alpha + (size_t(fi) * pd.d1 + sp.s0) * 2;
+        const double er = a[0] * sp.w0 + a[2] * sp.w1 + a[4] * sp.w2;
+        const double ei = a[1] * sp.w0 + a[3] * sp.w1 + a[5] * sp.w2;
+        dk.x += cs * er - sn * ei;
+        dk.y += cs * ei + sn * er;
+    }
+    return dk;
+}
+constexpr int CTRL_THREADS = 128;
+__global__ void __launch_bounds__(CTRL_THREADS) k_controls(const ProbDev pd, const int pair) {
+    // a block takes CTRL_THREADS - 2 steps and one more on either side (the changes of the controls
+    // over a step, in FP32)
+    __shared__ float2 ds[MAXQ][CTRL_THREADS];
+    const int64_t per = CTRL_THREADS - 2;
+    for (int64_t n0 = int64_t(blockIdx.x) * per; n0 < pd.nsteps; n0 += int64_t(gridDim.x) * per) {
+        const int t = threadIdx.x;
+        const int64_t n = min(max(n0 + t - 1, int64_t(0)), pd.nsteps - 1);
+        const bool own = t >= 1 && t <= per && n0 + t - 1 < pd.nsteps;
+        const SplineAt sp = spline_at(pd, (double(n) + 0.5) * pd.h);
+        float mag = 0.f;   // sum_k |d_k| for the contraction bound
         for (int k = 0; k < pd.q; ++k) {
-            double2 dk = make_double2(0.0, 0.0);
-            for (int fi = pd.cof[k]; fi < pd.cof[k + 1]; ++fi) {
-                const double2 ph = pd.phase[size_t(n) * pd.nfsum + fi];
-                const double cs = ph.x, sn = ph.y;
-                const double* a = pd.alpha + (size_t(fi) * pd.d1 + sp.s0) * 2;
-                const double er = a[0] * sp.w0 + a[2] * sp.w1 + a[4] * sp.w2;
-                const double ei = a[1] * sp.w0 + a[3] * sp.w1 + a[5] * sp.w2;
-                dk.x += cs * er - sn * ei;
-                dk.y += cs * ei + sn * er;
+            const double2 dk = control_at(pd, n, k, sp);
+            const float2 df = make_float2(float(dk.x), float(dk.y));
+            ds[k][t] = df;
+            mag += sqrtf(df.x * df.x + df.y * df.y);
+            if (own) {
+                pd.ctrl[size_t(n) * pd.q + k] = dk;
+                if (pd.coef)
+                    for (int j = 1; j < pd.L; ++j) {
+                        const double s = pd.sc[2 * j + 1];   // (h/2) sqrt(j)
+                        pd.coef[(size_t(n) * pd.q + k) * (pd.L - 1) + j - 1] =
+                            split_scaled(make_double2(s * dk.x, s * dk.y), 0);
+                    }
             }
-            pd.ctrl[size_t(n) * pd.q + k] = dk;
-            mag += sqrt(dk.x * dk.x + dk.y * dk.y);
         }
-        const float rho = float(0.5 * pd.h * pd.lam * mag + pd.rho_ex) * 1.0001f;
-        pd.spl[n] = Spline4{sp.s0, step_counts(pd.solver, pair, rho, float(pd.kap)), sp.w0, sp.w1, sp.w2};
+        __syncthreads();
+        if (own) {
+            float dm = 0.f, dp = 0.f;
+            for (int k = 0; k < pd.q; ++k) {
+                const float2 b = ds[k][t - 1], c = ds[k][t], e = ds[k][t + 1];
+                dm += sqrtf((c.x - b.x) * (c.x - b.x) + (c.y - b.y) * (c.y - b.y));
+                dp += sqrtf((c.x - e.x) * (c.x - e.x) + (c.y - e.y) * (c.y - e.y));
+            }
+            const float hl = float(0.5 * pd.h * pd.lam);
+            const float rho = (hl * mag + float(pd.rho_ex)) * 1.0001f;
+            const float drho = hl * (fmaxf(dm, dp) + 1e-6f * mag) * 1.0001f;
+            pd.spl[n] = Spline4{sp.s0, step_counts(pd.solver, pair, rho, float(pd.kap), drho), sp.w0, sp.w1, sp.w2};
+        }
+        __syncthreads();
     }
 }
 
@@ -127,19 +165,33 @@ __global__ void k_phases(const ProbDev pd) {
     }
 }
 
-// block-wide sum with a fixed reduction order (deterministic)
-template <int NT>
-__device__ double block_sum(double v, double* sh) {
-    sh[threadIdx.x] = v;
+// block-wide sums of K values with a fixed reduction order (deterministic): lanes by shuffles, then
+// the warps' sums in order; sh: K NT / 32 doubles
+template <int NT, int K>
+__device__ __forceinline__ void block_sums(double (&v)[K], double* sh) {
+    constexpr int NW = NT / 32;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k) sh[(threadIdx.x >> 5) * K + k] = v[k];
     __syncthreads();
 #pragma unroll
-    for (int o = NT / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
+    for (int k = 0; k < K; ++k) {
+        double s = sh[k];
+#pragma unroll
+        for (int w = 1; w < NW; ++w) s += sh[w * K + k];
+        v[k] = s;
     }
-    const double r = sh[0];
     __syncthreads();
-    return r;
+}
+template <int NT>
+__device__ double block_sum(double v, double* sh) {
+    double a[1] = {v};
+    block_sums<NT, 1>(a, sh);
+    return a[0];
 }
 
 // ------------------------------------------------------------------ slices of a window
@@ -152,7 +204,7 @@ __device__ double block_sum(double v, double* sh) {
 // sweeps of n steps.  The products are FP64.
 constexpr int COMPOSE_THREADS = 256;
 // thread t works on row t / JG and the terms congruent to t % JG mod JG of its sum (JG adjacent
-// lanes share a row): short chains, since a chain of FP64 operations costs ~70 cycles each
+// lanes share a row): short chains, since an FP64 instruction takes a warp ~64 cycles
 struct ComposeGeom {
     int R, JG;
 };
@@ -164,85 +216,130 @@ __host__ __device__ inline ComposeGeom compose_geom(int N) {
     JG = JG < 1 ? 1 : (JG > n2 ? n2 : JG);
     return ComposeGeom{R, JG > 32 ? 32 : JG};
 }
-// xs <- Phi xs (BWD: Phi^+ xs) for one propagator; every thread of the block takes part
-template <bool BWD>
-__device__ __forceinline__ void compose_step(const double2* __restrict__ Phi, int N, const ComposeGeom& ge,
-                                             double2* xs) {
+// The chain of `links` products x <- Phi x (BWD: Phi^+ x) on one column, phi(s) the propagator of
+// link s, visit(s, x) called with the state before link s (and with s = links at the end).  xs: two
+// buffers of N entries, the state in the first.  Every thread of the block takes part; one barrier
+// a link.  A link waits for nothing but its FP64 operations: where a thread has at most PRE terms
+// (N <= 32) it loads the next link's while it does this one's (QFT-8: 1.17 us a link without).
+template <bool BWD, class Phi, class Visit>
+__device__ __forceinline__ void compose_chain(int N, int links, double2* xs, Phi phi, Visit visit) {
+    constexpr int PRE = 4;
+    const ComposeGeom ge = compose_geom(N);
     const int i = threadIdx.x / ge.JG, g = threadIdx.x % ge.JG;
-    double2 y0 = make_double2(0.0, 0.0), y1 = y0;
-    if (i < N) {
-        // the terms in two running sums (shorter chains)
-        const double2* p = BWD ? Phi + size_t(i) * N : Phi + i;
-        const int st = BWD ? 1 : N;
-        int j = g;
+    const int st = BWD ? 1 : N;
+    const size_t off = BWD ? size_t(i) * N : size_t(i);
+    const bool pre = N <= PRE * ge.JG;
+    double2 nx[PRE];
+    auto fetch = [&](int s) {
+#pragma unroll
+        for (int u = 0; u < PRE; ++u) {
+            const int j = g + u * ge.JG;
+            nx[u] = i < N && j < N ? phi(s)[off + size_t(j) * st] : make_double2(0.0, 0.0);
+        }
+    };
+    if (pre && links > 0) fetch(0);
+    for (int s = 0; s < links; ++s) {
+        const double2* x = xs + (s & 1 ? N : 0);
+        double2* xn = xs + (s & 1 ? 0 : N);
+        visit(s, x);
+        double2 y = make_double2(0.0, 0.0);
+        if (pre) {
+            double2 c[PRE];
+#pragma unroll
+            for (int u = 0; u < PRE; ++u) c[u] = nx[u];
+            if (s + 1 < links) fetch(s + 1);
+#pragma unroll
+            for (int u = 0; u < PRE; ++u) {
+                const int j = g + u * ge.JG;
+                if (u * ge.JG >= N) break;   // uniform
+                const double2 z = x[j < N ? j : 0];
+                const double ci = BWD ? -c[u].y : c[u].y;
+                y.x = fma(c[u].x, z.x, fma(-ci, z.y, y.x));
+                y.y = fma(c[u].x, z.y, fma(ci, z.x, y.y));
+            }
+        } else if (i < N) {
+            // two running sums (shorter chains)
+            const double2* p = phi(s) + off;
+            double2 w = make_double2(0.0, 0.0);
+            int j = g;
 #pragma unroll 4
-        for (; j + ge.JG < N; j += 2 * ge.JG) {
-            const double2 a = p[size_t(j) * st], b = p[size_t(j + ge.JG) * st];
-            const double2 x = xs[j], z = xs[j + ge.JG];
-            const double ai = BWD ? -a.y : a.y, bi = BWD ? -b.y : b.y;
-            y0.x = fma(a.x, x.x, fma(-ai, x.y, y0.x));
-            y0.y = fma(a.x, x.y, fma(ai, x.x, y0.y));
-            y1.x = fma(b.x, z.x, fma(-bi, z.y, y1.x));
-            y1.y = fma(b.x, z.y, fma(bi, z.x, y1.y));
+            for (; j + ge.JG < N; j += 2 * ge.JG) {
+                const double2 a = p[size_t(j) * st], b = p[size_t(j + ge.JG) * st];
+                const double2 z = x[j], z2 = x[j + ge.JG];
+                const double ai = BWD ? -a.y : a.y, bi = BWD ? -b.y : b.y;
+                y.x = fma(a.x, z.x, fma(-ai, z.y, y.x));
+                y.y = fma(a.x, z.y, fma(ai, z.x, y.y));
+                w.x = fma(b.x, z2.x, fma(-bi, z2.y, w.x));
+                w.y = fma(b.x, z2.y, fma(bi, z2.x, w.y));
+            }
+            if (j < N) {
+                const double2 a = p[size_t(j) * st], z = x[j];
+                const double ai = BWD ? -a.y : a.y;
+                y.x = fma(a.x, z.x, fma(-ai, z.y, y.x));
+                y.y = fma(a.x, z.y, fma(ai, z.x, y.y));
+            }
+            y.x += w.x;
+            y.y += w.y;
         }
-        if (j < N) {
-            const double2 a = p[size_t(j) * st], x = xs[j];
-            const double ai = BWD ? -a.y : a.y;
-            y0.x = fma(a.x, x.x, fma(-ai, x.y, y0.x));
-            y0.y = fma(a.x, x.y, fma(ai, x.x, y0.y));
+        // the row's lanes: the first exchange leaves the real part in one half, the imaginary part
+        // in the other
+        if (ge.JG > 1) {
+            int o = ge.JG >> 1;
+            const bool up = g & o;
+            double v = (up ? y.y : y.x) + __shfl_xor_sync(0xffffffffu, up ? y.x : y.y, o);
+            for (o >>= 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (i < N && (g & ((ge.JG >> 1) - 1)) == 0) reinterpret_cast<double*>(xn + i)[up ? 1 : 0] = v;
+        } else if (i < N) {
+            xn[i] = y;
         }
+        __syncthreads();
     }
-    double yr = y0.x + y1.x, yi = y0.y + y1.y;
-    for (int o = ge.JG >> 1; o > 0; o >>= 1) {
-        yr += __shfl_xor_sync(0xffffffffu, yr, o);
-        yi += __shfl_xor_sync(0xffffffffu, yi, o);
-    }
-    __syncthreads();   // xs has been read
-    if (i < N && g == 0) xs[i] = make_double2(yr, yi);
-    __syncthreads();
+    visit(links, xs + (links & 1 ? N : 0));
 }
 // One block per (column, window, problem).  Forward: Ubeg of every slice from W^{m-1} (identity
 // embedding for the whole problem's first window) and U^m(t_m); backward: Lend of every slice from
 // Lambda^m(t_m) and Lambda^m(t_{m-1}).
-__global__ void __launch_bounds__(COMPOSE_THREADS) k_compose(const ProbDev* pds, const int* list, const int bwd) {
-    __shared__ double2 xs[256];
+template <bool BWD>
+__global__ void __launch_bounds__(COMPOSE_THREADS) k_compose(const ProbDev* pds, const int* list) {
+    __shared__ double2 xs[2 * 256];
     const ProbDev& pd = pds[list ? list[blockIdx.z] : blockIdx.z];
     const int col = blockIdx.x, m = blockIdx.y, N = pd.N, E = pd.E, C = pd.C;
     if (C == 1 || m >= pd.M || col >= E) return;
-    const ComposeGeom ge = compose_geom(N);
     const size_t wcol = (size_t(m) * E + col) * N;
     for (int i = threadIdx.x; i < N; i += blockDim.x)
-        xs[i] = bwd ? pd.Lterm[wcol + i]
+        xs[i] = BWD ? pd.Lterm[wcol + i]
                     : (m + pd.m_off == 0 ? make_double2(pd.emb[col] == i ? 1.0 : 0.0, 0.0)
                                          : pd.W[(size_t(m) - 1) * E * N + size_t(col) * N + i]);
     __syncthreads();
-    for (int s = 0; s < C; ++s) {
-        const size_t v = size_t(m) * C + (bwd ? C - 1 - s : s);
-        double2* keep = (bwd ? pd.Lend : pd.Ubeg) + (v * E + col) * N;
-        for (int i = threadIdx.x; i < N; i += blockDim.x) keep[i] = xs[i];
-        const double2* Phi = pd.Phi + v * N * N;
-        if (bwd)
-            compose_step<true>(Phi, N, ge, xs);
-        else
-            compose_step<false>(Phi, N, ge, xs);
-    }
-    for (int i = threadIdx.x; i < N; i += blockDim.x) (bwd ? pd.Lam0 : pd.Uend)[wcol + i] = xs[i];
+    const double2* Phi = pd.Phi;
+    double2* keep = BWD ? pd.Lend : pd.Ubeg;
+    double2* end = BWD ? pd.Lam0 : pd.Uend;
+    auto slice = [&](int s) { return size_t(m) * C + (BWD ? C - 1 - s : s); };
+    compose_chain<BWD>(
+        N, C, xs, [&](int s) { return Phi + slice(s) * N * N; },
+        [&](int s, const double2* x) {
+            double2* dst = s < C ? keep + (slice(s) * E + col) * N : end + wcol;
+            for (int i = threadIdx.x; i < N; i += blockDim.x) dst[i] = x[i];
+        });
 }
 // The roll-out's chain over the propagators of windows w0 .. w0 + nw - 1 (C a window), one block a
 // column: from the identity embedding (w0 = 0) or the state W^{w0} an earlier launch stored, the
 // states W^{w+1} at the windows' ends (but the last window's).
 __global__ void __launch_bounds__(COMPOSE_THREADS) k_compose_rollout(const ProbDev pd, const double2* Phi, int C, int w0,
                                                                      int nw, double2* W) {
-    __shared__ double2 xs[256];
+    __shared__ double2 xs[2 * 256];
     const int col = blockIdx.x, N = pd.N, E = pd.E;
-    const ComposeGeom ge = compose_geom(N);
     for (int i = threadIdx.x; i < N; i += blockDim.x)
         xs[i] = w0 == 0 ? make_double2(pd.emb[col] == i ? 1.0 : 0.0, 0.0) : W[(size_t(w0 - 1) * E + col) * N + i];
     __syncthreads();
-    for (int w = 0; w < nw && w0 + w < pd.M - 1; ++w) {
-        for (int s = 0; s < C; ++s) compose_step<false>(Phi + (size_t(w) * C + s) * N * N, N, ge, xs);
-        for (int i = threadIdx.x; i < N; i += blockDim.x) W[(size_t(w0 + w) * E + col) * N + i] = xs[i];
-    }
+    const int links = min(nw, pd.M - 1 - w0) * C;
+    compose_chain<false>(
+        N, links, xs, [&](int s) { return Phi + size_t(s) * N * N; },
+        [&](int s, const double2* x) {
+            if (s == 0 || s % C) return;
+            double2* dst = W + (size_t(w0 + s / C - 1) * E + col) * N;
+            for (int i = threadIdx.x; i < N; i += blockDim.x) dst[i] = x[i];
+        });
 }
 
 constexpr int TERM_THREADS = 256;
@@ -276,9 +373,9 @@ __global__ void __launch_bounds__(TERM_THREADS) k_terminal(const ProbDev pd, con
             gi = fma(v.x, u.y, fma(-v.y, u.x, gi));
             nr = fma(u.x, u.x, fma(u.y, u.y, nr));
         }
-        gr = block_sum<TERM_THREADS>(gr, sh);
-        gi = block_sum<TERM_THREADS>(gi, sh);
-        nr = block_sum<TERM_THREADS>(nr, sh);
+        double t[3] = {gr, gi, nr};
+        block_sums<TERM_THREADS, 3>(t, sh);
+        gr = t[0], gi = t[1], nr = t[2];
         const double E = pd.E;
         if (threadIdx.x == 0) pd.term[m - 1] = nr / E - (gr * gr + gi * gi) / (E * E);
         if (want_lambda) {
@@ -372,12 +469,12 @@ __global__ void __launch_bounds__(OUT_THREADS) k_gradient_outputs(const ProbDev 
             g1 = fma(w, fma(ph.x, ab.x, ph.y * ab.y), g1);
             g2 = fma(w, fma(ph.x, ab.y, -ph.y * ab.x), g2);
         }
-        g1 = block_sum<OUT_THREADS>(g1, sh);
-        g2 = block_sum<OUT_THREADS>(g2, sh);
+        double g[2] = {g1, g2};
+        block_sums<OUT_THREADS, 2>(g, sh);
         if (threadIdx.x == 0) {
             const size_t i = (size_t(fi) * pd.d1 + s) * 2;
-            ga[i] = -2.0 * pd.h * g1;
-            ga[i + 1] = -2.0 * pd.h * g2;
+            ga[i] = -2.0 * pd.h * g[0];
+            ga[i + 1] = -2.0 * pd.h * g[1];
         }
         return;
     }

@@ -46,6 +46,7 @@ struct msqoc_problem {
     double* alpha_dev = nullptr;   // the evaluation's inputs (copied from the caller's arrays)
     double* W_dev = nullptr;
     double2* ctrl = nullptr;
+    float4* coef = nullptr;
     msqoc::Spline4* spl = nullptr;
     double2* phase = nullptr;
     double2* hist = nullptr;       // allocated by the first gradient evaluation

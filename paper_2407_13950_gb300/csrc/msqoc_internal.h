@@ -95,6 +95,8 @@ struct ProbDev {
                                  // first window's initial state at index -1)
     // scratch
     double2* ctrl;               // [nsteps][q] d_k(t_{n+1/2})
+    float4* coef;                // [nsteps][q][L-1] (h/2) sqrt(j) d_k split into two floats (hi.x, hi.y,
+                                 // lo.x, lo.y), j = 1 .. L-1; nullptr: the sweeps form it from ctrl
     Spline4* spl;                // [nsteps] (first spline index, solver counts, w0, w1, w2)
     double2* phase;              // [nsteps][nfsum] exp(i Omega t_{n+1/2})
     // sliced problems (C > 1): slice i of window m is virtual window m C + i (0-based) and every per-

@@ -96,11 +96,15 @@ __device__ __forceinline__ void apply_off(const T2* __restrict__ buf, const T2* 
         w[l].x = 0;
         w[l].y = 0;
     }
+    // (the a_k^+ coefficient of a pair of levels is the a_k one with its real part negated)
     constexpr int kl = Q - 1;
 #pragma unroll
-    for (int l = 0; l < L; ++l) {
-        if (l < L - 1) cmac(w[l], cf[(kl * L + l) * 2 + 0], xr[l + 1]);
-        if (l > 0) cmac(w[l], cf[(kl * L + l) * 2 + 1], xr[l - 1]);
+    for (int l = 0; l < L - 1; ++l) {
+        const T2 c = cf[(kl * L + l) * 2 + 0];
+        T2 cm = c;
+        cm.x = -c.x;
+        cmac(w[l], c, xr[l + 1]);
+        cmac(w[l + 1], cm, xr[l]);
     }
 #pragma unroll
     for (int k = 0; k < Fiber<L, Q>::NFIX; ++k) {
@@ -108,7 +112,7 @@ __device__ __forceinline__ void apply_off(const T2* __restrict__ buf, const T2* 
         const T2* p1 = buf + fb.nb1[k];
 #pragma unroll
         for (int l = 0; l < L; ++l) cmac(w[l], c1, p1[l]);
-        if (fb.two[k]) {
+        if (L > 2 && fb.two[k]) {
             const T2 c2 = cf[fb.sl2[k]];
             const T2* p2 = buf + fb.nb2[k];
 #pragma unroll
@@ -119,6 +123,7 @@ __device__ __forceinline__ void apply_off(const T2* __restrict__ buf, const T2* 
     // w += i (h/2) J x_src
     if constexpr (L == 2 && Q >= 2) {
         using R = typename cx<T2>::T;
+#pragma unroll 1
         for (int e = 0; e < ex.n; ++e) {                       // uniform
             R c;
             if constexpr (sizeof(R) == 4)
@@ -138,28 +143,48 @@ __device__ __forceinline__ void apply_off(const T2* __restrict__ buf, const T2* 
 
 
 // ------------------------------------------------------------------ per-step coefficients
-// Warp 0: slot (k, l, dir) -> i (h/2) sqrt(l+1) d_k (dir 0, a_k) or i (h/2) sqrt(l) conj(d_k)
-// (dir 1, a_k^+); lane k' < NSLOT holds d_k of its slot's subsystem.  The coefficients go out
-// in FP64 (FP64 solver) or in FP32 and split into two floats (mixed solver).  The iteration counts
-// of the step (packed by step_counts in the controls kernel) are unpacked into prm; prm[3] holds
-// the solver-range flag (bit 0) and the coarse-step flag (bit 1).
+// Slot (k, l, dir) -> i (h/2) sqrt(l+1) d_k (dir 0, a_k) or i (h/2) sqrt(l) conj(d_k) (dir 1,
+// a_k^+), one lane a slot.  What a lane loads for its slot ahead of the step: d_k, or from the mixed
+// solver's table the split (h/2) sqrt(j) d_k (ProbDev::coef), as the same 16 bytes.
+template <int L, int Q>
+__device__ __forceinline__ float4 load_coefficient(const ProbDev& pd, int lane, int64_t n) {
+    constexpr int NSLOT = Q * L * 2;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < NSLOT) {
+        const int k = lane / (2 * L), l = (lane >> 1) % L, j = (lane & 1) ? l : l + 1;
+        if (pd.coef == nullptr)
+            v = *reinterpret_cast<const float4*>(pd.ctrl + size_t(n) * pd.q + k);
+        else if (j >= 1 && j < L)
+            v = pd.coef[(size_t(n) * pd.q + k) * (L - 1) + j - 1];
+    }
+    return v;
+}
+// The coefficients go out in FP64 (FP64 solver) or in FP32 and split into two floats (mixed solver).
+// The iteration counts of the step (packed by step_counts in the controls kernel) are unpacked into
+// prm; prm[3] holds the solver-range flag (bit 0) and the coarse-step flag (bit 1).
 template <int L, int Q, int SOLVER>
-__device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, double2 dk, int cnt, double2* cfd,
+__device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, const float4& in, int cnt, double2* cfd,
                                                   float2* cff, float4* cfs, int* prm) {
     constexpr int NSLOT = Q * L * 2;
     if (lane < NSLOT) {
         const int dir = lane & 1;
         const int l = (lane >> 1) % L;
         const bool valid = dir == 0 ? (l < L - 1) : (l > 0);
-        const double s = pd.sc[2 * l + dir];
-        double2 v = make_double2(0.0, 0.0);
-        if (valid) v = dir == 0 ? make_double2(-s * dk.y, s * dk.x) : make_double2(s * dk.y, s * dk.x);
-        if constexpr (SOLVER == SOLVER_FP64) {
-            cfd[lane] = v;
-        } else {
-            const float4 sp = split_scaled(v, 0);
+        if (SOLVER == SOLVER_MIXED && pd.coef != nullptr) {
+            const float4 sp = dir == 0 ? make_float4(-in.y, in.x, -in.w, in.z) : make_float4(in.y, in.x, in.w, in.z);
             cff[lane] = make_float2(sp.x, sp.y);
             cfs[lane] = sp;
+        } else {
+            const double2 dk = *reinterpret_cast<const double2*>(&in);
+            const double s = valid ? pd.sc[2 * l + dir] : 0.0;
+            const double2 v = dir == 0 ? make_double2(-s * dk.y, s * dk.x) : make_double2(s * dk.y, s * dk.x);
+            if constexpr (SOLVER == SOLVER_FP64) {
+                cfd[lane] = v;
+            } else {
+                const float4 sp = split_scaled(v, 0);
+                cff[lane] = make_float2(sp.x, sp.y);
+                cfs[lane] = sp;
+            }
         }
     }
     if (lane == 0) {
@@ -187,14 +212,13 @@ __device__ __forceinline__ void apply_off_df(const float4* __restrict__ buf, con
     // the first term of each entry's sum initialises it (no two-sum with zero)
     constexpr int kl = Q - 1;
 #pragma unroll
-    for (int l = 0; l < L; ++l) {
-        if (l < L - 1) cmul_df(xr[l + 1], cf[(kl * L + l) * 2 + 0], w[l][0], w[l][1]);
-        if (l > 0) {
-            if (l < L - 1)
-                cmac_df(w[l], cf[(kl * L + l) * 2 + 1], xr[l - 1]);
-            else
-                cmul_df(xr[l - 1], cf[(kl * L + l) * 2 + 1], w[l][0], w[l][1]);
-        }
+    for (int l = 0; l < L - 1; ++l) {
+        const float4 c = cf[(kl * L + l) * 2 + 0], cm = make_float4(-c.x, c.y, -c.z, c.w);
+        if (l == 0)
+            cmul_df(xr[l + 1], c, w[l][0], w[l][1]);
+        else
+            cmac_df(w[l], c, xr[l + 1]);
+        cmul_df(xr[l], cm, w[l + 1][0], w[l + 1][1]);
     }
 #pragma unroll
     for (int k = 0; k < Fiber<L, Q>::NFIX; ++k) {
@@ -202,7 +226,7 @@ __device__ __forceinline__ void apply_off_df(const float4* __restrict__ buf, con
         const float4* p1 = buf + fb.nb1[k];
 #pragma unroll
         for (int l = 0; l < L; ++l) cmac_df(w[l], c1, p1[l]);
-        if (fb.two[k]) {
+        if (L > 2 && fb.two[k]) {
             const float4 c2 = cf[fb.sl2[k]];
             const float4* p2 = buf + fb.nb2[k];
 #pragma unroll
@@ -210,6 +234,7 @@ __device__ __forceinline__ void apply_off_df(const float4* __restrict__ buf, con
         }
     }
     if constexpr (L == 2 && Q >= 2) {
+#pragma unroll 1
         for (int e = 0; e < ex.n; ++e) {   // uniform
             const float2 c = ex.cs[e];
             const int mask = ex.mask[e];
@@ -310,6 +335,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     double2* D1 = reinterpret_cast<double2*>(smem + lay.D1);
     float2* FA = reinterpret_cast<float2*>(smem + lay.FA);
     float2* FB = reinterpret_cast<float2*>(smem + lay.FB);
+    float2* DP = reinterpret_cast<float2*>(smem + lay.DP);
     double2* H = reinterpret_cast<double2*>(smem + lay.H);
 
     const int tid = threadIdx.x;
@@ -489,13 +515,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     // the slot's next step in registers (lane -> subsystem of its slot)
     const bool coef_warp = warp < nslot;
     const int cslot = coef_warp ? warp : 0;
-    const int my_k = (lane < NSLOT) ? (lane / (2 * L)) : 0;
-    double2 dk_next = make_double2(0.0, 0.0);
+    float4 cf_next = make_float4(0.f, 0.f, 0.f, 0.f);
     int cnt_next = 0;
     auto load_ctrl = [&](int jj) {
         if (coef_warp) {
             const int64_t n = step_of(cslot, jj);
-            dk_next = lane < NSLOT ? pd.ctrl[size_t(n) * pd.q + my_k] : make_double2(0.0, 0.0);
+            cf_next = load_coefficient<L, Q>(pd, lane, n);
             cnt_next = pd.spl[n].cnt;
         }
     };
@@ -513,11 +538,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     if (nit > 0) load_ctrl(0);
 
     int hpos = 0;   // position of iteration jj in its history group
+    bool fresh = true;   // no d of the step before: the first sweep starts from zero
     for (int jj = 0; jj < nit; ++jj) {
         const int par = jj & 1;
         const bool live = jj < my_cnt;
         if (coef_warp) {
-            const double2 dk = dk_next;
+            const float4 dk = cf_next;
             const int cnt = cnt_next;
             if (jj + 1 < nit) load_ctrl(jj + 1);
             step_coefficients<L, Q, SOLVER>(pd, lane, dk, cnt, coef_d + (par * 2 + cslot) * NSLOT,
@@ -527,6 +553,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
         // checkpoint: the state at the start of every segment (forward over whole windows)
         // (the state is rounded to what is stored, so that a segment recomputed from its checkpoint
         // repeats these steps bit for bit)
+        if (want_ckpt && jj % pd.kseg == 0) fresh = true;
         if (want_ckpt && live && jj % pd.kseg == 0) {
             double2* ck = pd.ckpt + ((size_t(m - 1) * pd.nseg + jj / pd.kseg) * E + col) * N + f * L;
 #pragma unroll
@@ -600,15 +627,18 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             // estimate m0 gives z = U + m0 exactly (two floats), the right-hand side at that z is
             // formed once in compensated FP32 (m1), and the correction delta = z* - z solves
             // (I + i kappa - s w) delta = R = m1 - m0, small (the FP32 rounding of m0 and what its
-            // sweeps left) and therefore FP32: m = m1 + (delta - R).  The state and every
+            // sweeps left) and therefore FP32: m = m1 + (delta - R).  The sweeps of the estimate
+            // start from the step before's: one sweep a step fewer.  The state and every
             // increment's leading part are never rounded; see step_counts for the counts.
             float2 m0[L], d[L], y[L];
 #pragma unroll
             for (int l = 0; l < L; ++l) {
-                // G u0 and, as the first sweep's point, P u0 = u0 + G u0
+                // G u0, and the first sweep's point P u0 + d = u0 + G u0 + d from the d of the step
+                // before
                 m0[l] = make_float2(fmaf(Gf[l].x, v[l][0].a, -Gf[l].y * v[l][1].a),
                                     fmaf(Gf[l].x, v[l][1].a, Gf[l].y * v[l][0].a));
-                y[l] = make_float2(v[l][0].a + m0[l].x, v[l][1].a + m0[l].y);
+                d[l] = fresh ? make_float2(0.f, 0.f) : DP[fb.xo + l];
+                y[l] = make_float2((v[l][0].a + m0[l].x) + d[l].x, (v[l][1].a + m0[l].y) + d[l].y);
             }
             // s P w for P = 1 + G
             auto precond = [&](int l, const float2& w) {
@@ -630,10 +660,11 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             // coarse steps (uniform over a slot) go to FP64 below
             const bool coarse0 = prm0[3] & 2, coarse1 = nslot > 1 ? (prm1[3] & 2) != 0 : coarse0;
             if (!coarse0 || !coarse1) {
-                const int j1 = prm[0], j2 = prm[1], R = prm[2];
+                const int more = fresh ? FRESH_SWEEPS : 0;
+                const int j1 = prm[0] + more, j2 = prm[1], R = prm[2];
                 const bool two = nslot > 1 && !coarse0 && !coarse1;
                 const int* pm = coarse0 ? prm1 : prm0;
-                const int j1max = two ? max(prm0[0], prm1[0]) : pm[0];
+                const int j1max = (two ? max(prm0[0], prm1[0]) : pm[0]) + more;
                 const int j2max = two ? max(prm0[1], prm1[1]) : pm[1];
                 const int Rmax = two ? max(prm0[2], prm1[2]) : pm[2];
                 for (int it = 0;;) {
@@ -653,6 +684,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                 DF mr[L], mi[L];   // the current z - U
 #pragma unroll
                 for (int l = 0; l < L; ++l) {
+                    if (act) DP[fb.xo + l] = d[l];
                     mr[l] = DF{m0[l].x + d[l].x, 0.f};
                     mi[l] = DF{m0[l].y + d[l].y, 0.f};
                     const DF zr = two_sum(v[l][0].a, mr[l].s), zi = two_sum(v[l][1].a, mi[l].s);
@@ -669,7 +701,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                     // barrier-free
                     if (want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
                     tile_sync();
-                    float2 r[L], pr[L], e[L];
+                    float2 r[L], gr[L], e[L];
                     {
                         DF w[L][2];
                         apply_off_df<L, Q>(D0s, cfs, fb, zf, w, ex_s);
@@ -686,12 +718,17 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                                 mr[l] = kr;
                                 mi[l] = ki;
                             }
-                            // P R, the first sweep's point
-                            pr[l] = make_float2(fmaf(Gf[l].x, r[l].x, fmaf(-Gf[l].y, r[l].y, r[l].x)),
-                                                fmaf(Gf[l].x, r[l].y, fmaf(Gf[l].y, r[l].x, r[l].y)));
-                            e[l] = pr[l];
+                            // G R, and the first sweep's point P R = R + G R
+                            gr[l] = make_float2(fmaf(Gf[l].x, r[l].x, -Gf[l].y * r[l].y),
+                                                fmaf(Gf[l].x, r[l].y, Gf[l].y * r[l].x));
+                            e[l] = make_float2(r[l].x + gr[l].x, r[l].y + gr[l].y);
                         }
                     }
+                    // delta = R + g, g = G R + s P w(delta) (e: delta; g is added to the increment, so
+                    // it is kept apart from R, whose size would round it)
+                    float2 g[L];
+#pragma unroll
+                    for (int l = 0; l < L; ++l) g[l] = gr[l];
                     for (int it = 0; it < j2max; ++it) {
                         float2* Fe = exchange(e);
                         float2 w[L];
@@ -700,15 +737,17 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
 #pragma unroll
                             for (int l = 0; l < L; ++l) {
                                 const float2 t = precond(l, w[l]);
-                                e[l] = make_float2(pr[l].x + t.x, pr[l].y + t.y);
+                                g[l] = make_float2(gr[l].x + t.x, gr[l].y + t.y);
+                                e[l] = make_float2(r[l].x + g[l].x, r[l].y + g[l].y);
                             }
                         }
                     }
                     if (pass < R) {
 #pragma unroll
                         for (int l = 0; l < L; ++l) {
-                            mr[l].c = fadd_n(mr[l].c, fsub_n(e[l].x, r[l].x));
-                            mi[l].c = fadd_n(mi[l].c, fsub_n(e[l].y, r[l].y));
+                            mr[l].c = fadd_n(mr[l].c, g[l].x);
+                            mi[l].c = fadd_n(mi[l].c, g[l].y);
+                            if (!want_hist && Rmax == 1) continue;   // z is needed no more
                             const DF zr = two_sum(zf[l].x, e[l].x), zi = two_sum(zf[l].y, e[l].y);
                             zf[l] = make_float4(zr.s, zi.s, fadd_n(zf[l].z, zr.c), fadd_n(zf[l].w, zi.c));
                         }
@@ -728,6 +767,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             } else if (want_hist && tid == 0 && hpos == 0) {
                 bulk_wait_read_all();   // (the coarse step's barriers follow)
             }
+            fresh = coarse0 || coarse1;
             if (coarse0 || coarse1) {
                 const bool mine = prm[3] & 2;
                 const int Kmax = max(coarse0 ? prm0[0] : 0, coarse1 ? (nslot > 1 ? prm1[0] : prm0[0]) : 0);

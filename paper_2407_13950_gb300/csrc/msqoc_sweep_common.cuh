@@ -103,6 +103,8 @@ __device__ __forceinline__ int column_shift(int ce) {
     const int sh = ce - 1018;
     return sh > SCALE_SHIFT_MAX ? SCALE_SHIFT_MAX : (sh < -SCALE_SHIFT_MAX ? -SCALE_SHIFT_MAX : sh);
 }
+// sweeps a step adds where it has no estimate of the step before to start from (step_counts)
+constexpr int FRESH_SWEEPS = 2;
 // tile columns at most (E = 2^q for 2-level shapes, q <= MAXQ)
 constexpr int MAX_TILE_COLS = 1 << MAXQ;
 
@@ -252,7 +254,7 @@ struct Fiber {
 // keep each coefficient in the form of either part, so their coefficient arrays are twice as
 // large.
 struct SweepSmem {
-    size_t coef_d, coef_f, coef_s, params, D0, D1, FA, FB, H, total;
+    size_t coef_d, coef_f, coef_s, params, D0, D1, FA, FB, DP, H, total;
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -275,6 +277,8 @@ __host__ __device__ inline SweepSmem sweep_layout(int q, int L, int N, int cpt, 
     s.D1 = o;     o = align16(o + (solver == SOLVER_FP64 ? buf_d : 0));
     s.FA = o;     o = align16(o + (solver == SOLVER_MIXED ? buf_f : 0));
     s.FB = o;     o = align16(o + (solver == SOLVER_MIXED ? buf_f : 0));
+    // the mixed solver's one-thread families: the step before's FP32 estimate
+    s.DP = o;     o = align16(o + (!pair && solver == SOLVER_MIXED ? size_t(cpt) * N * 8 : 0));
     s.H = o;      o = align16(o + size_t(hdepth) * cpt * N * 16);   // history staging: hdepth blocks of cpt N states
     s.total = o;
     return s;

@@ -119,16 +119,17 @@ class _CudaDevice:
         self.torch.cuda.synchronize()
 
 
-def session_columns(spec) -> int:
-    """Columns per sweep tile of a served problem (0: the library's choice).  An evaluation that
-    takes milliseconds and does not fill the GPU gets the widest one-window tiles of at most 8
-    warps: it holds a quarter of the SMs that the fastest tiles for it alone would (4 transmons at
-    16 windows: 32 tiles of 8 columns, 4.1 us a step, against 64 of 4 columns, 3.4 us), and the
-    other sessions' launches run beside it."""
+def session_tiles(spec) -> dict:
+    """Tile options of a served problem ({}: the library's choice, the fastest for an evaluation
+    alone).  An evaluation that takes milliseconds and does not fill the GPU gets the tiles with
+    the most columns per SM and time instead, so that the other sessions' launches run beside it:
+    4 transmons at 16 windows take 19 tiles of 14 columns at 6.0 us a step (2.3 columns a
+    microsecond and SM) against 64 tiles of 4 columns at 3.4 us (1.2)."""
     F = spec.N // spec.L
-    cb = max((c for c in range(1, spec.E + 1) if spec.E % c == 0 and c * F <= 256), default=0)
-    return cb if cb and eval_flops(spec, True) >= 1e9 and spec.M * spec.E // cb < 128 else 0
-
+    cb = min(spec.E, 384 // F)
+    if eval_flops(spec, True) < 1e9 or spec.M * spec.E >= 128 * cb:
+        return {}
+    return {"col_block": cb, "layout": msqoc.LAYOUT_FIBER_LEAN}
 
 
 class Server:
@@ -164,13 +165,13 @@ class Server:
     # ------------------------------------------------------------------ sessions
     def admit(self, spec, ckpt_interval: int = 0, solver: int = msqoc.SOLVER_DEFAULT) -> int:
         """Create a session for `spec` if its device memory fits; returns the session id."""
-        cb = session_columns(spec)
+        tiles = session_tiles(spec)
         try:
-            p = msqoc.Problem(spec, ckpt_interval=ckpt_interval, solver=solver, col_block=cb)
+            p = msqoc.Problem(spec, ckpt_interval=ckpt_interval, solver=solver, **tiles)
         except msqoc.MsqocError:
-            if not cb:
+            if not tiles:
                 raise
-            p = msqoc.Problem(spec, ckpt_interval=ckpt_interval, solver=solver)
+            p = msqoc.Problem(spec, ckpt_interval=ckpt_interval, solver=solver)   # (not admitted)
         if self.used + p.device_bytes > self.budget:
             need = p.device_bytes
             p.close()
