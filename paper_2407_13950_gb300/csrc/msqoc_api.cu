@@ -257,10 +257,12 @@ bool quad_admitted(const ProbDev& pd) { return pd.L == 2 && pd.nex <= MAXEXF; }
 // Tiles that do not fit at once run in waves of the CTAs an SM holds (the kernels' occupancy at
 // that width).
 // A tile over two windows pays a second coefficient set each step and wider class mixing in its
-// warps: about one more warp's work per step, so its cost is taken (w + 1) / w times that of w
-// warps (measured on the 4-transmon tiles: 6-warp two-window tiles as slow as 7-warp one-window
-// ones, at 64 windows; 8-warp two-window tiles in three waves 7% faster than 7-warp one-window
-// tiles in four, at 256 windows, where (w + 1) / w predicts 4%).  Candidates are ranked by
+// warps.  Alone or in pairs on an SM it is charged (w + 1) / w for its w warps (4 transmons at 8
+// windows: 4.44 us a step with 7-column two-window tiles of 6 warps, 3.97 with 8-column one-window
+// tiles of 7); among three or more, which hide it, 1.06 (3 transmons at full load: 12 warps an SM
+// take 0.749 ms for 7-column two-window tiles and 0.71 for 8-column ones).  The lean build's
+// narrower register budget costs 1.08 (4 transmons at 64 windows, 8-column tiles: 0.688 against
+// 0.632 ms).  Candidates are ranked by
 //   1. the makespan: an SM's ceil(tiles / SMs) tiles in waves of `resident`, summed over the
 //      waves;
 //   2. tiles that stay inside one window;
@@ -321,16 +323,17 @@ TileChoice choose_tile_layout(const std::vector<TileCand>& cands, int M, int E, 
         const long waves = (per_sm + t.resident - 1) / t.resident;
         const long last = per_sm - (waves - 1) * t.resident;
         const int cb = (E % t.cpt) ? 1 : 0;
-        const double two = cb ? double(t.warps + 1) / double(t.warps) : 1.0;
+        const double lean = t.lean && !fp64 ? 1.08 : 1.0;
+        auto two = [&](long n) { return !cb ? 1.0 : n >= 3 && !fp64 && !t.pair ? 1.06 : double(t.warps + 1) / t.warps; };
         const bool free_warps = !fp64 && !t.pair && t.warps == 1 && t.cpt >= 2 && t.cpt * F == 32;
         auto wave = [&](long n) {
             const double w = double(n * t.warps);
-            if (fp64 || t.pair) return std::max(w * c_load / 4.0, c_alone);
-            return (w <= 4.0 ? 1.0 : 1.0 + 0.09 * (w - 4.0)) * (free_warps ? 0.85 : 1.0);
+            if (fp64 || t.pair) return two(n) * std::max(w * c_load / 4.0, c_alone);
+            return two(n) * lean * (w <= 4.0 ? 1.0 : 1.0 + 0.09 * (w - 4.0)) * (free_warps ? 0.85 : 1.0);
         };
-        const double ca = two * (double(waves - 1) * wave(t.resident) + wave(last));
+        const double ca = double(waves - 1) * wave(t.resident) + wave(last);
         const double cc = 1.0 - double((1 << t.pair) * t.cpt * F) / (32.0 * t.warps);
-        const bool at_floor = ca <= two * double(waves) * c_alone + 1e-9;
+        const bool at_floor = ca <= two(1) * lean * double(waves) * c_alone + 1e-9;
         const int cw = !at_floor ? 0
                        : fp64    ? ((t.warps == 2 || t.warps == 3) ? 0 : (t.warps == 1 ? 1 : 2))
                                  : -std::min(t.warps, 4);
@@ -1240,7 +1243,7 @@ msqoc_status msqoc_rollout_estimate(msqoc_problem* p, double* est_out, void* str
     const bool dev = is_device_ptr(est_out);
     // a spare slot at the end of the output staging (the other slots hold the last results)
     double* dst = dev ? est_out : p->out_dev + out_layout(p->npen, p->pd.d, p->nW).total - 1;
-    k_rollout_estimate<<<1, 32, 0, s>>>(p->pd, dst);
+    k_rollout_estimate<<<1, OUT_THREADS, 0, s>>>(p->pd, dst);
     CUDA_TRY(cudaGetLastError());
     if (dev) return MSQOC_OK;
     CUDA_TRY(cudaMemcpyAsync(est_out, dst, sizeof(double), cudaMemcpyDeviceToHost, s));

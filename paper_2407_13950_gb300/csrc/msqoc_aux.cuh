@@ -417,11 +417,13 @@ __global__ void __launch_bounds__(OUT_THREADS) k_objective_outputs(const ProbDev
 
 // Roll-out infidelity estimate (Eq. rollout-infid-est) from the last evaluation's window terms:
 //   J + (2 / sqrt(n)) sqrt(J) S + S^2 / n,  S = sum_{m<M} ||C^m||_F,  ||C^m||_F = sqrt(2 pen_m / mu),
-// with n := E (as in the generalized infidelity).  Window order sum (deterministic).
-__global__ void k_rollout_estimate(const ProbDev pd, double* est) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double S = 0.0;
-        for (int m = 1; m < pd.M; ++m) S += sqrt(2.0 * pd.term[m - 1] / pd.mu);
+// with n := E (as in the generalized infidelity).  One block, fixed order (deterministic).
+__global__ void __launch_bounds__(OUT_THREADS) k_rollout_estimate(const ProbDev pd, double* est) {
+    __shared__ double sh[OUT_THREADS];
+    double S = 0.0;
+    for (int m = 1 + threadIdx.x; m < pd.M; m += OUT_THREADS) S += sqrt(2.0 * pd.term[m - 1] / pd.mu);
+    S = block_sum<OUT_THREADS>(S, sh);
+    if (threadIdx.x == 0) {
         const double J = pd.term[pd.M - 1];
         const double n = pd.E;
         *est = J + 2.0 / sqrt(n) * sqrt(fmax(J, 0.0)) * S + S * S / n;

@@ -388,13 +388,13 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     const size_t wcol = (size_t(m - 1) * E + col) * N;   // (window, column) in [M][E][N] arrays
 
     Fiber<L, Q> fb;
-    fb.init(c, f, pd, a.cpt * N);
+    fb.init(c, f, pd, a.cpt * col_pitch(N));
     __shared__ ExTab ex_s;   // (ordered before its first read by the first barrier of the time loop)
     fill_exchange(ex_s, pd);
     // the apply buffers' zero entry (read by the exchange terms a fiber entry does not have; the
     // first barrier of the time loop orders these stores before any read)
     if (tid == 0) {
-        const size_t z = size_t(a.cpt) * N;
+        const size_t z = size_t(a.cpt) * col_pitch(N);
         D0[z] = make_double2(0.0, 0.0);
         if (SOLVER == SOLVER_FP64) D1[z] = make_double2(0.0, 0.0);
         if (SOLVER == SOLVER_MIXED) {
@@ -777,7 +777,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                     io.u[l][0] = v[l][0];
                     io.u[l][1] = v[l][1];
                 }
-                coarse_step<L, Q, S, BWD>(D0, coef_d, pd, ex_s, c, f, a.cpt * N, step_of(0, jj), step_of(nslot - 1, jj),
+                coarse_step<L, Q, S, BWD>(D0, coef_d, pd, ex_s, c, f, a.cpt * col_pitch(N), step_of(0, jj), step_of(nslot - 1, jj),
                                           nslot, slot, act, mine, mine ? prm[0] : 0, Kmax, sh, io);
                 if (mine) {
 #pragma unroll
@@ -811,12 +811,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             }
             if (act && live) {
                 if constexpr (SOLVER == SOLVER_MIXED) {
-                    float4* Hs = reinterpret_cast<float4*>(H) + size_t(hpos) * hstride + fb.xo;
+                    float4* Hs = reinterpret_cast<float4*>(H) + size_t(hpos) * hstride + c * N + f * L;
 #pragma unroll
                     for (int l = 0; l < L; ++l) Hs[l] = zf[l];
                 } else {
 #pragma unroll
-                    for (int l = 0; l < L; ++l) H[size_t(hpos) * hstride + fb.xo + l] = z[l];
+                    for (int l = 0; l < L; ++l) H[size_t(hpos) * hstride + c * N + f * L + l] = z[l];
                 }
             }
             fence_proxy_async_smem();

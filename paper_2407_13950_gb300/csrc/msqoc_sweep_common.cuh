@@ -15,6 +15,10 @@ __host__ __device__ constexpr int ipow_c(int b, int e) { return e == 0 ? 1 : b *
 __host__ __device__ constexpr int next_pow2_c(int v) { return v <= 1 ? 1 : 2 * next_pow2_c((v + 1) / 2); }
 __host__ __device__ constexpr int log2_c(int v) { return v <= 1 ? 0 : 1 + log2_c(v / 2); }
 
+// Entries between the columns of the shared apply buffers: odd, so that lanes on the same fiber of
+// different columns meet different banks (N = 16: four columns 128 bytes apart would meet one)
+__host__ __device__ constexpr int col_pitch(int N) { return N | 1; }
+
 // ------------------------------------------------------------------ precision conversions
 // f64 -> f32 rounded to nearest (ties away from zero) for |x| in [2^-126, 2^127); smaller
 // magnitudes become signed zero.  Pure integer operations.
@@ -188,7 +192,7 @@ struct Fiber {
     static constexpr int NFIX = Q - 1;
     static constexpr int NA = NFIX > 0 ? NFIX : 1;
     int f;             // fiber index
-    int xo;            // offset of the fiber's first entry in a [cb][N] buffer
+    int xo;            // offset of the fiber's first entry in a [cb][pitch] buffer
     int nb1[NA];       // offset of neighbour fiber (first entry) for subsystem k, entry 1
     int nb2[NA];       // entry 2 (exists when the level is interior)
     int sl1[NA];       // coefficient slot of entry 1
@@ -204,24 +208,24 @@ struct Fiber {
 
     // c: tile column, f: fiber, zero: index of the shared buffers' zero entry
     __device__ void init(int c, int f, const ProbDev& pd, int zero) {
-        constexpr int N = ipow_c(L, Q);
+        constexpr int CP = col_pitch(ipow_c(L, Q));
         this->f = f;
-        xo = c * N + f * L;
+        xo = c * CP + f * L;
 #pragma unroll
         for (int k = 0; k < NFIX; ++k) {
             const int sf = ipow_c(L, Q - 2 - k);   // stride of subsystem k in fiber units
             const int lk = (f / sf) % L;
             if (lk < L - 1) {
-                nb1[k] = c * N + (f + sf) * L;
+                nb1[k] = c * CP + (f + sf) * L;
                 sl1[k] = (k * L + lk) * 2 + 0;
                 plus1[k] = true;
                 w1[k] = pd.wsq[2 * lk + 0];
                 two[k] = lk > 0;
-                nb2[k] = c * N + (f - (lk > 0 ? sf : 0)) * L;
+                nb2[k] = c * CP + (f - (lk > 0 ? sf : 0)) * L;
                 sl2[k] = (k * L + lk) * 2 + 1;
                 w2[k] = pd.wsq[2 * lk + 1];
             } else {
-                nb1[k] = c * N + (f - sf) * L;
+                nb1[k] = c * CP + (f - sf) * L;
                 sl1[k] = (k * L + lk) * 2 + 1;
                 plus1[k] = false;
                 w1[k] = pd.wsq[2 * lk + 1];
@@ -231,7 +235,7 @@ struct Fiber {
                 w2[k] = 0.0;
             }
         }
-        eb = c * N;
+        eb = c * CP;
         this->zero = zero;
 #pragma unroll
         for (int l = 0; l < L; ++l) {
@@ -263,9 +267,9 @@ __host__ __device__ inline SweepSmem sweep_layout(int q, int L, int N, int cpt, 
     SweepSmem s{};
     const int nslot = q * L * 2;
     const int ncoef = pair ? 2 : 1;
-    // apply buffers hold cpt N entries plus a zero entry (index cpt N, never written by the
+    // apply buffers hold cpt columns plus a zero entry (index cpt pitch, never written by the
     // sweeps: the source of the exchange terms an entry does not have)
-    const size_t buf_d = (size_t(cpt) * N + 1) * 16, buf_f = (size_t(cpt) * N + 1) * 8;
+    const size_t buf = size_t(cpt) * col_pitch(N) + 1, buf_d = buf * 16, buf_f = buf * 8;
     size_t o = 0;
     s.coef_d = o; o = align16(o + size_t(2) * 2 * ncoef * nslot * 16);  // [parity][slot][part][NSLOT]
     s.coef_f = o; o = align16(o + size_t(2) * 2 * ncoef * nslot * 8);
@@ -278,7 +282,7 @@ __host__ __device__ inline SweepSmem sweep_layout(int q, int L, int N, int cpt, 
     s.FA = o;     o = align16(o + (solver == SOLVER_MIXED ? buf_f : 0));
     s.FB = o;     o = align16(o + (solver == SOLVER_MIXED ? buf_f : 0));
     // the mixed solver's one-thread families: the step before's FP32 estimate
-    s.DP = o;     o = align16(o + (!pair && solver == SOLVER_MIXED ? size_t(cpt) * N * 8 : 0));
+    s.DP = o;     o = align16(o + (!pair && solver == SOLVER_MIXED ? buf_f : 0));
     s.H = o;      o = align16(o + size_t(hdepth) * cpt * N * 16);   // history staging: hdepth blocks of cpt N states
     s.total = o;
     return s;

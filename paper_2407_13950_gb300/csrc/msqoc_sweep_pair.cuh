@@ -224,13 +224,13 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     const size_t wcol = (size_t(m - 1) * E + col) * N;   // (window, column) in [M][E][N] arrays
 
     Fiber<L, Q> fb;
-    fb.init(c, f, pd, a.cpt * N);
+    fb.init(c, f, pd, a.cpt * col_pitch(N));
     __shared__ ExTab ex_s;   // (ordered before its first read by the first barrier of the time loop)
     fill_exchange(ex_s, pd);
     // the apply buffers' zero entry (read by the exchange terms a fiber entry does not have; the
     // first barrier of the time loop orders these stores before any read)
     if (tid == 0) {
-        const size_t z = size_t(a.cpt) * N;
+        const size_t z = size_t(a.cpt) * col_pitch(N);
         D0[z] = make_double2(0.0, 0.0);
         if (SOLVER == SOLVER_FP64) D1[z] = make_double2(0.0, 0.0);
         if (SOLVER == SOLVER_MIXED) {
@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                     tile_sync();
                 }
             }
-            if (act && live) store_part<LS, double2>(H + size_t(hpos) * hstride, fb.xo + le, part, z);
+            if (act && live) store_part<LS, double2>(H + size_t(hpos) * hstride, c * N + f * L + le, part, z);
             fence_proxy_async_smem();
         }
         if (live) {
