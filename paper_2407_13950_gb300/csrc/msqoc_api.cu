@@ -989,7 +989,7 @@ bool split_history(const ProbDev& pd) { return pd.solver == SOLVER_MIXED && pd.p
 
 // blocks of the quadrature kernel: per window, the chunk's steps in groups of its staged lanes
 int quad_blocks(const ProbDev& pd) {
-    const int most = pd.N <= 128 ? 32 : 16;   // quad_lanes
+    const int most = pd.N <= QUAD_ROWS_32 ? 32 : pd.N <= QUAD_ROWS_16 ? 16 : 8;   // quad_lanes
     int lanes = 1;
     while (lanes < pd.E && lanes < most) lanes <<= 1;
     const int per = most / lanes;
@@ -1062,9 +1062,11 @@ msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s) {
     return MSQOC_OK;
 }
 
+// a window's entries, at most TERM_THREADS (fewer warps: fewer partial sums in the chain)
+int terminal_threads(const ProbDev& pd) { return std::min(TERM_THREADS, (pd.N * pd.E + 31) / 32 * 32); }
 msqoc_status launch_terminal(msqoc_problem* p, bool want_lambda, cudaStream_t s) {
     Mark mk(p, MSQOC_KERNEL_TERMINAL, s);
-    k_terminal<<<p->pd.M, TERM_THREADS, 0, s>>>(p->pd, want_lambda ? 1 : 0);
+    k_terminal<<<p->pd.M, terminal_threads(p->pd), 0, s>>>(p->pd, want_lambda ? 1 : 0);
     CUDA_TRY(cudaGetLastError());
     return MSQOC_OK;
 }
@@ -1590,7 +1592,7 @@ msqoc_status eval_objective_noalloc(const msqoc_hamiltonian* H, const msqoc_cont
         CUDA_TRY(cudaGetLastError());
     }
     CUDA_TRY(launch_sweep(sweep_args(pd, pd_d, tiles_d, map_d, SWEEP_OBJECTIVE, 0), pd.ntiles, s));
-    k_terminal<<<pd.M, TERM_THREADS, 0, s>>>(pd, 0);
+    k_terminal<<<pd.M, terminal_threads(pd), 0, s>>>(pd, 0);
     CUDA_TRY(cudaGetLastError());
     k_objective_outputs<<<1, OUT_THREADS, 0, s>>>(pd, outs, outs + 1, M > 1 ? outs + 2 : nullptr);
     CUDA_TRY(cudaGetLastError());

@@ -166,14 +166,15 @@ __global__ void k_phases(const ProbDev pd) {
 }
 
 // block-wide sums of K values with a fixed reduction order (deterministic): lanes by shuffles, then
-// the warps' sums in order; sh: K NT / 32 doubles
-template <int NT, int K>
+// the warps' sums in order; sh: K doubles a warp
+template <int K>
 __device__ __forceinline__ void block_sums(double (&v)[K], double* sh) {
-    constexpr int NW = NT / 32;
+    const int nw = blockDim.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (nw == 1) return;
     if ((threadIdx.x & 31) == 0)
 #pragma unroll
         for (int k = 0; k < K; ++k) sh[(threadIdx.x >> 5) * K + k] = v[k];
@@ -181,16 +182,14 @@ __device__ __forceinline__ void block_sums(double (&v)[K], double* sh) {
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         double s = sh[k];
-#pragma unroll
-        for (int w = 1; w < NW; ++w) s += sh[w * K + k];
+        for (int w = 1; w < nw; ++w) s += sh[w * K + k];
         v[k] = s;
     }
     __syncthreads();
 }
-template <int NT>
-__device__ double block_sum(double v, double* sh) {
+__device__ __forceinline__ double block_sum(double v, double* sh) {
     double a[1] = {v};
-    block_sums<NT, 1>(a, sh);
+    block_sums(a, sh);
     return a[0];
 }
 
@@ -220,79 +219,88 @@ __host__ __device__ inline ComposeGeom compose_geom(int N) {
 // link s, visit(s, x) called with the state before link s (and with s = links at the end).  xs: two
 // buffers of N entries, the state in the first.  Every thread of the block takes part; one barrier
 // a link.  A link waits for nothing but its FP64 operations: where a thread has at most PRE terms
-// (N <= 32) it loads the next link's while it does this one's (QFT-8: 1.17 us a link without).
-template <bool BWD, class Phi, class Visit>
-__device__ __forceinline__ void compose_chain(int N, int links, double2* xs, Phi phi, Visit visit) {
-    constexpr int PRE = 4;
-    const ComposeGeom ge = compose_geom(N);
-    const int i = threadIdx.x / ge.JG, g = threadIdx.x % ge.JG;
-    const int st = BWD ? 1 : N;
-    const size_t off = BWD ? size_t(i) * N : size_t(i);
-    const bool pre = N <= PRE * ge.JG;
-    double2 nx[PRE];
-    auto fetch = [&](int s) {
-#pragma unroll
-        for (int u = 0; u < PRE; ++u) {
-            const int j = g + u * ge.JG;
-            nx[u] = i < N && j < N ? phi(s)[off + size_t(j) * st] : make_double2(0.0, 0.0);
-        }
-    };
-    if (pre && links > 0) fetch(0);
-    for (int s = 0; s < links; ++s) {
-        const double2* x = xs + (s & 1 ? N : 0);
-        double2* xn = xs + (s & 1 ? 0 : N);
-        visit(s, x);
-        double2 y = make_double2(0.0, 0.0);
-        if (pre) {
-            double2 c[PRE];
-#pragma unroll
-            for (int u = 0; u < PRE; ++u) c[u] = nx[u];
-            if (s + 1 < links) fetch(s + 1);
-#pragma unroll
-            for (int u = 0; u < PRE; ++u) {
-                const int j = g + u * ge.JG;
-                if (u * ge.JG >= N) break;   // uniform
-                const double2 z = x[j < N ? j : 0];
-                const double ci = BWD ? -c[u].y : c[u].y;
-                y.x = fma(c[u].x, z.x, fma(-ci, z.y, y.x));
-                y.y = fma(c[u].x, z.y, fma(ci, z.x, y.y));
-            }
-        } else if (i < N) {
-            // two running sums (shorter chains)
-            const double2* p = phi(s) + off;
-            double2 w = make_double2(0.0, 0.0);
-            int j = g;
-#pragma unroll 4
-            for (; j + ge.JG < N; j += 2 * ge.JG) {
-                const double2 a = p[size_t(j) * st], b = p[size_t(j + ge.JG) * st];
-                const double2 z = x[j], z2 = x[j + ge.JG];
-                const double ai = BWD ? -a.y : a.y, bi = BWD ? -b.y : b.y;
-                y.x = fma(a.x, z.x, fma(-ai, z.y, y.x));
-                y.y = fma(a.x, z.y, fma(ai, z.x, y.y));
-                w.x = fma(b.x, z2.x, fma(-bi, z2.y, w.x));
-                w.y = fma(b.x, z2.y, fma(bi, z2.x, w.y));
-            }
-            if (j < N) {
-                const double2 a = p[size_t(j) * st], z = x[j];
-                const double ai = BWD ? -a.y : a.y;
-                y.x = fma(a.x, z.x, fma(-ai, z.y, y.x));
-                y.y = fma(a.x, z.y, fma(ai, z.x, y.y));
-            }
-            y.x += w.x;
-            y.y += w.y;
-        }
+// (N <= 32) it loads the propagators AHEAD links early, longer than a load from L2 takes (QFT-4:
+// 0.85 us a link one link ahead).
+template <bool BWD>
+struct ComposeRow {
+    int N, i, g, JG, st;
+    size_t off;
+    // the finished row sums into xn, from this thread's part y of row i
+    __device__ __forceinline__ void finish(double2 y, double2* xn) const {
         // the row's lanes: the first exchange leaves the real part in one half, the imaginary part
         // in the other
-        if (ge.JG > 1) {
-            int o = ge.JG >> 1;
+        if (JG > 1) {
+            int o = JG >> 1;
             const bool up = g & o;
             double v = (up ? y.y : y.x) + __shfl_xor_sync(0xffffffffu, up ? y.x : y.y, o);
             for (o >>= 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (i < N && (g & ((ge.JG >> 1) - 1)) == 0) reinterpret_cast<double*>(xn + i)[up ? 1 : 0] = v;
+            if (i < N && (g & ((JG >> 1) - 1)) == 0) reinterpret_cast<double*>(xn + i)[up ? 1 : 0] = v;
         } else if (i < N) {
             xn[i] = y;
         }
         __syncthreads();
+    }
+    __device__ __forceinline__ static void mac(double2& y, double2 c, double2 z) {
+        const double ci = BWD ? -c.y : c.y;
+        y.x = fma(c.x, z.x, fma(-ci, z.y, y.x));
+        y.y = fma(c.x, z.y, fma(ci, z.x, y.y));
+    }
+};
+template <bool BWD, int PRE, class Phi, class Visit>
+__device__ __forceinline__ void compose_ahead(const ComposeRow<BWD>& r, int links, double2* xs, Phi phi, Visit visit) {
+    constexpr int AHEAD = 4;
+    double2 nx[AHEAD][PRE];
+    auto fetch = [&](int s, double2 (&to)[PRE]) {
+#pragma unroll
+        for (int u = 0; u < PRE; ++u) {
+            const int j = r.g + u * r.JG;
+            to[u] = s < links && r.i < r.N && j < r.N ? phi(s)[r.off + size_t(j) * r.st] : make_double2(0.0, 0.0);
+        }
+    };
+#pragma unroll
+    for (int a = 0; a < AHEAD; ++a) fetch(a, nx[a]);
+    for (int s0 = 0; s0 < links; s0 += AHEAD) {
+#pragma unroll
+        for (int a = 0; a < AHEAD; ++a) {
+            const int s = s0 + a;
+            if (s >= links) break;   // uniform
+            const double2* x = xs + (s & 1 ? r.N : 0);
+            visit(s, x);
+            double2 y = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int u = 0; u < PRE; ++u) {
+                const int j = r.g + u * r.JG;
+                r.mac(y, nx[a][u], x[j < r.N ? j : 0]);
+            }
+            fetch(s + AHEAD, nx[a]);
+            r.finish(y, xs + (s & 1 ? 0 : r.N));
+        }
+    }
+    visit(links, xs + (links & 1 ? r.N : 0));
+}
+template <bool BWD, class Phi, class Visit>
+__device__ __forceinline__ void compose_chain(int N, int links, double2* xs, Phi phi, Visit visit) {
+    const ComposeGeom ge = compose_geom(N);
+    const int i = threadIdx.x / ge.JG, g = threadIdx.x % ge.JG;
+    const ComposeRow<BWD> r{N, i, g, ge.JG, BWD ? 1 : N, BWD ? size_t(i) * N : size_t(i)};
+    if (N <= ge.JG) return compose_ahead<BWD, 1>(r, links, xs, phi, visit);
+    if (N <= 2 * ge.JG) return compose_ahead<BWD, 2>(r, links, xs, phi, visit);
+    if (N <= 4 * ge.JG) return compose_ahead<BWD, 4>(r, links, xs, phi, visit);
+    for (int s = 0; s < links; ++s) {
+        const double2* x = xs + (s & 1 ? N : 0);
+        visit(s, x);
+        double2 y = make_double2(0.0, 0.0), w = y;   // two running sums (shorter chains)
+        if (i < N) {
+            const double2* p = phi(s) + r.off;
+            int j = g;
+#pragma unroll 4
+            for (; j + ge.JG < N; j += 2 * ge.JG) {
+                r.mac(y, p[size_t(j) * r.st], x[j]);
+                r.mac(w, p[size_t(j + ge.JG) * r.st], x[j + ge.JG]);
+            }
+            if (j < N) r.mac(y, p[size_t(j) * r.st], x[j]);
+        }
+        r.finish(make_double2(y.x + w.x, y.y + w.y), xs + (s & 1 ? 0 : N));
     }
     visit(links, xs + (links & 1 ? N : 0));
 }
@@ -349,7 +357,7 @@ constexpr int TERM_THREADS = 256;
 //   m = M: gamma = <V, U^M>, J = ||U^M||^2/E - |gamma|^2/E^2, Lambda^M(t_M) = (gamma V - E U^M)/E^2
 // (m and M global: a shard's last window is the problem's last only when it ends the grid)
 __global__ void __launch_bounds__(TERM_THREADS) k_terminal(const ProbDev pd, const int want_lambda) {
-    __shared__ double sh[TERM_THREADS];
+    __shared__ double sh[3 * TERM_THREADS / 32];
     const int m = blockIdx.x + 1;
     const size_t ne = size_t(pd.N) * pd.E;
     const double2* U = pd.Uend + size_t(m - 1) * ne;
@@ -357,30 +365,30 @@ __global__ void __launch_bounds__(TERM_THREADS) k_terminal(const ProbDev pd, con
     if (m + pd.m_off < pd.M_glob) {
         const double2* Wm = pd.W + size_t(m - 1) * ne;
         double s = 0.0;
-        for (size_t e = threadIdx.x; e < ne; e += TERM_THREADS) {
+        for (size_t e = threadIdx.x; e < ne; e += blockDim.x) {
             const double2 u = U[e], w = Wm[e];
             const double cx = u.x - w.x, cy = u.y - w.y;
             s = fma(cx, cx, fma(cy, cy, s));
             if (want_lambda) Lt[e] = make_double2(-0.5 * pd.mu * cx, -0.5 * pd.mu * cy);
         }
-        s = block_sum<TERM_THREADS>(s, sh);
+        s = block_sum(s, sh);
         if (threadIdx.x == 0) pd.term[m - 1] = 0.5 * pd.mu * s;
     } else {
         double gr = 0.0, gi = 0.0, nr = 0.0;
-        for (size_t e = threadIdx.x; e < ne; e += TERM_THREADS) {
+        for (size_t e = threadIdx.x; e < ne; e += blockDim.x) {
             const double2 u = U[e], v = pd.V[e];
             gr = fma(v.x, u.x, fma(v.y, u.y, gr));
             gi = fma(v.x, u.y, fma(-v.y, u.x, gi));
             nr = fma(u.x, u.x, fma(u.y, u.y, nr));
         }
         double t[3] = {gr, gi, nr};
-        block_sums<TERM_THREADS, 3>(t, sh);
+        block_sums(t, sh);
         gr = t[0], gi = t[1], nr = t[2];
         const double E = pd.E;
         if (threadIdx.x == 0) pd.term[m - 1] = nr / E - (gr * gr + gi * gi) / (E * E);
         if (want_lambda) {
             const double inv = 1.0 / (E * E);
-            for (size_t e = threadIdx.x; e < ne; e += TERM_THREADS) {
+            for (size_t e = threadIdx.x; e < ne; e += blockDim.x) {
                 const double2 u = U[e], v = pd.V[e];
                 const double lx = (gr * v.x - gi * v.y) - E * u.x;
                 const double ly = (gr * v.y + gi * v.x) - E * u.y;
@@ -403,7 +411,7 @@ __device__ __forceinline__ void objective_outputs(const ProbDev& pd, double* P_o
         P += t;
         if (pen_out && m < npen) pen_out[m] = t;
     }
-    P = block_sum<OUT_THREADS>(P, sh);
+    P = block_sum(P, sh);
     if (threadIdx.x == 0) {
         if (P_out) *P_out = P;
         if (J_out) *J_out = has_last ? pd.term[pd.M - 1] : 0.0;
@@ -411,7 +419,7 @@ __device__ __forceinline__ void objective_outputs(const ProbDev& pd, double* P_o
 }
 __global__ void __launch_bounds__(OUT_THREADS) k_objective_outputs(const ProbDev pd, double* P_out, double* J_out,
                                                                     double* pen_out) {
-    __shared__ double sh[OUT_THREADS];
+    __shared__ double sh[2 * OUT_THREADS / 32];
     objective_outputs(pd, P_out, J_out, pen_out, sh);
 }
 
@@ -419,10 +427,10 @@ __global__ void __launch_bounds__(OUT_THREADS) k_objective_outputs(const ProbDev
 //   J + (2 / sqrt(n)) sqrt(J) S + S^2 / n,  S = sum_{m<M} ||C^m||_F,  ||C^m||_F = sqrt(2 pen_m / mu),
 // with n := E (as in the generalized infidelity).  One block, fixed order (deterministic).
 __global__ void __launch_bounds__(OUT_THREADS) k_rollout_estimate(const ProbDev pd, double* est) {
-    __shared__ double sh[OUT_THREADS];
+    __shared__ double sh[2 * OUT_THREADS / 32];
     double S = 0.0;
     for (int m = 1 + threadIdx.x; m < pd.M; m += OUT_THREADS) S += sqrt(2.0 * pd.term[m - 1] / pd.mu);
-    S = block_sum<OUT_THREADS>(S, sh);
+    S = block_sum(S, sh);
     if (threadIdx.x == 0) {
         const double J = pd.term[pd.M - 1];
         const double n = pd.E;
@@ -444,7 +452,7 @@ __global__ void __launch_bounds__(OUT_THREADS) k_rollout_estimate(const ProbDev 
 //     window k is its own, -2 Lambda^{k+1}(t_k) if window k + 1 is.
 __global__ void __launch_bounds__(OUT_THREADS) k_gradient_outputs(const ProbDev pd, double* P_out, double* ga,
                                                                    double2* gW, int wblocks, int nstates) {
-    __shared__ double sh[OUT_THREADS];
+    __shared__ double sh[2 * OUT_THREADS / 32];
     if (blockIdx.x == 0) {
         objective_outputs(pd, P_out, nullptr, nullptr, sh);
         return;
@@ -472,7 +480,7 @@ __global__ void __launch_bounds__(OUT_THREADS) k_gradient_outputs(const ProbDev 
             g2 = fma(w, fma(ph.x, ab.y, -ph.y * ab.x), g2);
         }
         double g[2] = {g1, g2};
-        block_sums<OUT_THREADS, 2>(g, sh);
+        block_sums(g, sh);
         if (threadIdx.x == 0) {
             const size_t i = (size_t(fi) * pd.d1 + s) * 2;
             ga[i] = -2.0 * pd.h * g[0];
@@ -514,7 +522,7 @@ constexpr int REG_CHUNK = 4;
 __global__ void __launch_bounds__(REG_THREADS) k_regularization(const ProbDev pd, const double* alpha,
                                                                  double gamma_tik, double gamma_energy,
                                                                  double* grad, double* epart) {
-    __shared__ double sh[REG_THREADS];
+    __shared__ double sh[REG_THREADS / 32];
     const int k = blockIdx.x / pd.d1, s = blockIdx.x % pd.d1;
     // steps whose midpoint lies in [(s - 2) dtau, (s + 1) dtau), widened by two steps on each side
     // (membership is decided exactly by spline_at below)
@@ -557,14 +565,14 @@ __global__ void __launch_bounds__(REG_THREADS) k_regularization(const ProbDev pd
             }
         }
         if (c0 == 0) {
-            const double se = block_sum<REG_THREADS>(en, sh);
+            const double se = block_sum(en, sh);
             if (threadIdx.x == 0) epart[blockIdx.x] = wt * se;
         }
 #pragma unroll
         for (int c = 0; c < REG_CHUNK; ++c) {
             if (c0 + c >= nfk) break;                  // block-uniform
-            const double sre = block_sum<REG_THREADS>(are[c], sh);
-            const double sim = block_sum<REG_THREADS>(aim[c], sh);
+            const double sre = block_sum(are[c], sh);
+            const double sim = block_sum(aim[c], sh);
             if (threadIdx.x == 0) {
                 const size_t i = (size_t(f0 + c0 + c) * pd.d1 + s) * 2;
                 grad[i] = gamma_tik * alpha[i] + 2.0 * gamma_energy * wt * sre;
@@ -578,12 +586,12 @@ __global__ void __launch_bounds__(REG_THREADS) k_regularization(const ProbDev pd
 __global__ void __launch_bounds__(REG_THREADS) k_regularization_total(const ProbDev pd, const double* alpha,
                                                                        double gamma_tik, double gamma_energy,
                                                                        const double* epart, double* R) {
-    __shared__ double sh[REG_THREADS];
+    __shared__ double sh[REG_THREADS / 32];
     double a2 = 0.0, en = 0.0;
     for (int i = threadIdx.x; i < pd.d; i += REG_THREADS) a2 += alpha[i] * alpha[i];
     for (int i = threadIdx.x; i < pd.q * pd.d1; i += REG_THREADS) en += epart[i];
-    a2 = block_sum<REG_THREADS>(a2, sh);
-    en = block_sum<REG_THREADS>(en, sh);
+    a2 = block_sum(a2, sh);
+    en = block_sum(en, sh);
     if (threadIdx.x == 0) *R = 0.5 * gamma_tik * a2 + gamma_energy * en;
 }
 

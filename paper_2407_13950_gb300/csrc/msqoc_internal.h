@@ -189,6 +189,8 @@ __host__ __device__ inline int64_t slice_start(const ProbDev& pd, int C, int v) 
     const int64_t n0 = win(w);
     return C == 1 ? n0 : n0 + ((v - 1 - w * C) * (win(w + 1) - n0)) / C;
 }
+// rows up to which the quadrature kernel stages 32 and 16 lanes (quad_lanes; more rows: 8)
+constexpr int QUAD_ROWS_32 = 32, QUAD_ROWS_16 = 128;
 // blocks a problem needs for its windows' chunks
 int quad_blocks(const ProbDev& pd);
 // nprob rows of `blocks` blocks each (0 blocks: only sets the kernel's attributes)

@@ -20,8 +20,8 @@
 // 4 transmons, 100000 steps: 2.08 ms (4.1 GB read, 2.0 TB/s; the products' FP32 operations alone
 // would take 0.8 ms), against 2.71 ms for one fiber a warp with a branch per level and 37% more
 // instructions.  Issue-bound: a staged CTA holds 85 KB, so two are resident on an SM.
-// LN = 32, or 16 for shapes whose staging would not fit (the half-warps then take alternate groups
-// of pairs).
+// LN = 32, 16 or 8 by the rows, so that several CTAs fit an SM and one's loads overlap the others'
+// products; below 32 the parts of a warp take alternate groups of pairs.
 #pragma once
 
 #include <type_traits>
@@ -76,13 +76,11 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 // staged lanes, warps and staging bytes of a CTA
 template <int L, int Q>
-__host__ __device__ constexpr int quad_lanes() { return ipow_c(L, Q) <= 128 ? 32 : 16; }
-template <int L, int Q>
-__host__ __device__ constexpr int quad_split() {   // warps that share one (k, j)
-    return ipow_c(L, Q) > 128 ? 2 : 1;
+__host__ __device__ constexpr int quad_lanes() {
+    return ipow_c(L, Q) <= QUAD_ROWS_32 ? 32 : ipow_c(L, Q) <= QUAD_ROWS_16 ? 16 : 8;
 }
 template <int L, int Q>
-__host__ __device__ constexpr int quad_warps() { return Q * (L - 1) * quad_split<L, Q>(); }
+__host__ __device__ constexpr int quad_warps() { return Q * (L - 1); }
 template <int L, int Q>
 __host__ __device__ constexpr size_t quad_smem() {
     constexpr size_t stage = size_t(ipow_c(L, Q)) * (quad_lanes<L, Q>() + 1) * 16 * 2;
@@ -106,7 +104,7 @@ __device__ __forceinline__ std::conditional_t<MODE == 2, double2, float4> quad_o
 template <int L, int Q, int MODE>
 __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs a) {
     constexpr int N = ipow_c(L, Q), F = N / L, NW = quad_warps<L, Q>(), LN = quad_lanes<L, Q>();
-    constexpr int WS = quad_split<L, Q>();
+    constexpr int SUB = 32 / LN;                             // parts of a warp
     constexpr int UN = L == 3 ? (F < 3 ? 1 : 3) : (F < 4 ? F : 4);   // pairs summed afresh; divides F
     constexpr int ROW = LN + 1;
     constexpr bool SPLIT = MODE > 0;
@@ -132,10 +130,10 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
     const int hi = min(min(ns, (a.seg + 1) * pd.kseg), lo + pd.kadj);
     if (lo + j0 >= hi) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int half = lane / LN;                              // 0, or the half-warp (LN = 16)
+    const int part = lane / LN;
     const int ln = lane % LN, sl = ln / EL, cl = ln % EL;    // staged lane; its step and column
     const bool live = lo + j0 + sl < hi;
-    const int k = warp / ((L - 1) * WS), j = 1 + (warp / WS) % (L - 1);
+    const int k = warp / (L - 1), j = 1 + warp % (L - 1);
     const int st = [&] {                                     // the stride of subsystem k's level
         int t = 1;
         for (int e = k; e < Q - 1; ++e) t *= L;
@@ -173,12 +171,11 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
         }
         cp_async_wait_all();
         __syncthreads();
-        // ---- the pairs, UN at a time; the warps (and half-warps) that share a (k, j) take turns
+        // ---- the pairs, UN at a time; the parts of the warp take turns
         GT R, I;
         gsum_zero(R);
         gsum_zero(I);
-        constexpr int TURNS = WS * (32 / LN);
-        for (int p0 = UN * ((warp % WS) * (32 / LN) + half); p0 < F; p0 += UN * TURNS) {
+        for (int p0 = UN * part; p0 < F; p0 += UN * SUB) {
             GT r, q;
 #pragma unroll
             for (int t = 0; t < UN; ++t) {
@@ -213,14 +210,15 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
         }
     }
 
-    // ---- sums over the step's lanes (and half-warps), weighted, then over the warps, fixed order
+    // ---- sums over the step's lanes and the warp's parts, weighted, then over the warps, fixed order
     for (int o = EL >> 1; o > 0; o >>= 1) {
         A = gsum_add(A, gsum_shfl_xor(A, o));
         B = gsum_add(B, gsum_shfl_xor(B, o));
     }
-    if constexpr (LN < 32) {
-        A = gsum_add(A, gsum_shfl_xor(A, LN));
-        B = gsum_add(B, gsum_shfl_xor(B, LN));
+#pragma unroll
+    for (int o = LN; o < 32; o <<= 1) {
+        A = gsum_add(A, gsum_shfl_xor(A, o));
+        B = gsum_add(B, gsum_shfl_xor(B, o));
     }
     if constexpr (MODE == 1) {
         A = df_scale_sqrt(A, j);
@@ -230,7 +228,7 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
         B *= sqrt_small(j);
     }
     __syncthreads();
-    if (half == 0 && cl == 0) {
+    if (part == 0 && cl == 0) {
         red[(warp * spw + sl) * 2] = A;
         red[(warp * spw + sl) * 2 + 1] = B;
     }
@@ -238,10 +236,10 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
     for (int e = threadIdx.x; e < spw * 2 * Q; e += 32 * NW) {
         const int kk = e / (2 * spw), r = e % (2 * spw), s = r >> 1;
         if (lo + j0 + s >= hi) continue;
-        const GT* q = red + size_t(kk) * (L - 1) * WS * spw * 2 + r;
+        const GT* q = red + size_t(kk) * (L - 1) * spw * 2 + r;
         GT t = q[0];
 #pragma unroll
-        for (int w = 1; w < (L - 1) * WS; ++w) t = gsum_add(t, q[w * spw * 2]);
+        for (int w = 1; w < L - 1; ++w) t = gsum_add(t, q[w * spw * 2]);
         double v;
         if constexpr (MODE == 1)
             v = df_to_f64_scaled(t, S);
