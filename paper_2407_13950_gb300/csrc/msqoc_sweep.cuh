@@ -308,6 +308,15 @@ static __device__ __noinline__ void coarse_step(double2* D0, double2* cfd, const
     }
 }
 
+// Tile-wide values (sweep_tile): per slot the window's first step, its steps in the launch, where
+// its history starts and the bytes of a step of it
+struct TileInfo {
+    int64_t n0[2];
+    double2* hist[2];
+    int cnt[2];
+    uint32_t bytes[2];
+};
+
 // ------------------------------------------------------------------ the sweep kernel
 // One CTA per tile.  A tile covers one or two windows ("slots"); each slot has its own step
 // range, per-step coefficients and iteration counts, computed by warp `slot` (the host only builds
@@ -364,11 +373,27 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     const int cnt_0 = max(0, min(wns_0, hi) - lo);
     const int cnt_1 = nslot > 1 ? max(0, min(wns_1, hi) - lo) : 0;
     const int nit = max(cnt_0, cnt_1);
+    // what only a few threads need in the loop, kept in shared memory instead of everyone's
+    // registers (written before the barrier ahead of the loop)
+    __shared__ TileInfo ti;
+    if (tid == 0) {
+        const size_t kh = BWD ? pd.kadj : pd.kseg;
+        double2* const base = PROP ? nullptr : BWD ? pd.lhist : pd.hist;
+        ti.n0[0] = wn0_0;
+        ti.n0[1] = wn0_1;
+        ti.cnt[0] = cnt_0;
+        ti.cnt[1] = cnt_1;
+        // slot s of a tile covers a contiguous column range of its window's block of a step
+        ti.hist[0] = base + (size_t(tile.m0 - 1) * kh * E + tile.c0) * N;
+        ti.hist[1] = base + size_t(tile.m0) * kh * E * N;
+        ti.bytes[0] = static_cast<uint32_t>(size_t(ncol0) * N * sizeof(double2));
+        ti.bytes[1] = static_cast<uint32_t>(size_t(ncol - ncol0) * N * sizeof(double2));
+    }
     // global step of slot s at iteration jj, clamped into the slot's range (a slot without steps
-    // in this launch maps to its window's first step, which exists)
+    // in this launch maps to its window's first step, or the grid's last)
     auto step_of = [&](int s, int jj) -> int64_t {
-        const int cnt = s ? cnt_1 : cnt_0;
-        const int64_t n0 = s ? wn0_1 : wn0_0;
+        const int cnt = ti.cnt[s];
+        const int64_t n0 = ti.n0[s];
         if (cnt <= 0) return min(n0, pd.nsteps - 1);
         const int jc = min(jj, cnt - 1);
         return BWD ? n0 + lo + cnt - 1 - jc : n0 + lo + jc;
@@ -486,17 +511,9 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
         }
     }
 
-    // ---- history blocks: slot s of a tile covers a contiguous column range of its window
+    // ---- history
     const bool want_hist = !PROP && (BWD || (mode == SWEEP_HISTORY && pd.nseg == 1) || mode == SWEEP_RECOMPUTE);
     const bool want_ckpt = !BWD && !PROP && mode == SWEEP_HISTORY && pd.nseg > 1;
-    const uint32_t bytes_0 = static_cast<uint32_t>(size_t(ncol0) * N * sizeof(double2));
-    const uint32_t bytes_1 = static_cast<uint32_t>(size_t(ncol - ncol0) * N * sizeof(double2));
-    auto hist_ptr = [&](int s, int jj) -> double2* {
-        const int64_t n0 = s ? wn0_1 : wn0_0;
-        const int jr = static_cast<int>(step_of(s, jj) - n0) - lo;   // step within the segment (chunk)
-        return (BWD ? pd.lhist : pd.hist) +
-               ((size_t(tile.m0 + s - 1) * (BWD ? pd.kadj : pd.kseg) + jr) * E + (s ? 0 : tile.c0)) * N;
-    };
     // Steps per history synchronisation: the midpoint states are staged in H in groups of hd
     // iterations (g hd .. g hd + hd - 1), one block of the tile's cpt N states per iteration, and
     // a group is stored with one wait.
@@ -505,10 +522,11 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     // thread 0: store the staged group starting at iteration g0 (every slot with a step)
     auto publish_group = [&](int g0) {
         const int g1 = min(g0 + hd, nit);
-        for (int j = g0; j < g1; ++j) {
-            const double2* src = H + size_t(j - g0) * hstride;
-            if (j < cnt_0) bulk_s2g(hist_ptr(0, j), src, bytes_0);
-            if (j < cnt_1) bulk_s2g(hist_ptr(1, j), src + size_t(ncol0) * N, bytes_1);
+        for (int s = 0; s < 2; ++s) {
+            const int cnt = ti.cnt[s];
+            const double2* src = H + (s ? size_t(ti.bytes[0] / sizeof(double2)) : 0);
+            for (int j = g0; j < min(g1, cnt); ++j)   // step j of the launch's, or from its end
+                bulk_s2g(ti.hist[s] + size_t(BWD ? cnt - 1 - j : j) * E * N, src + size_t(j - g0) * hstride, ti.bytes[s]);
         }
     };
     // warp s < nslot computes slot s's coefficients and keeps d_k and the iteration counts of
@@ -535,6 +553,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     int fsel = 0;
     double2* Dc = D0;   // FP64-solver ping-pong buffers
     double2* Dn = D1;
+    tile_sync();
     if (nit > 0) load_ctrl(0);
 
     int hpos = 0;   // position of iteration jj in its history group
@@ -550,21 +569,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                                             coef_f + (par * 2 + cslot) * NSLOT, coef_s + (par * 2 + cslot) * NSLOT,
                                             params + (par * 2 + cslot) * 4);
         }
-        // checkpoint: the state at the start of every segment (forward over whole windows)
-        // (the state is rounded to what is stored, so that a segment recomputed from its checkpoint
-        // repeats these steps bit for bit)
-        if (want_ckpt && jj % pd.kseg == 0) fresh = true;
-        if (want_ckpt && live && jj % pd.kseg == 0) {
+        // checkpoint: the state at the start of every segment (forward over whole windows), rounded
+        // to FP64 for the segment's recomputation; this sweep goes on with its own
+        if (want_ckpt && live && act && jj % pd.kseg == 0) {
             double2* ck = pd.ckpt + ((size_t(m - 1) * pd.nseg + jj / pd.kseg) * E + col) * N + f * L;
 #pragma unroll
-            for (int l = 0; l < L; ++l) {
-                const double2 o = state_out(l);
-                if (act) ck[l] = o;
-                if constexpr (SOLVER == SOLVER_MIXED) {
-                    v[l][0] = tf_split(o.x, sh);
-                    v[l][1] = tf_split(o.y, sh);
-                }
-            }
+            for (int l = 0; l < L; ++l) ck[l] = state_out(l);
         }
         const double2* cfd = coef_d + (par * 2 + slot) * NSLOT;
         const float2* cff = coef_f + (par * 2 + slot) * NSLOT;
