@@ -64,8 +64,7 @@ static cudaError_t launch_one(const SweepArgs& a, int ntiles, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     if (ntiles <= 0) return cudaSuccess;
-    kern<<<BOTH ? 2 * ntiles : ntiles, a.nthreads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(kern, BOTH ? 2 * ntiles : ntiles, a.nthreads, smem, s, a);
 }
 
 template <int SOLVER, bool BWD, int FAM>
@@ -123,8 +122,7 @@ static cudaError_t launch_quad_one(const QuadArgs& a, int blocks, int nprob, cud
         if (e != cudaSuccess) return e;
     }
     if (blocks <= 0 || nprob <= 0) return cudaSuccess;
-    kern<<<dim3(blocks, nprob), 32 * quad_warps<MSQOC_L, MSQOC_Q>(), smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3(blocks, nprob), 32 * quad_warps<MSQOC_L, MSQOC_Q>(), smem, s, a);
 }
 
 cudaError_t MSQOC_CAT(launch_quad, MSQOC_L, MSQOC_Q)(const QuadArgs& a, int blocks, int nprob, cudaStream_t s) {

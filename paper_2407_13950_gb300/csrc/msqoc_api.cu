@@ -49,6 +49,18 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// does p lie in the current device's own memory, at a multiple of `align` bytes?
+bool in_place(const void* p, size_t align) {
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (reinterpret_cast<uintptr_t>(p) % align) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 template <typename T>
 cudaError_t dalloc(T** p, size_t n) {
     *p = nullptr;
@@ -951,6 +963,18 @@ msqoc_status stage_inputs(msqoc_problem* p, const double* alpha, const double* W
     return MSQOC_OK;
 }
 
+// The same for an evaluation, whose kernels read arrays in this device's memory where they are (the
+// controls kernel copies the window states); others are copied and become null here.
+msqoc_status take_inputs(msqoc_problem* p, const double*& alpha, const double*& W, cudaStream_t s) {
+    if (!alpha || (p->nW > 0 && !W) || !in_place(alpha, sizeof(double)) || (p->nW > 0 && !in_place(W, sizeof(double2)))) {
+        const msqoc_status st = stage_inputs(p, alpha, W, s);
+        alpha = W = nullptr;
+        return st;
+    }
+    if (p->nW == 0) W = nullptr;
+    return MSQOC_OK;
+}
+
 // the histories, checkpoints and segment state, on the first gradient evaluation
 msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s) {
     if (p->hist) return MSQOC_OK;
@@ -1039,11 +1063,8 @@ SweepArgs prop_args(const SweepPlan& plan, const ProbDev& pd, const ProbDev* pds
 }
 cudaError_t launch_compose(const ProbDev* pds_dev, const int* list, int E, int M, int nprob, int N, bool bwd,
                            cudaStream_t s) {
-    if (bwd)
-        k_compose<true><<<dim3(E, M, nprob), compose_threads(N), 0, s>>>(pds_dev, list);
-    else
-        k_compose<false><<<dim3(E, M, nprob), compose_threads(N), 0, s>>>(pds_dev, list);
-    return cudaGetLastError();
+    return launch_chained(bwd ? k_compose<true> : k_compose<false>, dim3(E, M, nprob), compose_threads(N), 0, s, pds_dev,
+                          list);
 }
 
 // blocks of 256 threads for the phase table (grid-stride loop)
@@ -1054,11 +1075,14 @@ int phase_blocks(const ProbDev& pd) {
 int control_blocks(const ProbDev& pd) {
     return static_cast<int>(std::min<int64_t>((pd.nsteps + CTRL_THREADS - 3) / (CTRL_THREADS - 2), 8192));
 }
-msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s) {
-    const ProbDev& pd = p->pd;
+msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s, const double* alpha, const double* W) {
+    ProbDev pd = p->pd;
+    if (alpha) pd.alpha = alpha;
     Mark mk(p, MSQOC_KERNEL_CONTROLS, s);
-    k_controls<<<control_blocks(pd), CTRL_THREADS, 0, s>>>(pd, pair);
-    CUDA_TRY(cudaGetLastError());
+    const size_t nW = W ? p->nW / 2 : 0;
+    const int nctrl = control_blocks(pd), ncopy = static_cast<int>(std::min<size_t>((nW + 4 * CTRL_THREADS - 1) / (4 * CTRL_THREADS), 4096));
+    CUDA_TRY(launch_chained(k_controls, nctrl + ncopy, CTRL_THREADS, 0, s, pd, pair, nctrl,
+                            reinterpret_cast<const double2*>(W), reinterpret_cast<double2*>(p->W_dev), nW));
     return MSQOC_OK;
 }
 
@@ -1066,15 +1090,13 @@ msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s) {
 int terminal_threads(const ProbDev& pd) { return std::min(TERM_THREADS, (pd.N * pd.E + 31) / 32 * 32); }
 msqoc_status launch_terminal(msqoc_problem* p, bool want_lambda, cudaStream_t s) {
     Mark mk(p, MSQOC_KERNEL_TERMINAL, s);
-    k_terminal<<<p->pd.M, terminal_threads(p->pd), 0, s>>>(p->pd, want_lambda ? 1 : 0);
-    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(launch_chained(k_terminal, p->pd.M, terminal_threads(p->pd), 0, s, p->pd, want_lambda ? 1 : 0));
     return MSQOC_OK;
 }
 
 msqoc_status launch_objective_outputs(msqoc_problem* p, double* P, double* J, double* pen, cudaStream_t s) {
     Mark mk(p, MSQOC_KERNEL_FINALIZE, s);
-    k_objective_outputs<<<1, OUT_THREADS, 0, s>>>(p->pd, P, J, p->npen > 0 ? pen : nullptr);
-    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(launch_chained(k_objective_outputs, 1, OUT_THREADS, 0, s, p->pd, P, J, p->npen > 0 ? pen : nullptr));
     return MSQOC_OK;
 }
 
@@ -1083,16 +1105,15 @@ msqoc_status launch_gradient_outputs(msqoc_problem* p, double* P, double* ga, do
     Mark mk(p, MSQOC_KERNEL_FINALIZE, s);
     const size_t total = p->nWs > 0 ? p->ne * size_t(p->nWs) : 0;
     const int wblocks = static_cast<int>(std::min<size_t>((total + OUT_THREADS - 1) / OUT_THREADS, 8192));
-    k_gradient_outputs<<<1 + pd.nfsum * pd.d1 + wblocks, OUT_THREADS, 0, s>>>(
-        pd, P, ga, reinterpret_cast<double2*>(gw), wblocks, p->nWs);
-    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(launch_chained(k_gradient_outputs, 1 + pd.nfsum * pd.d1 + wblocks, OUT_THREADS, 0, s, pd, P, ga,
+                            reinterpret_cast<double2*>(gw), wblocks, p->nWs));
     return MSQOC_OK;
 }
 
 // controls, forward sweep over whole windows, terminal conditions
-msqoc_status launch_forward_part(msqoc_problem* p, int mode, cudaStream_t s) {
+msqoc_status launch_forward_part(msqoc_problem* p, int mode, cudaStream_t s, const double* alpha, const double* W) {
     for (bool& r : p->ran) r = false;
-    msqoc_status st = launch_controls(p, p->pd.pair, s);
+    msqoc_status st = launch_controls(p, p->pd.pair, s, alpha, W);
     if (st) return st;
     {
         Mark mk(p, MSQOC_KERNEL_FORWARD, s);
@@ -1137,9 +1158,9 @@ msqoc_status msqoc_eval_objective(msqoc_problem* p, const double* alpha, const d
     if (!p) return fail(MSQOC_ERR_INVALID_ARG, "problem is NULL");
     if (!P_out) return fail(MSQOC_ERR_INVALID_ARG, "P_out is NULL");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    msqoc_status st = stage_inputs(p, alpha, W, s);
+    msqoc_status st = take_inputs(p, alpha, W, s);
     if (st) return st;
-    st = launch_forward_part(p, SWEEP_OBJECTIVE, s);
+    st = launch_forward_part(p, SWEEP_OBJECTIVE, s, alpha, W);
     if (st) return st;
     const bool dP = is_device_ptr(P_out), dJ = !J_out || is_device_ptr(J_out), dpen = !pen_out || is_device_ptr(pen_out);
     double* o = p->out_dev;
@@ -1163,12 +1184,12 @@ msqoc_status msqoc_eval_gradient(msqoc_problem* p, const double* alpha, const do
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     msqoc_status st = ensure_gradient_buffers(p, s);
     if (st) return st;
-    st = stage_inputs(p, alpha, W, s);
+    st = take_inputs(p, alpha, W, s);
     if (st) return st;
     const ProbDev& pd = p->pd;
     // one history segment: every midpoint state in the forward sweep; otherwise checkpoints
     // at the segment starts, and each segment is recomputed before its adjoint sweep
-    st = launch_forward_part(p, SWEEP_HISTORY, s);
+    st = launch_forward_part(p, SWEEP_HISTORY, s, alpha, W);
     if (st) return st;
     {
         Mark mk(p, MSQOC_KERNEL_ADJOINT, s);
@@ -1210,12 +1231,15 @@ msqoc_status msqoc_rollout(msqoc_problem* p, const double* alpha, double* W_out,
     if (!alpha) return fail(MSQOC_ERR_INVALID_ARG, "alpha is NULL");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (p->pd.M == 1) return MSQOC_OK;
-    CUDA_TRY(cudaMemcpyAsync(p->alpha_dev, alpha, p->pd.d * sizeof(double), cudaMemcpyDefault, s));
+    if (!in_place(alpha, sizeof(double))) {
+        CUDA_TRY(cudaMemcpyAsync(p->alpha_dev, alpha, p->pd.d * sizeof(double), cudaMemcpyDefault, s));
+        alpha = nullptr;
+    }
     msqoc_status st;
     const bool dev = is_device_ptr(W_out) && reinterpret_cast<uintptr_t>(W_out) % 16 == 0;
     double* dst = dev ? W_out : p->out_dev + out_layout(p->npen, p->pd.d, p->nW).gw;
     for (bool& r : p->ran) r = false;
-    if ((st = launch_controls(p, 0, s))) return st;   // (propagators: one thread per fiber)
+    if ((st = launch_controls(p, 0, s, alpha, nullptr))) return st;   // (propagators: one thread per fiber)
     {
         // batches of windows whose propagators fit the buffer: their sweep, then the chain
         Mark mk(p, MSQOC_KERNEL_FORWARD, s);
@@ -1227,9 +1251,8 @@ msqoc_status msqoc_rollout(msqoc_problem* p, const double* alpha, double* W_out,
             const int nw = std::min(p->ro_windows, pd.M - 1 - w0);
             a.voff = w0 * p->ro_slices;
             CUDA_TRY(launch_sweep(a, p->ro.ntiles, s));
-            k_compose_rollout<<<pd.E, compose_threads(pd.N), 0, s>>>(pd, p->phi_ro, p->ro_slices, w0, nw,
-                                                                     reinterpret_cast<double2*>(dst));
-            CUDA_TRY(cudaGetLastError());
+            CUDA_TRY(launch_chained(k_compose_rollout, pd.E, compose_threads(pd.N), 0, s, pd, p->phi_ro, p->ro_slices, w0,
+                                    nw, reinterpret_cast<double2*>(dst)));
         }
     }
     if (dev) return MSQOC_OK;
@@ -1245,8 +1268,7 @@ msqoc_status msqoc_rollout_estimate(msqoc_problem* p, double* est_out, void* str
     const bool dev = is_device_ptr(est_out);
     // a spare slot at the end of the output staging (the other slots hold the last results)
     double* dst = dev ? est_out : p->out_dev + out_layout(p->npen, p->pd.d, p->nW).total - 1;
-    k_rollout_estimate<<<1, OUT_THREADS, 0, s>>>(p->pd, dst);
-    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(launch_chained(k_rollout_estimate, 1, OUT_THREADS, 0, s, p->pd, dst));
     if (dev) return MSQOC_OK;
     CUDA_TRY(cudaMemcpyAsync(est_out, dst, sizeof(double), cudaMemcpyDeviceToHost, s));
     return check_status_sync(p, s);
@@ -1268,10 +1290,10 @@ msqoc_status msqoc_eval_regularization(msqoc_problem* p, const double* alpha, do
     const bool dR = is_device_ptr(R_out);
     const bool dg = grad_alpha && is_device_ptr(grad_alpha);
     CUDA_TRY(cudaMemcpyAsync(a, alpha, pd.d * sizeof(double), cudaMemcpyDefault, s));
-    k_regularization<<<pd.q * pd.d1, REG_THREADS, 0, s>>>(pd, a, gamma_tik, gamma_energy, dg ? grad_alpha : g, ep);
-    CUDA_TRY(cudaGetLastError());
-    k_regularization_total<<<1, REG_THREADS, 0, s>>>(pd, a, gamma_tik, gamma_energy, ep, dR ? R_out : R);
-    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(launch_chained(k_regularization, pd.q * pd.d1, REG_THREADS, 0, s, pd, a, gamma_tik, gamma_energy,
+                            dg ? grad_alpha : g, ep));
+    CUDA_TRY(launch_chained(k_regularization_total, 1, REG_THREADS, 0, s, pd, a, gamma_tik, gamma_energy, ep,
+                            dR ? R_out : R));
     if (dR && (dg || !grad_alpha)) return MSQOC_OK;
     if (!dR) CUDA_TRY(cudaMemcpyAsync(R_out, R, sizeof(double), cudaMemcpyDeviceToHost, s));
     if (grad_alpha && !dg) CUDA_TRY(cudaMemcpyAsync(grad_alpha, g, pd.d * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1588,7 +1610,7 @@ msqoc_status eval_objective_noalloc(const msqoc_hamiltonian* H, const msqoc_cont
         const int threads = 256;
         k_phases<<<phase_blocks(pd), threads, 0, s>>>(pd);
         CUDA_TRY(cudaGetLastError());
-        k_controls<<<control_blocks(pd), CTRL_THREADS, 0, s>>>(pd, pd.pair);
+        k_controls<<<control_blocks(pd), CTRL_THREADS, 0, s>>>(pd, pd.pair, control_blocks(pd), nullptr, nullptr, 0);
         CUDA_TRY(cudaGetLastError());
     }
     CUDA_TRY(launch_sweep(sweep_args(pd, pd_d, tiles_d, map_d, SWEEP_OBJECTIVE, 0), pd.ntiles, s));

@@ -2,6 +2,7 @@
 // deterministic final reductions.
 #pragma once
 
+#include "msqoc_chain.cuh"
 #include "msqoc_internal.h"
 #include "msqoc_split.cuh"
 
@@ -105,12 +106,22 @@ __device__ __forceinline__ double2 control_at(const ProbDev& pd, int64_t n, int 
     return dk;
 }
 constexpr int CTRL_THREADS = 128;
-__global__ void __launch_bounds__(CTRL_THREADS) k_controls(const ProbDev pd, const int pair) {
+// Blocks nctrl and up copy the window states, nW entries of Wsrc, to Wdst (the caller's device
+// arrays are read in place of a copy of their own ahead of this kernel; pd.alpha is the caller's).
+__global__ void __launch_bounds__(CTRL_THREADS) k_controls(const ProbDev pd, const int pair, const int nctrl,
+                                                           const double2* Wsrc, double2* Wdst, const size_t nW) {
+    chain_wait();
+    chain_next();
+    if (blockIdx.x >= nctrl) {
+        const size_t stride = size_t(gridDim.x - nctrl) * CTRL_THREADS;
+        for (size_t e = size_t(blockIdx.x - nctrl) * CTRL_THREADS + threadIdx.x; e < nW; e += stride) Wdst[e] = Wsrc[e];
+        return;
+    }
     // a block takes CTRL_THREADS - 2 steps and one more on either side (the changes of the controls
     // over a step, in FP32)
     __shared__ float2 ds[MAXQ][CTRL_THREADS];
     const int64_t per = CTRL_THREADS - 2;
-    for (int64_t n0 = int64_t(blockIdx.x) * per; n0 < pd.nsteps; n0 += int64_t(gridDim.x) * per) {
+    for (int64_t n0 = int64_t(blockIdx.x) * per; n0 < pd.nsteps; n0 += int64_t(nctrl) * per) {
         const int t = threadIdx.x;
         const int64_t n = min(max(n0 + t - 1, int64_t(0)), pd.nsteps - 1);
         const bool own = t >= 1 && t <= per && n0 + t - 1 < pd.nsteps;
@@ -310,6 +321,7 @@ __device__ __forceinline__ void compose_chain(int N, int links, double2* xs, Phi
 template <bool BWD>
 __global__ void __launch_bounds__(COMPOSE_THREADS) k_compose(const ProbDev* pds, const int* list) {
     __shared__ double2 xs[2 * 256];
+    chain_wait();
     const ProbDev& pd = pds[list ? list[blockIdx.z] : blockIdx.z];
     const int col = blockIdx.x, m = blockIdx.y, N = pd.N, E = pd.E, C = pd.C;
     if (C == 1 || m >= pd.M || col >= E) return;
@@ -326,6 +338,7 @@ __global__ void __launch_bounds__(COMPOSE_THREADS) k_compose(const ProbDev* pds,
     compose_chain<BWD>(
         N, C, xs, [&](int s) { return Phi + slice(s) * N * N; },
         [&](int s, const double2* x) {
+            if (s == C - 1) chain_next();
             double2* dst = s < C ? keep + (slice(s) * E + col) * N : end + wcol;
             for (int i = threadIdx.x; i < N; i += blockDim.x) dst[i] = x[i];
         });
@@ -336,6 +349,7 @@ __global__ void __launch_bounds__(COMPOSE_THREADS) k_compose(const ProbDev* pds,
 __global__ void __launch_bounds__(COMPOSE_THREADS) k_compose_rollout(const ProbDev pd, const double2* Phi, int C, int w0,
                                                                      int nw, double2* W) {
     __shared__ double2 xs[2 * 256];
+    chain_wait();
     const int col = blockIdx.x, N = pd.N, E = pd.E;
     for (int i = threadIdx.x; i < N; i += blockDim.x)
         xs[i] = w0 == 0 ? make_double2(pd.emb[col] == i ? 1.0 : 0.0, 0.0) : W[(size_t(w0 - 1) * E + col) * N + i];
@@ -344,6 +358,7 @@ __global__ void __launch_bounds__(COMPOSE_THREADS) k_compose_rollout(const ProbD
     compose_chain<false>(
         N, links, xs, [&](int s) { return Phi + size_t(s) * N * N; },
         [&](int s, const double2* x) {
+            if (s == links - 1) chain_next();
             if (s == 0 || s % C) return;
             double2* dst = W + (size_t(w0 + s / C - 1) * E + col) * N;
             for (int i = threadIdx.x; i < N; i += blockDim.x) dst[i] = x[i];
@@ -358,6 +373,8 @@ constexpr int TERM_THREADS = 256;
 // (m and M global: a shard's last window is the problem's last only when it ends the grid)
 __global__ void __launch_bounds__(TERM_THREADS) k_terminal(const ProbDev pd, const int want_lambda) {
     __shared__ double sh[3 * TERM_THREADS / 32];
+    chain_wait();
+    chain_next();
     const int m = blockIdx.x + 1;
     const size_t ne = size_t(pd.N) * pd.E;
     const double2* U = pd.Uend + size_t(m - 1) * ne;
@@ -420,6 +437,8 @@ __device__ __forceinline__ void objective_outputs(const ProbDev& pd, double* P_o
 __global__ void __launch_bounds__(OUT_THREADS) k_objective_outputs(const ProbDev pd, double* P_out, double* J_out,
                                                                     double* pen_out) {
     __shared__ double sh[2 * OUT_THREADS / 32];
+    chain_wait();
+    chain_next();
     objective_outputs(pd, P_out, J_out, pen_out, sh);
 }
 
@@ -428,6 +447,8 @@ __global__ void __launch_bounds__(OUT_THREADS) k_objective_outputs(const ProbDev
 // with n := E (as in the generalized infidelity).  One block, fixed order (deterministic).
 __global__ void __launch_bounds__(OUT_THREADS) k_rollout_estimate(const ProbDev pd, double* est) {
     __shared__ double sh[2 * OUT_THREADS / 32];
+    chain_wait();
+    chain_next();
     double S = 0.0;
     for (int m = 1 + threadIdx.x; m < pd.M; m += OUT_THREADS) S += sqrt(2.0 * pd.term[m - 1] / pd.mu);
     S = block_sum(S, sh);
@@ -453,6 +474,8 @@ __global__ void __launch_bounds__(OUT_THREADS) k_rollout_estimate(const ProbDev 
 __global__ void __launch_bounds__(OUT_THREADS) k_gradient_outputs(const ProbDev pd, double* P_out, double* ga,
                                                                    double2* gW, int wblocks, int nstates) {
     __shared__ double sh[2 * OUT_THREADS / 32];
+    chain_wait();
+    chain_next();
     if (blockIdx.x == 0) {
         objective_outputs(pd, P_out, nullptr, nullptr, sh);
         return;
@@ -523,6 +546,8 @@ __global__ void __launch_bounds__(REG_THREADS) k_regularization(const ProbDev pd
                                                                  double gamma_tik, double gamma_energy,
                                                                  double* grad, double* epart) {
     __shared__ double sh[REG_THREADS / 32];
+    chain_wait();
+    chain_next();
     const int k = blockIdx.x / pd.d1, s = blockIdx.x % pd.d1;
     // steps whose midpoint lies in [(s - 2) dtau, (s + 1) dtau), widened by two steps on each side
     // (membership is decided exactly by spline_at below)
@@ -587,6 +612,8 @@ __global__ void __launch_bounds__(REG_THREADS) k_regularization_total(const Prob
                                                                        double gamma_tik, double gamma_energy,
                                                                        const double* epart, double* R) {
     __shared__ double sh[REG_THREADS / 32];
+    chain_wait();
+    chain_next();
     double a2 = 0.0, en = 0.0;
     for (int i = threadIdx.x; i < pd.d; i += REG_THREADS) a2 += alpha[i] * alpha[i];
     for (int i = threadIdx.x; i < pd.q * pd.d1; i += REG_THREADS) en += epart[i];

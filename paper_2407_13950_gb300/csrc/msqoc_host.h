@@ -141,7 +141,9 @@ msqoc_status stage_inputs(msqoc_problem* p, const double* alpha, const double* W
 msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s);
 int phase_blocks(const ProbDev& pd);   // blocks of 256 threads for k_phases
 // pair: the kernel family of the sweeps that follow (its iteration counts)
-msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s);
+// alpha, W: the inputs' device arrays where they are not the problem's own copies (null: they are)
+msqoc_status launch_controls(msqoc_problem* p, int pair, cudaStream_t s, const double* alpha = nullptr,
+                             const double* W = nullptr);
 msqoc_status launch_terminal(msqoc_problem* p, bool want_lambda, cudaStream_t s);
 // P, J (may be NULL), pen (may be NULL) of the last forward sweep into device arrays
 msqoc_status launch_objective_outputs(msqoc_problem* p, double* P, double* J, double* pen, cudaStream_t s);

@@ -24,6 +24,7 @@
 // products; below 32 the parts of a warp take alternate groups of pairs.
 #pragma once
 
+#include "msqoc_chain.cuh"
 #include <type_traits>
 
 #include "msqoc_sweep_common.cuh"
@@ -110,6 +111,7 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
     constexpr bool SPLIT = MODE > 0;
     using GT = std::conditional_t<MODE == 1, DF, double>;
     using ET = std::conditional_t<SPLIT, float4, double2>;
+    chain_wait();
     const ProbDev& pd = a.pds[a.list ? a.list[blockIdx.y] : blockIdx.y];
     const int E = pd.E;
     const int EL = E >= LN ? LN : (E <= 1 ? 1 : 1 << (32 - __clz(E - 1)));
@@ -210,6 +212,7 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
         }
     }
 
+    chain_next();
     // ---- sums over the step's lanes and the warp's parts, weighted, then over the warps, fixed order
     for (int o = EL >> 1; o > 0; o >>= 1) {
         A = gsum_add(A, gsum_shfl_xor(A, o));

@@ -32,6 +32,7 @@
 // sweeps a step; at 64 windows 6.97 -> 5.52 ms.
 #pragma once
 
+#include "msqoc_chain.cuh"
 #include <climits>
 
 #include "msqoc_sweep_common.cuh"
@@ -358,7 +359,10 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     // nothing to recompute; a sliced problem's objective comes from its propagators
     const bool idle_launch = !PROP && ((mode == SWEEP_RECOMPUTE && pd.nseg == 1) ||
                                        (mode == SWEEP_OBJECTIVE && C > 1));
-    if (idle_launch) return;
+    if (idle_launch) {
+        chain_wait();
+        return;
+    }
     const int v0 = tile.m0 + (PROP ? a.voff : 0);   // the first slot's virtual window, 1-based
 
     // ---- the slots' windows and step ranges (local step indices [lo, lo + cnt) of the window)
@@ -450,6 +454,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
         }
     }
 
+    chain_wait();   // (ahead of it: the tables of the problem's creation, and shared memory)
     // ---- initial state
     //   propagator            : unit vectors; a sliced problem: the slice's Ubeg, Lend (k_compose)
     //   forward, whole window : U^m(t_{m-1}) = W^{m-1} (identity embedding for the first window
@@ -561,6 +566,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     for (int jj = 0; jj < nit; ++jj) {
         const int par = jj & 1;
         const bool live = jj < my_cnt;
+        if (jj == nit - 1) chain_next();
         if (coef_warp) {
             const float4 dk = cf_next;
             const int cnt = cnt_next;

@@ -18,6 +18,7 @@
 // budget cost the adjoint 2-4%).
 #pragma once
 
+#include "msqoc_chain.cuh"
 #include <climits>
 
 #include "msqoc_sweep_common.cuh"
@@ -163,6 +164,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     constexpr int NSLOT = Q * L * 2;
     constexpr int S = BWD ? +1 : -1;       // sign of the preconditioned off-diagonal term
 
+    chain_wait();
     const Tile tile = a.tiles[blockIdx.x];
     const ProbDev& pd = a.pds[tile.prob];
 
