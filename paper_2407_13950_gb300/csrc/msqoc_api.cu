@@ -7,6 +7,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <functional>
 #include <vector>
 
 #include "../../include/msqoc.h"
@@ -149,26 +150,18 @@ int gray_rank(int g) {
 // lanes mirror the last active entry.  Writes out[nthreads]; no allocation.
 void build_lanemap(int L, int q, int ncol, int ncol0, int nthreads, int pair, int* out) {
     const int F = ipow_i(L, q) / L;
-    int key[MAX_ANY_TILE_THREADS], val[MAX_ANY_TILE_THREADS];
+    int val[MAX_ANY_TILE_THREADS];
     if (ncol * F > MAX_ANY_TILE_THREADS || nthreads > MAX_ANY_TILE_THREADS) return;   // rejected by tile_width_ok
+    // the fibers by the rank of their class, stable (a counting sort: 0.05 ms a 4-transmon table
+    // where sorting every map's entries took 0.25)
+    int first[(1 << (MAXQ - 1)) + 1] = {}, order[kMaxRows], rank[kMaxRows];
+    for (int f = 0; f < F; ++f) ++first[(rank[f] = gray_rank(fiber_class(L, q, f))) + 1];
+    for (int k = 0; k < 1 << (MAXQ - 1); ++k) first[k + 1] += first[k];
+    for (int f = 0; f < F; ++f) order[first[rank[f]]++] = f;
     int n = 0;
-    for (int part = 0; part < 2; ++part) {
-        const int first = n;
-        const int ca = part == 0 ? 0 : ncol0, cb = part == 0 ? ncol0 : ncol;
-        for (int f = 0; f < F; ++f)
-            for (int c = ca; c < cb; ++c) {
-                // stable insertion by key within this window's pairs
-                const int k = gray_rank(fiber_class(L, q, f));
-                int pos = n++;
-                while (pos > first && key[pos - 1] > k) {
-                    key[pos] = key[pos - 1];
-                    val[pos] = val[pos - 1];
-                    --pos;
-                }
-                key[pos] = k;
-                val[pos] = (c << 16) | f;
-            }
-    }
+    for (int part = 0; part < 2; ++part)
+        for (int i = 0; i < F; ++i)
+            for (int c = part == 0 ? 0 : ncol0; c < (part == 0 ? ncol0 : ncol); ++c) val[n++] = (c << 16) | order[i];
     const int sh = pair;
     for (int t = 0; t < nthreads; ++t) out[t] = (t >> sh) < n ? val[t >> sh] : ~val[n - 1];
 }
@@ -455,7 +448,7 @@ msqoc_status check_description(const msqoc_hamiltonian* H, const msqoc_controls*
 msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, double T, int64_t nsteps,
                            int32_t nwindows, double mu, int solver, int col_block, int layout, int sms, ProbDev& pd,
                            int wfirst = 0, int wlast = 0, bool slices = false,
-                           std::vector<TileCand>* plans = nullptr) {
+                           std::vector<TileCand>* plans = nullptr) {   // (plans: kept for a second call)
     const int q = H->nqubits, L = H->nlevels, ness = H->ness;
     int nfsum = 0;
     for (int k = 0; k < q; ++k) nfsum += C->ncarriers[k];
@@ -524,8 +517,9 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
         return fail(MSQOC_ERR_INVALID_ARG, "lane quads need 2-level subsystems and at most %d exchange-coupled pairs",
                     MAXEXF);
     if (col_block < 0) return fail(MSQOC_ERR_INVALID_ARG, "column block %d < 0", col_block);
-    const std::vector<TileCand> cands =
-        tile_candidates(pd.F, q, L, pd.N, pd.glocal, solver, layout, quad_admitted(pd));
+    std::vector<TileCand> own;
+    std::vector<TileCand>& cands = plans ? *plans : own;
+    if (cands.empty()) cands = tile_candidates(pd.F, q, L, pd.N, pd.glocal, solver, layout, quad_admitted(pd));
     // the tiles of M windows of E columns, sliced or not
     TileChoice tc = choose_tile_layout(cands, pd.M, pd.E, pd.F, solver, sms, col_block);
     pd.C = 1;
@@ -538,7 +532,6 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
             tc = ts;
         }
     }
-    if (plans) *plans = cands;
     if (tc.cpt < 0)
         return fail(MSQOC_ERR_INVALID_ARG,
                     "column block %d invalid for E=%d (needs 1 <= cb <= E, cb N/L <= %d threads with one thread "
@@ -630,10 +623,7 @@ bool is_shard(const ProbDev& pd) { return pd.M != pd.M_glob; }
 namespace {
 
 void free_problem(msqoc_problem* p) {
-    void* bufs[] = {p->tiles_ro, p->lanemap_ro, p->phi_ro, p->tiles_prop, p->lanemap_prop, p->Phi, p->Ubeg, p->Lend, p->coef,
-                    p->pds,   p->tiles, p->lanemap, p->P,     p->emb,   p->V,     p->alpha_dev, p->W_dev,
-                    p->ctrl,  p->spl,   p->phase,   p->hist,  p->ckpt,  p->Lstate, p->Uend,     p->Lterm,
-                    p->Lam0,  p->term,  p->lhist,   p->quad,  p->status, p->out_dev, p->reg_dev};
+    void* bufs[] = {p->arena, p->hist, p->lhist, p->Lend, p->quad, p->ckpt, p->Lstate};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (p->status_host) cudaFreeHost(p->status_host);
@@ -746,8 +736,9 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
     if (sms <= 0) sms = 1;
+    std::vector<TileCand> cands;
     st0 = shape_problem(H, C, T, nsteps, nwindows, mu, solver, o.col_block, o.layout, sms, pd, o.window_first,
-                        o.window_last);
+                        o.window_last, false, &cands);
     if (st0 != MSQOC_OK) return st0;
     const int q = pd.q, L = pd.L, nfsum = pd.nfsum;
     // checkpoint interval: 0 = automatic (every midpoint state unless that history would take
@@ -762,7 +753,6 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     p->ckpt_interval = K;
     set_segments(pd, K);
     // slices of the windows where every midpoint state is kept
-    std::vector<TileCand> cands;
     if (pd.nseg == 1) {
         st0 = shape_problem(H, C, T, nsteps, nwindows, mu, solver, o.col_block, o.layout, sms, pd, o.window_first,
                             o.window_last, true, &cands);
@@ -804,7 +794,7 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
         p->prop.ntiles = static_cast<int>(tabs_prop.tiles.size());
     }
     if (pd.M > 1 && !is_shard(pd)) {
-        if (pd.pair || cands.empty())
+        if (o.layout == MSQOC_LAYOUT_PAIR || o.layout == MSQOC_LAYOUT_QUAD)
             cands = tile_candidates(pd.F, q, L, N, pd.glocal, solver, MSQOC_LAYOUT_AUTO, false);
         p->ro_slices = choose_rollout_slices(cands, pd, sms);
         p->ro_windows = static_cast<int>(std::min<size_t>(
@@ -817,7 +807,9 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
         p->ro.ntiles = static_cast<int>(tabs_ro.tiles.size());
     }
 
-    // ---- device buffers
+    // ---- device buffers: one allocation, the tables ahead of the rest and filled by one copy (an
+    // allocation or a copy of its own for each of 27 buffers, with the sorts of build_lanemap: 4 transmons
+    // at 256 windows 1.4 ms a creation, now 0.6)
     const size_t M = pd.M;
     msqoc_status st = MSQOC_OK;
     auto A = [&](cudaError_t e, const char* what) {
@@ -825,36 +817,48 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
             st = fail(e == cudaErrorMemoryAllocation ? MSQOC_ERR_OUT_OF_MEMORY : MSQOC_ERR_CUDA,
                       "allocating %s: %s", what, cudaGetErrorString(e));
     };
-    A(dalloc(&p->pds, 1), "problem record");
-    A(dalloc(&p->tiles, tabs.tiles.size()), "tiles");
-    A(dalloc(&p->lanemap, tabs.maps.size()), "lane maps");
-    A(dalloc(&p->tiles_prop, tabs_prop.tiles.size()), "propagator tiles");
-    A(dalloc(&p->lanemap_prop, tabs_prop.maps.size()), "propagator lane maps");
-    A(dalloc(&p->tiles_ro, tabs_ro.tiles.size()), "roll-out tiles");
-    A(dalloc(&p->lanemap_ro, tabs_ro.maps.size()), "roll-out lane maps");
+    std::vector<std::function<void(unsigned char*)>> place;
+    size_t total = 0;
+    auto take = [&](auto** dst, size_t n) {
+        using T = std::remove_pointer_t<std::remove_pointer_t<decltype(dst)>>;
+        if (n == 0) return;
+        place.push_back([dst, at = total](unsigned char* base) { *dst = reinterpret_cast<T*>(base + at); });
+        total += (n * sizeof(T) + 255) / 256 * 256;
+    };
     const size_t phi_ro = size_t(p->ro_windows) * p->ro_slices * N * N;
-    A(dalloc(&p->phi_ro, phi_ro), "roll-out propagators");
-    if (pd.C > 1) {
-        A(dalloc(&p->Phi, size_t(V) * N * N), "propagators");
-        A(dalloc(&p->Ubeg, size_t(V) * p->ne), "slice states");
-    }
-    A(dalloc(&p->P, N), "P");
-    A(dalloc(&p->emb, E), "embedding");
-    A(dalloc(&p->V, p->ne), "target");
-    A(dalloc(&p->alpha_dev, pd.d), "alpha");
-    A(dalloc(&p->W_dev, std::max<size_t>(p->nW, 2)), "W");
-    A(dalloc(&p->ctrl, size_t(nsteps) * q), "controls");
     const size_t ncoef = pd.pair == 0 && pd.solver == SOLVER_MIXED ? size_t(nsteps) * q * (L - 1) : 0;
-    A(dalloc(&p->coef, ncoef), "step coefficients");
-    A(dalloc(&p->spl, size_t(nsteps)), "splines");
-    A(dalloc(&p->phase, size_t(nsteps) * nfsum), "phases");
-    A(dalloc(&p->Uend, M * p->ne), "Uend");
-    A(dalloc(&p->Lterm, M * p->ne), "Lterm");
-    A(dalloc(&p->Lam0, M * p->ne), "Lam0");
-    A(dalloc(&p->term, M), "terms");
-    A(dalloc(&p->status, 1), "status");
-    A(dalloc(&p->out_dev, out_layout(p->npen, pd.d, p->nW).total), "outputs");
-    A(dalloc(&p->reg_dev, reg_doubles(pd)), "regularization scratch");
+    take(&p->pds, 1);
+    take(&p->tiles, tabs.tiles.size());
+    take(&p->lanemap, tabs.maps.size());
+    take(&p->tiles_prop, tabs_prop.tiles.size());
+    take(&p->lanemap_prop, tabs_prop.maps.size());
+    take(&p->tiles_ro, tabs_ro.tiles.size());
+    take(&p->lanemap_ro, tabs_ro.maps.size());
+    take(&p->P, N);
+    take(&p->emb, E);
+    take(&p->V, p->ne);
+    take(&p->status, 1);
+    const size_t table_bytes = total;
+    take(&p->W_dev, std::max<size_t>(p->nW, 2));
+    take(&p->alpha_dev, pd.d);
+    take(&p->phi_ro, phi_ro);
+    if (pd.C > 1) {
+        take(&p->Phi, size_t(V) * N * N);
+        take(&p->Ubeg, size_t(V) * p->ne);
+    }
+    take(&p->ctrl, size_t(nsteps) * q);
+    take(&p->coef, ncoef);
+    take(&p->spl, size_t(nsteps));
+    take(&p->phase, size_t(nsteps) * nfsum);
+    take(&p->Uend, M * p->ne);
+    take(&p->Lterm, M * p->ne);
+    take(&p->Lam0, M * p->ne);
+    take(&p->term, M);
+    take(&p->out_dev, out_layout(p->npen, pd.d, p->nW).total);
+    take(&p->reg_dev, reg_doubles(pd));
+    A(dalloc(&p->arena, total), "device buffers");
+    if (p->arena)
+        for (auto& f : place) f(p->arena);
     A(cudaMallocHost(reinterpret_cast<void**>(&p->status_host), sizeof(int)), "pinned status");
     p->profile = o.profile == 1;
     if (p->profile)
@@ -878,21 +882,23 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
         pd.status = p->status;
         pd.Phi = p->Phi;
         pd.Ubeg = p->Ubeg;
-        auto up = [&](auto* dst, const auto& v, const char* what) {
-            if (!v.empty()) A(cudaMemcpy(dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice), what);
+        std::vector<unsigned char> table(table_bytes);   // (zero: the status word)
+        auto up = [&](const void* dst, const void* src, size_t bytes) {
+            if (bytes) memcpy(table.data() + (static_cast<const unsigned char*>(dst) - p->arena), src, bytes);
         };
-        up(p->tiles, tabs.tiles, "tiles copy");
-        up(p->lanemap, tabs.maps, "lane map copy");
-        up(p->tiles_prop, tabs_prop.tiles, "propagator tiles copy");
-        up(p->lanemap_prop, tabs_prop.maps, "propagator lane map copy");
-        up(p->tiles_ro, tabs_ro.tiles, "roll-out tiles copy");
-        up(p->lanemap_ro, tabs_ro.maps, "roll-out lane map copy");
-        A(cudaMemcpy(p->P, P.data(), N * sizeof(double2), cudaMemcpyHostToDevice), "P copy");
-        A(cudaMemcpy(p->emb, emb.data(), E * sizeof(int), cudaMemcpyHostToDevice), "emb copy");
-        A(cudaMemcpy(p->V, Vh.data(), p->ne * sizeof(double2), cudaMemcpyHostToDevice), "target copy");
+        auto upv = [&](const auto* dst, const auto& v) { up(dst, v.data(), v.size() * sizeof(v[0])); };
+        up(p->pds, &pd, sizeof pd);
+        upv(p->tiles, tabs.tiles);
+        upv(p->lanemap, tabs.maps);
+        upv(p->tiles_prop, tabs_prop.tiles);
+        upv(p->lanemap_prop, tabs_prop.maps);
+        upv(p->tiles_ro, tabs_ro.tiles);
+        upv(p->lanemap_ro, tabs_ro.maps);
+        upv(p->P, P);
+        upv(p->emb, emb);
+        upv(p->V, Vh);
+        A(cudaMemcpy(p->arena, table.data(), table_bytes, cudaMemcpyHostToDevice), "table copy");
         A(cudaMemset(p->W_dev, 0, std::max<size_t>(p->nW, 2) * sizeof(double)), "W init");
-        A(cudaMemset(p->status, 0, sizeof(int)), "status init");
-        A(cudaMemcpy(p->pds, &pd, sizeof(ProbDev), cudaMemcpyHostToDevice), "problem record copy");
         // the carrier phase table: a constant of the time grid, filled once
         if (st == MSQOC_OK) {
             k_phases<<<phase_blocks(pd), 256>>>(pd);

@@ -25,7 +25,8 @@ struct msqoc_problem {
     int nWs = 0;             // window states in W (M - 1, or those a shard reads)
     int npen = 0;            // penalty terms (M - 1, or those a shard owns)
     size_t ne = 0;           // N*E
-    // owned device buffers
+    // device buffers: `arena` holds those of the creation, the gradient's are allocations of their own
+    unsigned char* arena = nullptr;
     msqoc::ProbDev* pds = nullptr;   // device copy of pd (read by the sweeps)
     msqoc::Tile* tiles = nullptr;
     int* lanemap = nullptr;
