@@ -785,7 +785,21 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     const int V = pd.M * pd.C;   // (virtual) windows of the sweeps
     const TileTables tabs = tile_tables(L, q, V, E, pd.cb, pd.nthreads, pd.pair);
     // propagators of the slices, and of the roll-out's (one thread per fiber whatever the layout)
-    TileTables tabs_prop, tabs_ro;
+    TileTables tabs_prop, tabs_ro, tabs_both;
+    // A segment's recomputation and adjoint sweep do not depend on each other: one launch of both,
+    // in tiles for twice the windows, where the model has it faster than one after the other
+    // (4 transmons, 64 windows, checkpoints every 64 steps: 294 7-column lean tiles, two an SM, in
+    // place of 128 8-column tiles twice: 10.6 ms against 13.2 with the quadrature; at 16 windows, whose
+    // tiles fill neither launch, 4.5 against 8.0)
+    if (pd.nseg > 1 && pd.nsub == 1 && pd.pair == 0 && solver == SOLVER_MIXED && pd.hdepth == 1) {
+        const TileChoice t = choose_tile_layout(cands, 2 * pd.M, E, pd.F, solver, sms, o.col_block, true);
+        const TileChoice one = choose_tile_layout(cands, pd.M, E, pd.F, solver, sms, o.col_block);
+        if (t.cpt > 0 && t.cost < 2.0 * one.cost - 1e-9) {
+            p->both = SweepPlan{t.cpt, tile_threads(t.cpt, pd.F, 0), t.lean, 0};
+            tabs_both = tile_tables(L, q, pd.M, E, t.cpt, p->both.nthreads, 0);
+            p->both.ntiles = static_cast<int>(tabs_both.tiles.size());
+        }
+    }
     if (pd.C > 1) {
         const TileChoice t = choose_tile_layout(cands, V, N, pd.F, solver, sms, 0, true);
         if (t.cpt < 0) return fail(MSQOC_ERR_INTERNAL, "no tiles for the propagators");
@@ -832,6 +846,8 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     take(&p->lanemap, tabs.maps.size());
     take(&p->tiles_prop, tabs_prop.tiles.size());
     take(&p->lanemap_prop, tabs_prop.maps.size());
+    take(&p->tiles_both, tabs_both.tiles.size());
+    take(&p->lanemap_both, tabs_both.maps.size());
     take(&p->tiles_ro, tabs_ro.tiles.size());
     take(&p->lanemap_ro, tabs_ro.maps.size());
     take(&p->P, N);
@@ -892,6 +908,8 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
         upv(p->lanemap, tabs.maps);
         upv(p->tiles_prop, tabs_prop.tiles);
         upv(p->lanemap_prop, tabs_prop.maps);
+        upv(p->tiles_both, tabs_both.tiles);
+        upv(p->lanemap_both, tabs_both.maps);
         upv(p->tiles_ro, tabs_ro.tiles);
         upv(p->lanemap_ro, tabs_ro.maps);
         upv(p->P, P);
@@ -909,8 +927,8 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     if (st != MSQOC_OK) return st;
     p->bytes = sizeof(double2) * (N + p->ne * (1 + 3 * M) + size_t(nsteps) * (q + nfsum)) +
                sizeof(Spline4) * size_t(nsteps) + sizeof(double) * (pd.d + p->nW + M + out_layout(p->npen, pd.d, p->nW).total + reg_doubles(pd)) +
-               sizeof(int) * (E + 1 + tabs.maps.size() + tabs_prop.maps.size() + tabs_ro.maps.size()) +
-               sizeof(Tile) * (tabs.tiles.size() + tabs_prop.tiles.size() + tabs_ro.tiles.size()) +
+               sizeof(int) * (E + 1 + tabs.maps.size() + tabs_prop.maps.size() + tabs_both.maps.size() + tabs_ro.maps.size()) +
+               sizeof(Tile) * (tabs.tiles.size() + tabs_prop.tiles.size() + tabs_both.tiles.size() + tabs_ro.tiles.size()) +
                sizeof(double2) * phi_ro + sizeof(float4) * ncoef + slice_bytes(pd) + sizeof(ProbDev);
     p->grad_bytes = gradient_bytes(pd);
     *out = owner.release();
@@ -1057,15 +1075,19 @@ int compose_threads(int N) {
     const ComposeGeom g = compose_geom(N);
     return std::max(32, g.R * g.JG);
 }
-SweepArgs prop_args(const SweepPlan& plan, const ProbDev& pd, const ProbDev* pds_dev, const Tile* tiles,
-                    const int* lanemap) {
-    SweepArgs a = sweep_args(pd, pds_dev, tiles, lanemap, SWEEP_PROP, 0);
+SweepArgs plan_args(const SweepPlan& plan, const ProbDev& pd, const ProbDev* pds_dev, const Tile* tiles,
+                    const int* lanemap, int mode) {
+    SweepArgs a = sweep_args(pd, pds_dev, tiles, lanemap, mode, 0);
     a.cpt = plan.cpt;
     a.nthreads = plan.nthreads;
     a.lean = plan.lean;
     a.pair = 0;
     a.hdepth = 1;
     return a;
+}
+SweepArgs prop_args(const SweepPlan& plan, const ProbDev& pd, const ProbDev* pds_dev, const Tile* tiles,
+                    const int* lanemap) {
+    return plan_args(plan, pd, pds_dev, tiles, lanemap, SWEEP_PROP);
 }
 cudaError_t launch_compose(const ProbDev* pds_dev, const int* list, int E, int M, int nprob, int N, bool bwd,
                            cudaStream_t s) {
@@ -1201,6 +1223,13 @@ msqoc_status msqoc_eval_gradient(msqoc_problem* p, const double* alpha, const do
         Mark mk(p, MSQOC_KERNEL_ADJOINT, s);
         if (pd.C > 1) CUDA_TRY(launch_compose(p->pds, nullptr, pd.E, pd.M, 1, pd.N, true, s));
         for (int seg = pd.nseg - 1; seg >= 0; --seg) {
+            if (p->both.ntiles) {
+                SweepArgs a = plan_args(p->both, pd, p->pds, p->tiles_both, p->lanemap_both, SWEEP_BOTH);
+                a.seg = seg;
+                CUDA_TRY(launch_sweep(a, p->both.ntiles, s));
+                CUDA_TRY(launch_quad(quad_args(pd, p->pds, seg, 0), quad_blocks(pd), 1, s));
+                continue;
+            }
             if (pd.nseg > 1) {
                 st = sweep(p, SWEEP_RECOMPUTE, seg, s);
                 if (st) return st;

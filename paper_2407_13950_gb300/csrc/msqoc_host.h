@@ -33,6 +33,9 @@ struct msqoc_problem {
     msqoc::Tile* tiles_prop = nullptr;   // the propagator sweep of a sliced problem
     int* lanemap_prop = nullptr;
     msqoc::SweepPlan prop;
+    msqoc::Tile* tiles_both = nullptr;   // a segment's recomputation and adjoint in one launch
+    int* lanemap_both = nullptr;
+    msqoc::SweepPlan both;               // (ntiles = 0: two launches of the problem's tiles)
     msqoc::Tile* tiles_ro = nullptr;     // the roll-out's, for ro_windows windows of ro_slices slices
     int* lanemap_ro = nullptr;
     msqoc::SweepPlan ro;

@@ -865,13 +865,15 @@ template <int L, int Q, int SOLVER, bool BWD, bool PROP = false, int MAXT = MAX_
 __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
     sweep_tile<L, Q, SOLVER, BWD, PROP>(a, a.mode, blockIdx.x);
 }
-// The history and adjoint sweeps of sliced problems, which do not depend on each other: blocks
-// 0 .. n - 1 the forward tiles, n .. 2n - 1 the adjoint's.
+// The history sweep and the adjoint sweep in one launch, where neither needs the other: of a sliced
+// problem, or the recomputation and the adjoint of one checkpoint segment (the products of both
+// are k_quad's).  Blocks 0 .. n - 1 the forward tiles, n .. 2n - 1 the adjoint's.
 template <int L, int Q, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_sweep_both(const SweepArgs a) {
     const int n = gridDim.x / 2;
     if (blockIdx.x < n)
-        sweep_tile<L, Q, SOLVER_MIXED, false, false>(a, SWEEP_HISTORY, blockIdx.x);
+        sweep_tile<L, Q, SOLVER_MIXED, false, false>(a, a.pds[a.tiles[blockIdx.x].prob].nseg > 1 ? SWEEP_RECOMPUTE : SWEEP_HISTORY,
+                                                     blockIdx.x);
     else
         sweep_tile<L, Q, SOLVER_MIXED, true, false>(a, SWEEP_ADJOINT, blockIdx.x - n);
 }
