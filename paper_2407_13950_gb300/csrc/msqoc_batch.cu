@@ -34,6 +34,7 @@ struct msqoc_batch {
         SweepArgs args{};             // pds / tiles / lanemap / geometry of the group's launches
         int ntiles = 0;
         int nseg_max = 1, nsub_max = 1;
+        long slots = 1;               // tiles the GPU holds at a time
         bool quad_small = true;       // every member takes FP64 products (quad_fp64)
         int quad_blocks = 0;          // blocks of a row of the quadrature launch: the most of the members
         ProbDev* pds = nullptr;
@@ -133,6 +134,14 @@ struct GroupWork {
     int* list = nullptr;
     int ntiles = 0, nptiles = 0, nlist = 0;
 };
+// The history (or a segment's recomputation) and the adjoint sweep of n tiles each in one launch:
+// always for slices; for segments where that takes fewer waves (4 transmons, 16 windows, checkpoints
+// every 64 steps: one problem 11.7 -> 7.9 ms, but four, whose tiles fill the GPU, 15.0 -> 15.2).
+bool both_sweeps(const msqoc_batch::Group& g, long n) {
+    if (g.nsub_max != 1 || g.pair != 0 || g.solver != SOLVER_MIXED) return false;
+    auto waves = [&](long t) { return (t + g.slots - 1) / g.slots; };
+    return g.pthreads || (g.nseg_max > 1 && waves(2 * n) < 2 * waves(n));
+}
 // The launch sequence of one batched evaluation of the problems `sel`; work[g]: the part of group g;
 // set: the stream set of the groups.
 msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, const std::vector<GroupWork>& work,
@@ -176,17 +185,18 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, con
                 launch_compose(g.pds, work[gi].list, g.E_max, g.M_max, work[gi].nlist, ipow(g.L, g.q), true, gs);
             if (e != cudaSuccess) return e;
         }
+        const bool both = both_sweeps(g, work[gi].ntiles);
         for (int seg = g.nseg_max - 1; seg >= 0; --seg) {
             SweepArgs a = g.args;
             a.tiles = work[gi].tiles;
             a.seg = seg;
-            if (g.nseg_max > 1) {
+            if (g.nseg_max > 1 && !both) {
                 a.mode = SWEEP_RECOMPUTE;
                 const cudaError_t e = launch_sweep(a, work[gi].ntiles, gs);
                 if (e != cudaSuccess) return e;
             }
             for (int sub = g.nsub_max - 1; sub >= 0; --sub) {
-                a.mode = g.pthreads && g.nsub_max == 1 ? SWEEP_BOTH : SWEEP_ADJOINT;
+                a.mode = both ? SWEEP_BOTH : SWEEP_ADJOINT;
                 a.sub = sub;
                 cudaError_t e = launch_sweep(a, work[gi].ntiles, gs);
                 if (e != cudaSuccess) return e;
@@ -405,6 +415,11 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         if (g.pthreads) g.pargs = prop_args(plan, p0, g.pds, g.ptiles, g.plmap);
         SweepArgs adj = g.args;
         adj.mode = SWEEP_ADJOINT;
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        g.slots = std::max<long>(1, long(sms) * sweep_ctas_per_sm(adj));
+        SweepArgs both = g.args;
+        both.mode = SWEEP_BOTH;
         if (admission_bytes(g.q, g.L, p0.N, cpt, nthreads, gmax, g.solver, g.pair, g.args.hdepth) > 227 * 1024) {
             st = fail(MSQOC_ERR_UNSUPPORTED, "batched tiles need too much shared memory");
             break;
@@ -413,11 +428,8 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         // that a graph capture later makes no attribute calls
         if (launch_sweep(g.args, 0, nullptr) != cudaSuccess || launch_sweep(adj, 0, nullptr) != cudaSuccess ||
             launch_quad(quad_args(p0, g.pds, 0, 0), 0, 0, nullptr) != cudaSuccess ||
-            (g.pthreads && (launch_sweep(g.pargs, 0, nullptr) != cudaSuccess || [&] {
-                 SweepArgs both = g.args;
-                 both.mode = SWEEP_BOTH;
-                 return launch_sweep(both, 0, nullptr);
-             }() != cudaSuccess)))
+            (g.pthreads && launch_sweep(g.pargs, 0, nullptr) != cudaSuccess) ||
+            (both_sweeps(g, 1) && launch_sweep(both, 0, nullptr) != cudaSuccess))
             st = fail(MSQOC_ERR_CUDA, "sweep kernel attributes could not be set");
     }
     if (!st && (flags & MSQOC_BATCH_GRAPH) && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)

@@ -871,9 +871,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
 template <int L, int Q, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_sweep_both(const SweepArgs a) {
     const int n = gridDim.x / 2;
-    if (blockIdx.x < n)
-        sweep_tile<L, Q, SOLVER_MIXED, false, false>(a, a.pds[a.tiles[blockIdx.x].prob].nseg > 1 ? SWEEP_RECOMPUTE : SWEEP_HISTORY,
-                                                     blockIdx.x);
+    if (blockIdx.x < n)   // (nothing to recompute without segments: batches of both kinds)
+        sweep_tile<L, Q, SOLVER_MIXED, false, false>(
+            a, a.pds[a.tiles[blockIdx.x].prob].C > 1 ? SWEEP_HISTORY : SWEEP_RECOMPUTE, blockIdx.x);
     else
         sweep_tile<L, Q, SOLVER_MIXED, true, false>(a, SWEEP_ADJOINT, blockIdx.x - n);
 }

@@ -39,3 +39,23 @@ def test_segments_match_the_oracle(name):
         assert_grad_close(got["grad_W"], want["grad_W"], what="grad_W")
     assert got["P"] == again["P"] and np.array_equal(got["grad_alpha"], again["grad_alpha"])
     assert np.array_equal(got["grad_W"], again["grad_W"])
+
+
+def test_a_batch_of_checkpointed_and_whole_histories_equals_its_problems():
+    specs = [S.transmon_spec(3, 9.0, 607, 5, 6), S.transmon_spec(3, 6.0, 401, 7, 6), S.transmon_spec(3, 3.0, 203, 2, 6)]
+    probs = [msqoc.Problem(s, ckpt_interval=K, layout=msqoc.LAYOUT_FIBER, col_block=4) for s, K in zip(specs, (17, 64, 200))]
+    ins = [(S.random_alpha(s, 5 + i), S.random_W(s, 5 + i)) for i, s in enumerate(specs)]
+    want = [p.eval_gradient(*x) for p, x in zip(probs, ins)]
+    with msqoc.Batch(probs, graph=True) as b:
+        for i, x in enumerate(ins):
+            b.set_inputs(i, *x)
+        for _ in range(2):
+            b.eval_gradient()
+            for i, w in enumerate(want):
+                got = b.get_gradient(i)
+                assert all(np.array_equal(got[k], w[k]) for k in ("P", "grad_alpha", "grad_W"))
+        b.eval_subset([2, 0])
+        for i in (2, 0):
+            assert np.array_equal(b.get_gradient(i)["grad_alpha"], want[i]["grad_alpha"])
+    for p in probs:
+        p.close()
