@@ -5,8 +5,8 @@ Workload: 4 transmons x 3 levels (N=81 rows, E=16 essential columns), all-pair c
 2 carriers per transmon with 40 B-spline coefficients each (d=640), QFT_16 target,
 T=600 ns, 100000 implicit-midpoint steps, M windows (default 256), seeded synthetic controls
 and non-unitary window states.  A step of this benchmark is one full evaluation
-(controls, forward sweep of every window, terminal conditions, adjoint sweep with the fused
-gradient, reductions).  The midpoint-state history (2 GB) is far larger than L2, so no L2
+(controls, forward sweep of every window, terminal conditions, adjoint sweep, gradient quadrature,
+reductions).  The midpoint-state history (2 GB) is far larger than L2, so no L2
 flush is needed between steps.
 
 The default line also carries, measured in the same process:
@@ -108,13 +108,14 @@ class ClockSampler:
 
 
 SWEEP_SOURCES = ["msqoc_sweep.cuh", "msqoc_sweep_pair.cuh", "msqoc_sweep_common.cuh", "msqoc_split.cuh",
-                 "inst_sweep.cu", "msqoc_internal.h"]
+                 "msqoc_quad.cuh", "msqoc_chain.cuh", "inst_sweep.cu", "msqoc_internal.h"]
 PROFILES = os.path.join(ROOT, "profiles")
 LAYOUTS = {"auto": 0, "fiber": 1, "pair": 2, "quad": 3, "lean": 4}
 
 
 def sweep_traffic(kernel: str, windows: int, col_block: int, layout: int):
-    """DRAM bytes per launch of a sweep kernel from a committed ncu summary of the same tiles
+    """DRAM bytes of an evaluation's forward sweep, or of its adjoint sweeps and quadratures
+    together, from a committed ncu summary of the same tiles
     (a `capture_config:` line naming windows, columns per tile and kernel family, and a
     `traffic_per_launch_bytes:` line), or None when there is none or the kernel sources changed
     since that capture (their digest differs)."""
@@ -135,6 +136,17 @@ def sweep_traffic(kernel: str, windows: int, col_block: int, layout: int):
         if want in text and m and t and m.group(1) == digest:
             return float(t.group(1)), os.path.relpath(path, ROOT)
     return None, None
+
+
+def launches_per_evaluation(spec, tiles: int, col_block: int) -> int:
+    """Kernel launches of one gradient evaluation with every midpoint state kept.  Sliced windows:
+    controls, propagators, chain, terminal conditions, chain, both sweeps, quadrature, outputs.
+    Otherwise controls, forward sweep, terminal conditions, outputs, and an adjoint sweep and a
+    quadrature for each chunk of adjoint states (1 GiB at most, 16 steps at least)."""
+    if tiles * col_block > spec.M * spec.E + col_block:
+        return 8
+    chunk = max(16, (1 << 30) // (spec.M * spec.N * spec.E * 16))
+    return 4 + 2 * (-(-(-(-spec.nsteps // spec.M)) // chunk))
 
 
 def max_over_ranks(value: float, dist, device) -> float:
@@ -283,7 +295,7 @@ def solver_fp64_section(spec, dev, stream, peak, steps: int = 5, warmup: int = 2
         achieved = fl["adjoint"] / (kt["adjoint"] * 1e-3) / 1e12
         return {"value": 1e3 / ms, "unit": UNIT, "ms_per_eval": ms, "kernel_ms": kt,
                 "tiles": f"{FAMILY[p.layout]} x {p.col_block} columns ({p.tiles} CTAs)",
-                "roofline": {"kernel": "k_sweep (adjoint)", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                "roofline": {"kernel": "k_sweep (adjoint) + k_quad", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                              "frac": achieved / peak}}
 
 
@@ -373,7 +385,7 @@ def run_ours(args, spec):
                             else (None, None))
     dom_ms = kt[dom] / args.steps
     achieved = fl[dom] / (dom_ms * 1e-3) / 1e12
-    launches_per_eval = 6 if spec.M > 1 else 5
+    launches_per_eval = launches_per_evaluation(spec, prob.tiles, prob.col_block)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
@@ -386,10 +398,10 @@ def run_ours(args, spec):
             "layout": FAMILY[prob.layout], "ctas": prob.tiles, "threads_per_cta": prob.threads,
             "steps_per_sync": prob.steps_per_sync,
             **({"autotune": {"best": tuned, "ms_per_probe_eval": tune_ms}} if tuned else {})},
-        "roofline": {"bound": "alu", "kernel": f"k_sweep ({dom})", "achieved": achieved, "peak": peak_tflops,
+        "roofline": {"bound": "alu", "kernel": "k_sweep (forward)" if dom == "forward" else "k_sweep (adjoint) + k_quad", "achieved": achieved, "peak": peak_tflops,
                      "unit": "TFLOP/s", "frac": achieved / peak_tflops,
                      "traffic": traffic,
-                     "traffic_note": (f"DRAM bytes per launch from {traffic_src} (ncu capture of the same "
+                     "traffic_note": (f"DRAM bytes of the kernels' launches in one evaluation, from {traffic_src} (ncu capture of the same "
                                       "tiles and sweep sources)" if traffic else
                                       "null: no ncu summary of these tiles for the current sweep sources"),
                      "peak_source": "measured FP64 FMA microbenchmark (msqoc_measure_fp64_peak), same run",

@@ -73,10 +73,11 @@ typedef int32_t msqoc_status;
 
 /* Linear solver inside each implicit-midpoint step.
  *  MIXED: iterative refinement with FP32 inner corrections and a residual accurate to FP64
- *         round-off (formed in compensated FP32 where the step's contraction factor allows,
- *         else in FP64); the step is solved to FP64 round-off.  With one thread per fiber the
- *         state is kept as FP64 plus an FP32 carry and updated in compensated FP32 where the
- *         diagonal step |2 kappa| = h |D| <= 2^-4.5 (msqoc_selftest_carry).  Default.
+ *         round-off; the step is solved to FP64 round-off.  With one thread per fiber the
+ *         state is the exact sum of three floats and the step's increment is formed in
+ *         compensated FP32 (coarse steps, contraction factor above 2^-5 or diagonal step
+ *         |kappa| = h |D| / 2 above 2^-4, in FP64); the lane families form it in FP64.
+ *         Default.
  *  FP64 : diagonal-preconditioned fixed-point iteration carried out entirely in FP64. */
 #define MSQOC_SOLVER_DEFAULT 0
 #define MSQOC_SOLVER_FP64 1
@@ -108,8 +109,9 @@ typedef struct msqoc_options {
                               one-warp tile must divide E); 0 = automatic */
     int32_t ckpt_interval; /* K: forward states kept for the adjoint sweep.  1 = every midpoint
                               state (history of nsteps * E * N complex); K > 1 = the state every
-                              K steps of each window, each K-step segment recomputed before its
-                              adjoint sweep (one more forward sweep of work); 0 = automatic (1
+                              K steps of each window, each K-step segment recomputed before or
+                              beside its adjoint sweep (one more forward sweep of work); 0 =
+                              automatic (1
                               unless that history exceeds a quarter of the device memory, then
                               64) */
     int32_t profile;       /* 1 = record CUDA events around every kernel (msqoc_kernel_times) */
@@ -119,10 +121,9 @@ typedef struct msqoc_options {
                               0 and 0 = every window */
     int32_t window_last;
     int32_t steps_per_sync; /* time steps per synchronisation of a sweep tile with the midpoint
-                              history in device memory: the forward stages this many steps'
-                              states in shared memory and stores them with one wait, the adjoint
-                              fetches this many steps per mbarrier phase (one group ahead).
-                              1..8; 0 = 1.  Larger groups take more shared memory; a group that
+                              histories in device memory: the forward stages this many steps'
+                              (and the adjoint's) states in shared memory and stores them with
+                              one wait.  1..8; 0 = 1.  Larger groups take more shared memory; a group that
                               does not fit is MSQOC_ERR_INVALID_ARG */
 } msqoc_options;
 
@@ -147,10 +148,11 @@ typedef struct msqoc_options {
  * Roll-outs, roll-out estimates and batches take whole problems only (MSQOC_ERR_UNSUPPORTED). */
 
 /* Sweep kernel families.  FIBER: one thread per fiber (the L entries of a column along the last
- * subsystem), the choice for problems whose tiles fill the GPU.  PAIR: a lane pair per fiber,
- * one thread computing the real and one the imaginary component of every complex result: half
- * the FP64 instructions per thread, so steps run faster when the tiles are too few to fill the
- * GPU (small problems, the paper's QFT cases).  QUAD: 2-level subsystems only (and at most 6
+ * subsystem); with the mixed solver and every midpoint state kept, problems whose columns do not
+ * fill the GPU cut their windows into slices that run at the same time (the tiles are then of
+ * slices).  PAIR: a lane pair per fiber, one thread computing the real and one the imaginary
+ * component of every complex result: half the FP64 instructions per thread, so steps of the FP64
+ * solver run faster when the tiles are too few to fill the GPU.  QUAD: 2-level subsystems only (and at most 6
  * exchange-coupled pairs): a lane pair per entry of the fiber, four threads per fiber, a
  * quarter of its work per thread.  FIBER_LEAN: one thread per fiber like FIBER, compiled for
  * 168 registers a thread instead of 255: tiles of up to 384 threads, and two 6-warp tiles fit
@@ -168,7 +170,7 @@ typedef struct msqoc_options {
 #define MSQOC_KERNEL_CONTROLS 0  /* control evaluation at the step midpoints */
 #define MSQOC_KERNEL_FORWARD 1   /* forward sweep of every window */
 #define MSQOC_KERNEL_TERMINAL 2  /* window terminal conditions and objective terms */
-#define MSQOC_KERNEL_ADJOINT 3   /* adjoint sweep with the fused gradient quadrature */
+#define MSQOC_KERNEL_ADJOINT 3   /* adjoint sweep and gradient quadrature */
 #define MSQOC_KERNEL_FINALIZE 4  /* deterministic reductions and the W-gradient */
 #define MSQOC_NKERNELS 5
 
@@ -190,8 +192,8 @@ msqoc_status msqoc_create_problem(const msqoc_hamiltonian* H, const msqoc_contro
  * been evaluated.  Any pointer may be NULL. */
 msqoc_status msqoc_query(const msqoc_problem* p, int64_t* d, int64_t* nW, size_t* device_bytes);
 
-/* Sweep layout of a problem: columns per tile, tiles (CTAs) per sweep launch, threads per
- * tile, the checkpoint interval K, the kernel family (MSQOC_LAYOUT_FIBER, _PAIR, _QUAD or
+/* Sweep layout of a problem: columns per tile, tiles (CTAs) per sweep launch (of every slice of
+ * the windows), threads per tile, the checkpoint interval K, the kernel family (MSQOC_LAYOUT_FIBER, _PAIR, _QUAD or
  * _FIBER_LEAN) and the steps per history synchronisation in use (after automatic
  * choices).  Any pointer may be NULL. */
 msqoc_status msqoc_query_layout(const msqoc_problem* p, int32_t* col_block, int32_t* tiles,
@@ -205,18 +207,17 @@ msqoc_status msqoc_eval_objective(msqoc_problem* p, const double* alpha, const d
                                   double* P_out, double* J_out, double* pen_out, void* stream);
 
 /* Objective and gradient (forward sweep, terminal conditions Eq. terminal, discrete adjoint
- * sweep with the fused Eq. grad-int quadrature, Eq. dP-dW).  grad_alpha: d doubles;
+ * sweep, Eq. grad-int quadrature, Eq. dP-dW).  grad_alpha: d doubles;
  * grad_W: nW doubles, 2 N E (M-1) for a whole problem (may be NULL when nW = 0).  P_out may be
  * NULL. */
 msqoc_status msqoc_eval_gradient(msqoc_problem* p, const double* alpha, const double* W,
                                  double* P_out, double* grad_alpha, double* grad_W, void* stream);
 
 /* Roll-out (Sec. 5, initialisation of the window states): propagate the identity embedding
- * W^0 over the whole time grid [0, T] as one window under the controls alpha, sequentially in
- * time, and store the state at every window boundary: W_out^m = U(t_m), m = 1..M-1 (layout of
+ * W^0 over the whole time grid [0, T] as one window under the controls alpha and store the state at every window boundary: W_out^m = U(t_m), m = 1..M-1 (layout of
  * W).  With these window states every continuity penalty vanishes (to rounding) and the
- * objective equals the single-shooting infidelity.  This sweep cannot be parallelised over the
- * windows: it runs E / col_block tiles for all N_T steps.  W_out: host or device. */
+ * objective equals the single-shooting infidelity.  The windows' propagators (N columns each, cut
+ * into slices) are swept at the same time and then chained in order.  W_out: host or device. */
 msqoc_status msqoc_rollout(msqoc_problem* p, const double* alpha, double* W_out, void* stream);
 
 /* Roll-out infidelity estimate (Eq. rollout-infid-est) from the problem's last evaluation
@@ -300,10 +301,9 @@ msqoc_status msqoc_measure_fp64_peak(double* tflops);
  * way.  Synchronizes the device. */
 msqoc_status msqoc_selftest_bounded_wait(int64_t spins, int32_t arrive, double* seconds_out);
 
-/* Self-tests of the compensated FP32 arithmetic the mixed solver uses for the gradient products
- * of Eq. grad-int and for the implicit-midpoint state update (not operations of the paper), on
- * the host (on_device = 0)
- * or on the current device (on_device != 0: device copies, a kernel, copies back; synchronizes).
+/* Self-tests of compensated FP32 arithmetic: that of the mixed solver's gradient products of
+ * Eq. grad-int, and an implicit-midpoint state update with an FP32 carry, the form the solver had
+ * before its three-float state (not operations of the paper), on the host (on_device = 0) or on the current device (on_device != 0: device copies, a kernel, copies back; synchronizes).
  * All arrays are host arrays of n entries; -2000 <= scales <= 2000.
  *
  * msqoc_selftest_split: x_i 2^-sh as hi_i + lo_i, two floats: hi the value rounded to 24 bits
@@ -319,8 +319,7 @@ msqoc_status msqoc_selftest_bounded_wait(int64_t spins, int32_t arrive, double* 
  * one complex entry, U_{j+1} = R U_j + 2 d_j with R = 2P - 1, P = 1 / (1 + i kappa) the diagonal
  * preconditioner entry (P: 2 doubles, re and im; kappa = -Im P / Re P) and d_j the corrections
  * (d: n complex entries, 2n doubles, split into two floats in units 2^-sh as the solver's
- * corrections are), formed as the mixed solver forms it where |2 kappa| <= 2^-4.5: the state
- * an FP64 part u plus an FP32 carry, u' + carry' = u + carry + 2 kappa (Im b, -Re b) + 2 d_j with
+ * corrections are), for |2 kappa| <= 2^-4.5: the state an FP64 part u plus an FP32 carry, u' + carry' = u + carry + 2 kappa (Im b, -Re b) + 2 d_j with
  * b = P (u + carry) (R - 1 = -2 i kappa P).  u0: 2 doubles; out: the final u + carry (2 doubles).
  * -896 <= sh <= 896; Re P must lie in (1/2, 1] and (2 kappa)^2 <= 2^-9.
  *

@@ -6,8 +6,8 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
-#include <string>
 #include <functional>
+#include <string>
 #include <vector>
 
 #include "../../include/msqoc.h"
@@ -178,7 +178,6 @@ Tile tile_at(long t, int M, int E, int cpt, int prob) {
     x.c0 = static_cast<int>(g0 % E);
     x.ncol0 = std::min(x.ncol, E - x.c0);
     x.map = x.ncol == cpt ? x.ncol0 - 1 : cpt;
-    x.tloc = static_cast<int>(t);
     return x;
 }
 long tile_count(int M, int E, int cpt) { return (long(M) * E + cpt - 1) / cpt; }
@@ -248,7 +247,7 @@ bool quad_admitted(const ProbDev& pd) { return pd.L == 2 && pd.nex <= MAXEXF; }
 // Kernel family and columns per tile.  Makespan model calibrated on sweep timings, in units of the
 // step time of one one-thread-per-fiber warp alone on a sub-partition.
 //   Mixed solver: a step of an SM holding w warps of the one-thread families costs 1 up to four
-//     warps and 0.09 more for each further one (4 transmons: 3.3 us a step at 4 warps, 4.1 at 7, 6.0
+//     warps and 0.09 more for each further one (4 transmons: 2.7 us a step at 4 warps, 3.2 at 7, 4.9
 //     at 12: the steps are latency-bound).  One-warp tiles of at least two columns without
 //     idle lanes step without tile barriers and fall out of step: 0.85 (QFT-16 at 64 windows: 2.24
 //     us a step with 4-column one-warp tiles, 2.85 with 8-column ones).  The lane families do
@@ -361,13 +360,17 @@ TileChoice choose_tile_layout(const std::vector<TileCand>& cands, int M, int E, 
 // and chains: a step of one tile-model unit takes 1.2 us plus 0.13 us for each of a fiber's 2 q (L - 1)
 // terms (QFT-16 2.3 us, 3 transmons 2.6, 4 transmons 3.3), a launch LAUNCH us (its own start and a
 // sweep's set-up), and a link of the chain 0.35 us plus N^2 complex products at the FP64 rate of one
-// SM.  Slices have at least 4 steps, the propagators of a problem stay below SLICE_BYTES.
+// SM for each of the (window, column) chains that share it (QFT-16 at 64 windows, seven chains an SM:
+// 4.20 ms a gradient with 64 slices, 3.85 with 32; single shooting, one chain an SM: 4.36 ms with 384,
+// 6.04 with 192).  Slices have at least 4 steps, the propagators of a problem stay below SLICE_BYTES.
 constexpr double SLICE_LAUNCH = 5.0;
 double slice_unit_us(const ProbDev& pd) { return 1.2 + 0.13 * 2 * pd.q * (pd.L - 1); }
 constexpr size_t SLICE_BYTES = size_t(256) << 20;
 // propagators a roll-out holds at a time (whole windows; at least one)
 constexpr size_t ROLLOUT_BYTES = size_t(32) << 20;
-double slice_link_us(int N) { return 0.35 + double(N) * N * 4.0 / (1.9 * 2070.0); }
+double slice_link_us(int N, int64_t chains, int sms) {
+    return 0.35 + double(N) * N * 4.0 / (1.9 * 2070.0) * double((chains + sms - 1) / sms);
+}
 int choose_slices(const std::vector<TileCand>& cands, const ProbDev& pd, int M, int64_t steps, int sms) {
     const double unit = slice_unit_us(pd);
     auto sweep_us = [&](int windows, int cols, double n) {
@@ -382,7 +385,7 @@ int choose_slices(const std::vector<TileCand>& cands, const ProbDev& pd, int M, 
     for (int c2 = 4; c2 / 2 <= ns / 4.0; c2 += (c2 & (c2 - 1)) ? c2 / 3 : c2 / 2) {   // C = 2, 3, 4, 6, 8, 12, ..
         const int C = c2 / 2;
         if (size_t(M) * C * pd.N * pd.N * sizeof(double2) > SLICE_BYTES || int64_t(M) * C > (1 << 20)) break;
-        const double n = std::ceil(ns / C), chain = SLICE_LAUNCH + C * slice_link_us(pd.N);
+        const double n = std::ceil(ns / C), chain = SLICE_LAUNCH + C * slice_link_us(pd.N, int64_t(M) * pd.E, sms);
         const double objective = sweep_us(M * C, pd.N, n) + chain;
         if (objective > whole) continue;
         // (the history and adjoint sweeps run at the same time)
@@ -405,7 +408,7 @@ int choose_rollout_slices(const std::vector<TileCand>& cands, const ProbDev& pd,
         const double V = double(pd.M) * C;
         if (V > (1 << 20) && C > 1) break;
         const TileChoice t = choose_tile_layout(cands, static_cast<int>(V), pd.N, pd.F, pd.solver, sms, 0, true);
-        const double us = t.cost * std::ceil(ns / C) * slice_unit_us(pd) + V * slice_link_us(pd.N);
+        const double us = t.cost * std::ceil(ns / C) * slice_unit_us(pd) + V * slice_link_us(pd.N, pd.E, sms);
         if (us < best_us) {
             best_us = us;
             best = C;
@@ -497,8 +500,6 @@ msqoc_status shape_problem(const msqoc_hamiltonian* H, const msqoc_controls* C, 
     for (int l = 0; l < MAXL; ++l) {
         pd.sc[2 * l + 0] = 0.5 * pd.h * std::sqrt(double(l + 1));
         pd.sc[2 * l + 1] = 0.5 * pd.h * std::sqrt(double(l));
-        pd.wsq[2 * l + 0] = std::sqrt(double(l + 1));
-        pd.wsq[2 * l + 1] = std::sqrt(double(l));
     }
     // a window's part of the alpha-gradient: the splines active in one window (the most over the
     // windows, from each window's first active spline), plus a margin of two
@@ -788,7 +789,7 @@ msqoc_status create_problem(const msqoc_hamiltonian* H, const msqoc_controls* C,
     TileTables tabs_prop, tabs_ro, tabs_both;
     // A segment's recomputation and adjoint sweep do not depend on each other: one launch of both,
     // in tiles for twice the windows, where the model has it faster than one after the other
-    // (4 transmons, 64 windows, checkpoints every 64 steps: 294 7-column lean tiles, two an SM, in
+    // (4 transmons, 64 windows, checkpoints every 64 steps: 2 x 74 14-column lean tiles, one an SM, in
     // place of 128 8-column tiles twice: 10.6 ms against 13.2 with the quadrature; at 16 windows, whose
     // tiles fill neither launch, 4.5 against 8.0)
     if (pd.nseg > 1 && pd.nsub == 1 && pd.pair == 0 && solver == SOLVER_MIXED && pd.hdepth == 1) {

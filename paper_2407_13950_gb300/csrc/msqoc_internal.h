@@ -26,7 +26,7 @@ static_assert(MAX_TILE_THREADS <= MAX_ANY_TILE_THREADS && MAX_LEAN_TILE_THREADS 
 enum Solver { SOLVER_FP64 = 1, SOLVER_MIXED = 2 };
 
 // device status word bits
-enum Status { ST_OK = 0, ST_TIMEOUT = 1, ST_BAD_LAUNCH = 2, ST_SOLVER_RANGE = 4 };
+enum Status { ST_OK = 0, ST_TIMEOUT = 1, ST_SOLVER_RANGE = 4 };
 
 // Index of the first of the three quadratic B-splines (spacing dtau, d1 of them) active at time
 // t, clamped to the grid.  The controls kernel and the host take it from here.
@@ -83,7 +83,6 @@ struct ProbDev {
     double ex_c[MAXEX];
     double rho_ex;
     double kap;                  // max |(h/2) D_i| over the rows: the largest diagonal rotation of a step
-    double wsq[2 * MAXL];        // sqrt(l+1) [dir +] and sqrt(l) [dir -]: product weights
     // constant tables
     const double2* P;            // [N] (1 + i h/2 D_i)^-1
     const int* emb;              // [E] full row index of essential column e
@@ -126,10 +125,9 @@ struct ProbDev {
 // One sweep tile (one CTA): `ncol` consecutive columns of problem `prob` in window-major column
 // order, starting at column c0 of window m0 (1-based).  The first `ncol0` columns belong to
 // window m0, the rest to window m0 + 1 (a tile covers at most two windows).  `map` selects the
-// thread -> (column, fiber) assignment in the launch's lane maps; `tloc` is the tile's index
-// among its problem's tiles.
+// thread -> (column, fiber) assignment in the launch's lane maps.
 struct Tile {
-    int prob, m0, c0, ncol, ncol0, map, tloc, pad;
+    int prob, m0, c0, ncol, ncol0, map, pad[2];
 };
 
 // What a sweep launch does.

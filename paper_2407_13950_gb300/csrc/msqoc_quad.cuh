@@ -2,7 +2,7 @@
 //   A_k = Im z_k + Im y_k,  B_k = Re z_k - Re y_k,  z_k = <Lbar_n, a_k Ubar_n>_F,
 //   y_k = <Lbar_n, a_k^+ Ubar_n>_F  (summed over every column of the window),
 // from the midpoint states the forward and adjoint sweeps left in device memory.  The alpha-
-// gradient needs only these combinations (k_outputs folds them with the spline weights and the
+// gradient needs only these combinations (k_gradient_outputs folds them with the spline weights and the
 // carrier phases).
 //
 // Unlike the sweeps, the steps here are independent: the products run at the GPU's throughput
@@ -17,16 +17,17 @@
 // to [row][lane] (one padding lane a row: conflict-free both ways) with 16-byte asynchronous copies.
 // Split states sum a few pairs at a time in fresh two-float sums (their low parts round relative
 // to the partial sum) before those join the running sum.
-// 4 transmons, 100000 steps: 2.08 ms (4.1 GB read, 2.0 TB/s; the products' FP32 operations alone
-// would take 0.8 ms), against 2.71 ms for one fiber a warp with a branch per level and 37% more
-// instructions.  Issue-bound: a staged CTA holds 85 KB, so two are resident on an SM.
 // LN = 32, 16 or 8 by the rows, so that several CTAs fit an SM and one's loads overlap the others'
 // products; below 32 the parts of a warp take alternate groups of pairs.
+// 4 transmons, 100000 steps (4.15 GB read): 2.71 ms with one fiber a warp and a branch per level, 2.08
+// by row pairs with 32 lanes (two CTAs an SM), 1.91 with 16 (2.2 TB/s); 5 transmons with 8 lanes 0.85 ms
+// a segment of 64 steps at 100 windows.  Bound by instruction issue (73% of the slots, FMA pipe 52%,
+// DRAM 26-32%): ten FP32 operations a compensated term.
 #pragma once
 
-#include "msqoc_chain.cuh"
 #include <type_traits>
 
+#include "msqoc_chain.cuh"
 #include "msqoc_sweep_common.cuh"
 
 namespace msqoc {

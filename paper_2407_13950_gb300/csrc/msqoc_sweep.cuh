@@ -28,13 +28,13 @@
 //
 // What bounds the mixed step: instruction issue and the dependency latency inside its 4-5 barrier-
 // separated phases (no pipe is saturated).  4 transmons, 100000 steps at 256 windows on one GB300:
-// a forward sweep 5.22 -> 4.43 ms against the form with an FP64 state, an FP32 carry and two more
-// sweeps a step; at 64 windows 6.97 -> 5.52 ms.
+// a forward sweep 5.22 -> 3.85 ms against the form with an FP64 state, an FP32 carry and two more
+// sweeps a step; at 64 windows 6.97 -> 4.98 ms.
 #pragma once
 
-#include "msqoc_chain.cuh"
 #include <climits>
 
+#include "msqoc_chain.cuh"
 #include "msqoc_sweep_common.cuh"
 
 namespace msqoc {

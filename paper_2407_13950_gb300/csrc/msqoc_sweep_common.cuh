@@ -12,8 +12,6 @@
 namespace msqoc {
 
 __host__ __device__ constexpr int ipow_c(int b, int e) { return e == 0 ? 1 : b * ipow_c(b, e - 1); }
-__host__ __device__ constexpr int next_pow2_c(int v) { return v <= 1 ? 1 : 2 * next_pow2_c((v + 1) / 2); }
-__host__ __device__ constexpr int log2_c(int v) { return v <= 1 ? 0 : 1 + log2_c(v / 2); }
 
 // Entries between the columns of the shared apply buffers: odd, so that lanes on the same fiber of
 // different columns meet different banks (N = 16: four columns 128 bytes apart would meet one)
@@ -33,19 +31,7 @@ __device__ __forceinline__ float f32_of(double x) {
     fb = (ahi < 0x38100000u) ? (hi & 0x80000000u) : fb;
     return __uint_as_float(fb);
 }
-// f32 -> f64 exactly for normal floats (denormals become signed zero).  Integer operations.
-__device__ __forceinline__ double f64_of(float f) {
-    const unsigned int fb = __float_as_uint(f);
-    const unsigned int s = fb & 0x80000000u;
-    const unsigned int a = fb & 0x7fffffffu;
-    unsigned int hi = s | ((a >> 3) + 0x38000000u);
-    unsigned int lo = a << 29;
-    hi = (a < 0x00800000u) ? s : hi;
-    lo = (a < 0x00800000u) ? 0u : lo;
-    return __hiloint2double(static_cast<int>(hi), static_cast<int>(lo));
-}
 __device__ __forceinline__ float2 f32_of(double2 v) { return make_float2(f32_of(v.x), f32_of(v.y)); }
-__device__ __forceinline__ double2 f64_of(float2 v) { return make_double2(f64_of(v.x), f64_of(v.y)); }
 
 // The same conversions of a state entry with a per-column binary scale 2^-sh (|sh| <=
 // SCALE_SHIFT_MAX): f32_of_scaled gives x 2^-sh rounded to f32 as above, f64_of_scaled gives
@@ -198,9 +184,6 @@ struct Fiber {
     int sl1[NA];       // coefficient slot of entry 1
     int sl2[NA];
     bool two[NA];      // entry 2 exists (warp-uniform by construction)
-    bool plus1[NA];    // entry 1 is the a_k (lowering, "+") term
-    double w1[NA];     // product weight sqrt(level factor) of entry 1
-    double w2[NA];
     // dipole exchange of 2-level subsystems: the column's first entry, the buffers' zero entry and,
     // per entry of the fiber, the pairs that give it a term
     int eb, zero;
@@ -218,21 +201,15 @@ struct Fiber {
             if (lk < L - 1) {
                 nb1[k] = c * CP + (f + sf) * L;
                 sl1[k] = (k * L + lk) * 2 + 0;
-                plus1[k] = true;
-                w1[k] = pd.wsq[2 * lk + 0];
                 two[k] = lk > 0;
                 nb2[k] = c * CP + (f - (lk > 0 ? sf : 0)) * L;
                 sl2[k] = (k * L + lk) * 2 + 1;
-                w2[k] = pd.wsq[2 * lk + 1];
             } else {
                 nb1[k] = c * CP + (f - sf) * L;
                 sl1[k] = (k * L + lk) * 2 + 1;
-                plus1[k] = false;
-                w1[k] = pd.wsq[2 * lk + 1];
                 two[k] = false;
                 nb2[k] = nb1[k];
                 sl2[k] = sl1[k];
-                w2[k] = 0.0;
             }
         }
         eb = c * CP;
@@ -296,11 +273,6 @@ __device__ __forceinline__ void tile_sync() {
     else
         __syncthreads();
 }
-__device__ __forceinline__ int tile_sync_or(int p) {
-    if (blockDim.x == 32) return __any_sync(0xffffffffu, p);
-    return __syncthreads_or(p);
-}
-
 // first global step of local window m (1-based); window m owns [win_start(m), win_start(m + 1))
 // of the whole problem's grid
 __device__ __forceinline__ int64_t win_start(const ProbDev& pd, int m) {

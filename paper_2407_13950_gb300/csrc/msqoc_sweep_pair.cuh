@@ -1,5 +1,5 @@
 // Forward and adjoint sweeps with a lane pair per fiber (sm_103a): the variant of the sweeps of
-// msqoc_sweep.cuh (same tiles, step equation, solvers, history and fused gradient quadrature)
+// msqoc_sweep.cuh (same tiles, step equation, solvers and history; no propagators)
 // for problems whose tiles are too few to fill the GPU.
 //
 // A warp issues one FP64 instruction per 64 cycles on its SM sub-partition, so when an SM holds
@@ -18,9 +18,9 @@
 // budget cost the adjoint 2-4%).
 #pragma once
 
-#include "msqoc_chain.cuh"
 #include <climits>
 
+#include "msqoc_chain.cuh"
 #include "msqoc_sweep_common.cuh"
 
 namespace msqoc {
@@ -150,7 +150,7 @@ __device__ __forceinline__ void step_coefficients_pair(const ProbDev& pd, int la
 
 // ------------------------------------------------------------------ the sweep kernel
 // One CTA per tile.  A tile covers one or two windows ("slots"); each slot has its own step
-// range, per-step coefficients, iteration counts and gradient fold, computed by warp `slot`
+// range, per-step coefficients, iteration counts, computed by warp `slot`
 // (the host only builds two-slot tiles with at least two warps).  Loops run to the longer of
 // the slots' ranges; a thread whose slot has no step at an iteration keeps its state.  A lane
 // pair (parts 0 and 1) works on each (column, fiber) for SPLIT = 1, on each of its entries for

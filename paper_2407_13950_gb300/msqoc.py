@@ -256,7 +256,7 @@ class Problem:
         return {"P": float(P[0]), "grad_alpha": ga, "grad_W": gW[:self.nW].copy()}
 
     def rollout(self, alpha, stream=None) -> np.ndarray:
-        """Window states from a sequential roll-out of the identity under alpha (W^m = U(t_m))."""
+        """Window states from a roll-out of the identity under alpha (W^m = U(t_m))."""
         W = np.zeros(max(self.nW, 1))
         _check(load().msqoc_rollout(self.handle, _ptr(alpha), _ptr(W) if self.spec.M > 1 else None,
                                     _stream_handle(stream)))
@@ -345,7 +345,7 @@ def selftest_split(x, sh: int = 0, device: bool = False):
 
 
 def selftest_dot(x, y, shx: int = 0, shy: int = 0, device: bool = False) -> float:
-    """sum x_i y_i formed the way the mixed solver's adjoint forms its gradient products
+    """sum x_i y_i formed the way the mixed solver forms its gradient products
     (split operands, compensated FP32 accumulation, one double)."""
     x = np.ascontiguousarray(x, dtype=np.float64)
     y = np.ascontiguousarray(y, dtype=np.float64)
