@@ -64,7 +64,8 @@ static cudaError_t launch_one(const SweepArgs& a, int ntiles, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     if (ntiles <= 0) return cudaSuccess;
-    return launch_chained(kern, BOTH ? 2 * ntiles : ntiles, a.nthreads, smem, s, a);
+    return launch_carved(FAM == 3 ? cudaSharedmemCarveoutDefault : cudaSharedmemCarveoutMaxShared, kern,
+                         BOTH ? 2 * ntiles : ntiles, a.nthreads, smem, s, a);
 }
 
 template <int SOLVER, bool BWD, int FAM>

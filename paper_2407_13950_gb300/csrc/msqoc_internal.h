@@ -170,24 +170,42 @@ struct SweepArgs {
 // copies ahead of the first kernel left out (take_inputs), QFT-4's gradient of eight dependent
 // launches 116 -> 104 us, QFT-8's 372 -> 347, three transmons' 1060 -> 992, QFT-8's roll-out
 // 387 -> 323.  Captured launches are plain ones (a graph has its own edges).
+// carveout: percent of an SM's L1 kept as shared memory (not positive: the driver's choice).  Blocks of two kernels share an SM only
+// under one split, so every kernel asks for the same (the largest): QFT-4's gradient 104 -> 91 us,
+// QFT-8's 304 -> 266.  The lean sweeps leave it to the driver, since their spilled registers want the
+// L1 (QFT-16 at 64 windows 3.84 -> 4.00 ms with all of it shared).
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+cudaError_t launch_carved(int carveout, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                          A... args) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
         cudaGetLastError();
         cap = cudaStreamCaptureStatusActive;
     }
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2] = {};
+    int n = 0;
+    if (carveout > 0) {
+        at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        at[n++].val.sharedMemCarveout = static_cast<unsigned>(carveout);
+    }
+    if (cap == cudaStreamCaptureStatusNone) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
     cudaLaunchConfig_t c{};
     c.gridDim = grid;
     c.blockDim = dim3(threads);
     c.dynamicSmemBytes = smem;
     c.stream = s;
-    c.attrs = &at;
-    c.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
-    return cudaLaunchKernelEx(&c, kern, P(args)...);
+    c.attrs = at;
+    c.numAttrs = n;
+    const cudaError_t e = cudaLaunchKernelEx(&c, kern, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();   // returned here, not to the next caller that asks
+    return e;
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+    return launch_carved(cudaSharedmemCarveoutMaxShared, kern, grid, threads, smem, s, args...);
 }
 
 // shared-memory bytes of a sweep launch

@@ -162,22 +162,24 @@ __device__ __forceinline__ float4 load_coefficient(const ProbDev& pd, int lane, 
 }
 // The coefficients go out in FP64 (FP64 solver) or in FP32 and split into two floats (mixed solver).
 // The iteration counts of the step (packed by step_counts in the controls kernel) are unpacked into
-// prm; prm[3] holds the solver-range flag (bit 0) and the coarse-step flag (bit 1).
+// prm; prm[3] holds the solver-range flag (bit 0) and the coarse-step flag (bit 1).  sg: the sign s of
+// the step's off-diagonal term, which multiplies every coefficient (exactly).
 template <int L, int Q, int SOLVER>
-__device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, const float4& in, int cnt, double2* cfd,
-                                                  float2* cff, float4* cfs, int* prm) {
+__device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, const float4& in, int cnt, float sg,
+                                                  double2* cfd, float2* cff, float4* cfs, int* prm) {
     constexpr int NSLOT = Q * L * 2;
     if (lane < NSLOT) {
         const int dir = lane & 1;
         const int l = (lane >> 1) % L;
         const bool valid = dir == 0 ? (l < L - 1) : (l > 0);
         if (SOLVER == SOLVER_MIXED && pd.coef != nullptr) {
-            const float4 sp = dir == 0 ? make_float4(-in.y, in.x, -in.w, in.z) : make_float4(in.y, in.x, in.w, in.z);
+            const float sr = dir == 0 ? -sg : sg;
+            const float4 sp = make_float4(sr * in.y, sg * in.x, sr * in.w, sg * in.z);
             cff[lane] = make_float2(sp.x, sp.y);
             cfs[lane] = sp;
         } else {
             const double2 dk = *reinterpret_cast<const double2*>(&in);
-            const double s = valid ? pd.sc[2 * l + dir] : 0.0;
+            const double s = valid ? sg * pd.sc[2 * l + dir] : 0.0;
             const double2 v = dir == 0 ? make_double2(-s * dk.y, s * dk.x) : make_double2(s * dk.y, s * dk.x);
             if constexpr (SOLVER == SOLVER_FP64) {
                 cfd[lane] = v;
@@ -253,15 +255,15 @@ __device__ __forceinline__ void apply_off_df(const float4* __restrict__ buf, con
 // The mixed solver's step in FP64, for the steps step_counts flags as coarse: where the rotation
 // of a drift entry or the contraction factor is so large that the compensated increment's 2^-48
 // relative error would exceed the FP64 rounding of the state.  The fixed point z = P u + s P w(z)
-// takes K sweeps, U' = 2 z - U.  Out of line: it is rare, and everything it needs would cost the
+// (s in the coefficients) takes K sweeps, U' = 2 z - U.  Out of line: it is rare, and everything it needs would cost the
 // common step registers.  Every thread of the tile takes part in the barriers; `mine` says
 // whether the thread's slot is coarse at this step.  The buffer's zero entry stays zero.
 template <int L> struct CoarseIO {
     TF u[L][2];
     float4 z[L];
 };
-template <int L, int Q, int S, bool BWD>
-static __device__ __noinline__ void coarse_step(double2* D0, double2* cfd, const ProbDev& pd, const ExTab& ex, int c,
+template <int L, int Q>
+static __device__ __noinline__ void coarse_step(bool bwd, double2* D0, double2* cfd, const ProbDev& pd, const ExTab& ex, int c,
                                                 int f, int zero, int64_t n0, int64_t n1, int nslot, int slot, bool act,
                                                 bool mine, int K, int Kmax, int sh, CoarseIO<L>& io) {
     constexpr int NSLOT = Q * L * 2;
@@ -271,14 +273,14 @@ static __device__ __noinline__ void coarse_step(double2* D0, double2* cfd, const
     for (int t = threadIdx.x; t < nslot * NSLOT; t += blockDim.x) {
         const int i = t % NSLOT, dir = i & 1, l = (i >> 1) % L;
         const double2 d = pd.ctrl[size_t(t < NSLOT ? n0 : n1) * pd.q + i / (2 * L)];
-        const double s = (dir == 0 ? l < L - 1 : l > 0) ? pd.sc[2 * l + dir] : 0.0;
+        const double s = (dir == 0 ? l < L - 1 : l > 0) ? (bwd ? 1.0 : -1.0) * pd.sc[2 * l + dir] : 0.0;
         cfd[t] = dir == 0 ? make_double2(-s * d.y, s * d.x) : make_double2(s * d.y, s * d.x);
     }
     double2 u[L], b[L], z[L], P[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         P[l] = pd.P[f * L + l];
-        if (BWD) P[l].y = -P[l].y;
+        if (bwd) P[l].y = -P[l].y;
         u[l] = make_double2(tf_to_f64(io.u[l][0], sh), tf_to_f64(io.u[l][1], sh));
         b[l] = cmul(P[l], u[l]);
         z[l] = b[l];
@@ -294,7 +296,7 @@ static __device__ __noinline__ void coarse_step(double2* D0, double2* cfd, const
         apply_off<L, Q, double2>(D0, cfd + (nslot > 1 ? slot : 0) * NSLOT, fb, z, w, ex);
         if (it < K) {
 #pragma unroll
-            for (int l = 0; l < L; ++l) z[l] = cadd_scaled<S>(b[l], P[l], w[l]);
+            for (int l = 0; l < L; ++l) z[l] = cadd_scaled<1>(b[l], P[l], w[l]);
         }
     }
     tile_sync();
@@ -325,12 +327,14 @@ struct TileInfo {
 // whose slot has no step at an iteration keeps its state.
 // MAXT: the largest tile the instantiation serves; it sets the register budget (255 registers a
 // thread for MAX_TILE_THREADS, 168 for MAX_LEAN_TILE_THREADS: 12 warps on an SM).
-template <int L, int Q, int SOLVER, bool BWD, bool PROP>
-__device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, const int block) {
-    static_assert(!(BWD && PROP), "propagators are forward sweeps");
+// bwd: the adjoint sweep.  Nothing in the step depends on it: the adjoint's sign s = +1 (forward: -1)
+// is in the coefficients and its conj(P) in kappa and G, so k_sweep_both runs both sweeps through the
+// same instructions.
+template <int L, int Q, int SOLVER, bool PROP>
+__device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, const int block, const bool bwd) {
     constexpr int N = ipow_c(L, Q);
     constexpr int NSLOT = Q * L * 2;
-    constexpr int S = BWD ? +1 : -1;       // sign of the preconditioned off-diagonal term
+    const float sg = bwd ? 1.f : -1.f;     // sign s of the preconditioned off-diagonal term
 
     const Tile tile = a.tiles[block];
     const ProbDev& pd = a.pds[tile.prob];
@@ -372,8 +376,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     const int wns_1 = nslot > 1 ? static_cast<int>(slice_start(pd, C, v0 + 2) - wn0_1) : 0;
     // (an adjoint launch covers chunk `sub` of its segment)
     const int seg_hi = segmented ? (a.seg + 1) * pd.kseg : INT_MAX;
-    const int lo = segmented ? a.seg * pd.kseg + (BWD ? a.sub * pd.kadj : 0) : 0;
-    const int hi = BWD ? min(seg_hi, lo + pd.kadj) : seg_hi;
+    const int lo = segmented ? a.seg * pd.kseg + (bwd ? a.sub * pd.kadj : 0) : 0;
+    const int hi = bwd ? min(seg_hi, lo + pd.kadj) : seg_hi;
     const int cnt_0 = max(0, min(wns_0, hi) - lo);
     const int cnt_1 = nslot > 1 ? max(0, min(wns_1, hi) - lo) : 0;
     const int nit = max(cnt_0, cnt_1);
@@ -381,8 +385,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     // registers (written before the barrier ahead of the loop)
     __shared__ TileInfo ti;
     if (tid == 0) {
-        const size_t kh = BWD ? pd.kadj : pd.kseg;
-        double2* const base = PROP ? nullptr : BWD ? pd.lhist : pd.hist;
+        const size_t kh = bwd ? pd.kadj : pd.kseg;
+        double2* const base = PROP ? nullptr : bwd ? pd.lhist : pd.hist;
         ti.n0[0] = wn0_0;
         ti.n0[1] = wn0_1;
         ti.cnt[0] = cnt_0;
@@ -400,7 +404,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
         const int64_t n0 = ti.n0[s];
         if (cnt <= 0) return min(n0, pd.nsteps - 1);
         const int jc = min(jj, cnt - 1);
-        return BWD ? n0 + lo + cnt - 1 - jc : n0 + lo + jc;
+        return bwd ? n0 + lo + cnt - 1 - jc : n0 + lo + jc;
     };
 
     // ---- this thread's fiber
@@ -419,7 +423,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     Fiber<L, Q> fb;
     fb.init(c, f, pd, a.cpt * col_pitch(N));
     __shared__ ExTab ex_s;   // (ordered before its first read by the first barrier of the time loop)
-    fill_exchange(ex_s, pd);
+    fill_exchange(ex_s, pd, sg);
     // the apply buffers' zero entry (read by the exchange terms a fiber entry does not have; the
     // first barrier of the time loop orders these stores before any read)
     if (tid == 0) {
@@ -441,7 +445,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         double2 p = pd.P[f * L + l];
-        if (BWD) p.y = -p.y;
+        if (bwd) p.y = -p.y;
         if constexpr (SOLVER == SOLVER_FP64) {
             Pd[l] = p;
         } else {
@@ -470,7 +474,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             u[l] = make_double2(col == i ? 1.0 : 0.0, 0.0);
         } else if (my_cnt == 0) {
             u[l] = make_double2(0.0, 0.0);
-        } else if (BWD) {
+        } else if (bwd) {
             u[l] = C > 1 ? pd.Lend[wcol + i] : (lo + my_cnt == my_ns) ? pd.Lterm[wcol + i] : pd.Lstate[wcol + i];
         } else if (C > 1) {
             u[l] = pd.Ubeg[wcol + i];
@@ -509,7 +513,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     // the forward's history, per launch for the adjoint's
     if constexpr (SOLVER == SOLVER_MIXED) {
         if (!PROP && act && f == 0 && my_cnt > 0) {
-            if (BWD)
+            if (bwd)
                 pd.lsh[size_t(m - 1) * E + col] = sh;
             else if ((mode == SWEEP_HISTORY && pd.nseg == 1) || mode == SWEEP_RECOMPUTE)
                 pd.hsh[(size_t(m - 1) * pd.nseg + (mode == SWEEP_HISTORY ? 0 : a.seg)) * E + col] = sh;
@@ -517,8 +521,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     }
 
     // ---- history
-    const bool want_hist = !PROP && (BWD || (mode == SWEEP_HISTORY && pd.nseg == 1) || mode == SWEEP_RECOMPUTE);
-    const bool want_ckpt = !BWD && !PROP && mode == SWEEP_HISTORY && pd.nseg > 1;
+    const bool want_hist = !PROP && (bwd || (mode == SWEEP_HISTORY && pd.nseg == 1) || mode == SWEEP_RECOMPUTE);
+    const bool want_ckpt = !bwd && !PROP && mode == SWEEP_HISTORY && pd.nseg > 1;
     // Steps per history synchronisation: the midpoint states are staged in H in groups of hd
     // iterations (g hd .. g hd + hd - 1), one block of the tile's cpt N states per iteration, and
     // a group is stored with one wait.
@@ -531,7 +535,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             const int cnt = ti.cnt[s];
             const double2* src = H + (s ? size_t(ti.bytes[0] / sizeof(double2)) : 0);
             for (int j = g0; j < min(g1, cnt); ++j)   // step j of the launch's, or from its end
-                bulk_s2g(ti.hist[s] + size_t(BWD ? cnt - 1 - j : j) * E * N, src + size_t(j - g0) * hstride, ti.bytes[s]);
+                bulk_s2g(ti.hist[s] + size_t(bwd ? cnt - 1 - j : j) * E * N, src + size_t(j - g0) * hstride, ti.bytes[s]);
         }
     };
     // warp s < nslot computes slot s's coefficients and keeps d_k and the iteration counts of
@@ -571,7 +575,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             const float4 dk = cf_next;
             const int cnt = cnt_next;
             if (jj + 1 < nit) load_ctrl(jj + 1);
-            step_coefficients<L, Q, SOLVER>(pd, lane, dk, cnt, coef_d + (par * 2 + cslot) * NSLOT,
+            step_coefficients<L, Q, SOLVER>(pd, lane, dk, cnt, sg, coef_d + (par * 2 + cslot) * NSLOT,
                                             coef_f + (par * 2 + cslot) * NSLOT, coef_s + (par * 2 + cslot) * NSLOT,
                                             params + (par * 2 + cslot) * 4);
         }
@@ -631,7 +635,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                 apply_off<L, Q, double2>(Dc, cfd, fb, z, w, ex_s);
                 if (it < Kown) {
 #pragma unroll
-                    for (int l = 0; l < L; ++l) z[l] = cadd_scaled<S>(b[l], Pd[l], w[l]);
+                    for (int l = 0; l < L; ++l) z[l] = cadd_scaled<1>(b[l], Pd[l], w[l]);
                 }
                 double2* tmp = Dc;
                 Dc = Dn;
@@ -656,10 +660,10 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                 d[l] = fresh ? make_float2(0.f, 0.f) : DP[fb.xo + l];
                 y[l] = make_float2((v[l][0].a + m0[l].x) + d[l].x, (v[l][1].a + m0[l].y) + d[l].y);
             }
-            // s P w for P = 1 + G
+            // P w for P = 1 + G (s is in w)
             auto precond = [&](int l, const float2& w) {
                 const float x = fmaf(Gf[l].x, w.x, fmaf(-Gf[l].y, w.y, w.x)), yy = fmaf(Gf[l].x, w.y, fmaf(Gf[l].y, w.x, w.y));
-                return S > 0 ? make_float2(x, yy) : make_float2(-x, -yy);
+                return make_float2(x, yy);
             };
             auto exchange = [&](const float2 (&x)[L]) {
                 float2* Fb = fsel ? FB : FA;
@@ -723,11 +727,11 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                         apply_off_df<L, Q>(D0s, cfs, fb, zf, w, ex_s);
 #pragma unroll
                         for (int l = 0; l < L; ++l) {
-                            // m1 = -i kappa z + s w
+                            // m1 = -i kappa z + s w (s in the coefficients)
                             DF kr = kappa_mul(kh[l], kl[l], k3[l], zf[l].y, zf[l].w);
                             DF ki = df_neg(kappa_mul(kh[l], kl[l], k3[l], zf[l].x, zf[l].z));
-                            kr = df_add(kr, S > 0 ? w[l][0] : df_neg(w[l][0]));
-                            ki = df_add(ki, S > 0 ? w[l][1] : df_neg(w[l][1]));
+                            kr = df_add(kr, w[l][0]);
+                            ki = df_add(ki, w[l][1]);
                             r[l] = make_float2(fadd_n(fsub_n(kr.s, mr[l].s), fsub_n(kr.c, mr[l].c)),
                                                fadd_n(fsub_n(ki.s, mi[l].s), fsub_n(ki.c, mi[l].c)));
                             if (pass < R) {
@@ -793,7 +797,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                     io.u[l][0] = v[l][0];
                     io.u[l][1] = v[l][1];
                 }
-                coarse_step<L, Q, S, BWD>(D0, coef_d, pd, ex_s, c, f, a.cpt * col_pitch(N), step_of(0, jj), step_of(nslot - 1, jj),
+                coarse_step<L, Q>(bwd, D0, coef_d, pd, ex_s, c, f, a.cpt * col_pitch(N), step_of(0, jj), step_of(nslot - 1, jj),
                                           nslot, slot, act, mine, mine ? prm[0] : 0, Kmax, sh, io);
                 if (mine) {
 #pragma unroll
@@ -855,7 +859,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     } else if (act && my_cnt > 0 && C == 1 && mode != SWEEP_RECOMPUTE) {
         // forward: U^m(t_m); adjoint: Lambda at the launch's first step (Lambda^m(t_{m-1}) for
         // the window's first)
-        double2* dst = !BWD ? pd.Uend : (lo == 0 ? pd.Lam0 : pd.Lstate);
+        double2* dst = !bwd ? pd.Uend : (lo == 0 ? pd.Lam0 : pd.Lstate);
 #pragma unroll
         for (int l = 0; l < L; ++l) dst[wcol + f * L + l] = state_out(l);
     }
@@ -863,7 +867,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
 
 template <int L, int Q, int SOLVER, bool BWD, bool PROP = false, int MAXT = MAX_TILE_THREADS>
 __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
-    sweep_tile<L, Q, SOLVER, BWD, PROP>(a, a.mode, blockIdx.x);
+    static_assert(!(BWD && PROP), "propagators are forward sweeps");
+    sweep_tile<L, Q, SOLVER, PROP>(a, a.mode, blockIdx.x, BWD);
 }
 // The history sweep and the adjoint sweep in one launch, where neither needs the other: of a sliced
 // problem, or the recomputation and the adjoint of one checkpoint segment (the products of both
@@ -871,11 +876,21 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
 template <int L, int Q, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_sweep_both(const SweepArgs a) {
     const int n = gridDim.x / 2;
-    if (blockIdx.x < n)   // (nothing to recompute without segments: batches of both kinds)
-        sweep_tile<L, Q, SOLVER_MIXED, false, false>(
-            a, a.pds[a.tiles[blockIdx.x].prob].C > 1 ? SWEEP_HISTORY : SWEEP_RECOMPUTE, blockIdx.x);
-    else
-        sweep_tile<L, Q, SOLVER_MIXED, true, false>(a, SWEEP_ADJOINT, blockIdx.x - n);
+    const bool bwd = blockIdx.x >= n;
+    const int block = blockIdx.x - (bwd ? n : 0);
+    // (nothing to recompute without segments: batches of both kinds)
+    const int mode = bwd ? SWEEP_ADJOINT : a.pds[a.tiles[block].prob].C > 1 ? SWEEP_HISTORY : SWEEP_RECOMPUTE;
+    // One body for both, half the instructions to fetch: with two, 28% of QFT-4's 36 us went to fetches
+    // (27 us with one; two transmons from the host 248 -> 232 us, 5 transmons checkpointed 39.6 -> 38.9
+    // ms).  The lean 2-level sweeps spill more registers in one body (QFT-16 3.84 -> 3.89 ms).
+    if constexpr (L == 2 && MAXT == MAX_LEAN_TILE_THREADS) {
+        if (bwd)
+            sweep_tile<L, Q, SOLVER_MIXED, false>(a, SWEEP_ADJOINT, block, true);
+        else
+            sweep_tile<L, Q, SOLVER_MIXED, false>(a, mode, block, false);
+    } else {
+        sweep_tile<L, Q, SOLVER_MIXED, false>(a, mode, block, bwd);
+    }
 }
 
 }  // namespace msqoc

@@ -165,11 +165,12 @@ struct ExTab {
     float2 cs[MAXEX];   // (h/2) J split into two floats; x is its FP32 rounding
     double cd[MAXEX];
 };
-__device__ __forceinline__ void fill_exchange(ExTab& t, const ProbDev& pd) {
+// sg: +-1, a sign of every coefficient
+__device__ __forceinline__ void fill_exchange(ExTab& t, const ProbDev& pd, double sg = 1.0) {
     for (int e = threadIdx.x; e < pd.nex; e += blockDim.x) {
         t.mask[e] = (1 << (pd.q - 1 - pd.ex_j[e])) | (1 << (pd.q - 1 - pd.ex_k[e]));
-        t.cs[e] = split_scaled(pd.ex_c[e], 0);
-        t.cd[e] = pd.ex_c[e];
+        t.cs[e] = split_scaled(sg * pd.ex_c[e], 0);
+        t.cd[e] = sg * pd.ex_c[e];
     }
     if (threadIdx.x == 0) t.n = pd.nex;
 }
