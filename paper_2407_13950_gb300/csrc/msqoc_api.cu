@@ -666,7 +666,7 @@ size_t gradient_bytes(const ProbDev& pd) {
     b += size_t(pd.q) * pd.nsteps * sizeof(double2);
     if (pd.C > 1) b += V * ne * sizeof(double2);
     if (pd.nseg > 1) b += size_t(pd.M) * pd.nseg * ne * sizeof(double2);
-    if (pd.nseg * pd.nsub > 1) b += size_t(pd.M) * ne * sizeof(double2);
+    if (pd.nseg * pd.nsub > 1) b += V * ne * sizeof(double2);
     return b;
 }
 // propagators and slice states of a sliced problem
@@ -1010,7 +1010,7 @@ msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s) {
     if (e == cudaSuccess && pd.C > 1) e = dalloc(&p->Lend, V * p->ne);
     if (e == cudaSuccess) e = dalloc(&p->quad, size_t(pd.q) * pd.nsteps);
     if (e == cudaSuccess && pd.nseg > 1) e = dalloc(&p->ckpt, M * pd.nseg * p->ne);
-    if (e == cudaSuccess && pd.nseg * pd.nsub > 1) e = dalloc(&p->Lstate, M * p->ne);
+    if (e == cudaSuccess && pd.nseg * pd.nsub > 1) e = dalloc(&p->Lstate, V * p->ne);
     if (e != cudaSuccess) {
         for (double2** b : {&p->hist, &p->lhist, &p->Lend, &p->quad, &p->ckpt, &p->Lstate}) {
             if (*b) cudaFree(*b);

@@ -55,7 +55,7 @@ struct msqoc_problem {
     double2* phase = nullptr;
     double2* hist = nullptr;       // allocated by the first gradient evaluation
     double2* ckpt = nullptr;       // (with hist, when K > 1)
-    double2* Lstate = nullptr;     // (with hist, when K > 1)
+    double2* Lstate = nullptr;     // (with hist, when a window takes several adjoint launches)
     double2* Uend = nullptr;
     double2* Lterm = nullptr;
     double2* Lam0 = nullptr;

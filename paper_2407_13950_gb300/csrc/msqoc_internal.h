@@ -117,7 +117,7 @@ struct ProbDev {
     double2* Uend;               // [M][E][N] U^m(t_m)
     double2* Lterm;              // [M][E][N] Lambda^m(t_m)
     double2* Lam0;               // [M][E][N] Lambda^m(t_{m-1})
-    double2* Lstate;             // [M][E][N] adjoint state between segments
+    double2* Lstate;             // [M C][E][N] adjoint state between launches (chunks, segments)
     double* term;                // [M] pen_m (m < M), J (m = M)
     int* status;                 // status word (ST_* bits)
 };

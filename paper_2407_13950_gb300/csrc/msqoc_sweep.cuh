@@ -464,8 +464,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     //   forward, whole window : U^m(t_{m-1}) = W^{m-1} (identity embedding for the first window
     //                           of the whole problem)
     //   forward, recompute    : the segment's checkpoint
-    //   adjoint               : Lambda^m(t_m) for the window's last segment, else the state the
-    //                           previous (later) segment left
+    //   adjoint               : Lambda^m(t_m) (a slice: Lend) for the window's last steps, else the
+    //                           state the launch of the chunk or segment after these left
     double2 u[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
@@ -475,7 +475,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
         } else if (my_cnt == 0) {
             u[l] = make_double2(0.0, 0.0);
         } else if (bwd) {
-            u[l] = C > 1 ? pd.Lend[wcol + i] : (lo + my_cnt == my_ns) ? pd.Lterm[wcol + i] : pd.Lstate[wcol + i];
+            u[l] = lo + my_cnt < my_ns ? pd.Lstate[wcol + i] : C > 1 ? pd.Lend[wcol + i] : pd.Lterm[wcol + i];
         } else if (C > 1) {
             u[l] = pd.Ubeg[wcol + i];
         } else if (mode == SWEEP_RECOMPUTE) {
@@ -856,9 +856,9 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
 #pragma unroll
             for (int l = 0; l < L; ++l) dst[l] = state_out(l);
         }
-    } else if (act && my_cnt > 0 && C == 1 && mode != SWEEP_RECOMPUTE) {
+    } else if (act && my_cnt > 0 && mode != SWEEP_RECOMPUTE && (C == 1 || (bwd && lo > 0))) {
         // forward: U^m(t_m); adjoint: Lambda at the launch's first step (Lambda^m(t_{m-1}) for
-        // the window's first)
+        // the window's first); of a slice only the state between its chunks (k_compose has the rest)
         double2* dst = !bwd ? pd.Uend : (lo == 0 ? pd.Lam0 : pd.Lstate);
 #pragma unroll
         for (int l = 0; l < L; ++l) dst[wcol + f * L + l] = state_out(l);
