@@ -11,7 +11,7 @@ namespace msqoc {
 // Iteration counts of the implicit-midpoint solve of one step from the contraction bound
 // rho = ||P iX_C|| <= (h/2) lam sum_k |d_k(t_{n+1/2})| of the diagonally preconditioned
 // fixed point (P = (I + i kappa)^-1, kappa = (h/2) D) and kap = max |kappa|.  Packed as j1 | j2 << 8 |
-// passes << 16 | bad << 24 | coarse << 25.
+// passes << 16 | bad << 24 | coarse << 25 | nan << 26.
 //   FP64 solver : j1 = K sweeps with rho^(K+1) <= 2^-56.
 //   mixed solver, one thread per fiber: the FP32 estimate m0 of the increment m = z - U leaves the
 //     error e1 = u32 (2 kap + c rho) + rho^j1 del relative to |U| (its roundings plus truncation).
@@ -30,9 +30,12 @@ namespace msqoc {
 //     terms (rms), stays below the FP64 rounding of the state where kap <= 2^-4 and rho <= 2^-5;
 //     other steps are taken in FP64 (j1 = K sweeps as the FP64 solver).
 //   bad: rho >= 1/2, outside the range the counts are derived for.
+//   nan: a control is not a number.  The split coefficients cannot say so (msqoc_split.cuh), so the
+//     sweeps set the state of such a step (a coarse one) to NaN.
 __device__ inline int step_counts(int solver, int pair, float rho, float kap, float drho) {
     int a = 1, b = 1, r = 1, bad = 0;
-    const int coarse = solver == SOLVER_MIXED && !pair && (rho > 0.03125f || kap > 0.0625f) ? 1 : 0;
+    const int nan = rho != rho ? 1 : 0;
+    const int coarse = solver == SOLVER_MIXED && !pair && (nan || rho > 0.03125f || kap > 0.0625f) ? 1 : 0;
     if (rho > 1e-30f) {
         const float lr = logf(rho);
         if (solver == SOLVER_FP64 || coarse) {
@@ -69,7 +72,7 @@ __device__ inline int step_counts(int solver, int pair, float rho, float kap, fl
         }
         if (rho >= 0.5f) bad = 1;
     }
-    return a | (b << 8) | (r << 16) | (bad << 24) | (coarse << 25);
+    return a | (b << 8) | (r << 16) | (bad << 24) | (coarse << 25) | (nan << 26);
 }
 
 // The quadratic cardinal B-splines active at time t: on [j dtau, (j+1) dtau) the three

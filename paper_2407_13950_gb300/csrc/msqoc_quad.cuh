@@ -96,7 +96,9 @@ __device__ __forceinline__ double2 quad_operand(const double2& v) { return v; }
 template <int MODE>
 __device__ __forceinline__ std::conditional_t<MODE == 2, double2, float4> quad_operand(const float4& v) {
     if constexpr (MODE == 2)
-        return make_double2(df_to_f64_scaled(DF{v.x, v.z}, 0), df_to_f64_scaled(DF{v.y, v.w}, 0));
+        // (NaN has no place in the conversion's integer arithmetic)
+        return make_double2(v.x == v.x ? df_to_f64_scaled(DF{v.x, v.z}, 0) : NAN,
+                            v.y == v.y ? df_to_f64_scaled(DF{v.y, v.w}, 0) : NAN);
     else
         return v;
 }
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(32 * quad_warps<L, Q>()) k_quad(const QuadArgs
         for (int w = 1; w < L - 1; ++w) t = gsum_add(t, q[w * spw * 2]);
         double v;
         if constexpr (MODE == 1)
-            v = df_to_f64_scaled(t, S);
+            v = t.s == t.s ? df_to_f64_scaled(t, S) : NAN;
         else
             v = SPLIT ? ldexp(t, S) : t;
         reinterpret_cast<double*>(pd.quad)[2 * (size_t(kk) * pd.nsteps + n0 + lo + j0 + s) + (r & 1)] = v;

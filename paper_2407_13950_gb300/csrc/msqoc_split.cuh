@@ -243,8 +243,9 @@ __host__ __device__ __forceinline__ void tf_add(TF& u, float s, float t) {
     const DF q = fast_two_sum(p.c, r);
     u = TF{p.s, q.s, q.c};
 }
-// u 2^sh rounded to a double (|sh| <= 896)
+// u 2^sh rounded to a double (|sh| <= 896); NaN for a leading part that is NaN
 __host__ __device__ __forceinline__ double tf_to_f64(TF u, int sh) {
+    if (u.a != u.a) return NAN;
     return f64_of_float_scaled_normal(u.a, sh) +
            (f64_of_float_scaled_normal(u.b, sh) + f64_of_float_scaled_normal(u.c, sh));
 }

@@ -162,7 +162,8 @@ __device__ __forceinline__ float4 load_coefficient(const ProbDev& pd, int lane, 
 }
 // The coefficients go out in FP64 (FP64 solver) or in FP32 and split into two floats (mixed solver).
 // The iteration counts of the step (packed by step_counts in the controls kernel) are unpacked into
-// prm; prm[3] holds the solver-range flag (bit 0) and the coarse-step flag (bit 1).  sg: the sign s of
+// prm; prm[3] holds the solver-range flag (bit 0), the coarse-step flag (bit 1) and the flag of a
+// control that is NaN (bit 2).  sg: the sign s of
 // the step's off-diagonal term, which multiplies every coefficient (exactly).
 template <int L, int Q, int SOLVER>
 __device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, const float4& in, int cnt, float sg,
@@ -194,7 +195,7 @@ __device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, c
         prm[0] = cnt & 0xff;
         prm[1] = (cnt >> 8) & 0xff;
         prm[2] = (cnt >> 16) & 0xff;
-        prm[3] = (cnt >> 24) & 3;
+        prm[3] = (cnt >> 24) & 7;
     }
 }
 
@@ -488,9 +489,9 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     }
 
     // ---- the mixed solver's per-column scale, from the launch's initial state (column_shift)
-    int sh = 0;   // the column's scale exponent (ColScale cs below)
+    int sh = 0;   // the column's scale exponent
+    __shared__ int colexp_s[MAX_TILE_COLS];
     if constexpr (SOLVER == SOLVER_MIXED) {
-        __shared__ int colexp_s[MAX_TILE_COLS];
         for (int j = tid; j < MAX_TILE_COLS; j += blockDim.x) colexp_s[j] = 0;
         tile_sync();
         int ce = 0;
@@ -500,13 +501,15 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
         tile_sync();
         sh = column_shift(colexp_s[c < MAX_TILE_COLS ? c : 0]);
     }
-    // the mixed solver's state, units 2^sh
+    // the mixed solver's state, units 2^sh; a column with an entry that is not finite is NaN (a
+    // split has no form for it, and its scale leaves nothing of the others)
     TF v[L][2];
     if constexpr (SOLVER == SOLVER_MIXED) {
 #pragma unroll
         for (int l = 0; l < L; ++l) {
             v[l][0] = tf_split(u[l].x, sh);
             v[l][1] = tf_split(u[l].y, sh);
+            if (colexp_s[c < MAX_TILE_COLS ? c : 0] == EXP_NONFINITE) v[l][0].a = v[l][1].a = NAN;
         }
     }
     // the midpoint states' column scale exponent, read by the quadrature kernel: per segment for
@@ -802,6 +805,11 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                 if (mine) {
 #pragma unroll
                     for (int l = 0; l < L; ++l) {
+                        // (the control is NaN, or the state was: coarse_step's splits lose both)
+                        if ((prm[3] & 4) || v[l][0].a != v[l][0].a) {
+                            io.z[l] = make_float4(NAN, NAN, NAN, NAN);
+                            io.u[l][0].a = io.u[l][1].a = NAN;
+                        }
                         zf[l] = io.z[l];
                         if (live) {
                             v[l][0] = io.u[l][0];

@@ -78,7 +78,8 @@ __device__ __forceinline__ float2 f32_of_scaled(double2 v, const ColScale& cs) {
 __device__ __forceinline__ double2 f64_of_scaled(float2 v, const ColScale& cs) {
     return make_double2(f64_of_scaled(v.x, cs), f64_of_scaled(v.y, cs));
 }
-// biased exponent field of a double (0 for zero and subnormals)
+// biased exponent field of a double (0 for zero and subnormals, EXP_NONFINITE for infinities and NaN)
+constexpr int EXP_NONFINITE = 0x7ff;
 __device__ __forceinline__ int exp_field(double x) {
     return static_cast<int>(static_cast<unsigned long long>(__double_as_longlong(x)) >> 52) & 0x7ff;
 }

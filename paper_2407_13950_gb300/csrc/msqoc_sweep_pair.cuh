@@ -144,7 +144,7 @@ __device__ __forceinline__ void step_coefficients_pair(const ProbDev& pd, int la
         prm[0] = cnt & 0xff;
         prm[1] = (cnt >> 8) & 0xff;
         prm[2] = (cnt >> 16) & 0xff;
-        prm[3] = (cnt >> 24) & 1;
+        prm[3] = (cnt >> 24) & 5;   // the solver's range, and a control that is NaN
     }
 }
 
@@ -287,7 +287,12 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
         for (int l = 0; l < LS; ++l) ce = max(ce, exp_field(u[l]));
         if (act && ce > 0 && c < MAX_TILE_COLS) atomicMax(&colexp_s[c], ce);
         tile_sync();
-        sh = column_shift(colexp_s[c < MAX_TILE_COLS ? c : 0]);
+        const int cx = colexp_s[c < MAX_TILE_COLS ? c : 0];
+        sh = column_shift(cx);
+        if (cx == EXP_NONFINITE) {   // (the scale leaves nothing of the column's finite entries)
+#pragma unroll
+            for (int l = 0; l < LS; ++l) u[l] = NAN;
+        }
     }
     const ColScale cs = col_scale(sh);
     // this part's components of a [..][N] complex array at the fiber
@@ -505,9 +510,14 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 }
                 tile_sync();
             }
+            // (the FP32 corrections lose a NaN)
+            if (prm[3] & 4) {
+#pragma unroll
+                for (int l = 0; l < LS; ++l) z[l] = NAN;
+            }
         }
 
-        if (tid == 0 && (prm0[3] || (nslot > 1 && prm1[3]))) atomicOr(pd.status, ST_SOLVER_RANGE);
+        if (tid == 0 && ((prm0[3] & 1) || (nslot > 1 && (prm1[3] & 1)))) atomicOr(pd.status, ST_SOLVER_RANGE);
 
         // ---- midpoint states for the quadrature (async bulk store at the next step)
         if (want_hist) {
