@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(CTRL_THREADS) k_controls(const ProbDev pd, con
         return;
     }
     // a block takes CTRL_THREADS - 2 steps and one more on either side (the changes of the controls
-    // over a step, in FP32)
+    // over a step, in FP32: of (h/2) d, which has no unit, so that no choice of units leaves its range)
     __shared__ float2 ds[MAXQ][CTRL_THREADS];
     const int64_t per = CTRL_THREADS - 2;
     for (int64_t n0 = int64_t(blockIdx.x) * per; n0 < pd.nsteps; n0 += int64_t(nctrl) * per) {
@@ -129,10 +129,11 @@ __global__ void __launch_bounds__(CTRL_THREADS) k_controls(const ProbDev pd, con
         const int64_t n = min(max(n0 + t - 1, int64_t(0)), pd.nsteps - 1);
         const bool own = t >= 1 && t <= per && n0 + t - 1 < pd.nsteps;
         const SplineAt sp = spline_at(pd, (double(n) + 0.5) * pd.h);
-        float mag = 0.f;   // sum_k |d_k| for the contraction bound
+        float mag = 0.f;   // (h/2) sum_k |d_k| for the contraction bound
         for (int k = 0; k < pd.q; ++k) {
             const double2 dk = control_at(pd, n, k, sp);
-            const float2 df = make_float2(float(dk.x), float(dk.y));
+            const double2 hd = make_double2(pd.sc[0] * dk.x, pd.sc[0] * dk.y);   // sc[0] = h/2
+            const float2 df = make_float2(float(hd.x), float(hd.y));
             ds[k][t] = df;
             mag += sqrtf(df.x * df.x + df.y * df.y);
             if (own) {
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(CTRL_THREADS) k_controls(const ProbDev pd, con
                     for (int j = 1; j < pd.L; ++j) {
                         const double s = pd.sc[2 * j + 1];   // (h/2) sqrt(j)
                         pd.coef[(size_t(n) * pd.q + k) * (pd.L - 1) + j - 1] =
-                            split_scaled(make_double2(s * dk.x, s * dk.y), 0);
+                            split_scaled(j == 1 ? hd : make_double2(s * dk.x, s * dk.y), 0);
                     }
             }
         }
@@ -153,9 +154,9 @@ __global__ void __launch_bounds__(CTRL_THREADS) k_controls(const ProbDev pd, con
                 dm += sqrtf((c.x - b.x) * (c.x - b.x) + (c.y - b.y) * (c.y - b.y));
                 dp += sqrtf((c.x - e.x) * (c.x - e.x) + (c.y - e.y) * (c.y - e.y));
             }
-            const float hl = float(0.5 * pd.h * pd.lam);
-            const float rho = (hl * mag + float(pd.rho_ex)) * 1.0001f;
-            const float drho = hl * (fmaxf(dm, dp) + 1e-6f * mag) * 1.0001f;
+            const float lam = float(pd.lam);
+            const float rho = (lam * mag + float(pd.rho_ex)) * 1.0001f;
+            const float drho = lam * (fmaxf(dm, dp) + 1e-6f * mag) * 1.0001f;
             pd.spl[n] = Spline4{sp.s0, step_counts(pd.solver, pair, rho, float(pd.kap), drho), sp.w0, sp.w1, sp.w2};
         }
         __syncthreads();
