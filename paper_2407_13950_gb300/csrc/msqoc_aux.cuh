@@ -11,7 +11,7 @@ namespace msqoc {
 // Iteration counts of the implicit-midpoint solve of one step from the contraction bound
 // rho = ||P iX_C|| <= (h/2) lam sum_k |d_k(t_{n+1/2})| of the diagonally preconditioned
 // fixed point (P = (I + i kappa)^-1, kappa = (h/2) D) and kap = max |kappa|.  Packed as j1 | j2 << 8 |
-// passes << 16 | bad << 24 | coarse << 25 | nan << 26.
+// passes << 16 | bad << 24 | coarse << 25 | nan << 26 | wide << 27.
 //   FP64 solver : j1 = K sweeps with rho^(K+1) <= 2^-56.
 //   mixed solver, one thread per fiber: the FP32 estimate m0 of the increment m = z - U leaves the
 //     error e1 = u32 (2 kap + c rho) + rho^j1 del relative to |U| (its roundings plus truncation).
@@ -28,7 +28,9 @@ namespace msqoc {
 //     |P rhs|; each FP64 residual + FP32 correction multiplies it by phi = c u32 + rho^(j2+1).
 //   coarse (one thread per fiber): the compensated increment's error, about 2^-49 of its leading
 //     terms (rms), stays below the FP64 rounding of the state where kap <= 2^-4 and rho <= 2^-5;
-//     other steps are taken in FP64 (j1 = K sweeps as the FP64 solver).
+//     other steps keep the rotation apart (coarse_step): there only d is solved for, and no term but
+//     del's has the factor kap (the state changes by at most twice its norm).  wide: their last
+//     pass is in FP64, where rho > 2^-5.
 //   bad: rho >= 1/2, outside the range the counts are derived for.
 //   nan: a control is not a number.  The split coefficients cannot say so (msqoc_split.cuh), so the
 //     sweeps set the state of such a step (a coarse one) to NaN.
@@ -36,15 +38,17 @@ __device__ inline int step_counts(int solver, int pair, float rho, float kap, fl
     int a = 1, b = 1, r = 1, bad = 0;
     const int nan = rho != rho ? 1 : 0;
     const int coarse = solver == SOLVER_MIXED && !pair && (nan || rho > 0.03125f || kap > 0.0625f) ? 1 : 0;
+    const int wide = coarse && rho > 0.03125f ? 1 : 0;
     if (rho > 1e-30f) {
         const float lr = logf(rho);
-        if (solver == SOLVER_FP64 || coarse) {
+        if (solver == SOLVER_FP64) {
             a = int(ceilf(-38.8162f / lr)) - 1;   // log(2^-56) = -38.816
             a = a < 1 ? 1 : (a > 60 ? 60 : a);
         } else {
             const float u32 = 5.9604645e-8f, c = 4.f, target = 1.1102230e-16f;
-            const float f1 = pair ? c * u32 * rho : u32 * (2.f * kap + c * rho), f2 = pair ? c * u32 : f1;
-            const float del = pair ? rho : fminf(rho, 2.f * rho * (kap + rho) + drho);
+            const float f1 = pair || coarse ? c * u32 * rho : u32 * (2.f * kap + c * rho), f2 = pair ? c * u32 : f1;
+            const float del = pair ? rho : coarse ? 2.f * rho * fminf(kap + rho, 1.f) + drho
+                                                  : fminf(rho, 2.f * rho * (kap + rho) + drho);
             const int j0 = max(1, min(30, int(ceilf(logf(u32) / lr))));   // rho^j0 <= u32
             r = 0;
             for (int pass = 1; pass <= 6 && r == 0; ++pass) {
@@ -72,7 +76,7 @@ __device__ inline int step_counts(int solver, int pair, float rho, float kap, fl
         }
         if (rho >= 0.5f) bad = 1;
     }
-    return a | (b << 8) | (r << 16) | (bad << 24) | (coarse << 25) | (nan << 26);
+    return a | (b << 8) | (r << 16) | (bad << 24) | (coarse << 25) | (nan << 26) | (wide << 27);
 }
 
 // The quadratic cardinal B-splines active at time t: on [j dtau, (j+1) dtau) the three

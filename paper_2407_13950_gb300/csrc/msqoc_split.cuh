@@ -243,6 +243,35 @@ __host__ __device__ __forceinline__ void tf_add(TF& u, float s, float t) {
     const DF q = fast_two_sum(p.c, r);
     u = TF{p.s, q.s, q.c};
 }
+// The same for an increment s + t + r of any size against the state's.
+__host__ __device__ __forceinline__ void tf_add3(TF& u, float s, float t, float r) {
+    const DF x = two_sum(u.a, s);
+    const DF y = two_sum(u.b, x.c);
+    const DF z = two_sum(y.s, t);
+    const DF p = two_sum(x.s, z.s);
+    const DF q = two_sum(p.c, fadd_n(fadd_n(u.c, r), fadd_n(y.c, z.c)));
+    u = TF{p.s, q.s, q.c};
+}
+// x + y (two doubles, |y| <= ulp(x)) as three floats
+__host__ __device__ __forceinline__ TF tf_split_pair(double x, double y) {
+    const float2 h = split_scaled(x, 0);
+    return TF{h.x, h.y, static_cast<float>(((x - static_cast<double>(h.x)) - static_cast<double>(h.y)) + y)};
+}
+// a b and a + b of numbers of three floats, to about 2^-70 of the product, of the larger summand; the
+// parts of the result may overlap by a few bits
+__host__ __device__ __forceinline__ TF tf_mul(TF a, TF b) {
+    const float p = fmul_n(a.a, b.a), e = ffma_n(a.a, b.a, -p);
+    const float p1 = fmul_n(a.a, b.b), e1 = ffma_n(a.a, b.b, -p1);
+    const float p2 = fmul_n(a.b, b.a), e2 = ffma_n(a.b, b.a, -p2);
+    const DF x = two_sum(p1, p2), y = two_sum(x.s, e);
+    const float t = ffma_n(a.a, b.c, ffma_n(a.b, b.b, ffma_n(a.c, b.a, fadd_n(e1, e2))));
+    return TF{p, y.s, fadd_n(t, fadd_n(x.c, y.c))};
+}
+__host__ __device__ __forceinline__ TF tf_sum(TF a, TF b) {
+    const DF x = two_sum(a.a, b.a), y = two_sum(a.b, b.b), z = two_sum(y.s, x.c);
+    return TF{x.s, z.s, fadd_n(fadd_n(a.c, b.c), fadd_n(y.c, z.c))};
+}
+__host__ __device__ __forceinline__ TF tf_neg(TF a) { return TF{-a.a, -a.b, -a.c}; }
 // u 2^sh rounded to a double (|sh| <= 896); NaN for a leading part that is NaN
 __host__ __device__ __forceinline__ double tf_to_f64(TF u, int sh) {
     if (u.a != u.a) return NAN;

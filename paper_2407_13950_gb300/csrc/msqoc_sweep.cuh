@@ -162,8 +162,8 @@ __device__ __forceinline__ float4 load_coefficient(const ProbDev& pd, int lane, 
 }
 // The coefficients go out in FP64 (FP64 solver) or in FP32 and split into two floats (mixed solver).
 // The iteration counts of the step (packed by step_counts in the controls kernel) are unpacked into
-// prm; prm[3] holds the solver-range flag (bit 0), the coarse-step flag (bit 1) and the flag of a
-// control that is NaN (bit 2).  sg: the sign s of
+// prm; prm[3] holds the solver-range flag (bit 0), the coarse-step flag (bit 1), the flag of a
+// control that is NaN (bit 2) and that of a coarse step whose last pass is in FP64 (bit 3).  sg: the sign s of
 // the step's off-diagonal term, which multiplies every coefficient (exactly).
 template <int L, int Q, int SOLVER>
 __device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, const float4& in, int cnt, float sg,
@@ -195,7 +195,7 @@ __device__ __forceinline__ void step_coefficients(const ProbDev& pd, int lane, c
         prm[0] = cnt & 0xff;
         prm[1] = (cnt >> 8) & 0xff;
         prm[2] = (cnt >> 16) & 0xff;
-        prm[3] = (cnt >> 24) & 7;
+        prm[3] = (cnt >> 24) & 15;
     }
 }
 
@@ -253,61 +253,259 @@ __device__ __forceinline__ void apply_off_df(const float4* __restrict__ buf, con
 }
 
 // ------------------------------------------------------------------ coarse steps, out of line
-// The mixed solver's step in FP64, for the steps step_counts flags as coarse: where the rotation
-// of a drift entry or the contraction factor is so large that the compensated increment's 2^-48
-// relative error would exceed the FP64 rounding of the state.  The fixed point z = P u + s P w(z)
-// (s in the coefficients) takes K sweeps, U' = 2 z - U.  Out of line: it is rare, and everything it needs would cost the
-// common step registers.  Every thread of the tile takes part in the barriers; `mine` says
-// whether the thread's slot is coarse at this step.  The buffer's zero entry stays zero.
-template <int L> struct CoarseIO {
-    TF u[L][2];
-    float4 z[L];
-};
-template <int L, int Q>
-static __device__ __noinline__ void coarse_step(bool bwd, double2* D0, double2* cfd, const ProbDev& pd, const ExTab& ex, int c,
-                                                int f, int zero, int64_t n0, int64_t n1, int nslot, int slot, bool act,
-                                                bool mine, int K, int Kmax, int sh, CoarseIO<L>& io) {
-    constexpr int NSLOT = Q * L * 2;
+// The mixed solver's step where the rotation of a drift entry or the contraction factor is so large
+// that the common step's compensated increment, about 2^-48 of its terms, would exceed the FP64
+// rounding of the state (step_counts flags it).  Here the rotation is taken apart from the coupling:
+// with P = 1 + G, U' = U + 2 (G U + d) and d = s P w(P U + d).  G U is formed in three floats (G from
+// kappa, so that 1 + 2 G has modulus one to 2^-70); d, whose terms carry the contraction factor rho,
+// comes from the common step's FP32 sweeps and compensated passes, and where rho > 2^-5 its last pass
+// is formed in FP64.  Against the same fixed point carried out in FP64 (6 to 10 applies and every
+// state split and joined): 4 transmons over 600 ns at 256 windows, a gradient of 26000 steps 26.9 -> 4.5
+// ms, of 5000 steps (two passes, some in FP64) 6.9 -> 1.1; 5 transmons over 200 ns, 10000 steps 112 -> 17.
+// Out of line, with everything a thread carries through the step handed over and back in local
+// memory: it is rare, and what it needs would cost the common step registers (4 transmons' lean
+// sweeps 16 -> 216 bytes spilled and 4q-gradient 7% slower while the caller kept its own across the
+// call).  Every thread of the tile takes part in the barriers; a thread whose slot's step is not coarse
+// changes nothing.  The buffers' zero entries stay zero.
+template <int L, int Q> struct CoarseIO {
     Fiber<L, Q> fb;
-    fb.init(c, f, pd, zero);
-    // the step's coefficients of both slots in FP64
-    for (int t = threadIdx.x; t < nslot * NSLOT; t += blockDim.x) {
-        const int i = t % NSLOT, dir = i & 1, l = (i >> 1) % L;
-        const double2 d = pd.ctrl[size_t(t < NSLOT ? n0 : n1) * pd.q + i / (2 * L)];
-        const double s = (dir == 0 ? l < L - 1 : l > 0) ? (bwd ? 1.0 : -1.0) * pd.sc[2 * l + dir] : 0.0;
-        cfd[t] = dir == 0 ? make_double2(-s * d.y, s * d.x) : make_double2(s * d.y, s * d.x);
+    TF u[L][2];                       // the state
+    float4 z[L];                      // the midpoint state
+    float kh[L], kl[L], k3[L];        // kappa (-kappa for the adjoint)
+    float2 Gf[L];
+    TF g[L][2];                       // G, from the launch's first coarse step on
+    float2 d[L];                      // the last coarse step's d
+    bool have_g;
+};
+// par: parity of the step's coefficients; nslot, slot, act, live, bwd as in sweep_tile; later: not the
+// launch's first step; want_z: the midpoint state is wanted; n0, n1: the slots' global steps
+template <int L, int Q>
+static __device__ __noinline__ void coarse_step(CoarseIO<L, Q>& io, const ProbDev& pd, const ExTab& ex, int cpt, int par,
+                                                int nslot, int slot, bool act, bool live, bool bwd, bool later,
+                                                bool want_z, int64_t n0, int64_t n1) {
+    constexpr int NSLOT = Q * L * 2, N = ipow_c(L, Q);
+    extern __shared__ __align__(128) unsigned char smem[];
+    const SweepSmem lay = sweep_layout(Q, L, N, cpt, SOLVER_MIXED, 0, 1);   // (the history's part is not used)
+    double2* cfd = reinterpret_cast<double2*>(smem + lay.coef_d);
+    const float2* cff = reinterpret_cast<float2*>(smem + lay.coef_f) + (par * 2 + slot) * NSLOT;
+    const float4* cfs = reinterpret_cast<float4*>(smem + lay.coef_s) + (par * 2 + slot) * NSLOT;
+    const int* prm0 = reinterpret_cast<int*>(smem + lay.params) + par * 2 * 4;
+    const int* prm1 = prm0 + (nslot > 1 ? 4 : 0);
+    double2* D0 = reinterpret_cast<double2*>(smem + lay.D0);
+    float2* FA = reinterpret_cast<float2*>(smem + lay.FA);
+    float2* FB = reinterpret_cast<float2*>(smem + lay.FB);
+    if (!io.have_g) {
+        io.have_g = true;
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            // G = -i kappa / (1 + i kappa) = (-kappa^2 - i kappa) / (1 + kappa^2) in twice FP64
+            const double k = (double(io.kh[l]) + double(io.kl[l])) + double(io.k3[l]), k2 = k * k, s = 1.0 + k2;
+            const double e = (k2 > 1.0 ? (k2 - s) + 1.0 : (1.0 - s) + k2) + fma(k, k, -k2);
+            const double q = 1.0 / s, ql = (fma(-s, q, 1.0) - e * q) * q;
+            const double gy = -k * q, gyl = fma(-k, q, -gy) - k * ql;
+            const double gx = k * gy, gxl = fma(k, gy, -gx) + k * gyl;
+            io.g[l][0] = tf_split_pair(gx, gxl);
+            io.g[l][1] = tf_split_pair(gy, gyl);
+        }
     }
-    double2 u[L], b[L], z[L], P[L];
+    // counts and flags of the slots whose step is coarse
+    const int* prm = slot ? prm1 : prm0;
+    const bool c0 = prm0[3] & 2, c1 = prm1[3] & 2;
+    auto most = [&](int a, int b) { return max(c0 ? a : 0, c1 ? b : 0); };
+    auto narrow = [](const int* p) { return p[2] - (p[3] & 8 ? 1 : 0); };   // passes in compensated FP32
+    // the sweeps start from the d of the step before where that was a coarse one (its parameters are
+    // those of the other parity until the next step's first barrier)
+    auto warm = [&](const int* p) { return later && (p[par ? -8 + 3 : 8 + 3] & 2); };
+    auto first = [&](const int* p) { return p[0] + (warm(p) ? 0 : FRESH_SWEEPS); };
+    const int j1 = first(prm), j2 = prm[1], R = narrow(prm);
+    const bool mine = prm[3] & 2, nan = prm[3] & 4, wide = prm[3] & 8;      // (wide: a last pass in FP64)
+    const int j1max = most(first(prm0), first(prm1)), j2max = most(prm0[1], prm1[1]);
+    const int Rmax = most(narrow(prm0), narrow(prm1));
+    const bool any_wide = (c0 && prm0[3] & 8) || (c1 && prm1[3] & 8);
+
+    // (copies: what is read from io is read again after every barrier)
+    const Fiber<L, Q> fb = io.fb;
+    TF pu[L][2], d[L][2];   // P U = U + G U, and d
+    float2 gh[L], gl[L];    // G in two floats
 #pragma unroll
     for (int l = 0; l < L; ++l) {
-        P[l] = pd.P[f * L + l];
-        if (bwd) P[l].y = -P[l].y;
-        u[l] = make_double2(tf_to_f64(io.u[l][0], sh), tf_to_f64(io.u[l][1], sh));
-        b[l] = cmul(P[l], u[l]);
-        z[l] = b[l];
+        const TF gx = io.g[l][0], gy = io.g[l][1];
+        gh[l] = make_float2(gx.a, gy.a);
+        gl[l] = make_float2(gx.b, gy.b);
+        const TF x = tf_sum(tf_mul(gx, io.u[l][0]), tf_neg(tf_mul(gy, io.u[l][1])));
+        const TF y = tf_sum(tf_mul(gx, io.u[l][1]), tf_mul(gy, io.u[l][0]));
+        pu[l][0] = io.u[l][0];
+        pu[l][1] = io.u[l][1];
+        tf_add3(pu[l][0], x.a, x.b, x.c);
+        tf_add3(pu[l][1], y.a, y.b, y.c);
+        const float2 t = warm(prm) ? io.d[l] : make_float2(0.f, 0.f);
+        d[l][0] = TF{t.x, 0.f, 0.f};
+        d[l][1] = TF{t.y, 0.f, 0.f};
     }
-    for (int it = 0; it < Kmax; ++it) {
-        tile_sync();   // the buffer's readers are done (and the coefficients written)
+    auto precond = [&](int l, const float2& w) {
+        return make_float2(fmaf(gh[l].x, w.x, fmaf(-gh[l].y, w.y, w.x)), fmaf(gh[l].x, w.y, fmaf(gh[l].y, w.x, w.y)));
+    };
+    int sel = 0;
+    auto exchange = [&](const float2 (&x)[L]) {
+        float2* Fb = sel ? FB : FA;
+        sel ^= 1;
         if (act) {
 #pragma unroll
-            for (int l = 0; l < L; ++l) D0[fb.xo + l] = z[l];
+            for (int l = 0; l < L; ++l) Fb[fb.xo + l] = x[l];
+        }
+        tile_sync();
+        return Fb;
+    };
+    // the correction of a residual r of the d before: delta = r + g; g = s P w(delta)
+    auto correct = [&](const float2 (&r)[L], float2 (&g)[L]) {
+        float2 e[L];
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            e[l] = r[l];
+            g[l] = make_float2(0.f, 0.f);
+        }
+        for (int it = 0; it < j2max; ++it) {
+            const float2* Fe = exchange(e);
+            float2 w[L];
+            apply_off<L, Q, float2>(Fe, cff, fb, e, w, ex);
+            if (it < j2) {
+#pragma unroll
+                for (int l = 0; l < L; ++l) {
+                    g[l] = precond(l, w[l]);
+                    e[l] = make_float2(r[l].x + g[l].x, r[l].y + g[l].y);
+                }
+            }
+        }
+    };
+
+    // the buffers' earlier readers are done: at the end of the step before, or here where the other
+    // slot's step was not coarse
+    if (!(c0 && c1)) tile_sync();
+    // ---- FP32: d
+    {
+        float2 y[L];
+#pragma unroll
+        for (int l = 0; l < L; ++l) y[l] = make_float2(pu[l][0].a + d[l][0].a, pu[l][1].a + d[l][1].a);
+        for (int it = 0;;) {
+            const float2* Fb = exchange(y);
+            float2 w[L];
+            apply_off<L, Q, float2>(Fb, cff, fb, y, w, ex);
+            if (it < j1) {
+#pragma unroll
+                for (int l = 0; l < L; ++l) {
+                    const float2 t = precond(l, w[l]);
+                    d[l][0].a = t.x;
+                    d[l][1].a = t.y;
+                }
+            }
+            if (++it >= j1max) break;
+#pragma unroll
+            for (int l = 0; l < L; ++l) y[l] = make_float2(pu[l][0].a + d[l][0].a, pu[l][1].a + d[l][1].a);
+        }
+#pragma unroll
+        for (int l = 0; l < L; ++l) io.d[l] = make_float2(d[l][0].a, d[l][1].a);
+    }
+    // ---- passes in compensated FP32: d = s P w(z), z = P U + d in two floats
+    float4* D0s = reinterpret_cast<float4*>(D0);
+    for (int pass = 0; pass < Rmax; ++pass) {
+        const bool own = pass < R;
+        float4 zf[L];
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            const DF x = two_sum(pu[l][0].a, d[l][0].a), y = two_sum(pu[l][1].a, d[l][1].a);
+            zf[l] = make_float4(x.s, y.s, fadd_n(x.c, fadd_n(pu[l][0].b, d[l][0].b)),
+                                fadd_n(y.c, fadd_n(pu[l][1].b, d[l][1].b)));
+            if (act) D0s[fb.xo + l] = zf[l];
+        }
+        tile_sync();
+        float2 r[L], g[L];
+        {
+            DF w[L][2];
+            apply_off_df<L, Q>(D0s, cfs, fb, zf, w, ex);
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                DF n[2] = {w[l][0], w[l][1]};
+                df_mac(n[0], gh[l].x, gl[l].x, w[l][0].s, w[l][0].c);
+                df_mac(n[0], -gh[l].y, -gl[l].y, w[l][1].s, w[l][1].c);
+                df_mac(n[1], gh[l].x, gl[l].x, w[l][1].s, w[l][1].c);
+                df_mac(n[1], gh[l].y, gl[l].y, w[l][0].s, w[l][0].c);
+                r[l] = make_float2(fadd_n(fsub_n(n[0].s, d[l][0].a), fsub_n(n[0].c, d[l][0].b)),
+                                   fadd_n(fsub_n(n[1].s, d[l][1].a), fsub_n(n[1].c, d[l][1].b)));
+#pragma unroll
+                for (int p = 0; p < 2; ++p)
+                    if (own) d[l][p] = TF{n[p].s, n[p].c, 0.f};
+            }
+        }
+        correct(r, g);
+        if (own) {
+            // (two-sums: g is as large as rho r, more than a low part)
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                const DF x = two_sum(d[l][0].a, g[l].x), y = two_sum(d[l][1].a, g[l].y);
+                d[l][0] = TF{x.s, fadd_n(d[l][0].b, x.c), 0.f};
+                d[l][1] = TF{y.s, fadd_n(d[l][1].b, y.c), 0.f};
+            }
+        }
+    }
+    // z of three floats
+    auto midpoint = [&](int l, int p) {
+        TF t = pu[l][p];
+        tf_add3(t, d[l][p].a, d[l][p].b, d[l][p].c);
+        return t;
+    };
+    // ---- the last pass in FP64 (in units 2^sh, as everything here)
+    if (any_wide) {
+        for (int t = threadIdx.x; t < nslot * NSLOT; t += blockDim.x) {
+            const int i = t % NSLOT, dir = i & 1, l = (i >> 1) % L;
+            const double2 dk = pd.ctrl[size_t(t < NSLOT ? n0 : n1) * pd.q + i / (2 * L)];
+            const double s = (dir == 0 ? l < L - 1 : l > 0) ? (bwd ? 1.0 : -1.0) * pd.sc[2 * l + dir] : 0.0;
+            cfd[t] = dir == 0 ? make_double2(-s * dk.y, s * dk.x) : make_double2(s * dk.y, s * dk.x);
+        }
+        double2 z[L];
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            z[l] = make_double2(tf_to_f64(midpoint(l, 0), 0), tf_to_f64(midpoint(l, 1), 0));
+            if (act) D0[fb.xo + l] = z[l];
         }
         tile_sync();
         double2 w[L];
         apply_off<L, Q, double2>(D0, cfd + (nslot > 1 ? slot : 0) * NSLOT, fb, z, w, ex);
-        if (it < K) {
+        float2 r[L], g[L];
 #pragma unroll
-            for (int l = 0; l < L; ++l) z[l] = cadd_scaled<1>(b[l], P[l], w[l]);
+        for (int l = 0; l < L; ++l) {
+            double2 P = pd.P[fb.f * L + l];
+            if (bwd) P.y = -P.y;
+            const double2 x = cmul(P, w[l]);
+            const TF n[2] = {tf_split(x.x, 0), tf_split(x.y, 0)};
+            r[l] = make_float2(fadd_n(fsub_n(n[0].a, d[l][0].a), fsub_n(n[0].b, d[l][0].b)),
+                               fadd_n(fsub_n(n[1].a, d[l][1].a), fsub_n(n[1].b, d[l][1].b)));
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+                if (wide) d[l][p] = n[p];
+        }
+        correct(r, g);
+        if (wide) {
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                tf_add3(d[l][0], g[l].x, 0.f, 0.f);
+                tf_add3(d[l][1], g[l].y, 0.f, 0.f);
+            }
         }
     }
     tile_sync();
     if (mine) {
 #pragma unroll
         for (int l = 0; l < L; ++l) {
-            io.z[l] = split_scaled(z[l], sh);
-            const double2 v = reflect(z[l], u[l]);
-            io.u[l][0] = tf_split(v.x, sh);
-            io.u[l][1] = tf_split(v.y, sh);
+            TF z[2];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                z[p] = midpoint(l, p);
+                TF n = TF{2.f * z[p].a, 2.f * z[p].b, 2.f * z[p].c};   // U' = 2 z - U
+                tf_add3(n, -io.u[l][p].a, -io.u[l][p].b, -io.u[l][p].c);
+                if (nan) z[p].a = n.a = NAN;                          // (a control that is NaN)
+                if (live) io.u[l][p] = n;
+            }
+            if (want_z) io.z[l] = make_float4(z[0].a, z[1].a, z[0].b, z[1].b);
         }
     }
 }
@@ -570,6 +768,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
 
     int hpos = 0;   // position of iteration jj in its history group
     bool fresh = true;   // no d of the step before: the first sweep starts from zero
+    CoarseIO<L, Q> io;
+    io.have_g = false;
     for (int jj = 0; jj < nit; ++jj) {
         const int par = jj & 1;
         const bool live = jj < my_cnt;
@@ -680,7 +880,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             };
             float2* Fb = exchange(y);
             first_sync_work();
-            // coarse steps (uniform over a slot) go to FP64 below
+            // coarse steps (uniform over a slot) have a form of their own below
             const bool coarse0 = prm0[3] & 2, coarse1 = nslot > 1 ? (prm1[3] & 2) != 0 : coarse0;
             if (!coarse0 || !coarse1) {
                 const int more = fresh ? FRESH_SWEEPS : 0;
@@ -791,31 +991,35 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                 bulk_wait_read_all();   // (the coarse step's barriers follow)
             }
             fresh = coarse0 || coarse1;
-            if (coarse0 || coarse1) {
-                const bool mine = prm[3] & 2;
-                const int Kmax = max(coarse0 ? prm0[0] : 0, coarse1 ? (nslot > 1 ? prm1[0] : prm0[0]) : 0);
-                CoarseIO<L> io;
+            if (fresh) {
+                if (!io.have_g) {   // (what does not change goes once)
+                    io.fb = fb;
+#pragma unroll
+                    for (int l = 0; l < L; ++l) {
+                        io.kh[l] = kh[l];
+                        io.kl[l] = kl[l];
+                        io.k3[l] = k3[l];
+                        io.Gf[l] = Gf[l];
+                    }
+                }
 #pragma unroll
                 for (int l = 0; l < L; ++l) {
                     io.u[l][0] = v[l][0];
                     io.u[l][1] = v[l][1];
+                    if (want_hist && !(coarse0 && coarse1)) io.z[l] = zf[l];
                 }
-                coarse_step<L, Q>(bwd, D0, coef_d, pd, ex_s, c, f, a.cpt * col_pitch(N), step_of(0, jj), step_of(nslot - 1, jj),
-                                          nslot, slot, act, mine, mine ? prm[0] : 0, Kmax, sh, io);
-                if (mine) {
+                coarse_step<L, Q>(io, pd, ex_s, a.cpt, par, nslot, slot, act, live, bwd, jj > 0, want_hist, step_of(0, jj),
+                                  step_of(nslot - 1, jj));
+                fb = io.fb;
 #pragma unroll
-                    for (int l = 0; l < L; ++l) {
-                        // (the control is NaN, or the state was: coarse_step's splits lose both)
-                        if ((prm[3] & 4) || v[l][0].a != v[l][0].a) {
-                            io.z[l] = make_float4(NAN, NAN, NAN, NAN);
-                            io.u[l][0].a = io.u[l][1].a = NAN;
-                        }
-                        zf[l] = io.z[l];
-                        if (live) {
-                            v[l][0] = io.u[l][0];
-                            v[l][1] = io.u[l][1];
-                        }
-                    }
+                for (int l = 0; l < L; ++l) {
+                    v[l][0] = io.u[l][0];
+                    v[l][1] = io.u[l][1];
+                    if (want_hist) zf[l] = io.z[l];
+                    kh[l] = io.kh[l];
+                    kl[l] = io.kl[l];
+                    k3[l] = io.k3[l];
+                    Gf[l] = io.Gf[l];
                 }
             }
         }
