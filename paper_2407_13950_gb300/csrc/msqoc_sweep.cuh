@@ -255,7 +255,7 @@ __device__ __forceinline__ void apply_off_df(const float4* __restrict__ buf, con
 // ------------------------------------------------------------------ coarse steps, out of line
 // The mixed solver's step where the rotation of a drift entry or the contraction factor is so large
 // that the common step's compensated increment, about 2^-48 of its terms, would exceed the FP64
-// rounding of the state (step_counts flags it).  Here the rotation is taken apart from the coupling:
+// rounding of the state, or that one pass does not reach it (step_counts flags it).  Here the rotation is taken apart from the coupling:
 // with P = 1 + G, U' = U + 2 (G U + d) and d = s P w(P U + d).  G U is formed in three floats (G from
 // kappa, so that 1 + 2 G has modulus one to 2^-70); d, whose terms carry the contraction factor rho,
 // comes from the common step's FP32 sweeps and compensated passes, and where rho > 2^-5 its last pass
@@ -884,12 +884,11 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             const bool coarse0 = prm0[3] & 2, coarse1 = nslot > 1 ? (prm1[3] & 2) != 0 : coarse0;
             if (!coarse0 || !coarse1) {
                 const int more = fresh ? FRESH_SWEEPS : 0;
-                const int j1 = prm[0] + more, j2 = prm[1], R = prm[2];
+                const int j1 = prm[0] + more, j2 = prm[1];
                 const bool two = nslot > 1 && !coarse0 && !coarse1;
                 const int* pm = coarse0 ? prm1 : prm0;
                 const int j1max = (two ? max(prm0[0], prm1[0]) : pm[0]) + more;
                 const int j2max = two ? max(prm0[1], prm1[1]) : pm[1];
-                const int Rmax = two ? max(prm0[2], prm1[2]) : pm[2];
                 for (int it = 0;;) {
                     float2 w[L];
                     apply_off<L, Q, float2>(Fb, cff, fb, y, w, ex_s);
@@ -913,71 +912,62 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
                     const DF zr = two_sum(v[l][0].a, mr[l].s), zi = two_sum(v[l][1].a, mi[l].s);
                     zf[l] = make_float4(zr.s, zi.s, fadd_n(zr.c, v[l][0].b), fadd_n(zi.c, v[l][1].b));
                 }
-                for (int pass = 0;; ++pass) {
-                    if (act) {
+                if (act) {
 #pragma unroll
-                        for (int l = 0; l < L; ++l) D0s[fb.xo + l] = zf[l];
+                    for (int l = 0; l < L; ++l) D0s[fb.xo + l] = zf[l];
+                }
+                // the staged midpoints of the previous step must have been read by their bulk
+                // store (issued at this step's first barrier) before this step's are staged;
+                // waiting here, ahead of a barrier every step has, makes the staging
+                // barrier-free
+                if (want_hist && tid == 0 && hpos == 0) bulk_wait_read_all();
+                tile_sync();
+                float2 r[L], gr[L], e[L];
+                {
+                    DF w[L][2];
+                    apply_off_df<L, Q>(D0s, cfs, fb, zf, w, ex_s);
+#pragma unroll
+                    for (int l = 0; l < L; ++l) {
+                        // m1 = -i kappa z + s w (s in the coefficients)
+                        DF kr = kappa_mul(kh[l], kl[l], k3[l], zf[l].y, zf[l].w);
+                        DF ki = df_neg(kappa_mul(kh[l], kl[l], k3[l], zf[l].x, zf[l].z));
+                        kr = df_add(kr, w[l][0]);
+                        ki = df_add(ki, w[l][1]);
+                        r[l] = make_float2(fadd_n(fsub_n(kr.s, mr[l].s), fsub_n(kr.c, mr[l].c)),
+                                           fadd_n(fsub_n(ki.s, mi[l].s), fsub_n(ki.c, mi[l].c)));
+                        mr[l] = kr;
+                        mi[l] = ki;
+                        // G R, and the first sweep's point P R = R + G R
+                        gr[l] = make_float2(fmaf(Gf[l].x, r[l].x, -Gf[l].y * r[l].y),
+                                            fmaf(Gf[l].x, r[l].y, Gf[l].y * r[l].x));
+                        e[l] = make_float2(r[l].x + gr[l].x, r[l].y + gr[l].y);
                     }
-                    // the staged midpoints of the previous step must have been read by their bulk
-                    // store (issued at this step's first barrier) before this step's are staged;
-                    // waiting here, ahead of a barrier every step has, makes the staging
-                    // barrier-free
-                    if (want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
-                    tile_sync();
-                    float2 r[L], gr[L], e[L];
-                    {
-                        DF w[L][2];
-                        apply_off_df<L, Q>(D0s, cfs, fb, zf, w, ex_s);
+                }
+                // delta = R + g, g = G R + s P w(delta) (e: delta; g is added to the increment, so
+                // it is kept apart from R, whose size would round it)
+                float2 g[L];
+#pragma unroll
+                for (int l = 0; l < L; ++l) g[l] = gr[l];
+                for (int it = 0; it < j2max; ++it) {
+                    float2* Fe = exchange(e);
+                    float2 w[L];
+                    apply_off<L, Q, float2>(Fe, cff, fb, e, w, ex_s);
+                    if (it < j2) {
 #pragma unroll
                         for (int l = 0; l < L; ++l) {
-                            // m1 = -i kappa z + s w (s in the coefficients)
-                            DF kr = kappa_mul(kh[l], kl[l], k3[l], zf[l].y, zf[l].w);
-                            DF ki = df_neg(kappa_mul(kh[l], kl[l], k3[l], zf[l].x, zf[l].z));
-                            kr = df_add(kr, w[l][0]);
-                            ki = df_add(ki, w[l][1]);
-                            r[l] = make_float2(fadd_n(fsub_n(kr.s, mr[l].s), fsub_n(kr.c, mr[l].c)),
-                                               fadd_n(fsub_n(ki.s, mi[l].s), fsub_n(ki.c, mi[l].c)));
-                            if (pass < R) {
-                                mr[l] = kr;
-                                mi[l] = ki;
-                            }
-                            // G R, and the first sweep's point P R = R + G R
-                            gr[l] = make_float2(fmaf(Gf[l].x, r[l].x, -Gf[l].y * r[l].y),
-                                                fmaf(Gf[l].x, r[l].y, Gf[l].y * r[l].x));
-                            e[l] = make_float2(r[l].x + gr[l].x, r[l].y + gr[l].y);
+                            const float2 t = precond(l, w[l]);
+                            g[l] = make_float2(gr[l].x + t.x, gr[l].y + t.y);
+                            e[l] = make_float2(r[l].x + g[l].x, r[l].y + g[l].y);
                         }
                     }
-                    // delta = R + g, g = G R + s P w(delta) (e: delta; g is added to the increment, so
-                    // it is kept apart from R, whose size would round it)
-                    float2 g[L];
+                }
 #pragma unroll
-                    for (int l = 0; l < L; ++l) g[l] = gr[l];
-                    for (int it = 0; it < j2max; ++it) {
-                        float2* Fe = exchange(e);
-                        float2 w[L];
-                        apply_off<L, Q, float2>(Fe, cff, fb, e, w, ex_s);
-                        if (it < j2) {
-#pragma unroll
-                            for (int l = 0; l < L; ++l) {
-                                const float2 t = precond(l, w[l]);
-                                g[l] = make_float2(gr[l].x + t.x, gr[l].y + t.y);
-                                e[l] = make_float2(r[l].x + g[l].x, r[l].y + g[l].y);
-                            }
-                        }
-                    }
-                    if (pass < R) {
-#pragma unroll
-                        for (int l = 0; l < L; ++l) {
-                            mr[l].c = fadd_n(mr[l].c, g[l].x);
-                            mi[l].c = fadd_n(mi[l].c, g[l].y);
-                            if (!want_hist && Rmax == 1) continue;   // z is needed no more
-                            const DF zr = two_sum(zf[l].x, e[l].x), zi = two_sum(zf[l].y, e[l].y);
-                            zf[l] = make_float4(zr.s, zi.s, fadd_n(zf[l].z, zr.c), fadd_n(zf[l].w, zi.c));
-                        }
-                    }
-                    if (pass + 1 >= Rmax) break;
-                    // another pass rewrites D0: every thread must be done reading it
-                    tile_sync();
+                for (int l = 0; l < L; ++l) {
+                    mr[l].c = fadd_n(mr[l].c, g[l].x);
+                    mi[l].c = fadd_n(mi[l].c, g[l].y);
+                    if (!want_hist) continue;   // z is needed no more
+                    const DF zr = two_sum(zf[l].x, e[l].x), zi = two_sum(zf[l].y, e[l].y);
+                    zf[l] = make_float4(zr.s, zi.s, fadd_n(zf[l].z, zr.c), fadd_n(zf[l].w, zi.c));
                 }
                 // U' = U + 2 m
                 if (live && !(prm[3] & 2)) {
@@ -1077,8 +1067,13 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
     }
 }
 
+// Threads that set the register budget: 2-level shapes fit 168 registers in either build, and their
+// one-warp tiles need it: a sub-partition holds three warps of up to 168, two of more (QFT-8's 1536 tiles
+// of both sweeps at 176: two waves, a gradient 326 us in place of 267).
+template <int L, int MAXT>
+constexpr int budget_threads() { return L == 2 ? MAX_LEAN_TILE_THREADS : MAXT; }
 template <int L, int Q, int SOLVER, bool BWD, bool PROP = false, int MAXT = MAX_TILE_THREADS>
-__global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
+__global__ void __launch_bounds__(budget_threads<L, MAXT>(), 1) k_sweep(const SweepArgs a) {
     static_assert(!(BWD && PROP), "propagators are forward sweeps");
     sweep_tile<L, Q, SOLVER, PROP>(a, a.mode, blockIdx.x, BWD);
 }
@@ -1086,7 +1081,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_sweep(const SweepArgs a) {
 // problem, or the recomputation and the adjoint of one checkpoint segment (the products of both
 // are k_quad's).  Blocks 0 .. n - 1 the forward tiles, n .. 2n - 1 the adjoint's.
 template <int L, int Q, int MAXT>
-__global__ void __launch_bounds__(MAXT, 1) k_sweep_both(const SweepArgs a) {
+__global__ void __launch_bounds__(budget_threads<L, MAXT>(), 1) k_sweep_both(const SweepArgs a) {
     const int n = gridDim.x / 2;
     const bool bwd = blockIdx.x >= n;
     const int block = blockIdx.x - (bwd ? n : 0);
