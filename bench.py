@@ -108,7 +108,7 @@ class ClockSampler:
 
 
 SWEEP_SOURCES = ["msqoc_sweep.cuh", "msqoc_sweep_pair.cuh", "msqoc_sweep_common.cuh", "msqoc_split.cuh",
-                 "msqoc_quad.cuh", "msqoc_chain.cuh", "inst_sweep.cu", "msqoc_internal.h"]
+                 "msqoc_quad.cuh", "msqoc_chain.cuh", "msqoc_counts.cuh", "inst_sweep.cu", "msqoc_internal.h"]
 PROFILES = os.path.join(ROOT, "profiles")
 LAYOUTS = {"auto": 0, "fiber": 1, "pair": 2, "quad": 3, "lean": 4}
 

@@ -331,6 +331,13 @@ msqoc_status msqoc_selftest_dot(const double* x, const double* y, int64_t n, int
 msqoc_status msqoc_selftest_carry(const double* u0, const double* P, const double* d, int64_t n, int32_t sh,
                                   int32_t on_device, double* out);
 
+/* Self-test of the iteration counts of one step (on the host): solver (MSQOC_SOLVER_FP64 or _MIXED), pair
+ * (0: one thread per fiber, else a lane family), the contraction bound rho, the largest rotation kap = h
+ * max|D| / 2, and drho, the bound's part that the controls changed over the step before.
+ * out: FP32 (or FP64 solver: all) sweeps of the estimate, sweeps of a pass, passes, flags (1: rho out of
+ * range, 2: coarse step, 4: rho is NaN, 8: the last pass in FP64). */
+msqoc_status msqoc_selftest_step_counts(int32_t solver, int32_t pair, float rho, float kap, float drho, int32_t* out);
+
 /* ---------------------------------------------------------------------------------------
  * Batched evaluation (many problems per launch).
  *

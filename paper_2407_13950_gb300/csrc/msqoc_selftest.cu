@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "../../include/msqoc.h"
+#include "msqoc_counts.cuh"
 #include "msqoc_host.h"
 #include "msqoc_split.cuh"
 #include "msqoc_sweep_common.cuh"
@@ -256,5 +257,17 @@ extern "C" msqoc_status msqoc_selftest_bounded_wait(int64_t spins, int32_t arriv
     if (ce != cudaSuccess) return fail(MSQOC_ERR_CUDA, "bounded-wait self-test: %s", cudaGetErrorString(ce));
     if (seconds_out) *seconds_out = double(ms) * 1e-3;
     if (h & ST_TIMEOUT) return fail(MSQOC_ERR_TIMEOUT, "a bounded device wait gave up after %lld spins", (long long)spins);
+    return MSQOC_OK;
+}
+
+extern "C" msqoc_status msqoc_selftest_step_counts(int32_t solver, int32_t pair, float rho, float kap, float drho,
+                                                   int32_t* out) {
+    if (!out || (solver != SOLVER_FP64 && solver != SOLVER_MIXED))
+        return fail(MSQOC_ERR_INVALID_ARG, "step-count self-test: no output, or solver %d unknown", solver);
+    const int c = step_counts(solver, pair, rho, kap, drho);
+    out[0] = c & 0xff;
+    out[1] = (c >> 8) & 0xff;
+    out[2] = (c >> 16) & 0xff;
+    out[3] = (c >> 24) & 0xff;
     return MSQOC_OK;
 }

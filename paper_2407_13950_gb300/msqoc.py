@@ -29,7 +29,8 @@ EXPORTED = ["msqoc_create_problem", "msqoc_query", "msqoc_query_layout", "msqoc_
             "msqoc_get_objective", "msqoc_get_gradient", "msqoc_batch_eval_subset", "msqoc_autotune",
             "msqoc_rollout", "msqoc_rollout_estimate", "msqoc_eval_regularization", "msqoc_lbfgs_direction",
             "msqoc_lbfgs_trial", "msqoc_lbfgs_update", "msqoc_selftest_bounded_wait",
-            "msqoc_selftest_split", "msqoc_selftest_dot", "msqoc_selftest_carry"]
+            "msqoc_selftest_split", "msqoc_selftest_dot", "msqoc_selftest_carry",
+            "msqoc_selftest_step_counts"]
 BATCH_GRADIENT, BATCH_GRAPH = 1, 2
 KERNEL_NAMES = ["controls", "forward", "terminal", "adjoint", "finalize"]
 
@@ -90,6 +91,7 @@ def load(build_if_missing: bool = True):
             "msqoc_selftest_split": (i32, [vp, i64, i32, i32, vp, vp]),
             "msqoc_selftest_dot": (i32, [vp, vp, i64, i32, i32, i32, vp]),
             "msqoc_selftest_carry": (i32, [vp, vp, vp, i64, i32, i32, vp]),
+            "msqoc_selftest_step_counts": (i32, [i32, i32, ctypes.c_float, ctypes.c_float, ctypes.c_float, vp]),
             "msqoc_eval_objective_noalloc": (i32, [vp, vp, vp, ctypes.c_double, i64, i32, ctypes.c_double, i32,
                                                    vp, vp, vp, vp, vp, vp]),
             "msqoc_batch_create": (i32, [vp, i32, i32, vp]),
@@ -355,6 +357,13 @@ def selftest_dot(x, y, shx: int = 0, shy: int = 0, device: bool = False) -> floa
     _check(load().msqoc_selftest_dot(x.ctypes.data, y.ctypes.data, x.size, int(shx), int(shy), 1 if device else 0,
                                      ctypes.byref(out)))
     return out.value
+
+
+def selftest_step_counts(solver: int, pair: int, rho: float, kap: float, drho: float) -> tuple:
+    """(sweeps of the estimate, sweeps of a pass, passes, flags) of a step (msqoc_selftest_step_counts)."""
+    out = (ctypes.c_int32 * 4)()
+    _check(load().msqoc_selftest_step_counts(solver, pair, rho, kap, drho, out))
+    return tuple(out)
 
 
 def selftest_carry(u0, P, d, sh: int = 0, device: bool = False) -> complex:
