@@ -35,7 +35,7 @@ struct msqoc_batch {
         int ntiles = 0;
         int nseg_max = 1, nsub_max = 1;
         long slots = 1;               // tiles the GPU holds at a time
-        bool quad_small = true;       // every member takes FP64 products (quad_fp64)
+        int qmode = 0;                // the members' form of the gradient products (QuadArgs::mode)
         int quad_blocks = 0;          // blocks of a row of the quadrature launch: the most of the members
         ProbDev* pds = nullptr;
         Tile* tiles = nullptr;
@@ -201,7 +201,6 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, con
                 cudaError_t e = launch_sweep(a, work[gi].ntiles, gs);
                 if (e != cudaSuccess) return e;
                 QuadArgs qa = quad_args(b->probs[g.members[0]]->pd, g.pds, seg, sub);
-                if (qa.mode && !g.quad_small) qa.mode = 1;
                 qa.list = work[gi].list;
                 e = launch_quad(qa, g.quad_blocks, work[gi].nlist, gs);
                 if (e != cudaSuccess) return e;
@@ -287,13 +286,15 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
         for (msqoc_problem* p : b->probs)
             if (!st) st = ensure_gradient_buffers(p, nullptr);
     if (!st && cudaDeviceSynchronize() != cudaSuccess) st = fail(MSQOC_ERR_CUDA, "synchronize failed");
-    // groups by (levels, subsystems, solver, kernel family, tile threads, propagator tiles)
+    // groups by (levels, subsystems, solver, kernel family, tile threads, propagator tiles, form of the
+    // gradient products: a member's results do not depend on the others)
     for (int i = 0; i < n && !st; ++i) {
         const ProbDev& pd = b->probs[i]->pd;
+        const int qmode = flags & MSQOC_BATCH_GRADIENT ? quad_args(pd, nullptr, 0, 0).mode : 0;
         auto it = std::find_if(b->groups.begin(), b->groups.end(), [&](const msqoc_batch::Group& g) {
             return g.L == pd.L && g.q == pd.q && g.solver == pd.solver && g.pair == pd.pair && g.lean == pd.lean &&
                    g.nthreads == pd.nthreads && g.pthreads == b->probs[i]->prop.nthreads &&
-                   g.plean == b->probs[i]->prop.lean;
+                   g.plean == b->probs[i]->prop.lean && g.qmode == qmode;
         });
         if (it == b->groups.end()) {
             b->groups.emplace_back();
@@ -306,6 +307,7 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
             it->nthreads = pd.nthreads;
             it->pthreads = b->probs[i]->prop.nthreads;
             it->plean = b->probs[i]->prop.lean;
+            it->qmode = qmode;
         }
         it->members.push_back(i);
     }
@@ -327,7 +329,6 @@ msqoc_status batch_create(msqoc_problem* const* problems, int32_t n, int32_t fla
             g.nseg_max = std::max(g.nseg_max, pd.nseg);
             g.nsub_max = std::max(g.nsub_max, pd.nsub);
             g.quad_blocks = std::max(g.quad_blocks, quad_blocks(pd));
-            g.quad_small = g.quad_small && quad_fp64(pd);
         }
         std::vector<ProbDev> pds;
         std::vector<Tile> tiles, ptiles;

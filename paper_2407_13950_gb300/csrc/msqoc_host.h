@@ -123,7 +123,6 @@ cudaError_t launch_compose(const ProbDev* pds_dev, const int* list, int E, int M
                            cudaStream_t s);
 // quadrature launch arguments (SweepArgs of the same segment and chunk), see k_quad
 QuadArgs quad_args(const ProbDev& pd, const ProbDev* pds_dev, int seg, int sub);
-bool quad_fp64(const ProbDev& pd);
 // shared memory that admits a tile (see msqoc_api.cu)
 size_t admission_bytes(int q, int L, int N, int cpt, int nthreads, int g, int solver, int pair, int depth);
 
