@@ -228,7 +228,10 @@ struct Fiber {
     }
     // buffer entry of pair e's term for entry l of the fiber (the zero entry where it has none)
     __device__ __forceinline__ int exsrc(int e, int l, int mask) const {
-        return (exm[l] >> e) & 1u ? eb + ((f * L + l) ^ mask) : zero;
+        unsigned m = exm[0];   // (no index into exm, which would put the fiber in local memory)
+#pragma unroll
+        for (int t = 1; t < L; ++t) m = l == t ? exm[t] : m;
+        return (m >> e) & 1u ? eb + ((f * L + l) ^ mask) : zero;
     }
 };
 

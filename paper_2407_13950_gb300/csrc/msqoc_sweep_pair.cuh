@@ -54,12 +54,13 @@ __device__ __forceinline__ float pmac(float acc, float2 c, float xa, float xb) {
 // cf: this part's coefficient pairs of the step's slots, i(h/2)sqrt(.)d_k.
 //
 // SPLIT = 2 (lane quads, L = 2): the thread holds entry le of the fiber only (xa[0], w[0]); the
-// other entry of the in-fiber ladder term comes from the buffer.
+// other entry of the in-fiber ladder term comes from the buffer.  exo: the buffer entries of the first
+// MAXEXF exchange pairs' terms for the thread's entries (Fiber::exsrc).
 template <int L, int Q, typename T2, int SPLIT>
 __device__ __forceinline__ void apply_off_pair(const T2* __restrict__ buf, const T2* __restrict__ cf,
                                                const Fiber<L, Q>& fb, const typename cx<T2>::T (&xa)[L / SPLIT],
                                                typename cx<T2>::T (&w)[L / SPLIT], int p, int le,
-                                               const ExTab& ex) {
+                                               const ExTab& ex, const int (&exo)[MAXEXF][L / SPLIT]) {
     using R = typename cx<T2>::T;
     constexpr int LS = L / SPLIT;
     const R* ba = reinterpret_cast<const R*>(buf) + p;        // component p of entry i: ba[2 i]
@@ -95,15 +96,29 @@ __device__ __forceinline__ void apply_off_pair(const T2* __restrict__ buf, const
     // exchange-coupled problems are 2-level qubit models (the only shapes compiled with it):
     // w += (i (h/2) J x_src)_p, and (i c x)_p = (p ? c : -c) x_{1-p}
     if constexpr (L == 2 && Q >= 2) {
-        for (int e = 0; e < ex.n; ++e) {                       // uniform
-            R c;
+        auto coef = [&](int e) {
             if constexpr (sizeof(R) == 4)
-                c = p ? ex.cs[e].x : -ex.cs[e].x;
+                return p ? ex.cs[e].x : -ex.cs[e].x;
             else
-                c = p ? ex.cd[e] : -ex.cd[e];
-            const int mask = ex.mask[e];
+                return p ? ex.cd[e] : -ex.cd[e];
+        };
+        // Sources known ahead and an unrolled loop, so that the terms' loads overlap: with each
+        // pair's source worked out in a loop QFT-4 and QFT-8 with the FP64 solver (lane quads) took 0.51
+        // and 2.57 ms an objective in place of 0.48 and 2.49, QFT-16 with the mixed one 4.6 in place of 4.1.
 #pragma unroll
-            for (int l = 0; l < LS; ++l) w[l] += c * bb[2 * fb.exsrc(e, le + l, mask)];
+        for (int e = 0; e < MAXEXF; ++e) {
+            if (e >= ex.n) break;                              // uniform
+            const R c = coef(e);
+#pragma unroll
+            for (int l = 0; l < LS; ++l) w[l] += c * bb[2 * exo[e][l]];
+        }
+        if constexpr (SPLIT == 1) {
+            for (int e = MAXEXF; e < ex.n; ++e) {              // uniform (lane quads admit MAXEXF pairs)
+                const R c = coef(e);
+                const int mask = ex.mask[e];
+#pragma unroll
+                for (int l = 0; l < LS; ++l) w[l] += c * bb[2 * fb.exsrc(e, le + l, mask)];
+            }
         }
     }
 }
@@ -229,6 +244,16 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
     fb.init(c, f, pd, a.cpt * col_pitch(N));
     __shared__ ExTab ex_s;   // (ordered before its first read by the first barrier of the time loop)
     fill_exchange(ex_s, pd);
+    int exo[MAXEXF][LS] = {};
+    if constexpr (L == 2 && Q >= 2) {
+#pragma unroll
+        for (int e = 0; e < MAXEXF; ++e)
+            if (e < pd.nex) {
+                const int mask = (1 << (Q - 1 - pd.ex_j[e])) | (1 << (Q - 1 - pd.ex_k[e]));
+#pragma unroll
+                for (int l = 0; l < LS; ++l) exo[e][l] = fb.exsrc(e, le + l, mask);
+            }
+    }
     // the apply buffers' zero entry (read by the exchange terms a fiber entry does not have; the
     // first barrier of the time loop orders these stores before any read)
     if (tid == 0) {
@@ -401,7 +426,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                     tile_sync();
                 }
                 double w[LS];
-                apply_off_pair<L, Q, double2, SPLIT>(Dc, cfd, fb, z, w, part, le, ex_s);
+                apply_off_pair<L, Q, double2, SPLIT>(Dc, cfd, fb, z, w, part, le, ex_s, exo);
                 double wo[LS];
 #pragma unroll
                 for (int l = 0; l < LS; ++l) wo[l] = partner(w[l]);
@@ -428,7 +453,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 tile_sync();
                 first_sync_work();
                 float w[LS];
-                apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, ex_s);
+                apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, ex_s, exo);
 #pragma unroll
                 for (int l = 0; l < LS; ++l) {
                     const float wo = partner(w[l]);
@@ -447,7 +472,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 if (act) store_part<LS, float2>(Fb, fb.xo + le, part, y);
                 tile_sync();
                 float w[LS], wo[LS];
-                apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, ex_s);
+                apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, y, w, part, le, ex_s, exo);
 #pragma unroll
                 for (int l = 0; l < LS; ++l) wo[l] = partner(w[l]);
                 if (it < j1) {
@@ -471,7 +496,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                 if (want_hist && pass == 0 && tid == 0 && hpos == 0) bulk_wait_read_all();
                 tile_sync();
                 double w[LS];
-                apply_off_pair<L, Q, double2, SPLIT>(D0, cfd, fb, z, w, part, le, ex_s);
+                apply_off_pair<L, Q, double2, SPLIT>(D0, cfd, fb, z, w, part, le, ex_s, exo);
                 float rf[LS], e[LS];
 #pragma unroll
                 for (int l = 0; l < LS; ++l) {
@@ -486,7 +511,7 @@ __global__ void __launch_bounds__(SPLIT > 1 ? MAX_QUAD_TILE_THREADS : MAX_PAIR_T
                     if (act) store_part<LS, float2>(Fb, fb.xo + le, part, e);
                     tile_sync();
                     float wf[LS], wfo[LS];
-                    apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, e, wf, part, le, ex_s);
+                    apply_off_pair<L, Q, float2, SPLIT>(Fb, cff, fb, e, wf, part, le, ex_s, exo);
 #pragma unroll
                     for (int l = 0; l < LS; ++l) wfo[l] = partner(wf[l]);
                     if (it < j2) {
