@@ -64,7 +64,15 @@ static cudaError_t launch_one(const SweepArgs& a, int ntiles, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     if (ntiles <= 0) return cudaSuccess;
-    return launch_carved(FAM == 3 ? cudaSharedmemCarveoutDefault : cudaSharedmemCarveoutMaxShared, kern,
+    // Blocks placed while the kernel before still runs go where it leaves room.  That costs nothing where
+    // the tiles fill the GPU or a tile is an SM's, but a few one-warp tiles an SM gather on some SMs and
+    // share a sub-partition there: QFT-16 with the FP64 solver (1024 tiles, up to 20 an SM) 14.9 ms an
+    // objective in place of 9.0, at 256 windows with the mixed one 3.21 ms a gradient in place of 2.95.
+    // Slices (SWEEP_PROP, SWEEP_BOTH) are too short and too many for it, and gain the overlap; the lane
+    // families have no part ahead of chain_wait() and lose nothing by a plain launch.
+    const bool chained = (FAM == 0 || FAM == 3) &&
+                         (a.nthreads > 32 || a.mode == SWEEP_PROP || a.mode == SWEEP_BOTH || a.mode == SWEEP_RECOMPUTE);
+    return launch_carved(chained, FAM == 3 ? cudaSharedmemCarveoutDefault : cudaSharedmemCarveoutMaxShared, kern,
                          BOTH ? 2 * ntiles : ntiles, a.nthreads, smem, s, a);
 }
 

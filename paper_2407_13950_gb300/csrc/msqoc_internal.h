@@ -174,8 +174,9 @@ struct SweepArgs {
 // under one split, so every kernel asks for the same (the largest): QFT-4's gradient 104 -> 91 us,
 // QFT-8's 304 -> 266.  The lean sweeps leave it to the driver, since their spilled registers want the
 // L1 (QFT-16 at 64 windows 3.84 -> 4.00 ms with all of it shared).
+// chained: false for a plain launch, whose blocks are placed when the kernel before has ended.
 template <class... P, class... A>
-cudaError_t launch_carved(int carveout, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+cudaError_t launch_carved(bool chained, int carveout, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
                           A... args) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
@@ -188,7 +189,7 @@ cudaError_t launch_carved(int carveout, void (*kern)(P...), dim3 grid, int threa
         at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
         at[n++].val.sharedMemCarveout = static_cast<unsigned>(carveout);
     }
-    if (cap == cudaStreamCaptureStatusNone) {
+    if (chained && cap == cudaStreamCaptureStatusNone) {
         at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[n++].val.programmaticStreamSerializationAllowed = 1;
     }
@@ -205,7 +206,7 @@ cudaError_t launch_carved(int carveout, void (*kern)(P...), dim3 grid, int threa
 }
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
-    return launch_carved(cudaSharedmemCarveoutMaxShared, kern, grid, threads, smem, s, args...);
+    return launch_carved(true, cudaSharedmemCarveoutMaxShared, kern, grid, threads, smem, s, args...);
 }
 
 // shared-memory bytes of a sweep launch
