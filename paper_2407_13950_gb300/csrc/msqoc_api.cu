@@ -567,6 +567,11 @@ bool history_depth_ok(const ProbDev& pd, int depth) {
 // 16 steps).  1 GiB holds a whole segment of every workload but the largest, whose launches last
 // milliseconds a chunk.
 constexpr size_t ADJ_CHUNK_BYTES = size_t(1) << 30;
+constexpr int ADJ_CHUNK_STEPS = 16;
+void set_chunks(ProbDev& pd, int nsub) {
+    pd.nsub = nsub;
+    pd.kadj = (pd.kseg + nsub - 1) / nsub;
+}
 
 // history segmentation for a checkpoint interval K (1 = keep every midpoint state); slices come
 // with K = 1 only
@@ -575,9 +580,8 @@ void set_segments(ProbDev& pd, int K) {
     pd.kseg = (K <= 1 || K >= max_ns) ? static_cast<int>(max_ns) : K;
     pd.nseg = static_cast<int>((max_ns + pd.kseg - 1) / pd.kseg);
     const size_t step = size_t(pd.M) * pd.C * pd.N * pd.E * sizeof(double2);
-    const int64_t most = std::max<int64_t>(16, static_cast<int64_t>(ADJ_CHUNK_BYTES / step));
-    pd.nsub = static_cast<int>((pd.kseg + most - 1) / most);
-    pd.kadj = (pd.kseg + pd.nsub - 1) / pd.nsub;
+    const int64_t most = std::max<int64_t>(ADJ_CHUNK_STEPS, static_cast<int64_t>(ADJ_CHUNK_BYTES / step));
+    set_chunks(pd, static_cast<int>((pd.kseg + most - 1) / most));
 }
 
 // sweep launch arguments of a single problem
@@ -1006,11 +1010,23 @@ msqoc_status ensure_gradient_buffers(msqoc_problem* p, cudaStream_t s) {
     ProbDev& pd = p->pd;
     const size_t M = pd.M, V = M * pd.C;
     cudaError_t e = dalloc(&p->hist, V * pd.kseg * p->ne + hist_scale_blocks(pd));
-    if (e == cudaSuccess) e = dalloc(&p->lhist, V * pd.kadj * p->ne + adj_scale_blocks(pd));
     if (e == cudaSuccess && pd.C > 1) e = dalloc(&p->Lend, V * p->ne);
     if (e == cudaSuccess) e = dalloc(&p->quad, size_t(pd.q) * pd.nsteps);
     if (e == cudaSuccess && pd.nseg > 1) e = dalloc(&p->ckpt, M * pd.nseg * p->ne);
-    if (e == cudaSuccess && pd.nseg * pd.nsub > 1) e = dalloc(&p->Lstate, V * p->ne);
+    while (e == cudaSuccess) {
+        e = dalloc(&p->lhist, V * pd.kadj * p->ne + adj_scale_blocks(pd));
+        if (e == cudaSuccess && pd.nseg * pd.nsub > 1) e = dalloc(&p->Lstate, V * p->ne);
+        if (e != cudaErrorMemoryAllocation || pd.kadj < 2 * ADJ_CHUNK_STEPS) break;
+        // a chunk that does not fit: smaller ones, in more launches (the adjoint's states are kept
+        // between two kernels only; a history that leaves no room for 1 GiB of them still runs)
+        cudaGetLastError();
+        if (p->lhist) cudaFree(p->lhist);
+        p->lhist = nullptr;
+        set_chunks(pd, 2 * pd.nsub);
+        p->both = SweepPlan{};   // (its launches take a segment at once)
+        p->grad_bytes = gradient_bytes(pd);
+        e = cudaSuccess;
+    }
     if (e != cudaSuccess) {
         for (double2** b : {&p->hist, &p->lhist, &p->Lend, &p->quad, &p->ckpt, &p->Lstate}) {
             if (*b) cudaFree(*b);
