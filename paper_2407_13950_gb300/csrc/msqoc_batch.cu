@@ -142,12 +142,29 @@ bool both_sweeps(const msqoc_batch::Group& g, long n) {
     auto waves = [&](long t) { return (t + g.slots - 1) / g.slots; };
     return g.pthreads || (g.nseg_max > 1 && waves(2 * n) < 2 * waves(n));
 }
+// fn(pds, list, n) for the n members of a launch whose rows are problems, in parts of what a grid's y and z
+// dimensions hold
+template <class Fn>
+cudaError_t in_rows(const ProbDev* pds, const int* list, int n, Fn fn) {
+    constexpr int most = 65535;
+    for (int i = 0; i < n; i += most) {
+        const cudaError_t e = fn(list ? pds : pds + i, list ? list + i : nullptr, std::min(n - i, most));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
 // The launch sequence of one batched evaluation of the problems `sel`; work[g]: the part of group g;
 // set: the stream set of the groups.
 msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, const std::vector<GroupWork>& work,
                      bool grad, int set, cudaStream_t s) {
     std::vector<int> ntiles;
     for (const GroupWork& w : work) ntiles.push_back(w.ntiles);
+    auto compose = [&](int gi, bool bwd, cudaStream_t gs) {
+        const auto& g = b->groups[gi];
+        return in_rows(g.pds, work[gi].list, work[gi].nlist, [&](const ProbDev* pds, const int* list, int n) {
+            return launch_compose(pds, list, g.E_max, g.M_max, n, ipow(g.L, g.q), bwd, gs);
+        });
+    };
     msqoc_status st;
     for (msqoc_problem* p : sel)
         if ((st = launch_controls(p, p->pd.pair, s))) return st;
@@ -158,7 +175,7 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, con
             pa.tiles = work[gi].ptiles;
             cudaError_t e = launch_sweep(pa, work[gi].nptiles, gs);
             if (e == cudaSuccess)
-                e = launch_compose(g.pds, work[gi].list, g.E_max, g.M_max, work[gi].nlist, ipow(g.L, g.q), false, gs);
+                e = compose(gi, false, gs);
             if (e != cudaSuccess) return e;
         }
         if (g.pthreads && (!grad || g.nsub_max == 1)) return cudaSuccess;   // (history: with the adjoint)
@@ -181,8 +198,7 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, con
     st = for_groups(b, ntiles.data(), set, s, [&](int gi, cudaStream_t gs) {
         const auto& g = b->groups[gi];
         if (g.pthreads) {
-            const cudaError_t e =
-                launch_compose(g.pds, work[gi].list, g.E_max, g.M_max, work[gi].nlist, ipow(g.L, g.q), true, gs);
+            const cudaError_t e = compose(gi, true, gs);
             if (e != cudaSuccess) return e;
         }
         const bool both = both_sweeps(g, work[gi].ntiles);
@@ -201,8 +217,11 @@ msqoc_status enqueue(msqoc_batch* b, const std::vector<msqoc_problem*>& sel, con
                 cudaError_t e = launch_sweep(a, work[gi].ntiles, gs);
                 if (e != cudaSuccess) return e;
                 QuadArgs qa = quad_args(b->probs[g.members[0]]->pd, g.pds, seg, sub);
-                qa.list = work[gi].list;
-                e = launch_quad(qa, g.quad_blocks, work[gi].nlist, gs);
+                e = in_rows(g.pds, work[gi].list, work[gi].nlist, [&](const ProbDev* pds, const int* list, int n) {
+                    qa.pds = pds;
+                    qa.list = list;
+                    return launch_quad(qa, g.quad_blocks, n, gs);
+                });
                 if (e != cudaSuccess) return e;
             }
         }
