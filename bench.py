@@ -140,13 +140,16 @@ def sweep_traffic(kernel: str, windows: int, col_block: int, layout: int):
 
 def launches_per_evaluation(spec, tiles: int, col_block: int) -> int:
     """Kernel launches of one gradient evaluation with every midpoint state kept.  Sliced windows:
-    controls, propagators, chain, terminal conditions, chain, both sweeps, quadrature, outputs.
-    Otherwise controls, forward sweep, terminal conditions, outputs, and an adjoint sweep and a
-    quadrature for each chunk of adjoint states (1 GiB at most, 16 steps at least)."""
+    controls, propagators, chain, terminal conditions, chain, outputs, and both sweeps and a
+    quadrature, or where the adjoint states take several chunks (1 GiB at most, 16 steps at least) a
+    forward sweep, and an adjoint sweep and a quadrature a chunk.  Otherwise controls, forward sweep,
+    terminal conditions, outputs, and an adjoint sweep and a quadrature a chunk."""
+    slices = max(1, tiles * col_block // (spec.M * spec.E))
+    chunk = max(16, (1 << 30) // (spec.M * slices * spec.N * spec.E * 16))
+    chunks = -(-(-(-(-(-spec.nsteps // spec.M)) // slices)) // chunk)
     if tiles * col_block > spec.M * spec.E + col_block:
-        return 8
-    chunk = max(16, (1 << 30) // (spec.M * spec.N * spec.E * 16))
-    return 4 + 2 * (-(-(-(-spec.nsteps // spec.M)) // chunk))
+        return 8 if chunks == 1 else 7 + 2 * chunks
+    return 4 + 2 * chunks
 
 
 def max_over_ranks(value: float, dist, device) -> float:

@@ -331,6 +331,20 @@ msqoc_status msqoc_selftest_dot(const double* x, const double* y, int64_t n, int
 msqoc_status msqoc_selftest_carry(const double* u0, const double* P, const double* d, int64_t n, int32_t sh,
                                   int32_t on_device, double* out);
 
+/* Self-test of the arithmetic of the mixed solver's state, held as the exact sum of three floats a + b + c:
+ * out[3 i ..] = the three floats of one operation on x_i and y_i (each split exactly where its parts are
+ * normal floats): SPLIT x itself, ROUND x rounded to a double, ADD x + y for |y| <= |x| from y's two leading
+ * floats, ADD3 and SUM x + y, MUL x y, KAPPA x y from y's two leading floats, as two floats. */
+#define MSQOC_TRIPLE_SPLIT 0
+#define MSQOC_TRIPLE_ADD 1
+#define MSQOC_TRIPLE_ADD3 2
+#define MSQOC_TRIPLE_MUL 3
+#define MSQOC_TRIPLE_SUM 4
+#define MSQOC_TRIPLE_KAPPA 5
+#define MSQOC_TRIPLE_ROUND 6
+msqoc_status msqoc_selftest_triple(int32_t op, const double* x, const double* y, int64_t n, int32_t on_device,
+                                   float* out);
+
 /* Self-test of the iteration counts of one step (on the host): solver (MSQOC_SOLVER_FP64 or _MIXED), pair
  * (0: one thread per fiber, else a lane family), the contraction bound rho, the largest rotation kap = h
  * max|D| / 2, and drho, the bound's part that the controls changed over the step before.

@@ -172,8 +172,7 @@ struct SweepArgs {
 // 387 -> 323.  Captured launches are plain ones (a graph has its own edges).
 // carveout: percent of an SM's L1 kept as shared memory (not positive: the driver's choice).  Blocks of two kernels share an SM only
 // under one split, so every kernel asks for the same (the largest): QFT-4's gradient 104 -> 91 us,
-// QFT-8's 304 -> 266.  The lean sweeps leave it to the driver, since their spilled registers want the
-// L1 (QFT-16 at 64 windows 3.84 -> 4.00 ms with all of it shared).
+// QFT-8's 304 -> 266.  The lean sweeps leave it to the driver (LEANCARVE).
 // chained: false for a plain launch, whose blocks are placed when the kernel before has ended.
 template <class... P, class... A>
 cudaError_t launch_carved(bool chained, int carveout, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,

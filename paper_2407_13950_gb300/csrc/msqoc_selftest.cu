@@ -4,8 +4,8 @@
 //    hanging the GPU.  The context stays usable afterwards.
 //  * the compensated FP32 arithmetic of the mixed solver (msqoc_split.cuh), on the host or in a
 //    one-thread kernel: the split of doubles into two floats, a real dot product formed the way
-//    the gradient products are, and steps of the state update with an FP32 carry (the form of the
-//    update on an FP64 state, which the exported self-test defines).
+//    the gradient products are, the three-float arithmetic of the state, and steps of a state update
+//    with an FP32 carry (the form the solver had on an FP64 state, which the exported self-test defines).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -52,6 +52,33 @@ __host__ __device__ double dot_split(const double* x, const double* y, int64_t n
 
 __global__ void k_dot_probe(const double* x, const double* y, int64_t n, int shx, int shy, double* out) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *out = dot_split(x, y, n, shx, shy);
+}
+
+// One operation of the state's three-float arithmetic on two doubles, its result as three floats
+// (MSQOC_TRIPLE_* names them)
+__host__ __device__ TF triple_op(int op, double x, double y) {
+    TF a = tf_split(x, 0);
+    const TF b = tf_split(y, 0);
+    switch (op) {
+        case MSQOC_TRIPLE_ADD: tf_add(a, b.a, b.b); return a;
+        case MSQOC_TRIPLE_ADD3: tf_add3(a, b.a, b.b, b.c); return a;
+        case MSQOC_TRIPLE_MUL: return tf_mul(a, b);
+        case MSQOC_TRIPLE_SUM: return tf_sum(a, b);
+        case MSQOC_TRIPLE_KAPPA: {
+            const DF p = kappa_mul(a.a, a.b, a.c, b.a, b.b);
+            return TF{p.s, p.c, 0.f};
+        }
+        case MSQOC_TRIPLE_ROUND: return tf_split(tf_to_f64(a, 0), 0);
+        default: return a;   // MSQOC_TRIPLE_SPLIT
+    }
+}
+__global__ void k_triple_probe(int op, const double* x, const double* y, int64_t n, float* out) {
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+        const TF t = triple_op(op, x[i], y[i]);
+        out[3 * i] = t.a;
+        out[3 * i + 1] = t.b;
+        out[3 * i + 2] = t.c;
+    }
 }
 
 // ------------------------------------------------------------------ the compensated state update
@@ -269,5 +296,37 @@ extern "C" msqoc_status msqoc_selftest_step_counts(int32_t solver, int32_t pair,
     out[1] = (c >> 8) & 0xff;
     out[2] = (c >> 16) & 0xff;
     out[3] = (c >> 24) & 0xff;
+    return MSQOC_OK;
+}
+
+extern "C" msqoc_status msqoc_selftest_triple(int32_t op, const double* x, const double* y, int64_t n,
+                                              int32_t on_device, float* out) {
+    if (n < 0 || (n > 0 && (!x || !y || !out))) return fail(MSQOC_ERR_INVALID_ARG, "triple self-test: bad arrays");
+    if (op < MSQOC_TRIPLE_SPLIT || op > MSQOC_TRIPLE_ROUND)
+        return fail(MSQOC_ERR_INVALID_ARG, "triple self-test: unknown operation %d", op);
+    if (!on_device) {
+        for (int64_t i = 0; i < n; ++i) {
+            const TF t = triple_op(op, x[i], y[i]);
+            out[3 * i] = t.a;
+            out[3 * i + 1] = t.b;
+            out[3 * i + 2] = t.c;
+        }
+        return MSQOC_OK;
+    }
+    if (n == 0) return MSQOC_OK;
+    DevBufs d;
+    double *xd = nullptr, *yd = nullptr;
+    float* od = nullptr;
+    cudaError_t e = d.alloc(&xd, n);
+    if (e == cudaSuccess) e = d.alloc(&yd, n);
+    if (e == cudaSuccess) e = d.alloc(&od, 3 * n);
+    if (e == cudaSuccess) e = cudaMemcpy(xd, x, n * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(yd, y, n * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        k_triple_probe<<<static_cast<int>(std::min<int64_t>((n + 255) / 256, 1024)), 256>>>(op, xd, yd, n, od);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(out, od, 3 * n * sizeof(float), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return fail(MSQOC_ERR_CUDA, "triple self-test: %s", cudaGetErrorString(e));
     return MSQOC_OK;
 }

@@ -1,8 +1,9 @@
 // Double values as unevaluated sums of two or three floats, and compensated FP32 arithmetic on
 // them: the mixed solver holds its state, forms the midpoint increment and the gradient products of
-// Eq. grad-int with these instead of FP64 multiply-adds.  On this GPU a warp's FP64 instruction occupies the issuing warp for ~60 cycles
-// and the SM retires ~2 FP64 lanes a cycle, against 128 FP32 lanes.  Every function here runs on
-// the host too (the CPU tests pin them);
+// Eq. grad-int with these instead of FP64 multiply-adds.  On this GPU a warp's FP64 instruction occupies
+// the issuing warp for ~60 cycles and the SM retires ~2 FP64 lanes a cycle, against 128 FP32 lanes.
+// Every function here runs on the host too, where self-tests pin the split, the accumulation and the
+// three-float arithmetic of the state (tests/test_split_cpu.py, tests/test_triple.py);
 // the host side must be compiled without floating-point contraction (-ffp-contract=off), the
 // device side uses the _rn intrinsics, which the compiler never fuses.
 #pragma once

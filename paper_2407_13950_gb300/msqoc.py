@@ -30,7 +30,7 @@ EXPORTED = ["msqoc_create_problem", "msqoc_query", "msqoc_query_layout", "msqoc_
             "msqoc_rollout", "msqoc_rollout_estimate", "msqoc_eval_regularization", "msqoc_lbfgs_direction",
             "msqoc_lbfgs_trial", "msqoc_lbfgs_update", "msqoc_selftest_bounded_wait",
             "msqoc_selftest_split", "msqoc_selftest_dot", "msqoc_selftest_carry",
-            "msqoc_selftest_step_counts"]
+            "msqoc_selftest_step_counts", "msqoc_selftest_triple"]
 BATCH_GRADIENT, BATCH_GRAPH = 1, 2
 KERNEL_NAMES = ["controls", "forward", "terminal", "adjoint", "finalize"]
 
@@ -91,6 +91,7 @@ def load(build_if_missing: bool = True):
             "msqoc_selftest_split": (i32, [vp, i64, i32, i32, vp, vp]),
             "msqoc_selftest_dot": (i32, [vp, vp, i64, i32, i32, i32, vp]),
             "msqoc_selftest_carry": (i32, [vp, vp, vp, i64, i32, i32, vp]),
+            "msqoc_selftest_triple": (i32, [i32, vp, vp, i64, i32, vp]),
             "msqoc_selftest_step_counts": (i32, [i32, i32, ctypes.c_float, ctypes.c_float, ctypes.c_float, vp]),
             "msqoc_eval_objective_noalloc": (i32, [vp, vp, vp, ctypes.c_double, i64, i32, ctypes.c_double, i32,
                                                    vp, vp, vp, vp, vp, vp]),
@@ -357,6 +358,21 @@ def selftest_dot(x, y, shx: int = 0, shy: int = 0, device: bool = False) -> floa
     _check(load().msqoc_selftest_dot(x.ctypes.data, y.ctypes.data, x.size, int(shx), int(shy), 1 if device else 0,
                                      ctypes.byref(out)))
     return out.value
+
+
+TRIPLE_OPS = ("split", "add", "add3", "mul", "sum", "kappa", "round")   # MSQOC_TRIPLE_*
+
+
+def selftest_triple(op: str, x, y, device: bool = False) -> np.ndarray:
+    """The three floats [n][3] of an operation of the state's arithmetic (msqoc_selftest_triple)."""
+    x = np.ascontiguousarray(x, dtype=np.float64)
+    y = np.ascontiguousarray(y, dtype=np.float64)
+    if x.shape != y.shape:
+        raise ValueError("x and y differ in shape")
+    out = np.zeros((x.size, 3), dtype=np.float32)
+    _check(load().msqoc_selftest_triple(TRIPLE_OPS.index(op), x.ctypes.data, y.ctypes.data, x.size, 1 if device else 0,
+                                        out.ctypes.data))
+    return out
 
 
 def selftest_step_counts(solver: int, pair: int, rho: float, kap: float, drho: float) -> tuple:

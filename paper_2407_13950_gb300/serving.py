@@ -124,7 +124,13 @@ def session_tiles(spec) -> dict:
     alone).  An evaluation that takes milliseconds and does not fill the GPU gets the tiles with
     the most columns per SM and time instead, so that the other sessions' launches run beside it:
     4 transmons at 16 windows take 19 tiles of 14 columns at 6.0 us a step (2.3 columns a
-    microsecond and SM) against 64 tiles of 4 columns at 3.4 us (1.2)."""
+    microsecond and SM) against 64 tiles of 4 columns at 3.4 us (1.2).  16 sessions each of 2 to 5
+    transmons, 10 s of requests beyond capacity: 1081 completions with it against 1040 without in
+    arrival order (1.473 and 1.465 TFLOP/s), 1.51 against 1.42 TFLOP/s for throughput (4
+    transmons 488 against 401 requests); below capacity a 4-transmon request takes 8.5 ms against
+    6.4.  Lane pairs for the small sessions (fewer launches, no propagators) complete more of them in
+    arrival order (2 and 3 transmons 618 and 635 against 397 and 457) but fewer for throughput (1992
+    and 1988 against 2430 and 2386), and take 3 to 5 ms below capacity where slices take 0.5 to 1.4."""
     F = spec.N // spec.L
     cb = min(spec.E, 384 // F)
     if eval_flops(spec, True) < 1e9 or spec.M * spec.E >= 128 * cb:
