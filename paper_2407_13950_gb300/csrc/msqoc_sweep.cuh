@@ -294,6 +294,7 @@ static __device__ __noinline__ void coarse_step(CoarseIO<L, Q>& io, const ProbDe
     double2* D0 = reinterpret_cast<double2*>(smem + lay.D0);
     float2* FA = reinterpret_cast<float2*>(smem + lay.FA);
     float2* FB = reinterpret_cast<float2*>(smem + lay.FB);
+    float2* DP = reinterpret_cast<float2*>(smem + lay.DP);
     if (!io.have_g) {
         io.have_g = true;
 #pragma unroll
@@ -402,8 +403,13 @@ static __device__ __noinline__ void coarse_step(CoarseIO<L, Q>& io, const ProbDe
 #pragma unroll
             for (int l = 0; l < L; ++l) y[l] = make_float2(pu[l][0].a + d[l][0].a, pu[l][1].a + d[l][1].a);
         }
+        // (DP for a common step after this one: a window's results do not depend on what shares its
+        // tile, and beside a common step of the other slot this slot's DP holds nothing)
 #pragma unroll
-        for (int l = 0; l < L; ++l) io.d[l] = make_float2(d[l][0].a, d[l][1].a);
+        for (int l = 0; l < L; ++l) {
+            io.d[l] = make_float2(d[l][0].a, d[l][1].a);
+            if (act && mine) DP[fb.xo + l] = io.d[l];
+        }
     }
     // ---- passes in compensated FP32: d = s P w(z), z = P U + d in two floats
     float4* D0s = reinterpret_cast<float4*>(D0);
@@ -980,8 +986,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int mode, c
             } else if (want_hist && tid == 0 && hpos == 0) {
                 bulk_wait_read_all();   // (the coarse step's barriers follow)
             }
-            fresh = coarse0 || coarse1;
-            if (fresh) {
+            fresh = false;
+            if (coarse0 || coarse1) {
                 if (!io.have_g) {   // (what does not change goes once)
                     io.fb = fb;
 #pragma unroll
