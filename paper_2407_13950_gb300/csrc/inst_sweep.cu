@@ -72,8 +72,7 @@ static cudaError_t launch_one(const SweepArgs& a, int ntiles, cudaStream_t s) {
     // families have no part ahead of chain_wait() and lose nothing by a plain launch.
     const bool chained = (FAM == 0 || FAM == 3) &&
                          (a.nthreads > 32 || a.mode == SWEEP_PROP || a.mode == SWEEP_BOTH || a.mode == SWEEP_RECOMPUTE);
-    return launch_carved(chained, FAM == 3 ? cudaSharedmemCarveoutDefault : cudaSharedmemCarveoutMaxShared, kern,
-                         BOTH ? 2 * ntiles : ntiles, a.nthreads, smem, s, a);
+    return launch_split(chained, kern, BOTH ? 2 * ntiles : ntiles, a.nthreads, smem, s, a);
 }
 
 template <int SOLVER, bool BWD, int FAM>

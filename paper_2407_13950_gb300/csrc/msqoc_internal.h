@@ -170,12 +170,11 @@ struct SweepArgs {
 // copies ahead of the first kernel left out (take_inputs), QFT-4's gradient of eight dependent
 // launches 116 -> 104 us, QFT-8's 372 -> 347, three transmons' 1060 -> 992, QFT-8's roll-out
 // 387 -> 323.  Captured launches are plain ones (a graph has its own edges).
-// carveout: percent of an SM's L1 kept as shared memory (not positive: the driver's choice).  Blocks of two kernels share an SM only
-// under one split, so every kernel asks for the same (the largest): QFT-4's gradient 104 -> 91 us,
-// QFT-8's 304 -> 266.  The lean sweeps leave it to the driver (LEANCARVE).
+// Blocks of two kernels share an SM only under one split of its L1, so every kernel asks for the most
+// shared memory: QFT-4's gradient 104 -> 91 us, QFT-8's 304 -> 266.
 // chained: false for a plain launch, whose blocks are placed when the kernel before has ended.
 template <class... P, class... A>
-cudaError_t launch_carved(bool chained, int carveout, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+cudaError_t launch_split(bool chained, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
                           A... args) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
@@ -184,10 +183,8 @@ cudaError_t launch_carved(bool chained, int carveout, void (*kern)(P...), dim3 g
     }
     cudaLaunchAttribute at[2] = {};
     int n = 0;
-    if (carveout > 0) {
-        at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-        at[n++].val.sharedMemCarveout = static_cast<unsigned>(carveout);
-    }
+    at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
     if (chained && cap == cudaStreamCaptureStatusNone) {
         at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[n++].val.programmaticStreamSerializationAllowed = 1;
@@ -205,7 +202,7 @@ cudaError_t launch_carved(bool chained, int carveout, void (*kern)(P...), dim3 g
 }
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
-    return launch_carved(true, cudaSharedmemCarveoutMaxShared, kern, grid, threads, smem, s, args...);
+    return launch_split(true, kern, grid, threads, smem, s, args...);
 }
 
 // shared-memory bytes of a sweep launch

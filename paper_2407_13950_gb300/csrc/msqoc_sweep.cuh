@@ -27,9 +27,9 @@
 // Both sweeps store the midpoint states, from which msqoc_quad.cuh forms the gradient products.
 //
 // What bounds the mixed step: instruction issue and the dependency latency inside its 4-5 barrier-
-// separated phases (no pipe is saturated).  4 transmons, 100000 steps at 256 windows on one GB300:
-// a forward sweep 5.22 -> 3.85 ms against the form with an FP64 state, an FP32 carry and two more
-// sweeps a step; at 64 windows 6.97 -> 4.98 ms.
+// separated phases (no pipe is saturated).  4 transmons, 100000 steps at 256 windows on one GB300: an
+// objective 4.86 -> 3.60 ms against the form with an FP64 state, an FP32 carry and two more sweeps a
+// step; at 64 windows 6.97 -> 4.77 ms.
 #pragma once
 
 #include <climits>
@@ -1095,15 +1095,8 @@ __global__ void __launch_bounds__(budget_threads<L, MAXT>(), 1) k_sweep_both(con
     const int mode = bwd ? SWEEP_ADJOINT : a.pds[a.tiles[block].prob].C > 1 ? SWEEP_HISTORY : SWEEP_RECOMPUTE;
     // One body for both, half the instructions to fetch: with two, 28% of QFT-4's 36 us went to fetches
     // (27 us with one; two transmons from the host 248 -> 232 us, 5 transmons checkpointed 39.6 -> 38.9
-    // ms).  The lean 2-level sweeps spill more registers in one body (QFT-16 3.84 -> 3.89 ms).
-    if constexpr (L == 2 && MAXT == MAX_LEAN_TILE_THREADS) {
-        if (bwd)
-            sweep_tile<L, Q, SOLVER_MIXED, false>(a, SWEEP_ADJOINT, block, true);
-        else
-            sweep_tile<L, Q, SOLVER_MIXED, false>(a, mode, block, false);
-    } else {
-        sweep_tile<L, Q, SOLVER_MIXED, false>(a, mode, block, bwd);
-    }
+    // ms).
+    sweep_tile<L, Q, SOLVER_MIXED, false>(a, mode, block, bwd);
 }
 
 }  // namespace msqoc
