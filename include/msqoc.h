@@ -76,8 +76,9 @@ typedef int32_t msqoc_status;
  *         round-off; the step is solved to FP64 round-off.  With one thread per fiber the
  *         state is the exact sum of three floats and the step's increment is formed in
  *         compensated FP32 (coarse steps, contraction factor above 2^-5 or diagonal step
- *         |kappa| = h |D| / 2 above 2^-4, in FP64); the lane families form it in FP64.
- *         Default.
+ *         |kappa| = h |D| / 2 above 2^-4, keep the rotation apart in three floats and take their last
+ *         pass in FP64 where the contraction factor is); the lane families form it in FP64.
+ *         Inputs that are not finite give NaN.  Default.
  *  FP64 : diagonal-preconditioned fixed-point iteration carried out entirely in FP64. */
 #define MSQOC_SOLVER_DEFAULT 0
 #define MSQOC_SOLVER_FP64 1
